@@ -9,12 +9,14 @@ import glob
 import os
 import subprocess
 import sys
+from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libbwla.so")
 INCLUDE = os.path.join(_ROOT, "include")
+OBJ = os.path.join(_HERE, "_build")        # one object per source: an edit recompiles what it touched
 
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
               "-Xcompiler", "-fPIC", "-shared", "--use_fast_math=false"]
@@ -32,6 +34,10 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _newer(path: str, deps) -> bool:
+    return os.path.exists(path) and all(os.path.getmtime(d) <= os.path.getmtime(path) for d in deps)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return LIB
@@ -39,12 +45,25 @@ def build(force: bool = False, verbose: bool = False) -> str:
     flags = [f for f in NVCC_FLAGS if not f.startswith("--use_fast_math")]
     if verbose:
         flags += ["-Xptxas", "-v"]
-    cmd = [nvcc] + flags + ["-I", INCLUDE, "-I", CSRC, "-o", LIB] + sources() + ["-lcudart"]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if verbose or res.returncode != 0:
-        sys.stderr.write(res.stdout + res.stderr)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed building libbwla.so")
+    os.makedirs(OBJ, exist_ok=True)
+    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+
+    def run(cmd):
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if verbose or res.returncode != 0:
+            sys.stderr.write(res.stdout + res.stderr)
+        if res.returncode != 0:
+            raise RuntimeError("nvcc failed building libbwla.so")
+
+    def compile_one(src):
+        obj = os.path.join(OBJ, os.path.basename(src) + ".o")
+        if force or not _newer(obj, [src] + headers):
+            run([nvcc] + [f for f in flags if f != "-shared"] + ["-I", INCLUDE, "-I", CSRC, "-c", "-o", obj, src])
+        return obj
+
+    with ThreadPoolExecutor(max(2, os.cpu_count() or 2)) as pool:
+        objects = list(pool.map(compile_one, sources()))
+    run([nvcc] + flags + ["-o", LIB] + objects + ["-lcudart"])
     return LIB
 
 
