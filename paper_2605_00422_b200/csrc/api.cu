@@ -92,8 +92,8 @@ struct bwla_layer {
     const uint32_t* packed;
     const void *U, *V;
     uint8_t* prepared;
-    bool okt;                 // the tcgen05 rotation takes these factor sizes
-    OktGeom geom;
+    bool rot;                 // the tensor-core rotation takes these factor sizes
+    RotGeom geom;
     int asym;                 // activation quantiser: 0 symmetric, 1 asymmetric (per-token zero point)
     int32_t* rowsum;          // [N] sign sums of the rows, inside `prepared`
 };
@@ -113,7 +113,7 @@ int bwla_pack_signs(const void* w, int dtype, int64_t N, int64_t K, int64_t ldw,
 
 size_t bwla_binarize_workspace_bytes(int64_t K) {
     if (K <= 0 || K % 32 != 0 || K > 25600) return 0;
-    return binarize_workspace_bytes(K);
+    return kStatusBytes;
 }
 
 int bwla_binarize_rows(const void* w_res, int dtype, int64_t N, int64_t K, int64_t ldw, const float* P1, int n1,
@@ -128,7 +128,11 @@ int bwla_binarize_rows(const void* w_res, int dtype, int64_t N, int64_t K, int64
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < bwla_binarize_workspace_bytes(K)) return BWLA_ERR_WORKSPACE;
     int st = check_device();
     if (st != BWLA_OK) return st;
-    return launch_binarize(w_res, dtype, N, K, ldw, P1, n1, P2, n2, packed, alpha, mu, workspace, (cudaStream_t)stream);
+    RotGeom geom;
+    if (!rot_geometry(n1, n2, &geom)) return BWLA_ERR_UNSUPPORTED;
+    RotProblem pr{};
+    pr.P1 = P1; pr.P2 = P2; pr.packed = packed; pr.alpha = alpha; pr.mu = mu;
+    return launch_rot_binarize(geom, w_res, dtype, N, ldw, pr, (uint32_t*)workspace, (cudaStream_t)stream);
 }
 
 int bwla_rotate_quant_act(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, const float* P1, int n1,
@@ -140,6 +144,12 @@ int bwla_rotate_quant_act(const void* x_bf16, int64_t M, int64_t K, int64_t ldx,
     if (((uintptr_t)codes & 15) || ((uintptr_t)P1 & 15) || ((uintptr_t)P2 & 15)) return BWLA_ERR_INVALID_ARG;
     int st = check_device();
     if (st != BWLA_OK) return st;
+    RotGeom geom;
+    if (g_forced_rotation != BWLA_ROT_SIMT && rot_geometry(n1, n2, &geom)) {
+        RotProblem pr{};
+        pr.P1 = P1; pr.P2 = P2; pr.codes = codes; pr.scales = scales;
+        return launch_rot(geom, x_bf16, M, ldx, bits, 0, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
+    }
     return launch_prologue(x_bf16, M, K, ldx, P1, n1, P2, n2, bits, codes, 0, scales, nullptr, nullptr, 0, nullptr, nullptr, nullptr,
                            (cudaStream_t)stream);
 }
@@ -199,15 +209,14 @@ int bwla_w1ax_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, cons
     int8_t* codes = (int8_t*)(base + ws.codes);
     const int path = resolve_path(M, K, N, r, bits);
 
-    OktGeom geom;
-    if (g_forced_rotation != 1 && okt_geometry(n1, n2, &geom) && okt_accepts_x(x_bf16, ldx) && okt_prepared_bytes(geom) <= kOktPreparedMax) {
-        // the Kronecker factors are handed over raw: their bf16 terms go into the workspace first (a prepared layer
-        // does this once instead)
-        st = launch_prepare_okt(geom, P1, P2, base + ws.prep, s);
-        if (st != BWLA_OK) return st;
-        OktProblem pr{(const uint8_t*)(base + ws.prep), codes, path == BWLA_PATH_I8 ? 1 : 0, nullptr, 0, scales, qsum, nullptr};
+    RotGeom geom;
+    if (g_forced_rotation != BWLA_ROT_SIMT && rot_geometry(n1, n2, &geom)) {
+        // the Kronecker factors are handed over raw: every CTA of the rotation splits what it needs of them (a prepared
+        // layer has that done once)
+        RotProblem pr{};
+        pr.P1 = P1; pr.P2 = P2; pr.codes = codes; pr.codes_layout = path == BWLA_PATH_I8 ? 1 : 0; pr.scales = scales; pr.qsum = qsum;
         OktLowrank lr{V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status) + kLrCounterWord};
-        st = launch_okt(geom, x_bf16, M, ldx, bits, 0, 1, &pr, &lr, (uint32_t*)(base + ws.status), s);
+        st = launch_rot(geom, x_bf16, M, ldx, bits, 0, 1, &pr, &lr, (uint32_t*)(base + ws.status), s);
     } else {
         st = launch_prologue(x_bf16, M, K, ldx, P1, n1, P2, n2, bits, codes, path == BWLA_PATH_I8 ? 1 : 0, scales, qsum,
                              V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status), s);
@@ -273,9 +282,9 @@ int bwla_workspace_section(int64_t M, int64_t K, int64_t N, int r, int bits, int
 
 size_t bwla_layer_prepared_bytes(int64_t K, int64_t N, int n1, int n2, int r) {
     if (!valid_rotation_dims(K, n1, n2) || N < 0 || r < 0 || r > 256) return 0;
-    OktGeom g;
+    RotGeom g;
     // the terms of the Kronecker factors for the tensor-core rotation, then the sign sums of the rows
-    return (okt_geometry(n1, n2, &g) ? align_up(okt_prepared_bytes(g), 256) : 256) + align_up((size_t)N * 4, 256);
+    return (rot_geometry(n1, n2, &g) ? align_up(rot_prepared_bytes(g), 256) : 256) + align_up((size_t)N * 4, 256);
 }
 
 int bwla_layer_create(bwla_layer** layer, int64_t K, int64_t N, const float* P1, int n1, const float* P2, int n2, int bits,
@@ -296,11 +305,11 @@ int bwla_layer_create(bwla_layer** layer, int64_t K, int64_t N, const float* P1,
     L->K = K; L->N = N; L->n1 = n1; L->n2 = n2; L->bits = bits; L->r = r;
     L->P1 = P1; L->P2 = P2; L->packed = packed; L->alpha = alpha; L->mu = mu; L->U = U_bf16; L->V = V_bf16;
     L->prepared = (uint8_t*)prepared;
-    L->okt = okt_geometry(n1, n2, &L->geom);
+    L->rot = rot_geometry(n1, n2, &L->geom);
     L->asym = 0;
-    L->rowsum = (int32_t*)((uint8_t*)prepared + (L->okt ? align_up(okt_prepared_bytes(L->geom), 256) : 256));
-    if (L->okt) {
-        st = launch_prepare_okt(L->geom, P1, P2, prepared, (cudaStream_t)stream);
+    L->rowsum = (int32_t*)((uint8_t*)prepared + (L->rot ? align_up(rot_prepared_bytes(L->geom), 256) : 256));
+    if (L->rot) {
+        st = launch_prepare_rot(L->geom, P1, P2, prepared, (cudaStream_t)stream);
         if (st != BWLA_OK) { free(L); return st; }
     }
     st = launch_row_sums(packed, N, K, L->rowsum, (cudaStream_t)stream);
@@ -313,7 +322,7 @@ void bwla_layer_destroy(bwla_layer* layer) { free(layer); }
 
 int bwla_layer_set_activation_quant(bwla_layer* layer, int mode) {
     if (!layer || (mode != BWLA_ACT_SYMMETRIC && mode != BWLA_ACT_ASYMMETRIC)) return BWLA_ERR_INVALID_ARG;
-    if (mode == BWLA_ACT_ASYMMETRIC && !layer->okt) return BWLA_ERR_UNSUPPORTED;   // only the tensor-core rotation has it
+    if (mode == BWLA_ACT_ASYMMETRIC && !layer->rot) return BWLA_ERR_UNSUPPORTED;   // only the tensor-core rotation has it
     layer->asym = mode;
     return BWLA_OK;
 }
@@ -326,10 +335,11 @@ int bwla_layer_rotate_quant_asym(const bwla_layer* L, const void* x_bf16, int64_
     if (!x_bf16 || !codes || !scales || !zeros || ((uintptr_t)codes & 15)) return BWLA_ERR_INVALID_ARG;
     int st = check_device();
     if (st != BWLA_OK) return st;
-    if (!L->okt || !okt_accepts_x(x_bf16, ldx)) return BWLA_ERR_UNSUPPORTED;
+    if (!L->rot) return BWLA_ERR_UNSUPPORTED;
     // the kernel keeps u - 2^(b-1) so that codes fit int8; the bias puts u and the zero point back in [0, 2^b - 1]
-    OktProblem pr{L->prepared, (int8_t*)codes, 0, zeros, 1 << (L->bits - 1), scales, nullptr, y_f32};
-    return launch_okt(L->geom, x_bf16, M, ldx, L->bits, 1, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
+    RotProblem pr{};
+    pr.prepared = L->prepared; pr.codes = (int8_t*)codes; pr.zp = zeros; pr.code_bias = 1 << (L->bits - 1); pr.scales = scales; pr.y = y_f32;
+    return launch_rot(L->geom, x_bf16, M, ldx, L->bits, 1, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
 int bwla_layer_rotate_quant(const bwla_layer* L, const void* x_bf16, int64_t M, int64_t ldx, int8_t* codes, float* scales,
@@ -340,28 +350,26 @@ int bwla_layer_rotate_quant(const bwla_layer* L, const void* x_bf16, int64_t M, 
     if (!x_bf16 || !codes || !scales || ((uintptr_t)codes & 15)) return BWLA_ERR_INVALID_ARG;
     int st = check_device();
     if (st != BWLA_OK) return st;
-    if (L->okt && g_forced_rotation != BWLA_ROT_SIMT && okt_accepts_x(x_bf16, ldx)) {
-        OktProblem pr{L->prepared, codes, 0, nullptr, 0, scales, nullptr, y_f32};
-        return launch_okt(L->geom, x_bf16, M, ldx, L->bits, 0, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
+    if (L->rot && g_forced_rotation != BWLA_ROT_SIMT) {
+        RotProblem pr{};
+        pr.prepared = L->prepared; pr.codes = codes; pr.scales = scales; pr.y = y_f32;
+        return launch_rot(L->geom, x_bf16, M, ldx, L->bits, 0, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
     }
     if (y_f32) return BWLA_ERR_UNSUPPORTED;      // only the tensor-core kernel can hand out Y
     return launch_prologue(x_bf16, M, L->K, ldx, L->P1, L->n1, L->P2, L->n2, L->bits, codes, 0, scales, nullptr, nullptr, 0,
                            nullptr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
-struct A16Workspace { size_t status, Y, yhat, ysum, codes, scales, T, lr_part, total; };
+struct A16Workspace { size_t status, yhat, ysum, T, lr_part, total; };
 static A16Workspace a16_layout(const bwla_layer* L, int64_t M) {
     A16Workspace w{};
     size_t off = 0;
     w.status = off; off += kStatusBytes;
-    w.Y = off;      off += align_up((size_t)M * (size_t)L->K * 4, 256);
     w.yhat = off;   off += align_up((size_t)M * (size_t)L->K * 2, 256);
     w.ysum = off;   off += align_up((size_t)M * 4, 256);
-    w.codes = off;  off += align_up((size_t)M * (size_t)L->K, 256);
-    w.scales = off; off += align_up((size_t)M * 4, 256);
     const size_t lr_cols = (size_t)lowrank_cols(L->r);
     w.T = off;      off += align_up((size_t)M * lr_cols * 6, 256);
-    w.lr_part = off; off += L->r > 0 ? align_up(std::max((size_t)kLrKSplitMax * 16 * lr_cols * 4, lowrank_umma_part_bytes(M, L->K, L->r)), 256) : 0;
+    w.lr_part = off; off += lowrank_part_bytes(M, L->K, L->r);
     w.total = off;
     return w;
 }
@@ -380,24 +388,22 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < bwla_w1a16_workspace_bytes(L, M)) return BWLA_ERR_WORKSPACE;
     int st = check_device();
     if (st != BWLA_OK) return st;
-    if (!L->okt || !okt_accepts_x(x_bf16, ldx) || !a16_supports(M, L->K, L->N, L->r)) return BWLA_ERR_UNSUPPORTED;
+    if (!L->rot || !a16_supports(M, L->K, L->N, L->r)) return BWLA_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
     const A16Workspace w = a16_layout(L, M);
     char* base = (char*)workspace;
     uint32_t* status = (uint32_t*)(base + w.status);
-    // the rotation hands out Y in fp32 (its int8 codes, quantised at 8 bits, are a by-product nobody reads here)
-    OktProblem pr{L->prepared, (int8_t*)(base + w.codes), 0, nullptr, 0, (float*)(base + w.scales), nullptr, (float*)(base + w.Y)};
+    RotProblem pr{};
+    pr.prepared = L->prepared; pr.yhat = (__nv_bfloat16*)(base + w.yhat); pr.ysum = L->mu ? (float*)(base + w.ysum) : nullptr;
     OktLowrank lr{L->V, L->r, base + w.T, L->r > 0 ? (float*)(base + w.lr_part) : nullptr, status + kLrCounterWord};
-    st = launch_okt(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
+    st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
     if (st != BWLA_OK) return st;
-    st = launch_y_to_bf16((const float*)(base + w.Y), M, L->K, base + w.yhat, (float*)(base + w.ysum), s);
-    if (st != BWLA_OK) return st;
-    return launch_gemm_a16(base + w.yhat, (const float*)(base + w.ysum), M, L->K, L->N, L->packed, L->alpha, L->mu, L->U, L->r,
+    return launch_gemm_a16(base + w.yhat, pr.ysum, M, L->K, L->N, L->packed, L->alpha, L->mu, L->U, L->r,
                            L->r > 0 ? base + w.T : nullptr, out_bf16, ldo, status, s);
 }
 
 static bool valid_group(const bwla_layer* const* layers, int count) {
-    if (!layers || count < 1 || count > kOktMaxProblems) return false;
+    if (!layers || count < 1 || count > kRotMaxProblems) return false;
     for (int i = 0; i < count; ++i) {
         if (!layers[i]) return false;
         if (layers[i]->K != layers[0]->K || layers[i]->n1 != layers[0]->n1 || layers[i]->n2 != layers[0]->n2 ||
@@ -410,7 +416,7 @@ static bool valid_group(const bwla_layer* const* layers, int count) {
 size_t bwla_group_workspace_bytes(const bwla_layer* const* layers, int count, int64_t M) {
     if (!valid_group(layers, count) || M < 0) return 0;
     size_t total = 0;
-    for (int i = 0; i < count; ++i) total += workspace_layout(M, layers[i]->K, layers[i]->N, layers[i]->r, layers[i]->bits, false).total;
+    for (int i = 0; i < count; ++i) total += workspace_layout(M, layers[i]->K, layers[i]->N, layers[i]->r, layers[i]->bits).total;
     return total;
 }
 
@@ -433,31 +439,31 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
     // The status words of the whole call are the first layer's: only those 256 bytes start at zero.  Layer i keeps its
     // arrival counters for split sums of T in words 4 + 8 i .. 11 + 8 i of them.
     uint32_t* status = (uint32_t*)base;
-    Workspace ws[kOktMaxProblems];
-    char* wbase[kOktMaxProblems];
-    int path[kOktMaxProblems];
+    Workspace ws[kRotMaxProblems];
+    char* wbase[kRotMaxProblems];
+    int path[kRotMaxProblems];
     size_t off = 0;
     for (int i = 0; i < count; ++i) {
-        ws[i] = workspace_layout(M, layers[i]->K, layers[i]->N, layers[i]->r, layers[i]->bits, false);
+        ws[i] = workspace_layout(M, layers[i]->K, layers[i]->N, layers[i]->r, layers[i]->bits);
         wbase[i] = base + off;
         off += ws[i].total;
         path[i] = resolve_path(M, layers[i]->K, layers[i]->N, layers[i]->r, layers[i]->bits);
     }
-    bool okt = g_forced_rotation != BWLA_ROT_SIMT && okt_accepts_x(x_bf16, ldx);
-    for (int i = 0; i < count; ++i) okt = okt && layers[i]->okt;
-    if (L0->asym && !okt) return BWLA_ERR_UNSUPPORTED;     // the asymmetric quantiser lives in the tensor-core rotation
-    if (okt) {
-        OktProblem pr[kOktMaxProblems];
-        OktLowrank lr[kOktMaxProblems];
+    const bool rot = L0->rot && g_forced_rotation != BWLA_ROT_SIMT;      // (the layers share n1 and n2)
+    if (L0->asym && !rot) return BWLA_ERR_UNSUPPORTED;     // the asymmetric quantiser lives in the tensor-core rotation
+    if (rot) {
+        RotProblem pr[kRotMaxProblems];
+        OktLowrank lr[kRotMaxProblems];
         for (int i = 0; i < count; ++i) {
             const bwla_layer* L = layers[i];
-            pr[i] = OktProblem{L->prepared, (int8_t*)(wbase[i] + ws[i].codes), path[i] == BWLA_PATH_I8 ? 1 : 0,
-                               L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr, 0,
-                               (float*)(wbase[i] + ws[i].scales), (int32_t*)(wbase[i] + ws[i].qsum), nullptr};
+            pr[i] = RotProblem{};
+            pr[i].prepared = L->prepared; pr[i].codes = (int8_t*)(wbase[i] + ws[i].codes); pr[i].codes_layout = path[i] == BWLA_PATH_I8 ? 1 : 0;
+            pr[i].zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr;
+            pr[i].scales = (float*)(wbase[i] + ws[i].scales); pr[i].qsum = (int32_t*)(wbase[i] + ws[i].qsum);
             lr[i] = OktLowrank{L->V, L->r, wbase[i] + ws[i].T, L->r > 0 ? (float*)(wbase[i] + ws[i].lr_part) : nullptr,
                                status + 8 * i + kLrCounterWord};
         }
-        st = launch_okt(L0->geom, x_bf16, M, ldx, L0->bits, L0->asym, count, pr, lr, status, s);
+        st = launch_rot(L0->geom, x_bf16, M, ldx, L0->bits, L0->asym, count, pr, lr, status, s);
         if (st != BWLA_OK) return st;
     } else {
         for (int i = 0; i < count; ++i) {

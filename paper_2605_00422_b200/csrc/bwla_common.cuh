@@ -1,6 +1,7 @@
 // Shared declarations of the CUDA library: status handling, workspace layout, kernel launchers.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -78,9 +79,10 @@ constexpr int kLowrankPad = 64;          // T is kept as bf16 [3][M][64] (T = hi
 // of the token; unused parts are zero): the consumer adds them, the producers need no exchange.
 constexpr int kQsumParts = 8;
 
-// With few tokens and a large K the rows of V are read by several blocks that each take a part of K; their partial sums
-// of T meet in the workspace and the last block to arrive adds them in a fixed order (counters: status words 4..11).
-constexpr int kLrKSplitMax = 8;
+// With few tokens V is read by several blocks that each take a part of K; their partial sums of T meet in the workspace and
+// the last block to arrive adds them in a fixed order (counters: status words 4..11, one per tile of T).
+constexpr int kLrKSplitMax = 16;
+constexpr int kLrSplitTiles = 8;
 constexpr int kLrCounterWord = 4;
 
 __host__ __device__ inline int lowrank_cols(int r) { return r > kLowrankPad ? (r + 1) / 2 * 2 : kLowrankPad; }
@@ -94,15 +96,18 @@ size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r);
 int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_problems, const OktLowrank* lowrank,
                         uint32_t* status, cudaStream_t stream);
 
+// Bytes of partial sums of T: up to 64 tokens fp32 [tiles][parts][tile], beyond that what the tcgen05 kernel leaves.
+inline size_t lowrank_part_bytes(int64_t M, int64_t K, int r) {
+    if (r <= 0) return 0;
+    const size_t few = M <= 64 ? (size_t)((M + 15) / 16) * kLrKSplitMax * 16 * (size_t)lowrank_cols(r) * 4 : 0;
+    return align_up(std::max(few, lowrank_umma_part_bytes(M, K, r)), 256);
+}
+
 struct Workspace {
-    size_t status, scales, zp, qsum, T, lr_part, codes, prep, total;
+    size_t status, scales, zp, qsum, T, lr_part, codes, total;
 };
 
-// Room for the prepared Kronecker factors of one call (bf16 terms of P2^T and P1^T for the largest factor sizes the
-// tensor-core rotation takes): calls that are handed raw P1, P2 prepare them into the workspace every time.
-constexpr size_t kOktPreparedMax = 640 * 1024;
-
-inline Workspace workspace_layout(int64_t M, int64_t K, int64_t N, int r, int bits, bool with_prepared = true) {
+inline Workspace workspace_layout(int64_t M, int64_t K, int64_t N, int r, int bits) {
     Workspace w{};
     size_t off = 0;
     w.status = off; off += kStatusBytes;
@@ -111,10 +116,8 @@ inline Workspace workspace_layout(int64_t M, int64_t K, int64_t N, int r, int bi
     w.qsum = off;   off += align_up((size_t)M * 4 * kQsumParts, 256);
     const size_t lr_cols = (size_t)lowrank_cols(r);
     w.T = off;      off += align_up((size_t)M * lr_cols * 6, 256);     // bf16 [3][M][cols]
-    // partial sums of T: fp32 [KS][16][cols] for the few-token blocks, [tile][part][cols][128] for the tensor-core kernel
-    w.lr_part = off; off += r > 0 ? align_up(std::max((size_t)kLrKSplitMax * 16 * lr_cols * 4, lowrank_umma_part_bytes(M, K, r)), 256) : 0;
+    w.lr_part = off; off += lowrank_part_bytes(M, K, r);
     w.codes = off;  off += align_up((size_t)M * (size_t)K, 256);
-    w.prep = off;   off += with_prepared ? kOktPreparedMax : 0;
     (void)N; (void)bits;
     w.total = off;
     return w;
@@ -144,43 +147,56 @@ int launch_prologue(const void* x, int64_t M, int64_t K, int64_t ldx, const floa
                     int bits, int8_t* codes, int codes_layout, float* scales, int32_t* qsum, const void* V, int r,
                     void* Thl, float* lr_part, uint32_t* status, cudaStream_t stream);
 
-// ---- tcgen05 version of the rotation + quantiser (okt_umma.cu) ----
+// ---- rotation + quantiser on the warp-level tensor-core path (rot_mma.cu) ----
 // Geometry of the kernel for one pair of Kronecker factor sizes; computed on the host, passed to the kernels by value.
-struct OktGeom {
+struct RotGeom {
     int n1, n2, K;
-    int n1p, n2p;           // n1, n2 rounded up to 16: columns of Z^T / Y^T, contraction depth of the first stage
-    int atom2, atom1;       // bytes of one K-atom row (the swizzle span) of operands contracted over b / over a
-    int dt_count, dt_rows;  // tiles of the rows d of P2^T (= tensor-memory lanes) and rows per tile (a multiple of 8)
-    int cs_count, cs_cols;  // slabs of the rows c of P1^T (= output columns) and columns per slab (a multiple of 16)
-    int p2t_bytes, p1t_bytes, x_bytes;      // one tile of P2^T terms, one slab of P1^T terms, one token's X tile
-    int p1t_off, x_off, bar_off;            // shared-memory offsets (P2^T tile at 0)
-    int tmem_cols, smem_bytes;
+    int n2p;                // n2 rounded up to 16
+    int na;                 // 8-column tiles of a and c: n1 rounded up to 16, in eighths
+    int cw, ntw;            // warps the column tiles are dealt to (1, 2 or 4), tiles per warp
+    int dtc, dc;            // 16-row tiles of d per CTA, CTAs per token (cluster size, up to 8)
+    int warps;              // warps of one token in a CTA: a group
+    int max_groups;         // groups a CTA can hold
+    int s2, s1;             // bytes per row of operands contracted over b / over a
+    int p1_off, group_off, group_bytes;     // shared memory: P2^T terms at 0, P1^T terms, then per group
+    int z_rel, red_rel;                     // ... x at 0, Z^T, RotShared
+    int alias_z;            // Z^T takes the place of x
 };
-constexpr int kOktMaxProblems = 4;          // linears that share one x and are rotated by one launch
-struct OktProblem {
-    const uint8_t* prepared;    // bf16 terms of P2^T tiles and P1^T slabs (launch_prepare_okt)
+constexpr int kRotMaxProblems = 4;          // linears that share one x and are rotated by one launch
+struct RotProblem {
+    const uint8_t* prepared;    // terms of P2^T and P1^T (launch_prepare_rot), or NULL: P1 and P2 are split by every CTA
+    const float *P1, *P2;       // read only when `prepared` is NULL
+    // quantiser (yhat == NULL)
     int8_t* codes;              // [M][K]
     int codes_layout;           // 0: natural k order; 1: the interleaved order of the tensor-core contraction
     int32_t* zp;                // [M] zero points (asymmetric quantiser), or NULL
-    int code_bias;              // added to every stored code and to the stored zero point (see launch_okt)
+    int code_bias;              // added to every stored code and to the stored zero point (see launch_rot)
     float* scales;              // [M]
     int32_t* qsum;              // [M][kQsumParts] or NULL
-    float* y_debug;             // [M][K] fp32 rotated activations before the quantiser, or NULL
+    float* y;                   // [M][K] fp32 rotated activations before the quantiser, or NULL
+    // weight-only operating point
+    __nv_bfloat16* yhat;        // [M][K]
+    float* ysum;                // [M] sums of the rounded values, or NULL
+    // final binarisation
+    uint32_t* packed; float *alpha, *mu;
 };
 struct OktLowrank { const void* V; int r; void* Thl; float* lr_part; uint32_t* lr_count; };   // V == NULL: no T = V x blocks
-// false when the factor sizes are outside what the kernel takes (n2 a multiple of 8 up to 256, n1 up to 192, ...)
-bool okt_geometry(int n1, int n2, OktGeom* out);
-// false when x cannot be read by tiled TMA loads (16-byte aligned base, row stride a multiple of 8 elements)
-bool okt_accepts_x(const void* x, int64_t ldx);
-size_t okt_prepared_bytes(const OktGeom& g);
-int launch_prepare_okt(const OktGeom& g, const float* P1, const float* P2, void* prepared, cudaStream_t stream);
-// One launch for up to kOktMaxProblems linears that read the same x: rotation + quantiser for each, and the T = V x
+// false when the factor sizes are outside what the kernel takes (n2 a multiple of 8 up to 256, n1 up to 192)
+bool rot_geometry(int n1, int n2, RotGeom* out);
+// rows of x that start on 16 bytes (others are read element by element, and the tcgen05 V x kernel does not take them)
+bool rot_accepts_x(const void* x, int64_t ldx);
+size_t rot_prepared_bytes(const RotGeom& g);
+int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void* prepared, cudaStream_t stream);
+// One launch for up to kRotMaxProblems linears that read the same x: rotation + quantiser for each, and the T = V x
 // blocks of those with a low-rank branch.
 // asym == 0: symmetric codes in [-qmax, qmax], qmax = 2^(b-1) - 1.  asym == 1 (Sec. 4.1, per-token asymmetric): with
 // u in [0, 2^b - 1] and the integer zero point z of the token, the stored code is u - 2^(b-1) + code_bias and the
 // stored zero point z - 2^(b-1) + code_bias; a code minus the zero point times the scale is the value it stands for.
-int launch_okt(const OktGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
-               const OktProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream);
+int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
+               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream);
+// Rows of weights (fp32 or bf16): packed signs, scale and shift of every row.
+int launch_rot_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status,
+                        cudaStream_t stream);
 
 // qsum[t][0] = sum_k codes[t][k] (the other parts zero); optionally rewrites natural-order codes into the interleaved order.
 int launch_prepare_codes(const int8_t* codes, int64_t M, int64_t K, int8_t* codes_interleaved, int32_t* qsum,
@@ -213,18 +229,12 @@ struct GemmArgs {
 };
 enum { kDepChain = 0, kDepHead = 1, kDepSibling = 2 };
 
-// W1A16, the weight-only operating point (gemm_a16.cu): Y (fp32) -> bf16 + per-token sums; the bf16 contraction against
-// the packed signs with the fused epilogue.  Thl as for the int8 contractions (NULL when r == 0).
+// W1A16, the weight-only operating point (gemm_a16.cu): the bf16 contraction against the packed signs with the fused
+// epilogue.  Thl as for the int8 contractions (NULL when r == 0).
 bool a16_supports(int64_t M, int64_t K, int64_t N, int r);
-int launch_y_to_bf16(const float* Y, int64_t M, int64_t K, void* yhat, float* ysum, cudaStream_t stream);
 int launch_gemm_a16(const void* yhat, const float* ysum, int64_t M, int64_t K, int64_t N, const uint32_t* packed, const float* alpha,
                     const float* mu, const void* U, int r, const void* Thl, void* out, int64_t ldo, uint32_t* status,
                     cudaStream_t stream);
-
-// Final binarisation of weight rows in the rotated coordinates (binarize.cu).
-size_t binarize_workspace_bytes(int64_t K);
-int launch_binarize(const void* w, int dtype, int64_t N, int64_t K, int64_t ldw, const float* P1, int n1, const float* P2, int n2,
-                    uint32_t* packed, float* alpha, float* mu, void* workspace, cudaStream_t stream);
 
 int launch_gemm_simple(const GemmArgs& a, cudaStream_t stream);
 

@@ -2,7 +2,7 @@
 // activation is kept in bf16 instead of being quantised to integer codes, and meets the packed signs on the tcgen05
 // tensor cores as a bf16 contraction with fp32 accumulation:
 //
-//   yhat = bf16(Y)                                      (y_to_bf16_kernel; also sum_k yhat for the row-shift term)
+//   yhat = bf16(Y)                                      (rot_mma.cu; also sum_k yhat for the row-shift term)
 //   out[t][n] = bf16( alpha[n] * sum_k s[n][k] * yhat[t][k] + U[n,:] . T[t,:] + mu[n] * sum_k yhat[t][k] )
 //
 // Tile of one CTA: 128 tokens (the accumulator's lanes) x 128 weight rows (its columns) x all of K.
@@ -51,27 +51,6 @@ struct A16Params {
     __nv_bfloat16* out; int64_t ldo;
     uint32_t* status;
 };
-
-// One block per token: Y (fp32) -> bf16, and the sum of the rounded values (fp64 accumulation, one fp32 result).
-__global__ void __launch_bounds__(256) y_to_bf16_kernel(const float* __restrict__ Y, int64_t K, __nv_bfloat16* __restrict__ yhat,
-                                                       float* __restrict__ ysum) {
-    __shared__ double red[8];
-    const int64_t t = blockIdx.x;
-    double s = 0.0;
-    for (int64_t k = threadIdx.x; k < K; k += blockDim.x) {
-        const __nv_bfloat16 v = __float2bfloat16_rn(Y[t * K + k]);
-        yhat[t * K + k] = v;
-        s += (double)__bfloat162float(v);
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) a += red[i];
-        ysum[t] = (float)a;
-    }
-}
 
 // Eight sign bits (bit 1 = +1), given inverted in the low byte of `nbits` -> eight bf16 values +-1, two per word, the
 // lower k in the low half.  A pair of inverted bits t = b0 + 2 b1 times (2^15 + 2^30) puts b0 at bit 15 and b1 at bit
@@ -318,7 +297,7 @@ a16_gemm_kernel(const __grid_constant__ CUtensorMap y_map, const __grid_constant
         // not its token exists; only the stores look at the token)
         if (ok) {
             const bool live = t < p.M;
-            const float ys = live ? p.ysum[t] : 0.f;
+            const float ys = live && p.ysum ? p.ysum[t] : 0.f;
             const int c0 = 64 * half;
             __nv_bfloat16* dst = p.out + (live ? t : 0) * p.ldo + n0 + c0;
             const bool vec = ((reinterpret_cast<uintptr_t>(p.out) & 15) == 0) && (p.ldo % 8 == 0) && (n0 + c0 + 64 <= p.N);
@@ -371,12 +350,6 @@ a16_gemm_kernel(const __grid_constant__ CUtensorMap y_map, const __grid_constant
 // ---------------------------------------------------------------------------------------------
 bool a16_supports(int64_t M, int64_t K, int64_t N, int r) {
     return M >= 1 && N >= 1 && K % a16::kBlockK == 0 && r >= 0 && r <= kLowrankPad && M < ((int64_t)1 << 31);
-}
-
-int launch_y_to_bf16(const float* Y, int64_t M, int64_t K, void* yhat, float* ysum, cudaStream_t stream) {
-    ProfScope prof(kProfRotateQuant, stream);
-    y_to_bf16_kernel<<<(unsigned)M, 256, 0, stream>>>(Y, K, (__nv_bfloat16*)yhat, ysum);
-    return after_launch();
 }
 
 int launch_gemm_a16(const void* yhat, const float* ysum, int64_t M, int64_t K, int64_t N, const uint32_t* packed, const float* alpha,

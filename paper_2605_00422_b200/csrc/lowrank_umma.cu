@@ -43,11 +43,11 @@ constexpr int kTargetCtas = 160;          // parts are chosen so that tiles x pa
 struct LrUmmaParams {
     int64_t M;
     int K, ks, tiles, n_problems;
-    float* part[kOktMaxProblems];                 // [tile][part][column][lane] fp32 (ks > 1)
-    __nv_bfloat16* Thl[kOktMaxProblems];          // [3][M][64]
+    float* part[kRotMaxProblems];                 // [tile][part][column][lane] fp32 (ks > 1)
+    __nv_bfloat16* Thl[kRotMaxProblems];          // [3][M][64]
     uint32_t* status;
 };
-struct LrMaps { CUtensorMap v[kOktMaxProblems]; };
+struct LrMaps { CUtensorMap v[kRotMaxProblems]; };
 
 __device__ __forceinline__ void store_terms(__nv_bfloat16* Thl, int64_t M, int64_t t, int c0, const float (&s)[8]) {
     // three bf16 terms carry all 24 bits of an fp32 value; eight columns = 16 bytes per term
@@ -244,7 +244,7 @@ static int lowrank_umma_parts(int64_t M, int64_t K) {
 }
 
 bool lowrank_umma_supports(int64_t M, int64_t K, int r) {
-    return M >= 256 && r > 0 && r <= lru::kCols && lowrank_cols(r) == lru::kCols && K % lru::kBlockK == 0 && K >= lru::kBlockK;
+    return M > 64 && r > 0 && r <= lru::kCols && lowrank_cols(r) == lru::kCols && K % lru::kBlockK == 0 && K >= lru::kBlockK;
 }
 
 size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r) {
@@ -258,7 +258,7 @@ size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r) {
 int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_problems, const OktLowrank* lowrank,
                         uint32_t* status, cudaStream_t stream) {
     using namespace lru;
-    if (n_problems < 1 || n_problems > kOktMaxProblems || M >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
+    if (n_problems < 1 || n_problems > kRotMaxProblems || M >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
     LrUmmaParams p{};
     LrMaps maps{};
     p.M = M; p.K = (int)K; p.ks = lowrank_umma_parts(M, K); p.tiles = (int)((M + kTok - 1) / kTok); p.n_problems = n_problems;

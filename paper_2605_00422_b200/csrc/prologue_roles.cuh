@@ -41,10 +41,10 @@ struct PrologueParams {
     int sp_rest_off;    // split_y: where P2 starts
     // low-rank
     const __nv_bfloat16* V; int r; int lr_cols; __nv_bfloat16* Thl;   // [3][M][lr_cols]
-    int lr_wide;        // low-rank blocks: 0: 2 rows of V x 16 tokens (FMA), 1: 8 x 8 (FMA, many tokens), 2: 8 columns x 16 tokens on the
-                        // warp-level tensor-core path (few tokens), 3: all 64 columns x 16 tokens on that path (many tokens)
-    int lr_ks;          // lr_wide == 2: blocks that share a tile of T and split K (1: no split)
-    float* lr_part;     // [tiles][lr_ks][16 * 8] partial sums of those blocks
+    int lr_wide;        // low-rank blocks: 0: 2 rows of V x 16 tokens (FMA), 1: 8 x 8 (FMA, many tokens), 2, 4: 16 or 32 columns x 16
+                        // tokens on the warp-level tensor-core path, 3: all 64 columns x 16 tokens on that path (many tokens)
+    int lr_ks;          // lr_wide == 2, 4: blocks that share a tile of T and split K (1: no split)
+    float* lr_part;     // [tiles][lr_ks][16 * columns] partial sums of those blocks
     uint32_t* lr_count; // one arrival counter per tile, zero between calls
     int lr_stage;       // 1: a low-rank block copies its rows of V into shared memory before it waits for x
     int late_trigger;   // 1: the next kernel of the stream is let in only when this one is nearly done (see launch_prologue)
@@ -198,12 +198,11 @@ static __device__ void lowrank_role(const PrologueParams& p, int b, float* smem)
     }
 }
 
-// Few tokens: T for a tile of 16 tokens x 8 columns per block on the warp-level tensor-core path
-// (mma.sync m16n8k16, bf16 in, fp32 accumulate): far fewer instructions than the FMA version, so these blocks do not
-// take issue slots from the rotation blocks they share SMs with.  The warps of the block split K in chunks of 32; a
-// lane reads 16 bytes of two token rows and of one row of V per chunk, and the chunk is contracted by two MMAs whose
-// k order is permuted the same way for both operands (a sum over k does not care).  Partial tiles are added across
-// the warps in shared memory in warp order.
+// T = V x on the warp-level tensor-core path (mma.sync m16n8k16, bf16 in, fp32 accumulate): far fewer instructions than the
+// FMA version, so these blocks do not take issue slots from the rotation blocks they share SMs with.  The warps of a block
+// split K in chunks of 32; a lane reads 16 bytes of two token rows and of one row of V per chunk and column tile, and the
+// chunk is contracted by two MMAs whose k order is permuted the same way for both operands (a sum over k does not care).
+// Partial tiles are added across the warps in shared memory in warp order.
 __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                  uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
@@ -211,95 +210,86 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uin
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// Up to 64 tokens: T for a tile of 16 tokens x 8 NTC columns and a part of K per block.  What such a block costs is latency:
+// V comes from HBM and is requested before the preceding kernel has finished (two or four chunks per warp), x follows
+// in one round trip, and K is cut into as many parts as give every warp about that many.
+template <int NTC>
 static __device__ void lowrank_mma_role(const PrologueParams& p, int b, float* smem) {
-    const int jtiles = p.lr_cols / 8;
+    constexpr int COLS = 8 * NTC, U = 8 / NTC;            // U: chunks of a warp in registers at once
+    const int jtiles = (p.lr_cols + COLS - 1) / COLS;
     const int KS = p.lr_ks;
-    const int j0 = (b % jtiles) * 8;
+    const int jt = b % jtiles, j0 = jt * COLS;
     const int ks = (b / jtiles) % KS;
-    const int64_t t0 = (int64_t)(b / (jtiles * KS)) * 16;
+    const int tt = b / (jtiles * KS);
+    const int64_t t0 = (int64_t)tt * 16;
     if (t0 >= p.M) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int g = lane >> 2, tg = lane & 3;
     const int K = p.K;
+    const int chunks = K >> 5;
+    const int c_lo = (int)((int64_t)chunks * ks / KS), c_hi = (int)((int64_t)chunks * (ks + 1) / KS);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const uint4* vj = reinterpret_cast<const uint4*>(p.V) + tg;
+    const bool some = j0 < p.r;
+    uint4 v[U][NTC];
+    auto load_v = [&](int c0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int nt = 0; nt < NTC; ++nt) {
+                const int c = c0 + u * nwarps, j = j0 + 8 * nt + g;
+                v[u][nt] = (some && c < c_hi && j < p.r) ? __ldg(vj + (size_t)j * (K >> 3) + 4 * c) : zero;
+            }
+    };
+    load_v(c_lo + warp);
     griddep_launch_dependents();
     griddep_wait();                                           // x may be the output of the preceding kernel
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    if (j0 < p.r) {
-        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-        const bool row_lo = t0 + g < p.M, row_hi = t0 + g + 8 < p.M, col = j0 + g < p.r;
+    float run[NTC][4];
+#pragma unroll
+    for (int nt = 0; nt < NTC; ++nt)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) run[nt][i] = 0.f;
+    if (some) {
+        const bool row_lo = t0 + g < p.M, row_hi = t0 + g + 8 < p.M;
         const uint4* xlo = reinterpret_cast<const uint4*>(p.x + (t0 + (row_lo ? g : 0)) * p.ldx) + tg;
         const uint4* xhi = reinterpret_cast<const uint4*>(p.x + (t0 + (row_hi ? g + 8 : 0)) * p.ldx) + tg;
-        const uint4* vj = reinterpret_cast<const uint4*>(p.V + (int64_t)(j0 + (col ? g : 0)) * K) + tg;
-        const int chunks = K >> 5;
-        const int c_lo = (int)((int64_t)chunks * ks / KS), c_hi = (int)((int64_t)chunks * (ks + 1) / KS);
-        // The tensor core adds each group of 16 products into the accumulator with truncation; over the hundreds of
-        // steps of a large K that bias would reach 1e-5 of the sum.  Every four chunks the accumulator is added into a
-        // running fp32 sum with an ordinary rounded addition and starts from zero again.
-        float run[4] = {0.f, 0.f, 0.f, 0.f};
-        int since = 0;
-#pragma unroll 4
-        for (int c = c_lo + warp; c < c_hi; c += nwarps) {
-            const uint4 a = row_lo ? __ldg(xlo + 4 * c) : zero;
-            const uint4 h = row_hi ? __ldg(xhi + 4 * c) : zero;
-            const uint4 v = col ? __ldg(vj + 4 * c) : zero;
-            mma_bf16_16x8x16(acc, a.x, h.x, a.y, h.y, v.x, v.y);
-            mma_bf16_16x8x16(acc, a.z, h.z, a.w, h.w, v.z, v.w);
-            if (++since == 4) {
-                since = 0;
+        for (int c0 = c_lo + warp; c0 < c_hi; c0 += U * nwarps) {
+            if (c0 != c_lo + warp) load_v(c0);
+            uint4 a[U], h[U];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) { run[i] += acc[i]; acc[i] = 0.f; }
+            for (int u = 0; u < U; ++u) {
+                const int c = c0 + u * nwarps;
+                a[u] = (row_lo && c < c_hi) ? __ldg(xlo + 4 * c) : zero;
+                h[u] = (row_hi && c < c_hi) ? __ldg(xhi + 4 * c) : zero;
+            }
+            // The tensor core adds each group of 16 products into the accumulator with truncation; over the hundreds of steps
+            // of a large K that bias would reach 1e-5 of the sum.  After U chunks the accumulator is added into a running
+            // fp32 sum with an ordinary rounded addition and starts from zero again.
+#pragma unroll
+            for (int nt = 0; nt < NTC; ++nt) {
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    mma_bf16_16x8x16(acc, a[u].x, h[u].x, a[u].y, h[u].y, v[u][nt].x, v[u][nt].y);
+                    mma_bf16_16x8x16(acc, a[u].z, h[u].z, a[u].w, h[u].w, v[u][nt].z, v[u][nt].w);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) run[nt][i] += acc[i];
             }
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] += run[i];
     }
-    // acc: (token g, columns 2tg, 2tg+1), (token g+8, same columns)
-    float* red = smem;                                        // [nwarps][16 * 8]
-    red[warp * 128 + g * 8 + 2 * tg] = acc[0];
-    red[warp * 128 + g * 8 + 2 * tg + 1] = acc[1];
-    red[warp * 128 + (g + 8) * 8 + 2 * tg] = acc[2];
-    red[warp * 128 + (g + 8) * 8 + 2 * tg + 1] = acc[3];
+    // run: (token g, columns 2tg, 2tg+1), (token g+8, same columns) of every column tile
+    float* red = smem;                                        // [nwarps][16 * COLS]
+#pragma unroll
+    for (int nt = 0; nt < NTC; ++nt) {
+        float* r = red + warp * 16 * COLS + 8 * nt + 2 * tg;
+        r[g * COLS] = run[nt][0]; r[g * COLS + 1] = run[nt][1];
+        r[(g + 8) * COLS] = run[nt][2]; r[(g + 8) * COLS + 1] = run[nt][3];
+    }
     __syncthreads();
-    if (KS > 1) {
-        // Several blocks share this tile of T and split K.  Each leaves its partial tile in the workspace; the last one
-        // to arrive adds them in the order of the K parts (so the result does not depend on who came last).
-        const int tile = (int)(b / (jtiles * KS)) * jtiles + (b % jtiles);
-        float* mine = p.lr_part + ((size_t)tile * KS + ks) * 128;
-        for (int o = threadIdx.x; o < 128; o += blockDim.x) {
-            float s = 0.f;
-            for (int w = 0; w < nwarps; ++w) s += red[w * 128 + o];
-            mine[o] = s;
-        }
-        __threadfence();
-        __syncthreads();
-        __shared__ uint32_t arrived;
-        if (threadIdx.x == 0) arrived = atomicAdd(p.lr_count + tile, 1u);
-        __syncthreads();
-        if (arrived != (uint32_t)(KS - 1)) return;
-        __threadfence();
-        for (int o = threadIdx.x; o < 128; o += blockDim.x) {
-            const int i = o >> 3, j = o & 7;
-            float s = 0.f;
-            for (int k = 0; k < KS; ++k) s += __ldcg(p.lr_part + ((size_t)tile * KS + k) * 128 + o);
-            if (t0 + i < p.M) {
-                const __nv_bfloat16 hi = __float2bfloat16_rn(s);
-                const float r1 = s - __bfloat162float(hi);
-                const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-                const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-                const int64_t at = (t0 + i) * p.lr_cols + j0 + j;
-                p.Thl[at] = hi;
-                p.Thl[p.M * p.lr_cols + at] = mid;
-                p.Thl[2 * p.M * p.lr_cols + at] = lo;
-            }
-        }
-        if (threadIdx.x == 0) p.lr_count[tile] = 0;          // ready for the next call
-        return;
-    }
-    for (int o = threadIdx.x; o < 128; o += blockDim.x) {
-        const int i = o >> 3, j = o & 7;
-        if (t0 + i < p.M) {
-            float s = 0.f;
-            for (int w = 0; w < nwarps; ++w) s += red[w * 128 + o];
+    auto put = [&](int o, float s) {
+        const int i = o / COLS, j = o - i * COLS;
+        if (t0 + i < p.M && j0 + j < p.lr_cols) {
             // three bf16 terms carry all 24 bits of the fp32 sum
             const __nv_bfloat16 hi = __float2bfloat16_rn(s);
             const float r1 = s - __bfloat162float(hi);
@@ -310,6 +300,32 @@ static __device__ void lowrank_mma_role(const PrologueParams& p, int b, float* s
             p.Thl[p.M * p.lr_cols + at] = mid;
             p.Thl[2 * p.M * p.lr_cols + at] = lo;
         }
+    };
+    // Several blocks share this tile of T and split K.  Each leaves its partial tile in the workspace; the last one to arrive
+    // adds them in the order of the K parts (so the result does not depend on who came last).
+    const int tile = tt * jtiles + jt;
+    float* part = KS > 1 ? p.lr_part + (size_t)tile * KS * (16 * COLS) : nullptr;
+    for (int o = threadIdx.x; o < 16 * COLS; o += blockDim.x) {
+        float s = 0.f;
+        for (int w = 0; w < nwarps; ++w) s += red[w * 16 * COLS + o];
+        if (KS > 1) part[ks * (16 * COLS) + o] = s;
+        else put(o, s);
+    }
+    if (KS > 1) {
+        __threadfence();
+        __syncthreads();
+        __shared__ uint32_t arrived;
+        if (threadIdx.x == 0) arrived = atomicAdd(p.lr_count + tile, 1u);
+        __syncthreads();
+        if (arrived != (uint32_t)(KS - 1)) return;
+        __threadfence();
+        for (int o = threadIdx.x; o < 16 * COLS; o += blockDim.x) {
+            float s = 0.f;
+#pragma unroll 8
+            for (int k = 0; k < KS; ++k) s += __ldcg(part + k * (16 * COLS) + o);
+            put(o, s);
+        }
+        if (threadIdx.x == 0) p.lr_count[tile] = 0;          // ready for the next call
     }
 }
 
@@ -393,29 +409,41 @@ static __device__ void lowrank_mma_wide_role(const PrologueParams& p, int b, flo
     }
 }
 
+// One low-rank block of a launch.
+static __device__ __forceinline__ void lowrank_block(const PrologueParams& p, int b, float* smem) {
+    if (p.lr_wide == 1) lowrank_role<8, 8>(p, b, smem);
+    else if (p.lr_wide == 2) lowrank_mma_role<2>(p, b, smem);
+    else if (p.lr_wide == 4) lowrank_mma_role<4>(p, b, smem);
+    else lowrank_role<2, 16>(p, b, smem);
+}
+
 // Host side: chooses the kind of low-rank blocks for the problem in p (x, M, K, ldx, V, r, lr_cols, Thl set), fills the
-// lr_* fields and returns the number of blocks; *smem receives the dynamic shared memory one such block needs.
+// lr_* fields and returns the number of blocks, given their warps; *smem receives the dynamic shared memory one needs.
 // lr_part / lr_count (either may be NULL): workspace for blocks that share a tile of T and split K.
-inline int plan_lowrank(PrologueParams& p, float* lr_part, uint32_t* lr_count, size_t smem_limit, size_t* smem) {
+inline int plan_lowrank(PrologueParams& p, float* lr_part, uint32_t* lr_count, int warps, size_t smem_limit, size_t* smem) {
     const int64_t M = p.M;
     const int K = p.K;
     // few tokens: the tensor-core version (needs 16-byte rows); many tokens: tiles that re-read little
     const bool rows16 = ((reinterpret_cast<uintptr_t>(p.x) | reinterpret_cast<uintptr_t>(p.V)) & 15) == 0 && p.ldx % 8 == 0 &&
                         K % 32 == 0 && p.lr_cols % 8 == 0;
     // (the wide tiles read x once but need enough token tiles to fill the device: 16 tokens x 64 columns per block)
-    p.lr_wide = rows16 ? ((M >= 1024 && p.lr_cols == 64) ? 3 : 2) : ((M >= 64 && p.lr_cols % 8 == 0) ? 1 : 0);
+    p.lr_wide = rows16 ? ((M >= 1024 && p.lr_cols == 64) ? 3 : M > 32 ? 4 : 2) : ((M >= 64 && p.lr_cols % 8 == 0) ? 1 : 0);
+    const int cols = p.lr_wide == 4 ? 32 : 16;                // of one lr_wide 2 / 4 block
+    const int64_t tiles = ((p.lr_cols + cols - 1) / cols) * ((M + 15) / 16);
     int blocks = p.lr_wide == 1 ? (p.lr_cols / 8) * (int)((M + 7) / 8)
-               : p.lr_wide == 2 ? (p.lr_cols / 8) * (int)((M + 15) / 16)
+               : p.lr_wide == 2 || p.lr_wide == 4 ? (int)tiles
                : p.lr_wide == 3 ? (int)((M + 15) / 16) : (p.lr_cols / 2) * (int)((M + 15) / 16);
-    // One tile of 16 tokens and a large K: eight blocks would stream all of V (cold: from HBM) through eight SMs and
-    // become the longest part of the launch; more blocks take a part of K each.
+    // A block of few tokens that read all of V alone would stream it (cold: from HBM) through one SM and become the longest
+    // part of the launch; instead K is split so that a warp has about as many chunks as it can request at once.  There are as
+    // many arrival counters as eight tiles need (64 tokens of up to 64 columns).
     p.lr_ks = 1; p.lr_part = lr_part; p.lr_count = lr_count;
-    if (p.lr_wide == 2 && M <= 16 && lr_part && lr_count && p.lr_cols / 8 <= 8) {
-        const int ksplit = (int)std::min<int64_t>(kLrKSplitMax, (K >> 5) / 100);
-        if (ksplit > 1) { p.lr_ks = ksplit; blocks *= ksplit; }
+    const int per = warps * (p.lr_wide == 4 ? 2 : 4);         // chunks a block has in registers at once
+    if ((p.lr_wide == 2 || p.lr_wide == 4) && tiles <= kLrSplitTiles && lr_part && lr_count) {
+        p.lr_ks = (int)std::min<int64_t>(kLrKSplitMax, std::max(1, (K / 32 + per / 2) / per));
+        blocks *= p.lr_ks;
     }
     // shared memory of a low-rank block: per-warp partial sums, and its rows of V when those are staged (few tokens)
-    const size_t red_bytes = (size_t)kLrMaxWarps * 4 * (p.lr_wide == 3 ? 1024 : p.lr_wide == 2 ? 128 : 64);
+    const size_t red_bytes = (size_t)kLrMaxWarps * 4 * (p.lr_wide == 3 ? 1024 : p.lr_wide == 2 || p.lr_wide == 4 ? 16 * cols : 64);
     const size_t stage_bytes = (size_t)2 * (size_t)K * 2;
     p.lr_stage = (p.lr_wide == 0 && red_bytes + stage_bytes <= smem_limit) ? 1 : 0;
     *smem = red_bytes + (p.lr_stage ? stage_bytes : 0);

@@ -765,15 +765,13 @@ __device__ void rotate_role(const PrologueParams& p, float* smem) {
     finish_token(p, t, C, rank, Xs, slots, amax, rows, a_lo, red_max, &red_sum, true);
 }
 
-__global__ void prologue_kernel(PrologueParams p) {
+__global__ void __launch_bounds__(512) prologue_kernel(PrologueParams p) {
     extern __shared__ __align__(16) float smem[];
     const int b = (int)blockIdx.x;
     const int lr = p.rot_first ? b : b - p.rot_blocks;        // index among the low-rank blocks (when not a rotation block)
     if (b >= p.rot_first && b < p.rot_first + p.rot_blocks) rotate_role(p, smem);
-    else if (p.lr_wide == 1) lowrank_role<8, 8>(p, lr, smem);
-    else if (p.lr_wide == 2) lowrank_mma_role(p, lr, smem);
     else if (p.lr_wide == 3) lowrank_mma_wide_role(p, lr, smem);
-    else lowrank_role<2, 16>(p, lr, smem);
+    else lowrank_block(p, lr, smem);
 }
 
 // How many clusters of `c` prologue blocks (threads, dynamic shared memory) the device holds at once; cached.
@@ -983,7 +981,7 @@ int launch_prologue(const void* x, int64_t M, int64_t K, int64_t ldx, const floa
     int lr_blocks = 0;
     if (r > 0 && Thl) {
         size_t lr_smem = 0;
-        lr_blocks = plan_lowrank(p, lr_part, status ? status + kLrCounterWord : nullptr, kPrologueSmemFloats * 4, &lr_smem);
+        lr_blocks = plan_lowrank(p, lr_part, status ? status + kLrCounterWord : nullptr, threads / 32, kPrologueSmemFloats * 4, &lr_smem);
         smem = std::max(smem, lr_smem);
     }
     // A block with this much shared memory leaves no room on its SM for a block of the next kernel of the stream.  Let
