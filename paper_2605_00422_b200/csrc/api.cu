@@ -74,8 +74,12 @@ static int resolve_path(int64_t M, int64_t K, int64_t N, int r, int bits) {
 }
 
 static int run_contraction(int path, GemmArgs& g, const int8_t* codes, cudaStream_t stream) {
-    if (path == BWLA_PATH_I8) return launch_gemm_umma(g, codes, stream);
     g.codes = codes;
+    if (path == BWLA_PATH_I8) {
+        bool taken = false;
+        const int st = g.M <= 64 ? launch_gemm_small(&g, 1, 1, &taken, stream) : BWLA_OK;
+        return taken ? st : launch_gemm_umma(g, codes, stream);
+    }
     if (path == BWLA_PATH_BITPLANE) return launch_gemm_bitplane(g, stream);
     return launch_gemm_simple(g, stream);
 }
@@ -360,13 +364,16 @@ int bwla_layer_rotate_quant(const bwla_layer* L, const void* x_bf16, int64_t M, 
                            nullptr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
-struct A16Workspace { size_t status, yhat, ysum, T, lr_part, total; };
+// Up to how many tokens the weight-only operating point runs on three int8 digits per value (gemm_small.cu)
+constexpr int kDigitTokens = 32;
+struct A16Workspace { size_t status, yhat, ysum, scales, T, lr_part, total; };
 static A16Workspace a16_layout(const bwla_layer* L, int64_t M) {
     A16Workspace w{};
     size_t off = 0;
     w.status = off; off += kStatusBytes;
-    w.yhat = off;   off += align_up((size_t)M * (size_t)L->K * 2, 256);
-    w.ysum = off;   off += align_up((size_t)M * 4, 256);
+    w.yhat = off;   off += align_up((size_t)M * (size_t)L->K * (M <= kDigitTokens ? 3 : 2), 256);       // bf16, or three digits
+    w.ysum = off;   off += align_up((size_t)M * (M <= kDigitTokens ? 3 * kQsumParts * 4 : 4), 256);      // sums of either
+    w.scales = off; off += align_up((size_t)M * 4, 256);
     const size_t lr_cols = (size_t)lowrank_cols(L->r);
     w.T = off;      off += align_up((size_t)M * lr_cols * 6, 256);
     w.lr_part = off; off += lowrank_part_bytes(M, L->K, L->r);
@@ -393,9 +400,24 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
     const A16Workspace w = a16_layout(L, M);
     char* base = (char*)workspace;
     uint32_t* status = (uint32_t*)(base + w.status);
+    OktLowrank lr{L->V, L->r, base + w.T, L->r > 0 ? (float*)(base + w.lr_part) : nullptr, status + kLrCounterWord};
+    if (M <= kDigitTokens) {
+        GemmArgs g{};
+        g.codes = (const int8_t*)(base + w.yhat); g.scales = (const float*)(base + w.scales); g.qsum = (const int32_t*)(base + w.ysum);
+        g.M = M; g.K = L->K; g.N = L->N; g.bits = 8; g.packed = L->packed; g.alpha = L->alpha; g.mu = L->mu;
+        g.Thl = L->r > 0 ? base + w.T : nullptr; g.U = L->U; g.r = L->r; g.out = out_bf16; g.ldo = ldo; g.status = status;
+        if (gemm_small_fits(&g, 1, 3)) {
+            RotProblem pr{};
+            pr.prepared = L->prepared; pr.digits = 1; pr.codes = (int8_t*)(base + w.yhat); pr.codes_layout = 1;
+            pr.scales = (float*)(base + w.scales); pr.qsum = (int32_t*)(base + w.ysum);
+            st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
+            if (st != BWLA_OK) return st;
+            bool taken = false;
+            return launch_gemm_small(&g, 1, 3, &taken, s);
+        }
+    }
     RotProblem pr{};
     pr.prepared = L->prepared; pr.yhat = (__nv_bfloat16*)(base + w.yhat); pr.ysum = L->mu ? (float*)(base + w.ysum) : nullptr;
-    OktLowrank lr{L->V, L->r, base + w.T, L->r > 0 ? (float*)(base + w.lr_part) : nullptr, status + kLrCounterWord};
     st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
     if (st != BWLA_OK) return st;
     return launch_gemm_a16(base + w.yhat, pr.ysum, M, L->K, L->N, L->packed, L->alpha, L->mu, L->U, L->r,
@@ -475,25 +497,36 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
             if (st != BWLA_OK) return st;
         }
     }
-    // Several contractions that all go to the small-batch tensor-core kernel run beside one another (GemmArgs::dep_mode).
-    bool siblings = count > 1 && M <= 64;
-    for (int i = 0; i < count; ++i) siblings = siblings && path[i] == BWLA_PATH_I8;
-    // each sibling plans for its share of the SMs (by row tiles) when all of them fit the device at once
+    GemmArgs ga[kRotMaxProblems];
+    bool all_i8 = true;
+    for (int i = 0; i < count; ++i) {
+        const bwla_layer* L = layers[i];
+        GemmArgs& g = ga[i];
+        g = GemmArgs{};
+        g.codes = (int8_t*)(wbase[i] + ws[i].codes);
+        g.scales = (float*)(wbase[i] + ws[i].scales); g.qsum = (int32_t*)(wbase[i] + ws[i].qsum);
+        g.M = M; g.K = L->K; g.N = L->N; g.bits = L->bits; g.packed = L->packed; g.alpha = L->alpha; g.mu = L->mu;
+        g.zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr; g.rowsum = L->rowsum;
+        g.Thl = L->r > 0 ? wbase[i] + ws[i].T : nullptr; g.U = L->U; g.r = L->r; g.out = outs[i]; g.ldo = ldos[i];
+        g.status = status;
+        all_i8 = all_i8 && path[i] == BWLA_PATH_I8;
+    }
+    if (all_i8 && M <= 64) {
+        bool taken = false;
+        st = launch_gemm_small(ga, count, 1, &taken, s);
+        if (taken) return st;
+    }
+    // Several contractions that all go to the small-batch tcgen05 kernel run beside one another (GemmArgs::dep_mode); each
+    // plans for its share of the SMs (by row tiles) when all of them fit the device at once
+    const bool siblings = count > 1 && M <= 64 && all_i8;
     int64_t tiles_total = 0;
     for (int i = 0; i < count; ++i) tiles_total += (layers[i]->N + 127) / 128;
     const int sms_all = sm_count();
     const bool share = siblings && tiles_total <= sms_all;
     for (int i = 0; i < count; ++i) {
-        const bwla_layer* L = layers[i];
-        GemmArgs g{};
-        g.scales = (float*)(wbase[i] + ws[i].scales); g.qsum = (int32_t*)(wbase[i] + ws[i].qsum);
-        g.M = M; g.K = L->K; g.N = L->N; g.bits = L->bits; g.packed = L->packed; g.alpha = L->alpha; g.mu = L->mu;
-        g.zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr; g.rowsum = L->rowsum;
-        g.Thl = L->r > 0 ? wbase[i] + ws[i].T : nullptr; g.U = L->U; g.r = L->r; g.out = outs[i]; g.ldo = ldos[i];
-        g.acc_debug = nullptr; g.status = status;
-        g.dep_mode = siblings ? (i == 0 ? kDepHead : kDepSibling) : kDepChain;
-        g.sm_budget = share ? (int)(((int64_t)sms_all * ((L->N + 127) / 128)) / tiles_total) : 0;
-        st = run_contraction(path[i], g, (int8_t*)(wbase[i] + ws[i].codes), s);
+        ga[i].dep_mode = siblings ? (i == 0 ? kDepHead : kDepSibling) : kDepChain;
+        ga[i].sm_budget = share ? (int)(((int64_t)sms_all * ((layers[i]->N + 127) / 128)) / tiles_total) : 0;
+        st = run_contraction(path[i], ga[i], ga[i].codes, s);
         if (st != BWLA_OK) return st;
     }
     return BWLA_OK;

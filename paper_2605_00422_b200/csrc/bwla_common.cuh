@@ -174,7 +174,9 @@ struct RotProblem {
     float* scales;              // [M]
     int32_t* qsum;              // [M][kQsumParts] or NULL
     float* y;                   // [M][K] fp32 rotated activations before the quantiser, or NULL
-    // weight-only operating point
+    // weight-only operating point: bf16 values, or (digits; codes, scales and qsum are then [3][M][K], [M], [3][M][kQsumParts])
+    // their fixed-point digits
+    int digits;
     __nv_bfloat16* yhat;        // [M][K]
     float* ysum;                // [M] sums of the rounded values, or NULL
     // final binarisation
@@ -242,6 +244,12 @@ int launch_gemm_simple(const GemmArgs& a, cudaStream_t stream);
 // a.codes in natural k order.
 bool bitplane_supports(int64_t M, int64_t K, int64_t N, int r, int bits);
 int launch_gemm_bitplane(const GemmArgs& a, cudaStream_t stream);
+
+// Up to 64 tokens: warp-level int8 MMAs, all linears of a group (same M, K, bits; a.codes in the interleaved order) in one
+// launch.  planes == 3: three digit planes per token (the weight-only operating point, up to 32 tokens).  *taken is false, and
+// nothing has been launched, for shapes whose codes do not fit shared memory: those go to the tcgen05 kernels.
+bool gemm_small_fits(const GemmArgs* a, int n, int planes);
+int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStream_t stream);
 
 // tcgen05 path with the fused epilogue.  codes_interleaved: int8 [M][K] in the interleaved order.
 bool umma_supports(int64_t M, int64_t K, int64_t N, int r, int bits);

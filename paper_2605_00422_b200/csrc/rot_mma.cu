@@ -36,7 +36,7 @@
 
 namespace bwla {
 
-enum { kRotQuant = 0, kRotBf16 = 1, kRotBinarize = 2 };
+enum { kRotQuant = 0, kRotBf16 = 1, kRotBinarize = 2, kRotDigits = 3 };
 
 constexpr int kRotMaxWarps = 16;          // per CTA
 constexpr int kRotMaxSmem = 232448 - 128; // the 227 KB a block may have, less the static shared memory of the roles
@@ -49,7 +49,7 @@ struct RotShared {
     float amax[2][64], vmin[2][64];       // largest |Y| (asymmetric quantiser: largest and smallest Y)
     double wsum[kRotMaxWarps];
     double slot_sum[2][8];
-    int qsum[2];
+    int qsum[2][3];
 };
 static_assert(sizeof(RotShared) <= kRotRedBytes, "RotShared");
 
@@ -376,7 +376,8 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     // Where this lane's codes go, for its two columns (parity e) of tile 0 and row gq; a tile further is 8 n2 further, which
     // is a multiple of 64.  Interleaved layout: inside each group of 32, byte 4 (k % 8) + (k % 32) / 8; with n2 a multiple
     // of 16, rows gq and gq + 8 are neighbouring bytes.
-    const bool interleave = MODE == kRotQuant && pr.codes_layout != 0;
+    const bool interleave = (MODE == kRotQuant || MODE == kRotDigits) && pr.codes_layout != 0;
+    const bool pairs16 = interleave && (g.n2 & 15) == 0 && row_hi_ok;
     const bool plain_codes = interleave && (g.n2 & 15) == 0 && row_hi_ok && (nt0 + NTW) * 8 <= g.n1 && !pr.y;
     int lim[2], off_lo[2], off_hi[2];
 #pragma unroll
@@ -482,9 +483,12 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     // token `it`'s code sum leaves behind the first barrier of the token after it
     auto flush_qsum = [&](int64_t t, int par) {
         // every CTA of the cluster leaves its own part of the sum; the consumer adds the parts
-        if (MODE == kRotQuant && pr.qsum && tid < kQsumParts && (tid == rank || (rank == 0 && tid >= g.dc))) {
-            pr.qsum[t * kQsumParts + tid] = tid == rank ? sh.qsum[par] : 0;
-            if (tid == rank) sh.qsum[par] = 0;
+        if ((MODE == kRotQuant || MODE == kRotDigits) && pr.qsum && tid < kQsumParts && (tid == rank || (rank == 0 && tid >= g.dc))) {
+#pragma unroll
+            for (int pl = 0; pl < (MODE == kRotDigits ? 3 : 1); ++pl) {
+                pr.qsum[(pl * p.M + t) * kQsumParts + tid] = tid == rank ? sh.qsum[par][pl] : 0;
+                if (tid == rank) sh.qsum[par][pl] = 0;
+            }
         }
     };
 
@@ -611,6 +615,18 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             publish(sh.amax[par], __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax)));
             if (asym) publish(sh.vmin[par], __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(-vmin, 0.f))));
         }
+        if (MODE == kRotDigits && live) {
+            // the values of the weight-only operating point are bf16; their largest magnitude as bits, NaNs included
+            uint32_t top = 0u;
+#pragma unroll
+            for (int j = 0; j < NTW; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    acc[j][i] = __bfloat162float(__float2bfloat16_rn(acc[j][i]));
+                    top = max(top, __float_as_uint(acc[j][i]) & 0x7FFFFFFFu);
+                }
+            publish(sh.amax[par], __reduce_max_sync(0xFFFFFFFFu, top));
+        }
         // the next token's x has had the second contraction to arrive (and so have the constants, before the first)
         if (!F32) {
             cp_async_wait_all();
@@ -706,12 +722,61 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             if (pr.qsum) {
                 int local = (int)(usum - (uint32_t)counted * (0x4B400000u + (uint32_t)pr.code_bias));
                 local = __reduce_add_sync(0xFFFFFFFFu, local);
-                if (lane == 0 && local != 0) atomicAdd(&sh.qsum[par], local);
+                if (lane == 0 && local != 0) atomicAdd(&sh.qsum[par][0], local);
             }
             if (tid == 0 && rank == 0) {
                 pr.scales[t] = scale;
                 if (pr.zp) pr.zp[t] = shift_i;
             }
+        } else if (MODE == kRotDigits) {
+            // The weight-only operating point for few tokens (gemm_small.cu): q = rne(value * 2^(21 - exponent of the largest)), a
+            // 23-bit integer, as three signed base-256 digits.  Values down to 2^-14 of the largest are exact, smaller ones
+            // within 2^-23 of it: what an fp32 sum of the values would round away.  (A token with an infinity or a NaN in it
+            // gets a NaN scale.)
+            const uint32_t top = slots_max(sh.amax[par]);
+            const int es = min(21 - exponent_of(__uint_as_float(top)), 126);
+            const float mult = pow2f(es);
+            const int64_t plane = p.M * (int64_t)g.K;
+            int8_t* ct = pr.codes + t * (int64_t)g.K;
+            const int tile_step = 8 * g.n2;
+            int s0 = 0, s1 = 0, s2 = 0;               // sums of q, of q without its last digit, ... (wrap-around arithmetic)
+#pragma unroll
+            for (int j = 0; j < NTW; ++j) {
+                int q0[4], q1[4], q2[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    q0[i] = __float_as_int(__fadd_rn(acc[j][i] * mult, 12582912.f)) - 0x4B400000;      // (the product is exact)
+                    q1[i] = (q0[i] + 128) >> 8;
+                    q2[i] = (q1[i] + 128) >> 8;
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (8 * j < lim[e]) {
+                        s0 += q0[e]; s1 += q1[e]; s2 += q2[e];
+                        if (row_hi_ok) { s0 += q0[2 + e]; s1 += q1[2 + e]; s2 += q2[2 + e]; }
+                        if (pairs16) {
+                            int8_t* at = ct + off_lo[e] + j * tile_step;
+                            *reinterpret_cast<uint16_t*>(at) = (uint16_t)__byte_perm(q0[e], q0[2 + e], 0x0040);
+                            *reinterpret_cast<uint16_t*>(at + plane) = (uint16_t)__byte_perm(q1[e], q1[2 + e], 0x0040);
+                            *reinterpret_cast<uint16_t*>(at + 2 * plane) = (uint16_t)__byte_perm(q2[e], q2[2 + e], 0x0040);
+                        } else {
+                            int8_t* at = ct + off_lo[e] + j * tile_step;
+                            at[0] = (int8_t)q0[e]; at[plane] = (int8_t)q1[e]; at[2 * plane] = (int8_t)q2[e];
+                            if (row_hi_ok) {
+                                at = ct + off_hi[e] + j * tile_step;
+                                at[0] = (int8_t)q0[2 + e]; at[plane] = (int8_t)q1[2 + e]; at[2 * plane] = (int8_t)q2[2 + e];
+                            }
+                        }
+                    }
+                }
+            }
+            const int d[3] = {s0 - 256 * s1, s1 - 256 * s2, s2};
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) {
+                const int local = __reduce_add_sync(0xFFFFFFFFu, d[pl]);
+                if (lane == 0 && local != 0) atomicAdd(&sh.qsum[par][pl], local);
+            }
+            if (tid == 0 && rank == 0) pr.scales[t] = top >= 0x7F800000u ? __uint_as_float(0x7FC00000u) : pow2f(-es);
         } else if (MODE == kRotBf16) {
             // the weight-only operating point: bf16 values (layout 1: inside each group of 32, position 2 (k % 16) +
             // (k % 32) / 16), and where asked for their sum
@@ -776,7 +841,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             }
         }
     }
-    if (MODE == kRotQuant && ntok > 0) {
+    if ((MODE == kRotQuant || MODE == kRotDigits) && ntok > 0) {
         barrier();
         flush_qsum(tok0 + (int64_t)(ntok - 1) * stride, (ntok - 1) & 1);
     }
@@ -922,7 +987,7 @@ int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits
         }
     }
     for (int i = n_problems; i <= kRotMaxProblems; ++i) p.lr_begin[i] = lr_total;
-    RotKernel k = problems[0].yhat ? pick_kernel<kRotBf16, false>(g) : pick_kernel<kRotQuant, false>(g);
+    RotKernel k = problems[0].yhat ? pick_kernel<kRotBf16, false>(g) : problems[0].digits ? pick_kernel<kRotDigits, false>(g) : pick_kernel<kRotQuant, false>(g);
     return launch_rot_kernel(k, g, p, smem, lr_total, stream);
 }
 
