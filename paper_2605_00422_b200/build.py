@@ -16,6 +16,7 @@ _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libbwla.so")
 INCLUDE = os.path.join(_ROOT, "include")
+CALLS = os.path.join(_HERE, "_calls.so")   # the native half of the Python binding
 OBJ = os.path.join(_HERE, "_build")        # one object per source: an edit recompiles what it touched
 
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
@@ -39,6 +40,7 @@ def _newer(path: str, deps) -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_calls(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
@@ -65,6 +67,28 @@ def build(force: bool = False, verbose: bool = False) -> str:
         objects = list(pool.map(compile_one, sources()))
     run([nvcc] + flags + ["-o", LIB] + objects + ["-lcudart"])
     return LIB
+
+
+def build_calls(force: bool = False) -> str:
+    """csrc/python_calls.cpp against this interpreter's and PyTorch's headers (g++ only)."""
+    src = os.path.join(CSRC, "python_calls.cpp")
+    if not force and _newer(CALLS, [src, os.path.join(INCLUDE, "bwla.h")]):
+        return CALLS
+    import sysconfig
+
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    inc = [INCLUDE, os.path.join(troot, "include"), os.path.join(troot, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+    lib = os.path.join(troot, "lib")
+    cmd = (["g++", "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] +
+           [f"-I{d}" for d in inc] + ["-o", CALLS, src, f"-L{lib}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+                                      f"-Wl,-rpath,{lib}"])
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("g++ failed building _calls.so")
+    return CALLS
 
 
 def build_microbench() -> str:

@@ -1,7 +1,8 @@
 """Thin Python binding of the C ABI in ``include/bwla.h``.
 
 Argument marshalling only: each function here checks tensor types, takes ``data_ptr()`` and the current CUDA
-stream from PyTorch and calls the entry point of the same name in ``libbwla.so``.  Every step of the layer
+stream from PyTorch and calls the entry point of the same name in ``libbwla.so`` (the entry points that a program calls per
+step do that in native code, ``csrc/python_calls.cpp``).  Every step of the layer
 runs in the library's CUDA kernels.  There is no fallback: if the shared object is missing the import fails.
 """
 from __future__ import annotations
@@ -107,6 +108,24 @@ def _load() -> C.CDLL:
 _lib = _load()
 
 
+def _load_calls():
+    """The native half of the binding (csrc/python_calls.cpp), bound to the library that _load() found."""
+    import importlib.machinery
+    import importlib.util
+    path = os.path.join(_HERE, "_calls.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: build it with `python -m paper_2605_00422_b200.build`")
+    loader = importlib.machinery.ExtensionFileLoader("_calls", path)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_calls", loader))
+    loader.exec_module(mod)
+    mod.bind(*(C.cast(f, C.c_void_p).value for f in (_lib.bwla_w1ax_linear_group, _lib.bwla_w1ax_linear, _lib.bwla_layer_w1a16_linear,
+                                                     _lib.bwla_pack_signs)))
+    return mod
+
+
+_calls = _load_calls()
+
+
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else C.c_void_p(t.data_ptr())
 
@@ -165,16 +184,15 @@ def new_workspace(M: int, K: int, N: int, r: int, bits: int, device="cuda") -> t
 
 def bwla_pack_signs(w: torch.Tensor, packed: Optional[torch.Tensor] = None) -> torch.Tensor:
     """w: fp32 or bf16 [N][K] (row stride >= K) -> uint32 words stored as int32 [N][K/32]."""
-    if w.dtype not in (torch.float32, torch.bfloat16):
-        raise TypeError("w must be fp32 or bf16")
-    _need(w, w.dtype, "w", 2)
-    N, K = w.shape
     if packed is None:
+        if w.dtype not in (torch.float32, torch.bfloat16):
+            raise TypeError("w must be fp32 or bf16")
+        _need(w, w.dtype, "w", 2)
+        N, K = w.shape
         packed = torch.empty((N, K // 32), dtype=torch.int32, device=w.device)
-    _need(packed, torch.int32, "packed", 2)
-    st = _lib.bwla_pack_signs(_ptr(w), 0 if w.dtype == torch.float32 else 1, N, K, w.stride(0) if N > 0 else K,
-                              _ptr(packed), _stream())
-    _check(st, "bwla_pack_signs")
+    st = _calls.pack(w, packed)
+    if st:
+        _check(st, "bwla_pack_signs")
     return packed
 
 
@@ -249,14 +267,13 @@ def bwla_w1ax_linear(x: torch.Tensor, P1: torch.Tensor, P2: torch.Tensor, bits: 
                      mu: Optional[torch.Tensor] = None, out: Optional[torch.Tensor] = None,
                      workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """The whole layer: bf16 x [M][K] -> bf16 out [M][N]."""
-    M, K, N, r, out = _linear_args(x, P1, P2, packed, alpha, U, V, mu, out)
-    if workspace is None:
-        workspace = new_workspace(M, K, N, r, bits, x.device)
-    st = _lib.bwla_w1ax_linear(_ptr(x), M, K, x.stride(0) if M > 0 else K, _ptr(P1), P1.shape[0], _ptr(P2),
-                               P2.shape[0], bits, _ptr(packed), _ptr(alpha), _ptr(mu), _ptr(U), _ptr(V), r,
-                               _ptr(out), N, out.stride(0) if M > 0 else N, _ptr(workspace), workspace.numel(),
-                               _stream())
-    _check(st, "bwla_w1ax_linear")
+    if out is None or workspace is None:
+        M, K, N, r, out = _linear_args(x, P1, P2, packed, alpha, U, V, mu, out)
+        if workspace is None:
+            workspace = new_workspace(M, K, N, r, bits, x.device)
+    st = _calls.linear(x, P1, P2, bits, packed, alpha, U, V, mu, out, workspace)
+    if st:
+        _check(st, "bwla_w1ax_linear")
     return out
 
 
@@ -305,6 +322,7 @@ class Layer:
                                     _ptr(packed), _ptr(alpha), _ptr(mu), _ptr(U), _ptr(V), self.r, _ptr(self.prepared),
                                     nbytes, _stream())
         _check(st, "bwla_layer_create")
+        self._h = self.handle.value                  # (what the native calls read)
         if asymmetric:
             bwla_layer_set_activation_quant(self, BWLA_ACT_ASYMMETRIC)
 
@@ -313,6 +331,7 @@ class Layer:
         if h is not None and h.value and _lib is not None:      # (_lib is None while the interpreter shuts down)
             _lib.bwla_layer_destroy(h)
             self.handle = C.c_void_p()
+            self._h = 0
 
 
 def bwla_w1a16_workspace_bytes(layer: Layer, M: int) -> int:
@@ -322,16 +341,16 @@ def bwla_w1a16_workspace_bytes(layer: Layer, M: int) -> int:
 def bwla_layer_w1a16_linear(layer: Layer, x: torch.Tensor, out: Optional[torch.Tensor] = None,
                             workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """The weight-only layer (W1A16): bf16 x [M][K] -> bf16 out [M][N], rotated activations kept in bf16."""
-    _need(x, torch.bfloat16, "x", 2)
-    M = x.shape[0]
-    if out is None:
-        out = torch.empty((M, layer.N), dtype=torch.bfloat16, device=x.device)
-    _need(out, torch.bfloat16, "out", 2)
-    if workspace is None:
-        workspace = torch.zeros(max(256, bwla_w1a16_workspace_bytes(layer, M)), dtype=torch.uint8, device=x.device)
-    st = _lib.bwla_layer_w1a16_linear(layer.handle, _ptr(x), M, x.stride(0) if M > 0 else layer.K, _ptr(out),
-                                      out.stride(0) if M > 0 else layer.N, _ptr(workspace), workspace.numel(), _stream())
-    _check(st, "bwla_layer_w1a16_linear")
+    if out is None or workspace is None:
+        _need(x, torch.bfloat16, "x", 2)
+        M = x.shape[0]
+        if out is None:
+            out = torch.empty((M, layer.N), dtype=torch.bfloat16, device=x.device)
+        if workspace is None:
+            workspace = torch.zeros(max(256, bwla_w1a16_workspace_bytes(layer, M)), dtype=torch.uint8, device=x.device)
+    st = _calls.a16(layer, x, out, workspace)
+    if st:
+        _check(st, "bwla_layer_w1a16_linear")
     return out
 
 
@@ -397,19 +416,16 @@ def new_group_workspace(layers, M: int, device="cuda") -> torch.Tensor:
 
 def bwla_w1ax_linear_group(layers, x: torch.Tensor, outs=None, workspace: Optional[torch.Tensor] = None):
     """Layers that share x (q/k/v, gate/up) in one call; returns the list of bf16 outputs [M][N_i]."""
-    _need(x, torch.bfloat16, "x", 2)
-    M, K = x.shape
-    if outs is None:
-        outs = [torch.empty((M, l.N), dtype=torch.bfloat16, device=x.device) for l in layers]
-    for o in outs:
-        _need(o, torch.bfloat16, "out", 2)
-    if workspace is None:
-        workspace = new_group_workspace(layers, M, x.device)
-    optr = (C.c_void_p * len(layers))(*[o.data_ptr() for o in outs])
-    ldos = (C.c_int64 * len(layers))(*[(o.stride(0) if M > 0 else l.N) for o, l in zip(outs, layers)])
-    st = _lib.bwla_w1ax_linear_group(_handles(layers), len(layers), _ptr(x), M, x.stride(0) if M > 0 else K, optr, ldos,
-                                     _ptr(workspace), workspace.numel(), _stream())
-    _check(st, "bwla_w1ax_linear_group")
+    if outs is None or workspace is None:
+        _need(x, torch.bfloat16, "x", 2)
+        M = x.shape[0]
+        if outs is None:
+            outs = [torch.empty((M, l.N), dtype=torch.bfloat16, device=x.device) for l in layers]
+        if workspace is None:
+            workspace = new_group_workspace(layers, M, x.device)
+    st = _calls.group(layers, x, outs, workspace)
+    if st:
+        _check(st, "bwla_w1ax_linear_group")
     return outs
 
 

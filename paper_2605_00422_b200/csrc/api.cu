@@ -64,6 +64,9 @@ static int bitplane_max_tokens(int64_t K, int64_t N, int bits) {
     return (K % 128 != 0) ? 4 : 0;
 }
 
+// Up to how many tokens the warp-level MMA kernel (gemm_small.cu) runs the contraction.
+constexpr int kSmallTokens = 16;
+
 // Which kernel family runs the contraction.  A forced family that cannot take the shape falls back to the simple one.
 static int resolve_path(int64_t M, int64_t K, int64_t N, int r, int bits) {
     int path = g_forced_path;
@@ -77,7 +80,7 @@ static int run_contraction(int path, GemmArgs& g, const int8_t* codes, cudaStrea
     g.codes = codes;
     if (path == BWLA_PATH_I8) {
         bool taken = false;
-        const int st = g.M <= 64 ? launch_gemm_small(&g, 1, 1, &taken, stream) : BWLA_OK;
+        const int st = g.M <= kSmallTokens ? launch_gemm_small(&g, 1, 1, &taken, stream) : BWLA_OK;
         return taken ? st : launch_gemm_umma(g, codes, stream);
     }
     if (path == BWLA_PATH_BITPLANE) return launch_gemm_bitplane(g, stream);
@@ -511,7 +514,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         g.status = status;
         all_i8 = all_i8 && path[i] == BWLA_PATH_I8;
     }
-    if (all_i8 && M <= 64) {
+    if (all_i8 && M <= kSmallTokens) {
         bool taken = false;
         st = launch_gemm_small(ga, count, 1, &taken, s);
         if (taken) return st;

@@ -161,6 +161,7 @@ struct RotGeom {
     int p1_off, group_off, group_bytes;     // shared memory: P2^T terms at 0, P1^T terms, then per group
     int z_rel, red_rel;                     // ... x at 0, Z^T, RotShared
     int alias_z;            // Z^T takes the place of x
+    int pad;                // bytes added to every row against bank conflicts
 };
 constexpr int kRotMaxProblems = 4;          // linears that share one x and are rotated by one launch
 struct RotProblem {

@@ -9,33 +9,30 @@
 // tokens (256 weights per cycle at 8 tokens, 128 at 16), and the sign bits become its A operand in registers, with no trip
 // through tensor memory and no expander / issuer hand-over.
 //
-// Operand order.  A step is 128 values of k: lane t of a quad holds the sign word of the t-th 32 of them.  The interleaved code
-// layout puts k = j + 8 i of every 32 at byte 4 j + i, so byte i of (word >> j) & 0x01010101 meets code word j; an MMA takes
-// code words q and q + 4 of the four lanes.  With few tokens, where these instructions are the bound, 2 (or 4) neighbouring bit
-// positions are left where they are and have accumulators of their own (masks 0x01.., 0x02.., ... of a word shifted by
-// multiples of 2 (4) only), added with one shift each at the end.
+// Operand order.  An item is 32 rows x 512 values of k: lane t of a quad holds the four sign words of the t-th 128 of them, for
+// rows gq + 8 j.  The interleaved code layout puts k = j + 8 i of every 32 at byte 4 j + i, so byte i of (word >> j) & 0x01010101
+// meets code word j; an MMA takes code words q and q + 4 of the four lanes' words.  With few tokens, where these instructions
+// are the bound, 2 (or 4) neighbouring bit positions are left where they are and have accumulators of their own (masks 0x01..,
+// 0x02.., ... of a word shifted by multiples of 2 (4) only), added with one shift each at the end.
 //
-// Work split.  CTA = RW row groups of 32 rows x KW K slices (16 warps; from 33 tokens on also x 2 token halves), one CTA per
-// SM; it takes tiles of 32 RW rows in turn.  One thread streams the sign words by TMA (boxes of 32 RW rows x 1024 k, 128-byte
-// swizzle) into a ring as deep as shared memory allows, starting before the preceding kernel has finished (no warp of its own:
-// 16 warps may have 128 registers a thread, 17 only 96); the CTA's codes and T lie in shared memory for all its tiles (rows of
-// 128 bytes, swizzled the same way: every read is free of bank conflicts).  K is split over a cluster of S CTAs where the codes
-// would not fit or rows are few.  Partial sums meet in shared memory (of the CTA, then of the cluster), and the warps of a
-// group share out the epilogue, which also evaluates U T (bf16 MMAs, three terms of T).
+// Work split.  A CTA (16 warps, one CTA per SM) owns a run of 32-row groups; the items of a run go to the warps in equal
+// contiguous shares, with no barrier until all are done: a warp loads its sign words straight into registers, one item ahead,
+// and adds its sums to the CTA's in shared memory when it leaves a group.  (Tiles of 128 rows whose K was shared by four
+// warps, behind a TMA ring, spent half of their time at barriers and in the epilogue of every tile.)  The rows' sign words,
+// scales and rows of U are asked into the L2 before the preceding kernel has finished; the CTA's codes and T lie in shared
+// memory (rows of 128 bytes, permuted so that every read is free of bank conflicts).  K is split over a cluster of S CTAs
+// where the codes would not fit or rows are few.  The epilogue, once per run, also evaluates U T (bf16 MMAs, three terms of T).
 //
 // PL = 3 is the weight-only operating point: an activation is a 23-bit fixed-point number of a power-of-two scale, kept as
 // three signed base-256 digits (rot_mma.cu); the digits are contracted like three tokens' codes, exactly, and put together in
 // the epilogue.
-// Every wait is bounded (umma_wait.cuh).
 #include <cuda_bf16.h>
 
 #include <algorithm>
 
 #include "bwla_common.cuh"
 #include "rot_mma.cuh"
-#include "tensor_map.cuh"
 #include "umma_ptx.cuh"
-#include "umma_wait.cuh"
 
 namespace bwla {
 
@@ -43,32 +40,29 @@ using namespace ptx;
 
 namespace small_ {
 constexpr int kWarps = 16, kThreads = 32 * kWarps;
-constexpr int kUnit = 1024, kSteps = 8;                       // k per ring stage; steps of 128 k in it
-constexpr int kMaxStages = 12;
-constexpr int kSmemMax = 232448 - 1024 - 256;                 // (the base is aligned to 1024 bytes; barriers are static)
-// Warps a row group's tokens are dealt to: the accumulators of 64 tokens (12 tiles of digits) do not fit one warp's registers
-// (each then expands the sign bits for itself, which its MMAs cover).
-__host__ __device__ constexpr int token_warps(int NT) { return NT >= 8 ? 2 : 1; }
+constexpr int kUnit = 512, kSteps = 4;                        // k per item; code rows of 128 k in it
+constexpr int kSmemMax = 232448 - 256;
+// Sub-groups the tokens of a row group are dealt to: the accumulators of 64 tokens (12 tiles of digits) do not fit one warp's
+// registers (each then expands the sign bits for itself, which its MMAs cover).
+__host__ __device__ constexpr int token_parts(int NT) { return NT >= 8 ? 2 : 1; }
 }  // namespace small_
 
 struct SmallProblem {
-    const int8_t* codes;                  // [PL][M][K]
+    const uint32_t* packed; const int8_t* codes;              // codes [PL][M][K]
     const float* scales; const int32_t* qsum; const int32_t* zp; const int32_t* rowsum;
     const float* alpha; const float* mu;
     const __nv_bfloat16* U; const __nv_bfloat16* Thl;
     __nv_bfloat16* out; int64_t ldo; int32_t* acc_debug;
-    int N, r, tiles;
+    int N, r, groups;                     // 32-row groups
     int cluster_begin, clusters;          // clusters [cluster_begin, cluster_begin + clusters) of the launch
 };
 struct SmallParams {
     SmallProblem prob[kRotMaxProblems];
     int n_problems, M, K, units, S;
-    int stages;                           // of the sign-word ring
-    int flush;                            // rounds between cluster-wide reductions (S > 1)
-    int ring_off, t_off, tok_off, red_off, csum_off;
+    int run;                              // groups whose sums fit shared memory at a time
+    int t_off, tok_off, acc_off;
     uint32_t* status;
 };
-struct SmallMaps { CUtensorMap w[kRotMaxProblems]; };
 
 __device__ __forceinline__ void imma_16832(int32_t (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
@@ -79,77 +73,89 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
 }
-__device__ __forceinline__ void sts128(uint32_t addr, int32_t x, int32_t y, int32_t z, int32_t w) {
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+__device__ __forceinline__ void red_shared_add(uint32_t addr, int32_t v) { asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ int32_t ld_cluster_s32(uint32_t addr) {
+    int32_t v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+// sign words: read once, straight to registers
+__device__ __forceinline__ uint4 ldg_stream(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
 }
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// NTP: token tiles of 8; PL: digit planes per token; KW: warps that share a row group and split K; SPLIT: clusters split K
-template <int NTP, int PL, int KW, bool SPLIT>
-__global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const __grid_constant__ SmallMaps maps, const __grid_constant__ SmallParams p) {
+// NTP: token tiles of 8; PL: digit planes per token; SPLIT: clusters split K
+template <int NTP, int PL, bool SPLIT>
+__global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const __grid_constant__ SmallParams p) {
     using namespace small_;
-    constexpr int NT = NTP * PL, TW = token_warps(NT), NTPW = NTP / TW, NTW = NT / TW;        // ... W: of one warp
-    constexpr int RW = kWarps / (KW * TW), TOK = 8 * NT, SETS = NT == 1 ? 4 : NT <= 3 ? 2 : 1;
-    constexpr int CH = PL == 3 || NTPW < 2 ? 1 : 2, FR = 2 * CH;                              // token tiles, fragments reduced at a time
-    constexpr int kStageBytes = RW * 32 * 128;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t full[kMaxStages], empty[kMaxStages];
-    __shared__ int abort_word;
-    volatile int* abort_flag = &abort_word;
+    constexpr int NT = NTP * PL, TP = token_parts(NT), NTPW = NTP / TP, NTW = NT / TP;        // ... W: of one item
+    constexpr int TOK = 8 * NT, SETS = NT == 1 ? 4 : NT <= 3 ? 2 : 1;
+    extern __shared__ __align__(16) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
     const int cl_all = (int)blockIdx.x / p.S, rank = SPLIT ? (int)blockIdx.x - cl_all * p.S : 0;
     int pi = 0;
     while (pi + 1 < p.n_problems && cl_all >= p.prob[pi + 1].cluster_begin) ++pi;
     const SmallProblem& pr = p.prob[pi];
-    const int cl = cl_all - pr.cluster_begin, clusters = pr.clusters;
+    const int cl = cl_all - pr.cluster_begin;
     const int ub = (int)((int64_t)p.units * rank / p.S), un = (int)((int64_t)p.units * (rank + 1) / p.S) - ub;   // this CTA's units
-    const int rounds = (pr.tiles - cl + clusters - 1) / clusters;      // tiles cl, cl + clusters, ... (the same for a whole cluster)
+    const int g_lo = (int)((int64_t)pr.groups * cl / pr.clusters), g_hi = (int)((int64_t)pr.groups * (cl + 1) / pr.clusters);
+    const int row_bytes = p.K >> 3;
 
-    if (tid == 0) {
-        abort_word = 0;
-        for (int i = 0; i < p.stages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], kWarps); }
-        fence_barrier_init();
-        fence_proxy_async();
-    }
-    __syncthreads();
     griddep_launch_dependents();
-
-    // ---- sign words (constants of the layer): the ring is filled before the preceding kernel has finished, and refilled one
-    //      stage behind the consumption, when every warp has let go of the stage before
-    const int total = rounds * un;
-    auto request = [&](int c) {                       // stage number c of this CTA's sequence (thread 0)
-        const int i = c / un, u = c - i * un, st = c % p.stages;
-        mbar_expect_tx(&full[st], kStageBytes);
-        tma_load_2d_hint(smem + p.ring_off + st * kStageBytes, &maps.w[pi], (ub + u) * (kUnit / 32), (cl + i * clusters) * (32 * RW), &full[st],
-                         l2_policy_evict_first());
+    // ---- constants of the layer, before the preceding kernel has finished: this CTA's share of the sign words, and its rows' scales
+    //      and rows of U, into the L2
+    {
+        const int rows = min((g_hi - g_lo) * 32, pr.N - g_lo * 32);
+        const uint8_t* w = reinterpret_cast<const uint8_t*>(pr.packed) + (int64_t)g_lo * 32 * row_bytes + ub * (kUnit / 8);
+        const uint32_t bytes = (uint32_t)min(un * (kUnit / 8), row_bytes - ub * (kUnit / 8));
+        for (int i = tid; i < rows; i += kThreads) prefetch_l2_bulk(w + (int64_t)i * row_bytes, bytes);
+        for (int i = tid; i < (rows + 31) / 32; i += kThreads) {
+            const int n0 = (g_lo + i) * 32;
+            prefetch_l2_line(pr.alpha + n0);
+            if (pr.mu) prefetch_l2_line(pr.mu + n0);
+            if (pr.zp) prefetch_l2_line(pr.rowsum + n0);
+            if (pr.r > 0) {
+                const uintptr_t lo = reinterpret_cast<uintptr_t>(pr.U + (int64_t)n0 * pr.r);
+                const uintptr_t hi = reinterpret_cast<uintptr_t>(pr.U + (int64_t)min(n0 + 32, pr.N) * pr.r);
+                const uintptr_t a0 = (lo + 15) & ~(uintptr_t)15;
+                if (hi >= a0 + 16) prefetch_l2_bulk(reinterpret_cast<const void*>(a0), (uint32_t)((hi - a0) & ~(uintptr_t)15));
+            }
+        }
+    }
+    // this warp's items of a run of `n` groups from `g`: [lo, hi) in the order (group, token part, unit)
+    int g = g_lo, n = min(p.run, g_hi - g_lo), it, it_end;
+    auto share = [&]() {
+        const int all = n * TP * un;
+        it = all * warp / kWarps; it_end = all * (warp + 1) / kWarps;
     };
-    if (tid == 0) {
-        tma_prefetch_desc(&maps.w[pi]);
-        for (int c = 0; c < min(p.stages, total); ++c) request(c);
-    }
-    // the rows of U the epilogues will want come from HBM too: into the L2 before they are needed
-    if (pr.r > 0 && tid >= 32 && tid < 32 + rounds) {
-        const int n0 = (cl + (tid - 32) * clusters) * (32 * RW);
-        const uintptr_t lo = reinterpret_cast<uintptr_t>(pr.U + (int64_t)n0 * pr.r);
-        const uintptr_t hi = reinterpret_cast<uintptr_t>(pr.U + (int64_t)min(n0 + 32 * RW, pr.N) * pr.r);
-        const uintptr_t a0 = (lo + 15) & ~(uintptr_t)15;
-        if (hi >= a0 + 16) prefetch_l2_bulk(reinterpret_cast<const void*>(a0), (uint32_t)((hi - a0) & ~(uintptr_t)15));
-    }
-    __syncwarp();
+    share();
+    auto load_w = [&](uint4 (&w)[4], int item) {
+        const int sub = item / un, u = item - sub * un;
+        const int n0 = (g + sub / TP) * 32 + gq, k16 = (ub + u) * (kUnit / 128) + tq;            // 16-byte pieces of a row
+        const uint8_t* at = reinterpret_cast<const uint8_t*>(pr.packed) + 16 * k16;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            w[j] = 128 * k16 < p.K ? ldg_stream(at + (int64_t)min(n0 + 8 * j, pr.N - 1) * row_bytes) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    uint4 wn[4];
+    if (it < it_end) load_w(wn, it);
+    int32_t* const accs = reinterpret_cast<int32_t*>(smem + p.acc_off);      // [group of the run][row half][column tile][4][32 lanes]
+    for (int i = tid; i < p.run * 2 * NT * 32; i += kThreads) reinterpret_cast<uint4*>(accs)[i] = make_uint4(0u, 0u, 0u, 0u);
     griddep_wait();
-    if (lane == 0 && p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) *abort_flag = 1;      // the call already failed
-    // ---- codes (128-byte rows: step of 128 k, token), T (128-byte rows: term, token) and the per-token scalars; the 16-byte
-    //      pieces of a row are permuted by the token's low bits
+    // ---- codes (128-byte rows: 128 k, token), T (128-byte rows: term, token) and the per-token scalars; the 16-byte pieces of a
+    //      row are permuted by the token's low bits (and, for the codes, the row's place among the four of an item)
     const int pieces = min(un * (kUnit / 16), (p.K >> 4) - ub * (kUnit / 16));
     for (int t = warp; t < PL * p.M; t += kWarps) {
         const int plane = PL > 1 ? t / p.M : 0, row = plane * (8 * NTP) + (t - plane * p.M);
         const int8_t* src = pr.codes + (int64_t)t * p.K + (int64_t)ub * kUnit;
         const uint32_t dst = smem_u32(smem) + row * 128;
         for (int c = lane; c < pieces; c += 32)
-            cp_async16(dst + (uint32_t)((c >> 3) * (TOK * 128) + (((c & 7) ^ (row & 7)) << 4)), src + 16 * c);
+            cp_async16(dst + (uint32_t)((c >> 3) * (TOK * 128) + (((c & 7) ^ (row & 7) ^ (((c >> 3) & 3) << 1)) << 4)), src + 16 * c);
     }
     if (pr.r > 0)
         for (int i = tid; i < 3 * p.M * 8; i += kThreads) {
@@ -170,20 +176,14 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
         }
         sc_s[tid] = sc; qs_s[tid] = qs; zp_s[tid] = zp;
     }
+    // (behind the copies: the look at the status word is a trip to the L2)
+    const bool failed = p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0;       // the call already failed
     cp_async_wait_all();
     __syncthreads();
 
-    const int grp = warp / KW, kw = warp - grp * KW, rw = grp / TW, tw = grp - rw * TW;
-    // this lane's code pieces of a step: token gq, pieces 2 tq and 2 tq + 1; its sign words: rows gq + 8 j, piece = the step
-    const int b_lo = ((2 * tq) ^ gq) << 4, b_hi = ((2 * tq + 1) ^ gq) << 4;
-    const uint8_t* w_base = smem + p.ring_off + (rw * 32 + gq) * 128 + 4 * tq;
-    constexpr int SPW = kSteps / KW;                  // steps of a stage per warp
-    const uint32_t red = smem_u32(smem) + p.red_off + (uint32_t)(grp * KW * FR * PL * 512 + lane * 16);
-    const uint32_t csum = SPLIT ? smem_u32(smem) + p.csum_off + lane * 16 : 0u;
-
-    // one fragment (16 rows x 8 tokens) of a finished tile
-    auto epilogue = [&](int tile, int rg, int mt, int nt, const int32_t (&v)[PL][4]) {
-        const int n_lo = (tile * RW + rg) * 32 + 16 * mt + gq, n_hi = n_lo + 8;
+    // one fragment (16 rows x 8 tokens) of a finished group
+    auto epilogue = [&](int grp, int mt, int nt, const int32_t (&v)[PL][4]) {
+        const int n_lo = grp * 32 + 16 * mt + gq, n_hi = n_lo + 8;
         const bool ok_lo = n_lo < pr.N, ok_hi = n_hi < pr.N;
         float lr[4] = {0.f, 0.f, 0.f, 0.f};
         if (pr.r > 0) {
@@ -246,37 +246,40 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
         }
     };
 
-    int st = 0; uint32_t ph = 0;
-    bool ok = true;
+
+    const uint32_t b0 = smem_u32(smem) + (uint32_t)((tq * TOK + gq) * 128), b_swz = (uint32_t)((gq ^ (tq << 1)) << 4);
 #pragma unroll 1
-    for (int i = 0; i < rounds; ++i) {
-        const int tile = cl + i * clusters;
+    while (g < g_hi) {
         int32_t acc[SETS][2][NTW][4];
+        int sub = it < it_end ? it / un : 0, u = it - sub * un;
+        auto clear = [&]() {
 #pragma unroll
-        for (int s = 0; s < SETS; ++s)
+            for (int s = 0; s < SETS; ++s)
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+                for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                for (int nt = 0; nt < NTW; ++nt)
+                    for (int nt = 0; nt < NTW; ++nt)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[s][mt][nt][e] = 0;
+                        for (int e = 0; e < 4; ++e) acc[s][mt][nt][e] = 0;
+        };
+        clear();
 #pragma unroll 1
-        for (int u = 0; u < un; ++u) {
-            if (ok && !warp_wait(&full[st], ph, abort_flag)) { give_up(p.status, abort_flag, 0x420); ok = false; }
-            const uint8_t* w_stage = w_base + st * kStageBytes;
-            uint32_t w[SPW][4];
+        for (; it < it_end; ++it) {
+            uint4 w[4];
 #pragma unroll
-            for (int x = 0; x < SPW; ++x)
+            for (int j = 0; j < 4; ++j) w[j] = wn[j];
+            if (it + 1 < it_end) load_w(wn, it + 1);
+            const int part = TP > 1 ? sub % TP : 0;
+            // column tile j of the item: plane j / NTPW, token tile part * NTPW + j % NTPW
+            const uint32_t b_item = b0 + (uint32_t)((u * kSteps * TOK + 8 * NTPW * part) * 128);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) w[x][j] = *reinterpret_cast<const uint32_t*>(w_stage + j * 1024 + (((kw * SPW + x) ^ gq) << 4));
-            // column tile j of this warp: plane j / NTPW, token tile tw * NTPW + j % NTPW
-            const uint8_t* b_unit = smem + (8 * NTPW * tw + gq) * 128 + (u * kSteps + kw * SPW) * (TOK * 128);
-#pragma unroll
-            for (int x = 0; x < SPW; ++x) {
+            for (int x = 0; x < 4; ++x) {
                 uint32_t a[2][4][4];
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt) {
-                    const uint32_t lo = w[x][2 * mt], hi = w[x][2 * mt + 1];
+                    const uint4 lo4 = w[2 * mt], hi4 = w[2 * mt + 1];
+                    const uint32_t lo = x == 0 ? lo4.x : x == 1 ? lo4.y : x == 2 ? lo4.z : lo4.w;
+                    const uint32_t hi = x == 0 ? hi4.x : x == 1 ? hi4.y : x == 2 ? hi4.z : hi4.w;
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const int sh = q & ~(SETS - 1);
@@ -287,8 +290,8 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                 }
 #pragma unroll
                 for (int nt = 0; nt < NTW; ++nt) {
-                    const uint8_t* at = b_unit + (x * TOK + 8 * ((nt / NTPW) * NTP + nt % NTPW)) * 128;
-                    const uint4 c0 = *reinterpret_cast<const uint4*>(at + b_lo), c1 = *reinterpret_cast<const uint4*>(at + b_hi);
+                    const uint32_t at = b_item + (uint32_t)(8 * ((nt / NTPW) * NTP + nt % NTPW) * 128);
+                    const uint4 c0 = lds128(at + ((uint32_t)(32 * x) ^ b_swz)), c1 = lds128(at + ((uint32_t)(32 * x + 16) ^ b_swz));
                     const uint32_t bl[4] = {c0.x, c0.y, c0.z, c0.w}, bh[4] = {c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
@@ -297,119 +300,79 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                             imma_16832(acc[q & (SETS - 1)][mt][nt], a[mt][q][0], a[mt][q][1], a[mt][q][2], a[mt][q][3], bl[q], bh[q]);
                 }
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[st]);
-            if (tid == 0) {
-                const int c = i * un + u - 1;         // the stage before this one
-                if (c >= 0 && c + p.stages < total && !*abort_flag) {
-                    if (wait_or_abort(&empty[st > 0 ? st - 1 : p.stages - 1], st > 0 ? ph : ph ^ 1u, abort_flag)) request(c + p.stages);
-                    else give_up(p.status, abort_flag, 0x410);
-                }
-            }
-            if (++st == p.stages) { st = 0; ph ^= 1u; }
-        }
-        // ---- the KW slices of the tile meet, CH token tiles at a time
+            if (++u == un || it + 1 == it_end) {
+                // the group (or the warp's share of it) is done: into the CTA's sums
+                const uint32_t at = smem_u32(accs) + (uint32_t)(((sub / TP) * 2 * NT * 128 + lane) * 4);
 #pragma unroll
-        for (int c0 = 0; c0 < NTPW; c0 += CH) {
+                for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                for (int c = 0; c < CH; ++c)
-#pragma unroll
-                    for (int pl = 0; pl < PL; ++pl) {
-                        int32_t v[4];
+                    for (int nt = 0; nt < NTW; ++nt)
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            v[e] = acc[0][mt][pl * NTPW + c0 + c][e];
+                            int32_t v = acc[0][mt][nt][e];
 #pragma unroll
-                            for (int z = 1; z < SETS; ++z) v[e] += acc[z][mt][pl * NTPW + c0 + c][e] >> z;
+                            for (int z = 1; z < SETS; ++z) v += acc[z][mt][nt][e] >> z;
+                            const int col = (nt / NTPW) * NTP + NTPW * part + nt % NTPW;
+                            red_shared_add(at + (uint32_t)(((mt * NT + col) * 4 + e) * 128), v);
                         }
-                        sts128(red + (uint32_t)(((kw * FR + mt * CH + c) * PL + pl) * 512), v[0], v[1], v[2], v[3]);
-                    }
-            named_barrier(1 + grp, 32 * KW);
-#pragma unroll 1
-            for (int f = kw; f < FR; f += KW) {
-                int32_t v[PL][4];
-#pragma unroll
-                for (int pl = 0; pl < PL; ++pl) {
-                    v[pl][0] = v[pl][1] = v[pl][2] = v[pl][3] = 0;
-#pragma unroll
-                    for (int k = 0; k < KW; ++k) {
-                        const uint4 q = lds128(red + (uint32_t)(((k * FR + f) * PL + pl) * 512));
-                        v[pl][0] += (int32_t)q.x; v[pl][1] += (int32_t)q.y; v[pl][2] += (int32_t)q.z; v[pl][3] += (int32_t)q.w;
-                    }
-                }
-                const int mt = f / CH, nt = NTPW * tw + c0 + f - mt * CH;
-                if (!SPLIT) {
-                    if (!*abort_flag) epilogue(tile, rw, mt, nt, v);
-                } else {
-#pragma unroll
-                    for (int pl = 0; pl < PL; ++pl)
-                        sts128(csum + (uint32_t)(((((i % p.flush) * RW + rw) * 2 * NTP + 2 * nt + mt) * PL + pl) * 512), v[pl][0], v[pl][1], v[pl][2], v[pl][3]);
-                }
+                clear();
+                u = 0; ++sub;
             }
-            named_barrier(1 + grp, 32 * KW);          // (the buffer may be written again)
         }
-        if (SPLIT && ((i + 1) % p.flush == 0 || i + 1 == rounds)) {
-            // ---- the cluster's partial sums: every CTA takes its share of the fragments of the last rounds
-            cluster_arrive_release(); cluster_wait_acquire();
-            const int first = i / p.flush * p.flush, items = (i + 1 - first) * RW * 2 * NTP;
-#pragma unroll 1
-            for (int it = rank + p.S * warp; it < items && !*abort_flag; it += p.S * kWarps) {
-                const int rel = it / (2 * NTP), f = it - rel * 2 * NTP;
-                int32_t v[PL][4];
+        // the next run's first sign words are on their way while this one is finished
+        const int g_now = g, n_now = n;
+        g += n; n = min(p.run, g_hi - g);
+        if (g < g_hi) {
+            share();
+            if (it < it_end) load_w(wn, it);
+        }
+        if (SPLIT) { cluster_arrive_release(); cluster_wait_acquire(); }
+        else __syncthreads();
+        // ---- epilogue: the fragments of the run, dealt to the warps (of the whole cluster)
+        for (int f = SPLIT ? rank * kWarps + warp : warp; f < n_now * 2 * NTP && !failed; f += (SPLIT ? p.S : 1) * kWarps) {
+            const int grp = f / (2 * NTP), rest = f - grp * 2 * NTP, mt = rest / NTP, nt = rest - mt * NTP;
+            int32_t v[PL][4];
 #pragma unroll
-                for (int pl = 0; pl < PL; ++pl) {
-                    const uint32_t at = csum + (uint32_t)((it * PL + pl) * 512);
-                    uint4 q[8];
+            for (int pl = 0; pl < PL; ++pl) {
+                int32_t* at = accs + ((grp * 2 + mt) * NT + pl * NTP + nt) * 128 + lane;
 #pragma unroll
-                    for (int s = 0; s < 8; ++s)
-                        if (s < p.S) q[s] = ld_shared_cluster_v4(map_shared_rank(at, (uint32_t)s));
-                    v[pl][0] = v[pl][1] = v[pl][2] = v[pl][3] = 0;
+                for (int e = 0; e < 4; ++e) {
+                    if (!SPLIT) {
+                        v[pl][e] = at[32 * e];
+                        at[32 * e] = 0;
+                    } else {
+                        const uint32_t a = smem_u32(at + 32 * e);
+                        int32_t q[8];
 #pragma unroll
-                    for (int s = 0; s < 8; ++s)
-                        if (s < p.S) { v[pl][0] += (int32_t)q[s].x; v[pl][1] += (int32_t)q[s].y; v[pl][2] += (int32_t)q[s].z; v[pl][3] += (int32_t)q[s].w; }
+                        for (int s = 0; s < 8; ++s)
+                            if (s < p.S) q[s] = ld_cluster_s32(map_shared_rank(a, (uint32_t)s));
+                        v[pl][e] = 0;
+#pragma unroll
+                        for (int s = 0; s < 8; ++s)
+                            if (s < p.S) v[pl][e] += q[s];
+                    }
                 }
-                epilogue(cl + (first + rel / RW) * clusters, rel % RW, f & 1, f >> 1, v);
             }
-            cluster_arrive_release(); cluster_wait_acquire();       // everybody has read: the buffers may be written again
+            epilogue(g_now + grp, mt, nt, v);
+        }
+        if (SPLIT) {
+            cluster_arrive_release(); cluster_wait_acquire();       // everybody has read
+            if (g < g_hi) {
+                for (int i = tid; i < n_now * 2 * NT * 32; i += kThreads) reinterpret_cast<uint4*>(accs)[i] = make_uint4(0u, 0u, 0u, 0u);
+                __syncthreads();
+            }
+        } else if (g < g_hi) {
+            __syncthreads();
         }
     }
-    if (*abort_flag) for (int i = 0; i < 500; ++i) __nanosleep(100);   // let copies in flight land
 }
 
 // ---------------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------------
-struct SmallPlan { int S, KW, stages, flush, ring_off, t_off, tok_off, red_off, csum_off, smem; int clusters[kRotMaxProblems]; };
+struct SmallPlan { int S, run, t_off, tok_off, acc_off, smem; int clusters[kRotMaxProblems]; };
 
 static int token_tiles(int64_t M) { return M <= 8 ? 1 : M <= 16 ? 2 : M <= 32 ? 4 : 8; }
-static int tile_rows(int NT, int KW) { return 32 * (small_::kWarps / (KW * small_::token_warps(NT))); }
-
-// Shared memory for S CTAs per cluster and KW K slices; false when it does not fit.
-static bool small_layout(int NTP, int PL, int units, int S, int KW, bool lowrank, int rounds, int most_stages, SmallPlan* out) {
-    using namespace small_;
-    const int NT = NTP * PL, tok = 8 * NT, ch = PL == 3 || NTP / token_warps(NT) < 2 ? 1 : 2, rows = tile_rows(NT, KW);
-    SmallPlan pl{};
-    pl.S = S; pl.KW = KW;
-    int off = ((units + S - 1) / S) * kSteps * tok * 128;
-    pl.t_off = off; off += lowrank ? 3 * 8 * NTP * 128 : 0;
-    pl.red_off = off; off += kWarps * 2 * ch * PL * 512;
-    pl.csum_off = off;
-    pl.flush = 1;
-    const int stage = rows * 128, per_round = rows / 32 * 2 * NT * 512, tok_bytes = (12 * tok + 1023) / 1024 * 1024;
-    if (S > 1) {
-        pl.flush = std::max(1, std::min(rounds, (kSmemMax - off - tok_bytes - 4 * stage) / per_round));
-        off += pl.flush * per_round;
-    }
-    pl.tok_off = off; off += tok_bytes;
-    pl.ring_off = off = (off + 1023) / 1024 * 1024;
-    pl.stages = std::min(std::min(kMaxStages, most_stages), (kSmemMax - off) / stage);
-    if (pl.stages < std::min(2, most_stages)) return false;
-    pl.smem = off + pl.stages * stage + 1024;
-    *out = pl;
-    return true;
-}
 
 // How many clusters of S such CTAs the device holds at once.  (Clusters are placed inside a GPC, so this is less than SMs / S:
 // asked once per size and thread.)
@@ -419,71 +382,74 @@ static int resident_small_clusters(int S) {
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
     if (known_dev != dev) { for (int& k : known) k = -1; known_dev = dev; }
     if (known[S] < 0) {
-        auto kernel = gemm_small_kernel<2, 1, 4, true>;
+        auto kernel = gemm_small_kernel<2, 1, true>;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)(S * sm_count()), 1, 1);
         cfg.blockDim = dim3(small_::kThreads, 1, 1);
-        cfg.dynamicSmemBytes = small_::kSmemMax + 1024;
+        cfg.dynamicSmemBytes = small_::kSmemMax;
         cudaLaunchAttribute a[1];
         a[0].id = cudaLaunchAttributeClusterDimension;
         a[0].val.clusterDim.x = (unsigned)S; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
         cfg.attrs = a; cfg.numAttrs = 1;
         int n = 0;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, small_::kSmemMax + 1024) != cudaSuccess ||
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, small_::kSmemMax) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
         known[S] = n;
     }
     return known[S];
 }
 
-// Picks S and KW by an estimate of cycles: rounds x (stages per tile x MMA or ALU cycles of the 16 warps, plus the reduction
-// and epilogue of a round), plus filling the CTA's codes from the L2, plus the cluster barriers.
+// Picks S by an estimate of cycles: the items of the longest run chain at the measured rate of the loop (32 and 52 cycles per
+// 128 k, row group and scheduler-quarter at 8 and 16 tokens), a round of barriers and epilogue per run, filling the CTA's codes from
+// the L2, and the cluster's barriers.
 static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int n, bool lowrank, int sms, SmallPlan* best) {
     using namespace small_;
-    const int NT = NTP * PL;
+    const int NT = NTP * PL, tok = 8 * NT;
     double best_cost = 0.0;
     bool found = false;
-    for (int KW = 4; KW <= 8; KW *= 2)
-        for (int S = 1; S <= 8 && S <= units; ++S) {
-            const int rows = tile_rows(NT, KW);
-            const int per_cta = (units + S - 1) / S;
-            if (per_cta * kSteps * 8 * NT * 128 > kSmemMax) continue;
-            const int total = S == 1 ? sms : resident_small_clusters(S);      // clusters the device holds
-            if (total < n) break;
-            int tiles[kRotMaxProblems], cl[kRotMaxProblems], used = 0, rounds = 1;
-            int64_t all = 0;
-            for (int i = 0; i < n; ++i) { tiles[i] = (int)((N[i] + rows - 1) / rows); all += tiles[i]; }
-            // clusters per problem, by row tiles: at least one each, never more than tiles
-            for (int i = 0; i < n; ++i) {
-                cl[i] = (int)std::max<int64_t>(1, std::min<int64_t>(tiles[i], (int64_t)total * tiles[i] / all));
-                used += cl[i];
-            }
-            while (used > total) {                                    // (only through the minimum of one each)
-                int big = 0;
-                for (int i = 1; i < n; ++i) if (cl[i] > cl[big]) big = i;
-                --cl[big]; --used;
-            }
-            while (used < total) {                                    // what is left goes to whoever has most rounds
-                int worst = -1, wr = 1;
-                for (int i = 0; i < n; ++i) {
-                    const int r = (tiles[i] + cl[i] - 1) / cl[i];
-                    if (r > wr) { wr = r; worst = i; }
-                }
-                if (worst < 0) break;
-                ++cl[worst]; ++used;
-            }
-            for (int i = 0; i < n; ++i) rounds = std::max(rounds, (tiles[i] + cl[i] - 1) / cl[i]);
-            SmallPlan pl;
-            if (!small_layout(NTP, PL, units, S, KW, lowrank, rounds, rounds * per_cta, &pl)) continue;
-            // a stage is kSteps steps of the row groups: 4 x 2 x NT MMAs of 2 cycles, or about 60 ALU instructions of half a cycle
-            const double stage_cycles = kSteps * (rows / 32) * (NT == 1 ? 32.0 : 16.0 * NT + 6.0);
-            const double cost = rounds * (per_cta * stage_cycles + 900.0) + per_cta * kSteps * 8.0 * NT * 128.0 / 40.0 +
-                                (S > 1 ? 2500.0 * ((rounds + pl.flush - 1) / pl.flush) : 0.0);
-            if (!found || cost < best_cost) {
-                best_cost = cost; *best = pl; found = true;
-                for (int i = 0; i < n; ++i) best->clusters[i] = cl[i];
-            }
+    for (int S = 1; S <= 8 && S <= units; ++S) {
+        const int per_cta = (units + S - 1) / S;
+        SmallPlan pl{};
+        pl.S = S;
+        int off = per_cta * kSteps * tok * 128;
+        pl.t_off = off; off += lowrank ? 3 * 8 * NTP * 128 : 0;
+        pl.tok_off = off; off += (12 * tok + 15) / 16 * 16;
+        pl.acc_off = off;
+        const int group_bytes = 2 * NT * 512;
+        const int fit = (kSmemMax - off) / group_bytes;
+        if (fit < 1) continue;
+        const int total = S == 1 ? sms : resident_small_clusters(S);      // clusters the device holds
+        if (total < n) break;
+        int groups[kRotMaxProblems], used = 0, longest = 1;
+        int64_t all = 0;
+        for (int i = 0; i < n; ++i) { groups[i] = (int)((N[i] + 31) / 32); all += groups[i]; }
+        // clusters per problem, by row groups: at least one each, never more than groups
+        for (int i = 0; i < n; ++i) {
+            pl.clusters[i] = (int)std::max<int64_t>(1, std::min<int64_t>(groups[i], (int64_t)total * groups[i] / all));
+            used += pl.clusters[i];
         }
+        while (used > total) {                                    // (only through the minimum of one each)
+            int big = 0;
+            for (int i = 1; i < n; ++i) if (pl.clusters[i] > pl.clusters[big]) big = i;
+            --pl.clusters[big]; --used;
+        }
+        auto chain = [&](int i) { return (groups[i] + pl.clusters[i] - 1) / pl.clusters[i]; };
+        while (used < total) {                                    // what is left goes to whoever has the longest chain
+            int worst = 0;
+            for (int i = 1; i < n; ++i) if (chain(i) > chain(worst)) worst = i;
+            if (chain(worst) == 1) break;
+            ++pl.clusters[worst]; ++used;
+        }
+        for (int i = 0; i < n; ++i) longest = std::max(longest, chain(i));
+        pl.run = std::min(longest, fit);
+        pl.smem = off + pl.run * group_bytes;
+        const double step = NT == 1 ? 30.0 : 22.0 * NT + 8.0;     // cycles per SM and code row of an item
+        const int runs = (longest + pl.run - 1) / pl.run;
+        auto items = [&](int g) { return (double)((g * token_parts(NT) * per_cta + kWarps - 1) / kWarps) * kWarps / token_parts(NT); };
+        const double cost = (runs - 1) * items(pl.run) * kSteps * step + items(longest - (runs - 1) * pl.run) * kSteps * step +
+                            runs * (1500.0 + 60.0 * NT * pl.run / S) + per_cta * kSteps * tok * 128 / 40.0 + (S > 1 ? 1500.0 + 1000.0 * runs : 0.0);
+        if (!found || cost < best_cost) { best_cost = cost; *best = pl; found = true; }
+    }
     return found;
 }
 
@@ -513,7 +479,7 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     const int sms = sm_count();
     Known& slot = known[used % 16];
     slot.k = k;
-    slot.ok = sms > 0 && encode_tiled_fn() && small_plan_search(k.NTP, k.PL, k.units, k.N, n, k.lowrank != 0, sms, &slot.plan);
+    slot.ok = sms > 0 && small_plan_search(k.NTP, k.PL, k.units, k.N, n, k.lowrank != 0, sms, &slot.plan);
     ++used;
     *out = slot.plan;
     return slot.ok;
@@ -524,14 +490,14 @@ bool gemm_small_fits(const GemmArgs* a, int n, int planes) {
     return small_plan(a, n, planes, &pl);
 }
 
-template <int NTP, int PL, int KW, bool SPLIT>
-static int launch_small_t(const SmallMaps& maps, const SmallParams& p, int grid, int smem, cudaStream_t stream) {
-    auto kernel = gemm_small_kernel<NTP, PL, KW, SPLIT>;
+template <int NTP, int PL, bool SPLIT>
+static int launch_small_t(const SmallParams& p, int grid, int smem, cudaStream_t stream) {
+    auto kernel = gemm_small_kernel<NTP, PL, SPLIT>;
     static thread_local int configured = -1;
     int dev = 0;
     BWLA_CUDA_TRY(cudaGetDevice(&dev));
     if (configured != dev) {
-        BWLA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, small_::kSmemMax + 1024));
+        BWLA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, small_::kSmemMax));
         configured = dev;
     }
     cudaLaunchConfig_t cfg{};
@@ -547,14 +513,13 @@ static int launch_small_t(const SmallMaps& maps, const SmallParams& p, int grid,
     cfg.attrs = attrs;
     cfg.numAttrs = SPLIT ? 2 : 1;
     ProfScope prof(kProfContraction, stream);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, maps, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
     if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e); }
     return after_launch();
 }
 template <int NTP, int PL>
-static int launch_small_nt(const SmallMaps& maps, const SmallParams& p, int KW, int grid, int smem, cudaStream_t stream) {
-    if (KW == 4) return p.S > 1 ? launch_small_t<NTP, PL, 4, true>(maps, p, grid, smem, stream) : launch_small_t<NTP, PL, 4, false>(maps, p, grid, smem, stream);
-    return p.S > 1 ? launch_small_t<NTP, PL, 8, true>(maps, p, grid, smem, stream) : launch_small_t<NTP, PL, 8, false>(maps, p, grid, smem, stream);
+static int launch_small_nt(const SmallParams& p, int grid, int smem, cudaStream_t stream) {
+    return p.S > 1 ? launch_small_t<NTP, PL, true>(p, grid, smem, stream) : launch_small_t<NTP, PL, false>(p, grid, smem, stream);
 }
 
 // All problems have the same M, K and bits; a[i].codes: int8 [planes][M][K] in the interleaved order; a[i].Thl: bf16 [3][M][64].
@@ -565,40 +530,31 @@ int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStr
     if (!*taken) return BWLA_OK;
     const int M = (int)a[0].M, K = (int)a[0].K, NTP = token_tiles(M);
     SmallParams p{};
-    SmallMaps maps;
-    p.n_problems = n; p.M = M; p.K = K; p.units = (K + small_::kUnit - 1) / small_::kUnit; p.S = pl.S; p.stages = pl.stages; p.flush = pl.flush;
-    p.ring_off = pl.ring_off; p.t_off = pl.t_off; p.tok_off = pl.tok_off; p.red_off = pl.red_off; p.csum_off = pl.csum_off;
+    p.n_problems = n; p.M = M; p.K = K; p.units = (K + small_::kUnit - 1) / small_::kUnit; p.S = pl.S; p.run = pl.run;
+    p.t_off = pl.t_off; p.tok_off = pl.tok_off; p.acc_off = pl.acc_off;
     p.status = a[0].status;
-    const int rows = tile_rows(NTP * planes, pl.KW);
     int begin = 0;
     for (int i = 0; i < n; ++i) {
         SmallProblem& q = p.prob[i];
-        q.codes = a[i].codes; q.scales = a[i].scales; q.qsum = a[i].qsum; q.zp = a[i].zp; q.rowsum = a[i].rowsum;
+        q.packed = a[i].packed; q.codes = a[i].codes; q.scales = a[i].scales; q.qsum = a[i].qsum; q.zp = a[i].zp; q.rowsum = a[i].rowsum;
         q.alpha = a[i].alpha; q.mu = a[i].mu; q.U = (const __nv_bfloat16*)a[i].U; q.Thl = (const __nv_bfloat16*)a[i].Thl;
         q.out = (__nv_bfloat16*)a[i].out; q.ldo = a[i].ldo; q.acc_debug = a[i].acc_debug;
-        q.N = (int)a[i].N; q.r = a[i].r; q.tiles = ((int)a[i].N + rows - 1) / rows; q.cluster_begin = begin; q.clusters = pl.clusters[i];
+        q.N = (int)a[i].N; q.r = a[i].r; q.groups = ((int)a[i].N + 31) / 32; q.cluster_begin = begin; q.clusters = pl.clusters[i];
         begin += pl.clusters[i];
-        const uint64_t dims[2] = {(uint64_t)K / 32, (uint64_t)a[i].N};
-        const uint64_t strides[1] = {(uint64_t)K / 8};
-        const uint32_t box[2] = {32, (uint32_t)rows};
-        int st = make_map(&maps.w[i], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, a[i].packed, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-        if (st != BWLA_OK) return st;
     }
-    for (int i = n; i < kRotMaxProblems; ++i) maps.w[i] = maps.w[0];
     const int grid = begin * pl.S;
     if (planes == 3) {
         switch (NTP) {
-            case 1: return launch_small_nt<1, 3>(maps, p, pl.KW, grid, pl.smem, stream);
-            case 2: return launch_small_nt<2, 3>(maps, p, pl.KW, grid, pl.smem, stream);
-            default: return launch_small_nt<4, 3>(maps, p, pl.KW, grid, pl.smem, stream);
+            case 1: return launch_small_nt<1, 3>(p, grid, pl.smem, stream);
+            case 2: return launch_small_nt<2, 3>(p, grid, pl.smem, stream);
+            default: return launch_small_nt<4, 3>(p, grid, pl.smem, stream);
         }
     }
     switch (NTP) {
-        case 1: return launch_small_nt<1, 1>(maps, p, pl.KW, grid, pl.smem, stream);
-        case 2: return launch_small_nt<2, 1>(maps, p, pl.KW, grid, pl.smem, stream);
-        case 4: return launch_small_nt<4, 1>(maps, p, pl.KW, grid, pl.smem, stream);
-        default: return launch_small_nt<8, 1>(maps, p, pl.KW, grid, pl.smem, stream);
+        case 1: return launch_small_nt<1, 1>(p, grid, pl.smem, stream);
+        case 2: return launch_small_nt<2, 1>(p, grid, pl.smem, stream);
+        case 4: return launch_small_nt<4, 1>(p, grid, pl.smem, stream);
+        default: return launch_small_nt<8, 1>(p, grid, pl.smem, stream);
     }
 }
 

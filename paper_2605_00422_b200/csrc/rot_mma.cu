@@ -55,9 +55,30 @@ static_assert(sizeof(RotShared) <= kRotRedBytes, "RotShared");
 
 static int round_to(int v, int m) { return (v + m - 1) / m * m; }
 
+// A warp may have ntw column tiles at most; `alias`: Z^T takes the place of x, which is dead by then (the next token's x then
+// arrives late, which costs about a fifth).  Fills in what follows from dc and alias; false when it does not fit.
+static bool rot_layout(RotGeom& g, int dc, int alias, int pad) {
+    const int tiles = g.n2p / 16;
+    g.dtc = (tiles + dc - 1) / dc;
+    g.warps = g.dtc * g.cw;
+    if (g.warps > kRotMaxWarps || (dc - 1) * g.dtc >= tiles || dc * g.warps > 64) return false;
+    // Rows of an odd number of 16-byte chunks (pad 16): the eight rows of an ldmatrix then fall into different banks.  The
+    // largest factors only fit without that padding, and without the rows of x beyond n1.
+    g.pad = pad;
+    g.s2 = g.n2p * 2 + pad; g.s1 = g.na * 16 + pad;
+    const int x = (pad ? g.cw * g.ntw * 8 : g.n1) * g.s2, z = g.cw > 1 ? 2 * g.dtc * 16 * g.s1 : 0;
+    g.dc = dc; g.alias_z = alias;
+    g.p1_off = 3 * g.dtc * 16 * g.s2;
+    g.group_off = g.p1_off + 2 * g.na * 8 * g.s1;
+    g.group_bytes = (alias ? std::max(x, z) : x + z) + kRotRedBytes;
+    g.z_rel = alias ? 0 : x; g.red_rel = g.group_bytes - kRotRedBytes;
+    if (g.group_off + g.group_bytes > kRotMaxSmem) return false;
+    g.max_groups = dc == 1 ? std::min(std::min(kRotMaxWarps / g.warps, 8), (kRotMaxSmem - g.group_off) / g.group_bytes) : 1;   // (barriers 1..8)
+    return true;
+}
+
 // Chooses the split of a token over warps and CTAs: the one that keeps most warps busy on an SM (16 is what the registers
-// allow), counting that the last CTA of a cluster may have fewer rows.  Z^T may take the place of x, which is dead by then,
-// where both do not fit; the next token's x then arrives late, which costs about a fifth.
+// allow), counting that the last CTA of a cluster may have fewer rows.
 bool rot_geometry(int n1, int n2, RotGeom* out) {
     if (n1 < 1 || n2 < 8 || n2 % 8 != 0 || n2 > 256 || n1 > 192) return false;
     RotGeom g{};
@@ -65,39 +86,38 @@ bool rot_geometry(int n1, int n2, RotGeom* out) {
     g.n2p = round_to(n2, 16); g.na = round_to(n1, 16) / 8;
     g.cw = g.na <= 8 ? 1 : g.na <= 16 ? 2 : 4;
     g.ntw = (g.na + g.cw - 1) / g.cw;                         // (the last warp may have tiles beyond na, which it ignores)
-    const int tiles = g.n2p / 16;
     double best = 0.0;
-    // Rows of an odd number of 16-byte chunks: the eight rows of an ldmatrix then fall into different banks.  The largest
-    // factors only fit without that padding, and without the rows of x beyond n1.
-    for (int pad = 16; pad >= 0 && best == 0.0; pad -= 16) {
-        g.s2 = g.n2p * 2 + pad; g.s1 = g.na * 16 + pad;
-        const int p1 = 2 * g.na * 8 * g.s1, x = (pad ? g.cw * g.ntw * 8 : n1) * g.s2;
+    for (int pad = 16; pad >= 0 && best == 0.0; pad -= 16)
         for (int dc = 1; dc <= 8; ++dc)
             for (int alias = 0; alias <= (g.cw > 1 ? 1 : 0); ++alias) {
-                const int dtc = (tiles + dc - 1) / dc, warps = dtc * g.cw;
-                if (warps > kRotMaxWarps || (dc - 1) * dtc >= tiles || dc * warps > 64) continue;
-                const int consts = 3 * dtc * 16 * g.s2 + p1, z = g.cw > 1 ? 2 * dtc * 16 * g.s1 : 0;
-                const int group = (alias ? std::max(x, z) : x + z) + kRotRedBytes;
-                if (consts + group > kRotMaxSmem) continue;
-                int groups = 1, ctas = 1;
-                if (dc == 1) groups = std::min(std::min(kRotMaxWarps / warps, 8), (kRotMaxSmem - consts) / group);   // (barriers 1..8)
-                else ctas = std::min(kRotMaxWarps / warps, (kRotMaxSmem + 1024) / (consts + group + 1024));
-                const double score = (double)tiles * g.cw / dc * groups * ctas * (alias ? 0.8 : 1.0);
-                if (score > best * 1.001) {
-                    best = score;
-                    g.dc = dc; g.dtc = dtc; g.alias_z = alias; g.max_groups = groups; g.warps = warps;
-                    g.p1_off = 3 * dtc * 16 * g.s2; g.group_off = consts; g.group_bytes = group;
-                    g.z_rel = alias ? 0 : x; g.red_rel = group - kRotRedBytes;
-                }
+                RotGeom t = g;
+                if (!rot_layout(t, dc, alias, pad)) continue;
+                const int ctas = dc == 1 ? 1 : std::min(kRotMaxWarps / t.warps, (kRotMaxSmem + 1024) / (t.group_off + t.group_bytes + 1024));
+                const double score = (double)(g.n2p / 16) * g.cw / dc * t.max_groups * ctas * (alias ? 0.8 : 1.0);
+                if (score > best * 1.001) { best = score; *out = t; }
             }
+    return best != 0.0;
+}
+
+// Few tokens: what counts is the time of one token, so it is spread over more warps (up to 64 columns: two warps instead of
+// one) and, while every cluster finds SMs of its own, over more CTAs: MMAs of a CTA at 2 cycles each, against about 2000
+// cycles for the cluster's barriers.
+static RotGeom few_tokens_geometry(const RotGeom& base, int64_t clusters, int sms) {
+    RotGeom best = base;
+    double best_cost = 0.0;
+    const int ksteps = base.n2p / 16 + base.na / 2;
+    for (int dc = 1; dc <= 8 && clusters * dc <= sms; ++dc) {
+        RotGeom t = base;
+        if (t.na > 4 && t.na <= 8) { t.cw = 2; t.ntw = 4; }
+        if (!rot_layout(t, dc, 0, base.pad) && (t.cw == 1 || !rot_layout(t, dc, 1, base.pad))) continue;
+        const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 2000.0 : 0.0);
+        if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = t; }
     }
-    if (best == 0.0) return false;
-    *out = g;
-    return true;
+    return best;
 }
 
 size_t rot_prepared_bytes(const RotGeom& g) {
-    return kRotHeader + (size_t)3 * g.dc * g.dtc * 16 * g.s2 + (size_t)2 * g.na * 8 * g.s1;
+    return kRotHeader + (size_t)3 * g.n2p * g.s2 + (size_t)2 * g.na * 8 * g.s1;
 }
 
 // Exponent by which P1 is scaled: its largest magnitude goes to [2^13, 2^14).
@@ -166,7 +186,7 @@ __global__ void __launch_bounds__(256) prepare_rot_kernel(RotGeom g, const float
     __shared__ uint32_t red[8];
     const int e2 = exponent_of(block_absmax(P2, g.n2 * g.n2, red)), e1 = factor_exponent(block_absmax(P1, g.n1 * g.n1, red));
     if (blockIdx.x == 0 && threadIdx.x == 0) { reinterpret_cast<int*>(prepared)[0] = e2; reinterpret_cast<int*>(prepared)[1] = e1; }
-    const int rows2 = g.dc * g.dtc * 16, rows1 = g.na * 8;
+    const int rows2 = g.n2p, rows1 = g.na * 8;
     uint8_t* t2 = prepared + kRotHeader;
     uint8_t* t1 = t2 + (size_t)3 * rows2 * g.s2;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
@@ -243,9 +263,10 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     int e2, e1;
     if (pr.prepared) {
         const uint8_t* t2 = pr.prepared + kRotHeader + (size_t)rank * part2;
-        const size_t all2 = (size_t)g.dc * part2;
+        const size_t all2 = (size_t)g.n2p * g.s2;                     // (the last CTA of a cluster may have fewer rows)
+        const int own2 = min(part2, (g.n2p - rank * rows2) * g.s2);
         const uint8_t* t1 = pr.prepared + kRotHeader + 3 * all2;
-        for (int i = 16 * threadIdx.x; i < part2; i += 16 * blockDim.x) {
+        for (int i = 16 * threadIdx.x; i < own2; i += 16 * blockDim.x) {
             cp_async16(smem_u32(p2s + i), t2 + i);
             cp_async16(smem_u32(p2s + part2 + i), t2 + all2 + i);
             cp_async16(smem_u32(p2s + 2 * part2 + i), t2 + 2 * all2 + i);
@@ -268,6 +289,12 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         if (g.n2p != g.n2)
             for (int i = tid; i < g.n1; i += T) *reinterpret_cast<uint4*>(xs + i * g.s2 + 16 * cpr) = make_uint4(0u, 0u, 0u, 0u);
     };
+    // x may be what the preceding kernel is writing, so it is read only behind the wait below; but its lines can be asked into the
+    // L2, where those writes go anyway: address translation and, where x is older, the trip to HBM are over by then
+    if (tok0 < p.M) {
+        const uint8_t* xt = reinterpret_cast<const uint8_t*>(p.x) + tok0 * p.ldx * (F32 ? 4 : 2);
+        for (int i = 128 * tid; i < g.K * (F32 ? 4 : 2); i += 128 * T) prefetch_l2_line(xt + i);
+    }
     zero_padding();
     for (int i = tid; i < (int)(sizeof(RotShared) / 4); i += T) reinterpret_cast<uint32_t*>(&sh)[i] = 0u;
     __syncthreads();
@@ -275,12 +302,6 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     griddep_launch_dependents();
     griddep_wait();                                   // x may be the output of the preceding kernel
     int ntok = tok0 < p.M ? (int)((p.M - tok0 + stride - 1) / stride) : 0;
-    if (MODE == kRotBinarize) {
-        if (b == 0 && threadIdx.x < kStatusBytes / 4) p.status[threadIdx.x] = 0u;     // this call clears its status words itself
-    } else if (p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) {
-        ntok = 0;                                                                     // the call already failed
-    }
-
     // this thread's chunks of X: tid, tid + T, ...; (row, column) advance without divisions
     const int ch_a0 = tid / cpr, ch_c0 = tid - ch_a0 * cpr, ch_da = T / cpr, ch_dc = T - ch_da * cpr;
     auto for_chunks = [&](auto&& f) {
@@ -492,7 +513,16 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         }
     };
 
-    // Pass -1 only fetches the first token's x.
+    // (the look at the status word takes a trip to the L2: the first token's x is on its way by then)
+    if (!F32 && ntok > 0) fetch_x(tok0);
+    const int first_tokens = ntok;
+    if (MODE == kRotBinarize) {
+        if (b == 0 && threadIdx.x < kStatusBytes / 4) p.status[threadIdx.x] = 0u;     // this call clears its status words itself
+    } else if (p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) {
+        ntok = 0;                                                                     // the call already failed
+    }
+    if (ntok < first_tokens) cp_async_wait_all();
+    // Pass -1 only takes in the first token's x.
 #pragma unroll 1
     for (int it = F32 ? 0 : -1; it < ntok; ++it) {
         const int par = it & 1;
@@ -522,7 +552,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         if (it > 0) flush_qsum(t - stride, par ^ 1);
         }
         const bool fetch_late = EXCH && g.alias_z;
-        if (!F32 && more && (!live || !fetch_late)) fetch_x(t + stride);
+        if (!F32 && more && live && !fetch_late) fetch_x(t + stride);
         // ---- the two fp16 terms of Z^T: accumulators of two column tiles are one A operand (16 values of a)
         const int ex = exponent_of(__uint_as_float(slots_max(sh.xmax[par])));
         const int z_exp = max(-126, min(126, 15 - (32 - __clz(g.n2 - 1)) - (e2 + 1) - (ex + 1)));
@@ -861,6 +891,7 @@ static RotKernel pick_kernel(const RotGeom& g) {
     if (g.cw == 1)
         return g.ntw <= 2 ? rot_mma_kernel<2, false, MODE, F32> : g.ntw <= 4 ? rot_mma_kernel<4, false, MODE, F32>
              : g.ntw <= 6 ? rot_mma_kernel<6, false, MODE, F32> : rot_mma_kernel<8, false, MODE, F32>;
+    if (MODE != kRotBinarize && g.ntw <= 4) return rot_mma_kernel<MODE == kRotBinarize ? 5 : 4, true, MODE, F32>;
     return g.ntw <= 5 ? rot_mma_kernel<5, true, MODE, F32> : g.ntw <= 6 ? rot_mma_kernel<6, true, MODE, F32>
          : g.ntw <= 7 ? rot_mma_kernel<7, true, MODE, F32> : rot_mma_kernel<8, true, MODE, F32>;
 }
@@ -934,9 +965,10 @@ static int launch_rot_kernel(RotKernel k, const RotGeom& g, RotKernelParams& p, 
     return after_launch();
 }
 
-int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
+int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream) {
     if (M == 0 || n_problems == 0) return BWLA_OK;
+    const RotGeom g = M * n_problems <= sm_count() ? few_tokens_geometry(base, M * n_problems, sm_count()) : base;
     if (n_problems > kRotMaxProblems || M >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
     RotKernelParams p{};
     p.g = g; p.x = x; p.ldx = ldx; p.x_vec = rot_accepts_x(x, ldx); p.M = M; p.bits = bits; p.asym = asym; p.n_problems = n_problems;

@@ -41,6 +41,7 @@ __device__ __forceinline__ void add4(float (&c)[4], const float (&t)[4]) {
     add2(c[0], c[1], t[0], t[1]);
     add2(c[2], c[3], t[2], t[3]);
 }
+__device__ __forceinline__ void prefetch_l2_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void named_barrier(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
