@@ -181,24 +181,28 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
     cp_async_wait_all();
     __syncthreads();
 
-    // one fragment (16 rows x 8 tokens) of a finished group
-    auto epilogue = [&](int grp, int mt, int nt, const int32_t (&v)[PL][4]) {
+    // ---- epilogue of one fragment (16 rows x 8 tokens), in two halves: what it needs from global memory is requested a fragment
+    //      ahead (an L2 round trip each otherwise: rows of U, then the scales, then the shifts)
+    struct Rows { uint32_t ul[8], uh[8]; float al[2], mu[2]; int32_t rs[2]; };
+    const bool u_vec = (pr.r & 7) == 0 && (reinterpret_cast<uintptr_t>(pr.U) & 15) == 0;
+    auto fetch_rows = [&](Rows& w, int grp, int mt) {
         const int n_lo = grp * 32 + 16 * mt + gq, n_hi = n_lo + 8;
         const bool ok_lo = n_lo < pr.N, ok_hi = n_hi < pr.N;
-        float lr[4] = {0.f, 0.f, 0.f, 0.f};
+        w.al[0] = ok_lo ? __ldg(pr.alpha + n_lo) : 0.f; w.al[1] = ok_hi ? __ldg(pr.alpha + n_hi) : 0.f;
+        w.mu[0] = pr.mu && ok_lo ? __ldg(pr.mu + n_lo) : 0.f; w.mu[1] = pr.mu && ok_hi ? __ldg(pr.mu + n_hi) : 0.f;
+        w.rs[0] = pr.zp && ok_lo ? __ldg(pr.rowsum + n_lo) : 0; w.rs[1] = pr.zp && ok_hi ? __ldg(pr.rowsum + n_hi) : 0;
         if (pr.r > 0) {
             // U T with the 64 columns dealt to the quad's lanes, 16 each (a sum does not care in which order)
-            uint32_t ul[8], uh[8];
             const __nv_bfloat16* u_lo = pr.U + (int64_t)(ok_lo ? n_lo : 0) * pr.r + 16 * tq;
             const __nv_bfloat16* u_hi = pr.U + (int64_t)(ok_hi ? n_hi : 0) * pr.r + 16 * tq;
-            if ((pr.r & 7) == 0 && (reinterpret_cast<uintptr_t>(pr.U) & 15) == 0) {
+            if (u_vec) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const bool in = 16 * tq + 8 * h < pr.r;
                     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
                     const uint4 a = in ? __ldg(reinterpret_cast<const uint4*>(u_lo) + h) : z, b = in ? __ldg(reinterpret_cast<const uint4*>(u_hi) + h) : z;
-                    ul[4 * h] = a.x; ul[4 * h + 1] = a.y; ul[4 * h + 2] = a.z; ul[4 * h + 3] = a.w;
-                    uh[4 * h] = b.x; uh[4 * h + 1] = b.y; uh[4 * h + 2] = b.z; uh[4 * h + 3] = b.w;
+                    w.ul[4 * h] = a.x; w.ul[4 * h + 1] = a.y; w.ul[4 * h + 2] = a.z; w.ul[4 * h + 3] = a.w;
+                    w.uh[4 * h] = b.x; w.uh[4 * h + 1] = b.y; w.uh[4 * h + 2] = b.z; w.uh[4 * h + 3] = b.w;
                 }
             } else {
 #pragma unroll
@@ -206,32 +210,39 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                     const int c0 = 16 * tq + 2 * c;
                     const uint32_t a0 = c0 < pr.r ? __bfloat16_as_ushort(u_lo[2 * c]) : 0u, a1 = c0 + 1 < pr.r ? __bfloat16_as_ushort(u_lo[2 * c + 1]) : 0u;
                     const uint32_t b0 = c0 < pr.r ? __bfloat16_as_ushort(u_hi[2 * c]) : 0u, b1 = c0 + 1 < pr.r ? __bfloat16_as_ushort(u_hi[2 * c + 1]) : 0u;
-                    ul[c] = a0 | (a1 << 16); uh[c] = b0 | (b1 << 16);
-                }
-            }
-            const uint32_t tb = smem_u32(smem) + p.t_off + (8 * nt + gq) * 128;
-#pragma unroll
-            for (int h = 2; h >= 0; --h) {             // small terms first
-                const uint4 x = lds128(tb + h * (8 * NTP * 128) + (((2 * tq) ^ gq) << 4)), y = lds128(tb + h * (8 * NTP * 128) + (((2 * tq + 1) ^ gq) << 4));
-                const uint32_t t8[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const uint32_t ua[4] = {ul[2 * kk], uh[2 * kk], ul[2 * kk + 1], uh[2 * kk + 1]};
-                    mma_16816<false>(lr, ua, t8[2 * kk], t8[2 * kk + 1], lr);
+                    w.ul[c] = a0 | (a1 << 16); w.uh[c] = b0 | (b1 << 16);
                 }
             }
         }
-        const float al[2] = {ok_lo ? __ldg(pr.alpha + n_lo) : 0.f, ok_hi ? __ldg(pr.alpha + n_hi) : 0.f};
-        const float mu[2] = {pr.mu && ok_lo ? __ldg(pr.mu + n_lo) : 0.f, pr.mu && ok_hi ? __ldg(pr.mu + n_hi) : 0.f};
-        const int32_t rs[2] = {pr.zp && ok_lo ? __ldg(pr.rowsum + n_lo) : 0, pr.zp && ok_hi ? __ldg(pr.rowsum + n_hi) : 0};
+    };
+    auto epilogue = [&](const Rows& w, int grp, int mt, int nt, const int32_t (&v)[PL][4]) {
+        const int n_lo = grp * 32 + 16 * mt + gq, n_hi = n_lo + 8;
+        float lr[3][4];                                // the three terms of T side by side: three short chains instead of a long one
+#pragma unroll
+        for (int h = 0; h < 3; ++h) lr[h][0] = lr[h][1] = lr[h][2] = lr[h][3] = 0.f;
+        if (pr.r > 0) {
+            const uint8_t* tb = smem + p.t_off + (8 * nt + gq) * 128;
+#pragma unroll
+            for (int h = 0; h < 3; ++h) {
+                const uint4 x = *reinterpret_cast<const uint4*>(tb + h * (8 * NTP * 128) + (((2 * tq) ^ gq) << 4));
+                const uint4 y = *reinterpret_cast<const uint4*>(tb + h * (8 * NTP * 128) + (((2 * tq + 1) ^ gq) << 4));
+                const uint32_t t8[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint32_t ua[4] = {w.ul[2 * kk], w.uh[2 * kk], w.ul[2 * kk + 1], w.uh[2 * kk + 1]};
+                    mma_16816<false>(lr[h], ua, t8[2 * kk], t8[2 * kk + 1], lr[h]);
+                }
+            }
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = 8 * nt + 2 * tq + (i & 1), h = i >> 1, n = h ? n_hi : n_lo;
+            const bool live = t < p.M && n < pr.N;
             const float sc = sc_s[t];
             float accf, qsf;
             if constexpr (PL == 1) {
-                const int32_t qs = qs_s[t], zp = zp_s[t], acc = 2 * v[0][i] - qs - zp * rs[h];
-                if (pr.acc_debug && t < p.M && (h ? ok_hi : ok_lo)) pr.acc_debug[(int64_t)t * pr.N + n] = acc;
+                const int32_t qs = qs_s[t], zp = zp_s[t], acc = 2 * v[0][i] - qs - zp * w.rs[h];
+                if (pr.acc_debug && live) pr.acc_debug[(int64_t)t * pr.N + n] = acc;
                 accf = (float)acc; qsf = (float)(qs - p.K * zp);
             } else {
                 // the low two digits' sums together are still exact in int32 (|sum of a digit| <= 128 K)
@@ -239,14 +250,12 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                 accf = fmaf((float)(2 * v[PL - 1][i] - q2), 65536.f, (float)(256 * (2 * v[PL / 2][i] - q1) + (2 * v[0][i] - q0)));
                 qsf = fmaf((float)q2, 65536.f, (float)(256 * q1 + q0));
             }
-            if (t < p.M && (h ? ok_hi : ok_lo) && pr.out) {
-                const float y = fmaf(__fmul_rn(mu[h], sc), qsf, __fmul_rn(__fmul_rn(al[h], sc), accf) + lr[i]);
+            if (live && pr.out) {
+                const float y = fmaf(__fmul_rn(w.mu[h], sc), qsf, __fmul_rn(__fmul_rn(w.al[h], sc), accf) + (lr[0][i] + (lr[1][i] + lr[2][i])));
                 pr.out[(int64_t)t * pr.ldo + n] = __float2bfloat16_rn(y);
             }
         }
     };
-
-
     const uint32_t b0 = smem_u32(smem) + (uint32_t)((tq * TOK + gq) * 128), b_swz = (uint32_t)((gq ^ (tq << 1)) << 4);
 #pragma unroll 1
     while (g < g_hi) {
@@ -319,8 +328,11 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                 u = 0; ++sub;
             }
         }
-        // the next run's first sign words are on their way while this one is finished
-        const int g_now = g, n_now = n;
+        // the next run's first sign words, and what the first fragment of this one needs, are on their way while the warps meet
+        const int g_now = g, n_now = n, frags = n_now * 2 * NTP, f_step = (SPLIT ? p.S : 1) * kWarps;
+        int f = SPLIT ? rank * kWarps + warp : warp;
+        Rows rows;
+        if (f < frags) fetch_rows(rows, g_now + f / (2 * NTP), f / NTP & 1);
         g += n; n = min(p.run, g_hi - g);
         if (g < g_hi) {
             share();
@@ -329,8 +341,11 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
         if (SPLIT) { cluster_arrive_release(); cluster_wait_acquire(); }
         else __syncthreads();
         // ---- epilogue: the fragments of the run, dealt to the warps (of the whole cluster)
-        for (int f = SPLIT ? rank * kWarps + warp : warp; f < n_now * 2 * NTP && !failed; f += (SPLIT ? p.S : 1) * kWarps) {
-            const int grp = f / (2 * NTP), rest = f - grp * 2 * NTP, mt = rest / NTP, nt = rest - mt * NTP;
+#pragma unroll 1
+        for (; f < frags && !failed; f += f_step) {
+            const int grp = f / (2 * NTP), mt = f / NTP & 1, nt = f % NTP;
+            const Rows now = rows;
+            if (f + f_step < frags) fetch_rows(rows, g_now + (f + f_step) / (2 * NTP), (f + f_step) / NTP & 1);
             int32_t v[PL][4];
 #pragma unroll
             for (int pl = 0; pl < PL; ++pl) {
@@ -353,7 +368,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                     }
                 }
             }
-            epilogue(g_now + grp, mt, nt, v);
+            epilogue(now, g_now + grp, mt, nt, v);
         }
         if (SPLIT) {
             cluster_arrive_release(); cluster_wait_acquire();       // everybody has read
@@ -402,7 +417,7 @@ static int resident_small_clusters(int S) {
 // Picks S by an estimate of cycles: the items of the longest run chain at the measured rate of the loop (32 and 52 cycles per
 // 128 k, row group and scheduler-quarter at 8 and 16 tokens), a round of barriers and epilogue per run, filling the CTA's codes from
 // the L2, and the cluster's barriers.
-static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int n, bool lowrank, int sms, SmallPlan* best) {
+static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int n, bool lowrank, int sms, int spare, SmallPlan* best) {
     using namespace small_;
     const int NT = NTP * PL, tok = 8 * NT;
     double best_cost = 0.0;
@@ -418,7 +433,7 @@ static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int 
         const int group_bytes = 2 * NT * 512;
         const int fit = (kSmemMax - off) / group_bytes;
         if (fit < 1) continue;
-        const int total = S == 1 ? sms : resident_small_clusters(S);      // clusters the device holds
+        const int total = std::min((sms - spare) / S, S == 1 ? sms : resident_small_clusters(S));      // clusters the device holds
         if (total < n) break;
         int groups[kRotMaxProblems], used = 0, longest = 1;
         int64_t all = 0;
@@ -456,7 +471,7 @@ static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int 
 // The plans of the shapes a thread has called lately: a decode loop asks for the same few on every step.
 static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     using namespace small_;
-    struct Key { int dev, NTP, PL, units, n, lowrank; int64_t N[kRotMaxProblems]; };
+    struct Key { int dev, NTP, PL, units, n, lowrank, spare; int64_t N[kRotMaxProblems]; };
     struct Known { Key k; bool ok; SmallPlan plan; };
     static thread_local Known known[16];
     static thread_local int used = 0;
@@ -470,8 +485,11 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     }
     if (cudaGetDevice(&k.dev) != cudaSuccess) { cudaGetLastError(); return false; }
     k.NTP = token_tiles(M); k.PL = planes; k.units = (int)((K + kUnit - 1) / kUnit); k.n = n;
+    // With very few tokens the rotation kernels before and after have a handful of CTAs: a few SMs are left to them, so that this
+    // kernel starts whole while the one before still runs, and the next one's constants arrive under this one.
+    k.spare = M <= 2 ? 8 : 0;
     auto same = [&](const Key& o) {
-        return o.dev == k.dev && o.NTP == k.NTP && o.PL == k.PL && o.units == k.units && o.n == k.n && o.lowrank == k.lowrank &&
+        return o.dev == k.dev && o.NTP == k.NTP && o.PL == k.PL && o.units == k.units && o.n == k.n && o.lowrank == k.lowrank && o.spare == k.spare &&
                std::equal(k.N, k.N + kRotMaxProblems, o.N);
     };
     for (int i = 0; i < 16 && i < used; ++i)
@@ -479,7 +497,7 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     const int sms = sm_count();
     Known& slot = known[used % 16];
     slot.k = k;
-    slot.ok = sms > 0 && small_plan_search(k.NTP, k.PL, k.units, k.N, n, k.lowrank != 0, sms, &slot.plan);
+    slot.ok = sms > 0 && small_plan_search(k.NTP, k.PL, k.units, k.N, n, k.lowrank != 0, sms, k.spare, &slot.plan);
     ++used;
     *out = slot.plan;
     return slot.ok;

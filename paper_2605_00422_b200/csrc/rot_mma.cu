@@ -100,8 +100,8 @@ bool rot_geometry(int n1, int n2, RotGeom* out) {
 }
 
 // Few tokens: what counts is the time of one token, so it is spread over more warps (up to 64 columns: two warps instead of
-// one) and, while every cluster finds SMs of its own, over more CTAs: MMAs of a CTA at 2 cycles each, against about 2000
-// cycles for the cluster's barriers.
+// one) and, while every cluster finds SMs of its own, over more CTAs: MMAs of a CTA at 2 cycles each, against about 5000
+// cycles for the cluster's barriers and its later start (64 x 128, one token: 6.7 us on eight CTAs, 5.2 on one).
 static RotGeom few_tokens_geometry(const RotGeom& base, int64_t clusters, int sms) {
     RotGeom best = base;
     double best_cost = 0.0;
@@ -110,7 +110,7 @@ static RotGeom few_tokens_geometry(const RotGeom& base, int64_t clusters, int sm
         RotGeom t = base;
         if (t.na > 4 && t.na <= 8) { t.cw = 2; t.ntw = 4; }
         if (!rot_layout(t, dc, 0, base.pad) && (t.cw == 1 || !rot_layout(t, dc, 1, base.pad))) continue;
-        const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 2000.0 : 0.0);
+        const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 5000.0 + 300.0 * dc : 0.0);
         if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = t; }
     }
     return best;
