@@ -76,11 +76,11 @@ static int resolve_path(int64_t M, int64_t K, int64_t N, int r, int bits) {
     return path;
 }
 
-static int run_contraction(int path, GemmArgs& g, const int8_t* codes, int busy, cudaStream_t stream) {
+static int run_contraction(int path, GemmArgs& g, const int8_t* codes, cudaStream_t stream) {
     g.codes = codes;
     if (path == BWLA_PATH_I8) {
         bool taken = false;
-        const int st = g.M <= kSmallTokens ? launch_gemm_small(&g, 1, 1, busy, &taken, stream) : BWLA_OK;
+        const int st = g.M <= kSmallTokens ? launch_gemm_small(&g, 1, 1, &taken, stream) : BWLA_OK;
         return taken ? st : launch_gemm_umma(g, codes, stream);
     }
     if (path == BWLA_PATH_BITPLANE) return launch_gemm_bitplane(g, stream);
@@ -217,14 +217,13 @@ int bwla_w1ax_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, cons
     const int path = resolve_path(M, K, N, r, bits);
 
     RotGeom geom;
-    int busy = -1;
     if (g_forced_rotation != BWLA_ROT_SIMT && rot_geometry(n1, n2, &geom)) {
         // the Kronecker factors are handed over raw: every CTA of the rotation splits what it needs of them (a prepared
         // layer has that done once)
         RotProblem pr{};
         pr.P1 = P1; pr.P2 = P2; pr.codes = codes; pr.codes_layout = path == BWLA_PATH_I8 ? 1 : 0; pr.scales = scales; pr.qsum = qsum;
         OktLowrank lr{V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status) + kLrCounterWord};
-        st = launch_rot(geom, x_bf16, M, ldx, bits, 0, 1, &pr, &lr, (uint32_t*)(base + ws.status), s, &busy);
+        st = launch_rot(geom, x_bf16, M, ldx, bits, 0, 1, &pr, &lr, (uint32_t*)(base + ws.status), s);
     } else {
         st = launch_prologue(x_bf16, M, K, ldx, P1, n1, P2, n2, bits, codes, path == BWLA_PATH_I8 ? 1 : 0, scales, qsum,
                              V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status), s);
@@ -234,7 +233,7 @@ int bwla_w1ax_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, cons
     g.scales = scales; g.qsum = qsum; g.M = M; g.K = K; g.N = N; g.bits = bits; g.packed = packed; g.alpha = alpha;
     g.mu = mu; g.Thl = r > 0 ? Thl : nullptr; g.U = U_bf16; g.r = r; g.out = out_bf16; g.ldo = ldo; g.acc_debug = nullptr;
     g.status = (uint32_t*)(base + ws.status);
-    return run_contraction(path, g, codes, busy, s);
+    return run_contraction(path, g, codes, s);
 }
 
 int bwla_w1a_gemm_codes(const int8_t* codes, const float* scales, int64_t M, int64_t K, int bits,
@@ -270,7 +269,7 @@ int bwla_w1a_gemm_codes(const int8_t* codes, const float* scales, int64_t M, int
     g.scales = scales; g.qsum = qsum; g.M = M; g.K = K; g.N = N; g.bits = bits; g.packed = packed; g.alpha = alpha;
     g.mu = mu; g.Thl = r > 0 ? Thl : nullptr; g.U = U_bf16; g.r = r; g.out = out_bf16; g.ldo = ldo; g.acc_debug = acc_debug;
     g.status = (uint32_t*)(base + ws.status);
-    return run_contraction(path, g, inter ? inter : codes, -1, s);
+    return run_contraction(path, g, inter ? inter : codes, s);
 }
 
 int bwla_workspace_section(int64_t M, int64_t K, int64_t N, int r, int bits, int which, size_t* offset, size_t* bytes) {
@@ -414,11 +413,10 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
             RotProblem pr{};
             pr.prepared = L->prepared; pr.digits = 1; pr.codes = (int8_t*)(base + w.yhat); pr.codes_layout = 1;
             pr.scales = (float*)(base + w.scales); pr.qsum = (int32_t*)(base + w.ysum);
-            int busy = -1;
-            st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s, &busy);
+            st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
             if (st != BWLA_OK) return st;
             bool taken = false;
-            return launch_gemm_small(&g, 1, 3, busy, &taken, s);
+            return launch_gemm_small(&g, 1, 3, &taken, s);
         }
     }
     RotProblem pr{};
@@ -478,7 +476,6 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
     }
     const bool rot = L0->rot && g_forced_rotation != BWLA_ROT_SIMT;      // (the layers share n1 and n2)
     if (L0->asym && !rot) return BWLA_ERR_UNSUPPORTED;     // the asymmetric quantiser lives in the tensor-core rotation
-    int busy = -1;
     if (rot) {
         RotProblem pr[kRotMaxProblems];
         OktLowrank lr[kRotMaxProblems];
@@ -491,7 +488,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
             lr[i] = OktLowrank{L->V, L->r, wbase[i] + ws[i].T, L->r > 0 ? (float*)(wbase[i] + ws[i].lr_part) : nullptr,
                                status + 8 * i + kLrCounterWord};
         }
-        st = launch_rot(L0->geom, x_bf16, M, ldx, L0->bits, L0->asym, count, pr, lr, status, s, &busy);
+        st = launch_rot(L0->geom, x_bf16, M, ldx, L0->bits, L0->asym, count, pr, lr, status, s);
         if (st != BWLA_OK) return st;
     } else {
         for (int i = 0; i < count; ++i) {
@@ -519,7 +516,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
     }
     if (all_i8 && M <= kSmallTokens) {
         bool taken = false;
-        st = launch_gemm_small(ga, count, 1, busy, &taken, s);
+        st = launch_gemm_small(ga, count, 1, &taken, s);
         if (taken) return st;
     }
     // Several contractions that all go to the small-batch tcgen05 kernel run beside one another (GemmArgs::dep_mode); each
@@ -532,7 +529,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
     for (int i = 0; i < count; ++i) {
         ga[i].dep_mode = siblings ? (i == 0 ? kDepHead : kDepSibling) : kDepChain;
         ga[i].sm_budget = share ? (int)(((int64_t)sms_all * ((layers[i]->N + 127) / 128)) / tiles_total) : 0;
-        st = run_contraction(path[i], ga[i], ga[i].codes, busy, s);
+        st = run_contraction(path[i], ga[i], ga[i].codes, s);
         if (st != BWLA_OK) return st;
     }
     return BWLA_OK;

@@ -194,10 +194,9 @@ int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void*
 // blocks of those with a low-rank branch.
 // asym == 0: symmetric codes in [-qmax, qmax], qmax = 2^(b-1) - 1.  asym == 1 (Sec. 4.1, per-token asymmetric): with
 // u in [0, 2^b - 1] and the integer zero point z of the token, the stored code is u - 2^(b-1) + code_bias and the
-// rot_ctas (may be NULL) receives the number of CTAs that rotate.
 // stored zero point z - 2^(b-1) + code_bias; a code minus the zero point times the scale is the value it stands for.
 int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
-               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream, int* rot_ctas = nullptr);
+               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream);
 // Rows of weights (fp32 or bf16): packed signs, scale and shift of every row.
 int launch_rot_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status,
                         cudaStream_t stream);
@@ -248,10 +247,10 @@ bool bitplane_supports(int64_t M, int64_t K, int64_t N, int r, int bits);
 int launch_gemm_bitplane(const GemmArgs& a, cudaStream_t stream);
 
 // Up to 64 tokens: warp-level int8 MMAs, all linears of a group (same M, K, bits; a.codes in the interleaved order) in one
-// launch.  busy: CTAs of the kernel before that hold their SMs to its end (-1: not known).  planes == 3: three digit planes per token (the weight-only operating point, up to 32 tokens).  *taken is false, and
+// launch.  planes == 3: three digit planes per token (the weight-only operating point, up to 32 tokens).  *taken is false, and
 // nothing has been launched, for shapes whose codes do not fit shared memory: those go to the tcgen05 kernels.
 bool gemm_small_fits(const GemmArgs* a, int n, int planes);
-int launch_gemm_small(const GemmArgs* a, int n, int planes, int busy, bool* taken, cudaStream_t stream);
+int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStream_t stream);
 
 // tcgen05 path with the fused epilogue.  codes_interleaved: int8 [M][K] in the interleaved order.
 bool umma_supports(int64_t M, int64_t K, int64_t N, int r, int bits);

@@ -61,7 +61,6 @@ struct SmallParams {
     int n_problems, M, K, units, S;
     int run;                              // groups whose sums fit shared memory at a time
     int t_off, tok_off, acc_off;
-    int early;                            // CTAs that are expected on the device before the preceding kernel has finished
     uint32_t* status;
 };
 
@@ -95,7 +94,6 @@ template <int NTP, int PL, bool SPLIT>
 __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const __grid_constant__ SmallParams p) {
     using namespace small_;
     constexpr int NT = NTP * PL, TP = token_parts(NT), NTPW = NTP / TP, NTW = NT / TP;        // ... W: of one item
-    constexpr bool AHEAD = NT <= 2;                   // (registers: beyond that the rows of a fragment are fetched when its turn comes)
     constexpr int TOK = 8 * NT, SETS = NT == 1 ? 4 : NT <= 3 ? 2 : 1;
     extern __shared__ __align__(16) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
@@ -147,9 +145,42 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
     uint4 wn[4];
     if (it < it_end) load_w(wn, it);
     int32_t* const accs = reinterpret_cast<int32_t*>(smem + p.acc_off);      // [group of the run][row half][column tile][4][32 lanes]
+    for (int i = tid; i < p.run * 2 * NT * 32; i += kThreads) reinterpret_cast<uint4*>(accs)[i] = make_uint4(0u, 0u, 0u, 0u);
+    griddep_wait();
+    // ---- codes (128-byte rows: 128 k, token), T (128-byte rows: term, token) and the per-token scalars; the 16-byte pieces of a
+    //      row are permuted by the token's low bits (and, for the codes, the row's place among the four of an item)
+    const int pieces = min(un * (kUnit / 16), (p.K >> 4) - ub * (kUnit / 16));
+    for (int t = warp; t < PL * p.M; t += kWarps) {
+        const int plane = PL > 1 ? t / p.M : 0, row = plane * (8 * NTP) + (t - plane * p.M);
+        const int8_t* src = pr.codes + (int64_t)t * p.K + (int64_t)ub * kUnit;
+        const uint32_t dst = smem_u32(smem) + row * 128;
+        for (int c = lane; c < pieces; c += 32)
+            cp_async16(dst + (uint32_t)((c >> 3) * (TOK * 128) + (((c & 7) ^ (row & 7) ^ (((c >> 3) & 3) << 1)) << 4)), src + 16 * c);
+    }
+    if (pr.r > 0)
+        for (int i = tid; i < 3 * p.M * 8; i += kThreads) {
+            const int row = i >> 3, c = i & 7, h = row / p.M, t = row - h * p.M;
+            cp_async16(smem_u32(smem) + (uint32_t)(p.t_off + (h * 8 * NTP + t) * 128 + ((c ^ (t & 7)) << 4)), pr.Thl + (int64_t)row * kLowrankPad + 8 * c);
+        }
     float* sc_s = reinterpret_cast<float*>(smem + p.tok_off);
     int32_t *qs_s = reinterpret_cast<int32_t*>(sc_s) + TOK, *zp_s = qs_s + TOK;
-    bool failed = false, dry = false;
+    if (tid < TOK) {
+        float sc = 0.f; int32_t qs = 0, zp = 0;
+        const int plane = tid / (8 * NTP), t = tid - plane * (8 * NTP);
+        if (t < p.M) {
+            sc = pr.scales[t];
+            const int4* parts = reinterpret_cast<const int4*>(pr.qsum + ((size_t)plane * p.M + t) * kQsumParts);
+            const int4 a = parts[0], b = parts[1];
+            qs = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
+            if (pr.zp) zp = pr.zp[t];
+        }
+        sc_s[tid] = sc; qs_s[tid] = qs; zp_s[tid] = zp;
+    }
+    // (behind the copies: the look at the status word is a trip to the L2)
+    const bool failed = p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0;       // the call already failed
+    cp_async_wait_all();
+    __syncthreads();
+
     // ---- epilogue of one fragment (16 rows x 8 tokens), in two halves: what it needs from global memory is requested a fragment
     //      ahead (an L2 round trip each otherwise: rows of U, then the scales, then the shifts)
     struct Rows { uint32_t ul[8], uh[8]; float al[2], mu[2]; int32_t rs[2]; };
@@ -206,7 +237,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = 8 * nt + 2 * tq + (i & 1), h = i >> 1, n = h ? n_hi : n_lo;
-            const bool live = t < p.M && n < pr.N && !dry;
+            const bool live = t < p.M && n < pr.N;
             const float sc = sc_s[t];
             float accf, qsf;
             if constexpr (PL == 1) {
@@ -226,48 +257,6 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
         }
     };
     const uint32_t b0 = smem_u32(smem) + (uint32_t)((tq * TOK + gq) * 128), b_swz = (uint32_t)((gq ^ (tq << 1)) << 4);
-    // A CTA that is on its SM before the preceding kernel has finished first takes one item and one fragment through the code
-    // below, on whatever shared memory holds and without storing anything: instructions, address translations and rows of U
-    // are then where they are needed (cold, they cost several microseconds of a launch this short).
-#pragma unroll 1
-    for (int pass = (int)blockIdx.x < p.early ? 0 : 1; pass < 2; ++pass) {
-    dry = pass == 0;
-    if (!dry) {
-        __syncthreads();                              // (the sums may still be read by the pass before)
-        for (int i = tid; i < p.run * 2 * NT * 32; i += kThreads) reinterpret_cast<uint4*>(accs)[i] = make_uint4(0u, 0u, 0u, 0u);
-        griddep_wait();
-        // ---- codes (128-byte rows: 128 k, token), T (128-byte rows: term, token) and the per-token scalars; the 16-byte pieces of a
-        //      row are permuted by the token's low bits (and, for the codes, the row's place among the four of an item)
-        const int pieces = min(un * (kUnit / 16), (p.K >> 4) - ub * (kUnit / 16));
-        for (int t = warp; t < PL * p.M; t += kWarps) {
-            const int plane = PL > 1 ? t / p.M : 0, row = plane * (8 * NTP) + (t - plane * p.M);
-            const int8_t* src = pr.codes + (int64_t)t * p.K + (int64_t)ub * kUnit;
-            const uint32_t dst = smem_u32(smem) + row * 128;
-            for (int c = lane; c < pieces; c += 32)
-                cp_async16(dst + (uint32_t)((c >> 3) * (TOK * 128) + (((c & 7) ^ (row & 7) ^ (((c >> 3) & 3) << 1)) << 4)), src + 16 * c);
-        }
-        if (pr.r > 0)
-            for (int i = tid; i < 3 * p.M * 8; i += kThreads) {
-                const int row = i >> 3, c = i & 7, h = row / p.M, t = row - h * p.M;
-                cp_async16(smem_u32(smem) + (uint32_t)(p.t_off + (h * 8 * NTP + t) * 128 + ((c ^ (t & 7)) << 4)), pr.Thl + (int64_t)row * kLowrankPad + 8 * c);
-            }
-        if (tid < TOK) {
-            float sc = 0.f; int32_t qs = 0, zp = 0;
-            const int plane = tid / (8 * NTP), t = tid - plane * (8 * NTP);
-            if (t < p.M) {
-                sc = pr.scales[t];
-                const int4* parts = reinterpret_cast<const int4*>(pr.qsum + ((size_t)plane * p.M + t) * kQsumParts);
-                const int4 a = parts[0], b = parts[1];
-                qs = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
-                if (pr.zp) zp = pr.zp[t];
-            }
-            sc_s[tid] = sc; qs_s[tid] = qs; zp_s[tid] = zp;
-        }
-        // (behind the copies: the look at the status word is a trip to the L2)
-        failed = p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0;       // the call already failed
-        cp_async_wait_all();
-        __syncthreads();
-    }
 #pragma unroll 1
     while (g < g_hi) {
         int32_t acc[SETS][2][NTW][4];
@@ -283,13 +272,12 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                         for (int e = 0; e < 4; ++e) acc[s][mt][nt][e] = 0;
         };
         clear();
-        const int it_stop = dry ? min(it + 1, it_end) : it_end, it_first = it;
 #pragma unroll 1
-        for (; it < it_stop; ++it) {
+        for (; it < it_end; ++it) {
             uint4 w[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) w[j] = wn[j];
-            if (it + 1 < it_stop) load_w(wn, it + 1);
+            if (it + 1 < it_end) load_w(wn, it + 1);
             const int part = TP > 1 ? sub % TP : 0;
             // column tile j of the item: plane j / NTPW, token tile part * NTPW + j % NTPW
             const uint32_t b_item = b0 + (uint32_t)((u * kSteps * TOK + 8 * NTPW * part) * 128);
@@ -321,7 +309,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                             imma_16832(acc[q & (SETS - 1)][mt][nt], a[mt][q][0], a[mt][q][1], a[mt][q][2], a[mt][q][3], bl[q], bh[q]);
                 }
             }
-            if (++u == un || it + 1 == it_stop) {
+            if (++u == un || it + 1 == it_end) {
                 // the group (or the warp's share of it) is done: into the CTA's sums
                 const uint32_t at = smem_u32(accs) + (uint32_t)(((sub / TP) * 2 * NT * 128 + lane) * 4);
 #pragma unroll
@@ -344,15 +332,11 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
         const int g_now = g, n_now = n, frags = n_now * 2 * NTP, f_step = (SPLIT ? p.S : 1) * kWarps;
         int f = SPLIT ? rank * kWarps + warp : warp;
         Rows rows;
-        if (AHEAD && f < frags) fetch_rows(rows, g_now + f / (2 * NTP), f / NTP & 1);
-        if (dry) {
-            it = it_first;                            // (its sign words are still in registers)
-        } else {
-            g += n; n = min(p.run, g_hi - g);
-            if (g < g_hi) {
-                share();
-                if (it < it_end) load_w(wn, it);
-            }
+        if (f < frags) fetch_rows(rows, g_now + f / (2 * NTP), f / NTP & 1);
+        g += n; n = min(p.run, g_hi - g);
+        if (g < g_hi) {
+            share();
+            if (it < it_end) load_w(wn, it);
         }
         if (SPLIT) { cluster_arrive_release(); cluster_wait_acquire(); }
         else __syncthreads();
@@ -360,9 +344,8 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
 #pragma unroll 1
         for (; f < frags && !failed; f += f_step) {
             const int grp = f / (2 * NTP), mt = f / NTP & 1, nt = f % NTP;
-            if (!AHEAD) fetch_rows(rows, g_now + grp, mt);
             const Rows now = rows;
-            if (AHEAD && f + f_step < frags) fetch_rows(rows, g_now + (f + f_step) / (2 * NTP), (f + f_step) / NTP & 1);
+            if (f + f_step < frags) fetch_rows(rows, g_now + (f + f_step) / (2 * NTP), (f + f_step) / NTP & 1);
             int32_t v[PL][4];
 #pragma unroll
             for (int pl = 0; pl < PL; ++pl) {
@@ -386,15 +369,16 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                 }
             }
             epilogue(now, g_now + grp, mt, nt, v);
-            if (dry) break;
         }
-        if (SPLIT) { cluster_arrive_release(); cluster_wait_acquire(); }       // everybody has read
-        if (dry) break;
-        if (SPLIT && g < g_hi) {
-            for (int i = tid; i < n_now * 2 * NT * 32; i += kThreads) reinterpret_cast<uint4*>(accs)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (SPLIT) {
+            cluster_arrive_release(); cluster_wait_acquire();       // everybody has read
+            if (g < g_hi) {
+                for (int i = tid; i < n_now * 2 * NT * 32; i += kThreads) reinterpret_cast<uint4*>(accs)[i] = make_uint4(0u, 0u, 0u, 0u);
+                __syncthreads();
+            }
+        } else if (g < g_hi) {
+            __syncthreads();
         }
-        if (g < g_hi) __syncthreads();
-    }
     }
 }
 
@@ -557,9 +541,8 @@ static int launch_small_nt(const SmallParams& p, int grid, int smem, cudaStream_
 }
 
 // All problems have the same M, K and bits; a[i].codes: int8 [planes][M][K] in the interleaved order; a[i].Thl: bf16 [3][M][64].
-// busy: CTAs of the kernel before that hold their SMs to its end (-1: not known).  *taken is false where the shapes do not fit
-// (nothing has been launched then).
-int launch_gemm_small(const GemmArgs* a, int n, int planes, int busy, bool* taken, cudaStream_t stream) {
+// *taken is false where the shapes do not fit (nothing has been launched then).
+int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStream_t stream) {
     SmallPlan pl;
     *taken = small_plan(a, n, planes, &pl);
     if (!*taken) return BWLA_OK;
@@ -578,7 +561,6 @@ int launch_gemm_small(const GemmArgs* a, int n, int planes, int busy, bool* take
         begin += pl.clusters[i];
     }
     const int grid = begin * pl.S;
-    p.early = busy >= 0 ? std::max(0, std::min(grid, sm_count() - busy)) / pl.S * pl.S : 0;
     if (planes == 3) {
         switch (NTP) {
             case 1: return launch_small_nt<1, 3>(p, grid, pl.smem, stream);

@@ -966,7 +966,7 @@ static int launch_rot_kernel(RotKernel k, const RotGeom& g, RotKernelParams& p, 
 }
 
 int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
-               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream, int* rot_ctas) {
+               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream) {
     if (M == 0 || n_problems == 0) return BWLA_OK;
     const RotGeom g = M * n_problems <= sm_count() ? few_tokens_geometry(base, M * n_problems, sm_count()) : base;
     if (n_problems > kRotMaxProblems || M >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
@@ -1020,9 +1020,7 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
     }
     for (int i = n_problems; i <= kRotMaxProblems; ++i) p.lr_begin[i] = lr_total;
     RotKernel k = problems[0].yhat ? pick_kernel<kRotBf16, false>(g) : problems[0].digits ? pick_kernel<kRotDigits, false>(g) : pick_kernel<kRotQuant, false>(g);
-    const int st = launch_rot_kernel(k, g, p, smem, lr_total, stream);
-    if (rot_ctas) *rot_ctas = p.rot_ctas;
-    return st;
+    return launch_rot_kernel(k, g, p, smem, lr_total, stream);
 }
 
 int launch_rot_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status,
