@@ -94,6 +94,7 @@ template <int NTP, int PL, bool SPLIT>
 __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const __grid_constant__ SmallParams p) {
     using namespace small_;
     constexpr int NT = NTP * PL, TP = token_parts(NT), NTPW = NTP / TP, NTW = NT / TP;        // ... W: of one item
+    constexpr bool AHEAD = NT == 1;                   // (registers: beyond that the rows of a fragment are fetched when its turn comes)
     constexpr int TOK = 8 * NT, SETS = NT == 1 ? 4 : NT <= 3 ? 2 : 1;
     extern __shared__ __align__(16) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
@@ -119,12 +120,11 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
             prefetch_l2_line(pr.alpha + n0);
             if (pr.mu) prefetch_l2_line(pr.mu + n0);
             if (pr.zp) prefetch_l2_line(pr.rowsum + n0);
-            if (pr.r > 0) {
-                const uintptr_t lo = reinterpret_cast<uintptr_t>(pr.U + (int64_t)n0 * pr.r);
-                const uintptr_t hi = reinterpret_cast<uintptr_t>(pr.U + (int64_t)min(n0 + 32, pr.N) * pr.r);
-                const uintptr_t a0 = (lo + 15) & ~(uintptr_t)15;
-                if (hi >= a0 + 16) prefetch_l2_bulk(reinterpret_cast<const void*>(a0), (uint32_t)((hi - a0) & ~(uintptr_t)15));
-            }
+        }
+        // (line by line: bulk prefetches of U behind those of the sign words were seen to arrive late)
+        if (pr.r > 0) {
+            const uint8_t* u = reinterpret_cast<const uint8_t*>(pr.U) + (int64_t)g_lo * 32 * pr.r * 2;
+            for (int i = 128 * tid; i < rows * pr.r * 2; i += 128 * kThreads) prefetch_l2_line(u + i);
         }
     }
     // this warp's items of a run of `n` groups from `g`: [lo, hi) in the order (group, token part, unit)
@@ -146,6 +146,14 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
     if (it < it_end) load_w(wn, it);
     int32_t* const accs = reinterpret_cast<int32_t*>(smem + p.acc_off);      // [group of the run][row half][column tile][4][32 lanes]
     for (int i = tid; i < p.run * 2 * NT * 32; i += kThreads) reinterpret_cast<uint4*>(accs)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (warp == 0) {
+        if (lane == 0 && p.status) touch(p.status);
+        if (lane == 1) touch(pr.codes);
+        if (lane == 2 && pr.r > 0) touch(pr.U + (int64_t)g_lo * 32 * pr.r);
+        if (lane == 3) touch(pr.alpha + g_lo * 32);
+        if (lane == 4 && pr.out) touch(pr.out + g_lo * 32);
+        if (lane == 5 && pr.r > 0) touch(pr.Thl);
+    }
     griddep_wait();
     // ---- codes (128-byte rows: 128 k, token), T (128-byte rows: term, token) and the per-token scalars; the 16-byte pieces of a
     //      row are permuted by the token's low bits (and, for the codes, the row's place among the four of an item)
@@ -332,7 +340,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
         const int g_now = g, n_now = n, frags = n_now * 2 * NTP, f_step = (SPLIT ? p.S : 1) * kWarps;
         int f = SPLIT ? rank * kWarps + warp : warp;
         Rows rows;
-        if (f < frags) fetch_rows(rows, g_now + f / (2 * NTP), f / NTP & 1);
+        if (AHEAD && f < frags) fetch_rows(rows, g_now + f / (2 * NTP), f / NTP & 1);
         g += n; n = min(p.run, g_hi - g);
         if (g < g_hi) {
             share();
@@ -344,8 +352,9 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
 #pragma unroll 1
         for (; f < frags && !failed; f += f_step) {
             const int grp = f / (2 * NTP), mt = f / NTP & 1, nt = f % NTP;
+            if (!AHEAD) fetch_rows(rows, g_now + grp, mt);
             const Rows now = rows;
-            if (f + f_step < frags) fetch_rows(rows, g_now + (f + f_step) / (2 * NTP), (f + f_step) / NTP & 1);
+            if (AHEAD && f + f_step < frags) fetch_rows(rows, g_now + (f + f_step) / (2 * NTP), (f + f_step) / NTP & 1);
             int32_t v[PL][4];
 #pragma unroll
             for (int pl = 0; pl < PL; ++pl) {

@@ -300,7 +300,6 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     __syncthreads();
     if (g.dc > 1) { cluster_arrive_release(); cluster_wait_acquire(); }   // every CTA of the cluster runs: its slots may be written
     griddep_launch_dependents();
-    griddep_wait();                                   // x may be the output of the preceding kernel
     int ntok = tok0 < p.M ? (int)((p.M - tok0 + stride - 1) / stride) : 0;
     // this thread's chunks of X: tid, tid + T, ...; (row, column) advance without divisions
     const int ch_a0 = tid / cpr, ch_c0 = tid - ch_a0 * cpr, ch_da = T / cpr, ch_dc = T - ch_da * cpr;
@@ -513,6 +512,16 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         }
     };
 
+    // (what the lanes need to know of their places is worked out by now, with the preceding kernel still running)
+    uint32_t pin[6] = {a2_addr, bx_addr, b1_addr, az_addr, (uint32_t)off_lo[0], (uint32_t)off_hi[1]};
+    asm volatile("" ::"r"(pin[0]), "r"(pin[1]), "r"(pin[2]), "r"(pin[3]), "r"(pin[4]), "r"(pin[5]), "r"(ntok), "r"(ch_a0), "r"(ch_da), "r"(lim[0]), "r"(lim[1]) : "memory");
+    if (warp == 0 && tok0 < p.M) {
+        if (lane == 0) touch(reinterpret_cast<const uint8_t*>(p.x) + tok0 * p.ldx * (F32 ? 4 : 2));
+        if (lane == 1 && p.status) touch(p.status);
+        if (lane == 2 && (MODE == kRotQuant || MODE == kRotDigits)) touch(pr.codes + tok0 * (int64_t)g.K);
+        if (lane == 3 && MODE == kRotBf16) touch(pr.yhat + tok0 * (int64_t)g.K);
+    }
+    griddep_wait();                                   // x may be the output of the preceding kernel
     // (the look at the status word takes a trip to the L2: the first token's x is on its way by then)
     if (!F32 && ntok > 0) fetch_x(tok0);
     const int first_tokens = ntok;
