@@ -102,6 +102,10 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     const int my_tiles = (int)blockIdx.x < tiles ? (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int units = (p.K + kUnitK - 1) / kUnitK;
     const int kblocks = p.K / kBlockK;
+    // CTAs that work on the same token tile read the same codes: each starts at a unit of its own and goes round (the sums are
+    // integers, the order does not matter), so that they do not all ask the same slices of the L2 at the same time.
+    const int u0 = (int)(((int64_t)blockIdx.x * units) / gridDim.x);
+    auto unit_at = [&](int j) { const int u = u0 + j; return u < units ? u : u - units; };
     const bool lowrank = p.r > 0;
     // tile i of this CTA: row tiles fastest, so that the CTAs working at the same time share a token tile's codes in the L2
     auto tile_n0 = [&](int i) { return (((int)blockIdx.x + i * (int)gridDim.x) % p.row_tiles) * kRows; };
@@ -143,7 +147,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                         if (!wait_or_abort(&w_empty[ws], wph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x110); break; }
                     }
                     mbar_expect_tx(&w_full[ws], w_bytes);
-                    tma_load_2d_hint(wbuf + ws * w_bytes, &w_map, u * (kUnitK / 32), n0, &w_full[ws], stream_once);
+                    tma_load_2d_hint(wbuf + ws * w_bytes, &w_map, unit_at(u) * (kUnitK / 32), n0, &w_full[ws], stream_once);
                     if (++ws == WS) { ws = 0; wph ^= 1; }
                 }
             }
@@ -178,11 +182,13 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&tok_full[buf]);
-                for (int kb = 0; kb < kblocks; ++kb) {
+                int kb = u0 * (kUnitK / kBlockK);
+                for (int c = 0; c < kblocks; ++c) {
                     if (!wait_or_abort(&b_empty[bs], bph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x121); ok = false; break; }
                     mbar_expect_tx(&b_full[bs], b_bytes);
                     tma_load_2d(bbuf + bs * b_bytes, &b_map, kb * kBlockK, t0, &b_full[bs]);
                     if (++bs == BS) { bs = 0; bph ^= 1; }
+                    if (++kb == kblocks) kb = 0;
                 }
                 // T is first needed when the K loop is over; the previous tile's low-rank MMAs have long read theirs
                 if (ok && lowrank) {
@@ -366,7 +372,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             for (int u = 0; u < units && ok; ++u) {
                 if (!warp_wait(&w_full[ws], wph, abort_flag)) { give_up(p.status, abort_flag, 0x150); ok = false; break; }
                 const uint8_t* wrow = wbuf + ws * w_bytes + row * 128;
-                const int ns = min(kUnitK / kBlockK, (p.K - u * kUnitK) / kBlockK);
+                const int ns = min(kUnitK / kBlockK, (p.K - unit_at(u) * kUnitK) / kBlockK);
                 // Block g of this CTA (a running count over its tiles) belongs to part g % EW and to stage g % AS.  AS is a
                 // multiple of EW, so a stage always has the same owner and the owner is never more than one phase ahead of
                 // the stage's consumer: a parity wait cannot tell a phase from the one two before it.  (The last unit of a
