@@ -31,16 +31,19 @@ constexpr int kRows = 128;                // output rows per tile
 constexpr int kTok = 128;                 // tokens per tile
 constexpr int kUnitK = 1024;              // weights per row in one sign-word stage
 constexpr int kBlockK = 128;              // K per code stage and per operand stage
-constexpr int WS = 2, BS = 5, AS = 4, EW = 4;
+// A stage is a k-block's codes in shared memory and its expanded signs in tensor memory, under one pair of barriers: the issuing
+// thread runs one wait and one commit per k-block.  (With a ring and barriers for each operand the loop took 590 cycles per
+// k-block, 500 of them also without any of the copies, stores and MMAs: the issuing thread's waits and commits were the bound.)
+constexpr int WS = 2, AS = 4, EW = 4;
 static_assert(AS % EW == 0, "an operand stage must keep one owner among the expander parts");
 constexpr int kEpiFirst = 128, kExpFirst = 256;
 constexpr int kThreads = kExpFirst + 128 * EW;       // 768
 constexpr int w_bytes = kRows * 128, b_bytes = kTok * 128;
-constexpr int u_off = WS * w_bytes + BS * b_bytes;
+constexpr int u_off = WS * w_bytes + AS * b_bytes;
 constexpr int t_off = u_off + kRows * 128;
 constexpr int o_off = t_off + 3 * b_bytes;           // finished outputs [token][row] bf16
 constexpr int bars_off = o_off + kTok * kRows * 2;
-constexpr int n_bars = 2 * WS + 2 * BS + 2 * AS + 12;
+constexpr int n_bars = 2 * WS + 2 * AS + 12;
 constexpr int misc_off = bars_off + n_bars * 8;
 constexpr int tok_off = misc_off + 16;               // [2][scales, code sums, zero points][kTok]
 constexpr int used = tok_off + 2 * 12 * kTok;
@@ -79,11 +82,9 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + bars_off);
     uint64_t* w_full = bars;                 // [WS]
     uint64_t* w_empty = w_full + WS;
-    uint64_t* b_full = w_empty + WS;         // [BS]
-    uint64_t* b_empty = b_full + BS;
-    uint64_t* a_full = b_empty + BS;         // [AS]
-    uint64_t* a_empty = a_full + AS;
-    uint64_t* d_full = a_empty + AS;         // the tile's MMAs (low-rank ones included) have completed
+    uint64_t* s_full = w_empty + WS;         // [AS] codes landed and signs expanded
+    uint64_t* s_empty = s_full + AS;         // [AS] the MMAs that read both have completed
+    uint64_t* d_full = s_empty + AS;         // the tile's MMAs (low-rank ones included) have completed
     uint64_t* acc_free = d_full + 1;         // the epilogue has read the tile's accumulators
     uint64_t* u_full = acc_free + 1;         // the tile's rows of U are staged
     uint64_t* u_empty = u_full + 1;          // the low-rank MMAs have read them
@@ -114,8 +115,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         for (int i = 0; i < WS; ++i) { mbar_init(&w_full[i], 1); mbar_init(&w_empty[i], 4 * EW); }
-        for (int i = 0; i < BS; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], 1); }
-        for (int i = 0; i < AS; ++i) { mbar_init(&a_full[i], 4); mbar_init(&a_empty[i], 1); }
+        for (int i = 0; i < AS; ++i) { mbar_init(&s_full[i], 5); mbar_init(&s_empty[i], 1); }      // four expander warps and the copy
         mbar_init(d_full, 1); mbar_init(acc_free, 4);
         mbar_init(u_full, 4); mbar_init(u_empty, 1);
         mbar_init(t_full, 1); mbar_init(t_empty, 1);
@@ -184,10 +184,10 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 mbar_arrive(&tok_full[buf]);
                 int kb = u0 * (kUnitK / kBlockK);
                 for (int c = 0; c < kblocks; ++c) {
-                    if (!wait_or_abort(&b_empty[bs], bph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x121); ok = false; break; }
-                    mbar_expect_tx(&b_full[bs], b_bytes);
-                    tma_load_2d(bbuf + bs * b_bytes, &b_map, kb * kBlockK, t0, &b_full[bs]);
-                    if (++bs == BS) { bs = 0; bph ^= 1; }
+                    if (!wait_or_abort(&s_empty[bs], bph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x121); ok = false; break; }
+                    mbar_expect_tx(&s_full[bs], b_bytes);
+                    tma_load_2d(bbuf + bs * b_bytes, &b_map, kb * kBlockK, t0, &s_full[bs]);
+                    if (++bs == AS) { bs = 0; bph ^= 1; }
                     if (++kb == kblocks) kb = 0;
                 }
                 // T is first needed when the K loop is over; the previous tile's low-rank MMAs have long read theirs
@@ -211,7 +211,6 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             const uint64_t desc_hi = smem_desc_sw128(0u, 0u);
             const uint32_t b_lo0 = (smem_u32(bbuf) & 0x3FFFFu) >> 4;
             int as = 0; uint32_t aph = 0;
-            int bs = 0; uint32_t bph = 0;
             bool ok = true;
             griddep_wait();                           // everything this thread waits for follows the preceding kernel
             for (int i = 0; i < my_tiles && ok; ++i) {
@@ -221,20 +220,17 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 const uint32_t d_addr = tmem_base + D_COL + (uint32_t)(i & 1) * kTok;
                 uint32_t acc = 0;
                 for (int kb = 0; kb < kblocks && ok; ++kb) {
-                    if (!wait_or_abort(&b_full[bs], bph, abort_flag)) { give_up(p.status, abort_flag, 0x131); ok = false; break; }
-                    if (!wait_or_abort(&a_full[as], aph, abort_flag)) { give_up(p.status, abort_flag, 0x132); ok = false; break; }
+                    if (!wait_or_abort(&s_full[as], aph, abort_flag)) { give_up(p.status, abort_flag, 0x132); ok = false; break; }
                     tc_fence_after();
-                    const uint64_t desc = desc_hi | (uint64_t)(b_lo0 + (uint32_t)bs * (b_bytes >> 4));
+                    const uint64_t desc = desc_hi | (uint64_t)(b_lo0 + (uint32_t)as * (b_bytes >> 4));
                     const uint32_t a_addr = a_base + 32 * as;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         mma_i8_ts(d_addr, a_addr + 8 * j, desc + 2 * j, idesc, acc);
                         acc = 1u;
                     }
-                    tc_commit(&a_empty[as]);
-                    tc_commit(&b_empty[bs]);
+                    tc_commit(&s_empty[as]);
                     if (++as == AS) { as = 0; aph ^= 1u; }
-                    if (++bs == BS) { bs = 0; bph ^= 1u; }
                 }
                 // The epilogue of the tile before has had this tile's whole K loop to read its accumulators; it is waited for
                 // here, before this tile's MMAs are committed, so that completions of acc_free are seen strictly in order
@@ -388,9 +384,9 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                         for (int j = 0; j < 8; ++j) v[8 * c + j] = (w[c] << (7 - j)) & 0x80808080u;
                     const int as = (kb_base + s) % AS;
                     const uint32_t aph = (uint32_t)(((kb_base + s) / AS) & 1);
-                    if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(&a_empty[as], aph ^ 1u))) {
+                    if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(&s_empty[as], aph ^ 1u))) {
                         griddep_wait();
-                        if (!warp_wait(&a_empty[as], aph ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x151); ok = false; }
+                        if (!warp_wait(&s_empty[as], aph ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x151); ok = false; }
                     }
                     if (ok) {
                         tc_fence_after();
@@ -398,7 +394,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                         tc_wait_st();
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(&a_full[as]);
+                        if (lane == 0) mbar_arrive(&s_full[as]);
                     }
                 }
                 // the stage is released only after every word of it that this warp needs has gone through the expansion
