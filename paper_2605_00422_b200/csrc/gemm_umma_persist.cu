@@ -68,6 +68,12 @@ struct PersistParams {
     uint32_t* status;
 };
 
+__device__ __forceinline__ uint4 lds_words(const uint8_t* p) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+
 __global__ void __launch_bounds__(persist::kThreads, 1)
 umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap b_map,
                            const __grid_constant__ CUtensorMap t_map, PersistParams p) {
@@ -137,7 +143,9 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         // ---------------- packed sign words (independent of the preceding kernel) ----------------
         if (elect_one()) {
             tma_prefetch_desc(&w_map);
+            // one token tile: every word is read once; more: once per token tile, so they may stay
             const uint64_t stream_once = l2_policy_evict_first();
+            const bool once = p.tok_tiles == 1;
             int ws = 0; uint32_t wph = 0;
             for (int i = 0; i < my_tiles && !*abort_flag; ++i) {
                 const int n0 = tile_n0(i);
@@ -147,7 +155,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                         if (!wait_or_abort(&w_empty[ws], wph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x110); break; }
                     }
                     mbar_expect_tx(&w_full[ws], w_bytes);
-                    tma_load_2d_hint(wbuf + ws * w_bytes, &w_map, unit_at(u) * (kUnitK / 32), n0, &w_full[ws], stream_once);
+                    if (once) tma_load_2d_hint(wbuf + ws * w_bytes, &w_map, unit_at(u) * (kUnitK / 32), n0, &w_full[ws], stream_once);
+                    else tma_load_2d(wbuf + ws * w_bytes, &w_map, unit_at(u) * (kUnitK / 32), n0, &w_full[ws]);
                     if (++ws == WS) { ws = 0; wph ^= 1; }
                 }
             }
@@ -361,29 +370,56 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         const int part = (warp - 8) >> 2;             // which of the EW warps of the lane quarter
         const int row = q * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
+        // A warp's words of a unit (two blocks of eight) go to registers, a unit ahead, and the stage is let go at once: the copies
+        // then have three units of MMA time to arrive instead of one.  (Held until the unit was expanded, the two stages made the
+        // loop wait for the L2: 537 us for 4096 x 5120 x 25600 with and without MMAs, stores and code copies.)
+        // Block g of this CTA (a running count over its tiles) belongs to part g % EW and to stage g % AS.  AS is a multiple of
+        // EW, so a stage always has the same owner and the owner is never more than one phase ahead of the stage's consumer: a
+        // parity wait cannot tell a phase from the one two before it.  (The last unit of a row may hold fewer than eight
+        // blocks, which is why neither follows from the position inside the unit.)
+        constexpr int PER = kUnitK / kBlockK / EW;
         int ws = 0; uint32_t wph = 0;
-        int kb_base = 0;                              // k-blocks of this CTA before the current unit: block g lives in stage g % AS
+        const int total = my_tiles * units;
+        int c = 0, u_nxt = 0;                         // next unit to take: running number, position in its row
+        int base_nxt = 0;                             // blocks of this CTA before it
+        uint4 nxt[PER];
+        int ns_nxt = 0, first_nxt = 0, g_nxt = 0;
         bool ok = true;
-        for (int i = 0; i < my_tiles && ok; ++i) {
-            for (int u = 0; u < units && ok; ++u) {
-                if (!warp_wait(&w_full[ws], wph, abort_flag)) { give_up(p.status, abort_flag, 0x150); ok = false; break; }
-                const uint8_t* wrow = wbuf + ws * w_bytes + row * 128;
-                const int ns = min(kUnitK / kBlockK, (p.K - unit_at(u) * kUnitK) / kBlockK);
-                // Block g of this CTA (a running count over its tiles) belongs to part g % EW and to stage g % AS.  AS is a
-                // multiple of EW, so a stage always has the same owner and the owner is never more than one phase ahead of
-                // the stage's consumer: a parity wait cannot tell a phase from the one two before it.  (The last unit of a
-                // row may hold fewer than eight blocks, which is why neither follows from the position inside the unit.)
-#pragma unroll 1
-                for (int s = (part + EW - kb_base % EW) % EW; s < ns && ok; s += EW) {
-                    const uint4 w4 = *reinterpret_cast<const uint4*>(wrow + ((s ^ (row & 7)) << 4));
+        auto take = [&]() {                           // (the unit's stage is full)
+            ns_nxt = min(kUnitK / kBlockK, (p.K - unit_at(u_nxt) * kUnitK) / kBlockK);
+            first_nxt = (part + EW - base_nxt % EW) % EW;
+            g_nxt = base_nxt + first_nxt;
+            const uint8_t* wrow = wbuf + ws * w_bytes + row * 128;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) nxt[q] = lds_words(wrow + (((first_nxt + EW * q) ^ (row & 7)) << 4));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&w_empty[ws]);
+            if (++ws == WS) { ws = 0; wph ^= 1u; }
+            base_nxt += ns_nxt;
+            if (++u_nxt == units) u_nxt = 0;
+            ++c;
+        };
+        if (total > 0) {
+            if (!warp_wait(&w_full[ws], wph, abort_flag)) { give_up(p.status, abort_flag, 0x150); ok = false; }
+            else take();
+        }
+        for (int i = 0; i < total && ok; ++i) {
+            uint4 cur[PER];
+#pragma unroll
+            for (int q = 0; q < PER; ++q) cur[q] = nxt[q];
+            const int ns = ns_nxt, first = first_nxt, g = g_nxt;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                if (c == i + 1 && c < total && __all_sync(0xFFFFFFFFu, mbar_test_wait(&w_full[ws], wph))) take();
+                if (first + EW * q < ns && ok) {
                     uint32_t v[32];
-                    const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+                    const uint32_t w[4] = {cur[q].x, cur[q].y, cur[q].z, cur[q].w};
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
+                    for (int k = 0; k < 4; ++k)
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) v[8 * c + j] = (w[c] << (7 - j)) & 0x80808080u;
-                    const int as = (kb_base + s) % AS;
-                    const uint32_t aph = (uint32_t)(((kb_base + s) / AS) & 1);
+                        for (int j = 0; j < 8; ++j) v[8 * k + j] = (w[k] << (7 - j)) & 0x80808080u;
+                    const int as = (g + EW * q) % AS;
+                    const uint32_t aph = (uint32_t)(((g + EW * q) / AS) & 1);
                     if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(&s_empty[as], aph ^ 1u))) {
                         griddep_wait();
                         if (!warp_wait(&s_empty[as], aph ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x151); ok = false; }
@@ -397,11 +433,10 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                         if (lane == 0) mbar_arrive(&s_full[as]);
                     }
                 }
-                // the stage is released only after every word of it that this warp needs has gone through the expansion
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&w_empty[ws]);
-                if (++ws == WS) { ws = 0; wph ^= 1u; }
-                kb_base += ns;
+            }
+            if (c == i + 1 && c < total && ok) {
+                if (!warp_wait(&w_full[ws], wph, abort_flag)) { give_up(p.status, abort_flag, 0x152); ok = false; }
+                else take();
             }
         }
     }
