@@ -34,19 +34,18 @@ constexpr int kBlockK = 128;              // K per code stage and per operand st
 // A stage is a k-block's codes in shared memory and its expanded signs in tensor memory, under one pair of barriers: the issuing
 // thread runs one wait and one commit per k-block.  (With a ring and barriers for each operand the loop took 590 cycles per
 // k-block, 500 of them also without any of the copies, stores and MMAs: the issuing thread's waits and commits were the bound.)
-constexpr int WS = 2, AS = 4, EW = 4;
+constexpr int WS = 3, AS = 4, EW = 4;
 static_assert(AS % EW == 0, "an operand stage must keep one owner among the expander parts");
 constexpr int kEpiFirst = 128, kExpFirst = 256;
 constexpr int kThreads = kExpFirst + 128 * EW;       // 768
 constexpr int w_bytes = kRows * 128, b_bytes = kTok * 128;
 constexpr int u_off = WS * w_bytes + AS * b_bytes;
 constexpr int t_off = u_off + kRows * 128;
-constexpr int o_off = t_off + 3 * b_bytes;           // finished outputs [token][row] bf16
-constexpr int bars_off = o_off + kTok * kRows * 2;
+constexpr int bars_off = t_off + 3 * b_bytes;
 constexpr int n_bars = 2 * WS + 2 * AS + 12;
 constexpr int misc_off = bars_off + n_bars * 8;
-constexpr int tok_off = misc_off + 16;               // [2][scales, code sums, zero points][kTok]
-constexpr int used = tok_off + 2 * 12 * kTok;
+constexpr int tok_off = (misc_off + 31) / 16 * 16;   // [2][scales, code sums, zero points, corrections][kTok]
+constexpr int used = tok_off + 2 * 16 * kTok;
 constexpr int total = used + 1024;
 // tensor memory: two int32 accumulators (tiles alternate, so the MMAs of a tile never wait for the epilogue of the one
 // before), one fp32 low-rank accumulator (written at the very end of a tile's MMAs, long after the previous epilogue has
@@ -65,9 +64,15 @@ struct PersistParams {
     const __nv_bfloat16* U;
     __nv_bfloat16* out; int64_t ldo;
     int32_t* acc_debug;
+    int fast;                    // no zero points, no row shift, no accumulators wanted, sums below 2^22: the short epilogue
     uint32_t* status;
 };
 
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
 __device__ __forceinline__ uint4 lds_words(const uint8_t* p) {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
@@ -84,7 +89,6 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     uint8_t* bbuf = smem + WS * w_bytes;
     uint8_t* ubuf = smem + u_off;
     uint8_t* tbuf = smem + t_off;
-    __nv_bfloat16* otile = reinterpret_cast<__nv_bfloat16*>(smem + o_off);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + bars_off);
     uint64_t* w_full = bars;                 // [WS]
     uint64_t* w_empty = w_full + WS;
@@ -100,9 +104,12 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     uint64_t* epi_done = tok_full + 2;       // [2] the epilogue is through with them
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + misc_off);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + misc_off + 4);
-    auto tok_scale = [&](int buf) { return reinterpret_cast<float*>(smem + tok_off + buf * 12 * kTok); };
-    auto tok_qsum = [&](int buf) { return reinterpret_cast<int32_t*>(smem + tok_off + buf * 12 * kTok + 4 * kTok); };
-    auto tok_zp = [&](int buf) { return reinterpret_cast<int32_t*>(smem + tok_off + buf * 12 * kTok + 8 * kTok); };
+    // per token: scale, sum of the codes, zero point, and as a float what the epilogue takes from the raw sum (p.fast: 1.5 * 2^23 +
+    // sum of the codes) or what meets mu (otherwise: sum of the codes less K zero points)
+    auto tok_scale = [&](int buf) { return reinterpret_cast<float*>(smem + tok_off + buf * 16 * kTok); };
+    auto tok_qsum = [&](int buf) { return reinterpret_cast<int32_t*>(smem + tok_off + buf * 16 * kTok + 4 * kTok); };
+    auto tok_zp = [&](int buf) { return reinterpret_cast<int32_t*>(smem + tok_off + buf * 16 * kTok + 8 * kTok); };
+    auto tok_corr = [&](int buf) { return reinterpret_cast<float*>(smem + tok_off + buf * 16 * kTok + 12 * kTok); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles = p.row_tiles * p.tok_tiles;
@@ -186,7 +193,9 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                     qs = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
                 }
                 tok_qsum(buf)[j] = qs;
-                tok_zp(buf)[j] = (p.zp && t < p.M) ? p.zp[t] : 0;
+                const int32_t zp = (p.zp && t < p.M) ? p.zp[t] : 0;
+                tok_zp(buf)[j] = zp;
+                tok_corr(buf)[j] = p.fast ? 12582912.f + (float)qs : (float)(qs - p.K * zp);
             }
             __syncwarp();
             if (lane == 0) {
@@ -314,13 +323,34 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             if (ok && !warp_wait(d_full, (uint32_t)(i & 1), abort_flag)) { give_up(p.status, abort_flag, 0x142); ok = false; }
             if (ok) {
                 tc_fence_after();
-                const float* sc_s = tok_scale(buf);
-                const int32_t* qs_s = tok_qsum(buf);
-                const int32_t* zp_s = tok_zp(buf);
+                const float4* sc_s = reinterpret_cast<const float4*>(tok_scale(buf));
+                const float4* co_s = reinterpret_cast<const float4*>(tok_corr(buf));
+                const int4* qs_s = reinterpret_cast<const int4*>(tok_qsum(buf));
+                const int4* zp_s = reinterpret_cast<const int4*>(tok_zp(buf));
+                // Finished values go straight to global memory: a lane has one row and two tokens in a word, its neighbour the
+                // other row of the pair; they swap halves, and a store instruction writes 64 bytes of each token's outputs.
+                // (Through a shared-memory tile, one 16-bit store a value, with three scalar loads and two conversions beside
+                // it, the epilogue took 10.8 us a tile, longer than the K loop of 5120 it runs under.)
+                const int odd = lane & 1;
+                const uint32_t sel = odd ? 0x3276u : 0x5410u;
+                const int n_pair = n & ~1;
+                const bool pair_ok = ((reinterpret_cast<uintptr_t>(p.out) & 3) == 0) && (p.ldo & 1) == 0 && n_pair + 1 < p.N;
+                const uint32_t acc_addr = tmem_base + lane_addr + D_COL + (uint32_t)(i & 1) * kTok;
+                auto put = [&](uint32_t word, int tok) {          // word: tokens tok (low half) and tok + 1 of this lane's row
+                    const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 1);
+                    if (pair_ok) {
+                        const int t = t0 + tok + odd;
+                        if (t < p.M) *reinterpret_cast<uint32_t*>(p.out + (int64_t)t * p.ldo + n_pair) = __byte_perm(word, other, sel);
+                    } else if (valid_row) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            if (t0 + tok + h < p.M) p.out[(int64_t)(t0 + tok + h) * p.ldo + n] = __ushort_as_bfloat16((unsigned short)(word >> (16 * h)));
+                    }
+                };
 #pragma unroll 1
                 for (int c = 0; c < kTok / 16; ++c) {
                     uint32_t v[16], l[16];
-                    tmem_ld_32x16(tmem_base + lane_addr + D_COL + (uint32_t)(i & 1) * kTok + 16 * c, v);
+                    tmem_ld_32x16(acc_addr + 16 * c, v);
                     if (lowrank) tmem_ld_32x16(tmem_base + lane_addr + LR_COL + 16 * c, l);
                     tc_wait_ld();
                     if (c == kTok / 16 - 1) {
@@ -330,38 +360,47 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                         if (lane == 0) mbar_arrive(acc_free);
                     }
                     if (t0 + 16 * c >= p.M) continue;            // warp-uniform; nothing of this chunk is stored
+                    if (p.fast) {
+                        // the raw sum is -2^7 times the sum over the set bits; 2^23 * 1.5 + integer is a float by its bits, and
+                        // the difference to (2^23 * 1.5 + sum of the codes) is exact
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float sc = sc_s[16 * c + j];
-                        const int32_t qs = qs_s[16 * c + j], zp = zp_s[16 * c + j];
-                        const int32_t acc = -((int32_t)v[j] >> 6) - qs - zp * rs_n;
-                        if (p.acc_debug && valid_row && t0 + 16 * c + j < p.M) p.acc_debug[(int64_t)(t0 + 16 * c + j) * p.N + n] = acc;
-                        const float lr = lowrank ? __uint_as_float(l[j]) : 0.f;
-                        const float y = fmaf(__fmul_rn(mu_n, sc), (float)(qs - p.K * zp), __fmul_rn(__fmul_rn(alpha_n, sc), (float)acc) + lr);
-                        otile[(16 * c + j) * kRows + e] = __float2bfloat16_rn(y);
+                        for (int j = 0; j < 16; j += 4) {
+                            const float4 sc = sc_s[4 * c + (j >> 2)], co = co_s[4 * c + (j >> 2)];
+                            const float scs[4] = {sc.x, sc.y, sc.z, sc.w}, cos[4] = {co.x, co.y, co.z, co.w};
+                            float y[4];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                const float acc = __int_as_float(0x4B400000 - ((int32_t)v[j + h] >> 6)) - cos[h];
+                                y[h] = __fmul_rn(__fmul_rn(alpha_n, scs[h]), acc) + (lowrank ? __uint_as_float(l[j + h]) : 0.f);
+                            }
+                            put(pack_bf16x2(y[0], y[1]), 16 * c + j);
+                            put(pack_bf16x2(y[2], y[3]), 16 * c + j + 2);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; j += 4) {
+                            const float4 sc = sc_s[4 * c + (j >> 2)], co = co_s[4 * c + (j >> 2)];
+                            const int4 qs = qs_s[4 * c + (j >> 2)], zp = zp_s[4 * c + (j >> 2)];
+                            const float scs[4] = {sc.x, sc.y, sc.z, sc.w}, cos[4] = {co.x, co.y, co.z, co.w};
+                            const int32_t qss[4] = {qs.x, qs.y, qs.z, qs.w}, zps[4] = {zp.x, zp.y, zp.z, zp.w};
+                            float y[4];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                const int32_t acc = -((int32_t)v[j + h] >> 6) - qss[h] - zps[h] * rs_n;
+                                if (p.acc_debug && valid_row && t0 + 16 * c + j + h < p.M) p.acc_debug[(int64_t)(t0 + 16 * c + j + h) * p.N + n] = acc;
+                                y[h] = fmaf(__fmul_rn(mu_n, scs[h]), cos[h], __fmul_rn(__fmul_rn(alpha_n, scs[h]), (float)acc) + (lowrank ? __uint_as_float(l[j + h]) : 0.f));
+                            }
+                            if (p.out) {
+                                put(pack_bf16x2(y[0], y[1]), 16 * c + j);
+                                put(pack_bf16x2(y[2], y[3]), 16 * c + j + 2);
+                            }
+                        }
                     }
                 }
             } else if (!*abort_flag) {
                 *abort_flag = 1;
             }
-            asm volatile("bar.sync 1, 128;" ::: "memory");       // the output tile is complete (all epilogue warps, always)
-            if (ok && p.out) {
-                // 16 threads move one token's 128 outputs (256 bytes) with 128-bit stores
-                const bool vec = ((reinterpret_cast<uintptr_t>(p.out) & 15) == 0) && (p.ldo % 8 == 0) && (n0 + kRows <= p.N);
-                for (int tt = e >> 4; tt < kTok && t0 + tt < p.M; tt += 8) {
-                    const int c8 = (e & 15) * 8;
-                    __nv_bfloat16* dst = p.out + (int64_t)(t0 + tt) * p.ldo + n0 + c8;
-                    const uint4 val = *reinterpret_cast<const uint4*>(otile + tt * kRows + c8);
-                    if (vec) {
-                        *reinterpret_cast<uint4*>(dst) = val;
-                    } else {
-                        const __nv_bfloat16* sv = reinterpret_cast<const __nv_bfloat16*>(&val);
-                        for (int j = 0; j < 8; ++j)
-                            if (n0 + c8 + j < p.N) dst[j] = sv[j];
-                    }
-                }
-            }
-            asm volatile("bar.sync 1, 128;" ::: "memory");       // the tile buffer may be written again
+            __syncwarp();
             if (lane == 0) mbar_arrive(&epi_done[buf]);
         }
     } else if (warp >= 8) {
@@ -491,6 +530,7 @@ int launch_gemm_umma_persistent(const GemmArgs& a, const int8_t* codes_interleav
     p.M = M; p.N = N; p.K = K; p.row_tiles = (N + kRows - 1) / kRows; p.tok_tiles = (M + kTok - 1) / kTok; p.r = a.r;
     p.scales = a.scales; p.qsum = a.qsum; p.zp = a.zp; p.alpha = a.alpha; p.mu = a.mu; p.rowsum = a.rowsum;
     p.U = (const __nv_bfloat16*)a.U; p.out = (__nv_bfloat16*)a.out; p.ldo = a.ldo; p.acc_debug = a.acc_debug; p.status = a.status;
+    p.fast = !a.zp && !a.mu && !a.acc_debug && a.out && (int64_t)K << (a.bits - 1) < (int64_t)1 << 22;
     const int tiles = p.row_tiles * p.tok_tiles;
 
     static thread_local int configured = -1;
