@@ -36,8 +36,10 @@ constexpr int kBlockK = 128;              // K per code stage and per operand st
 // k-block, 500 of them also without any of the copies, stores and MMAs: the issuing thread's waits and commits were the bound.)
 constexpr int WS = 3, AS = 4, EW = 4;
 static_assert(AS % EW == 0, "an operand stage must keep one owner among the expander parts");
-constexpr int kEpiFirst = 128, kExpFirst = 256;
-constexpr int kThreads = kExpFirst + 128 * EW;       // 768
+// Two epilogue warps per lane quarter, 64 tokens each: one warp needs about eight cycles an instruction beside the expanders, and
+// with four warps the epilogue of a tile took 8 us, more than the K loop of 5120 it runs under.
+constexpr int kEpiFirst = 128, kExpFirst = 384;
+constexpr int kThreads = kExpFirst + 128 * EW;       // 896
 constexpr int w_bytes = kRows * 128, b_bytes = kTok * 128;
 constexpr int u_off = WS * w_bytes + AS * b_bytes;
 constexpr int t_off = u_off + kRows * 128;
@@ -104,8 +106,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     uint64_t* epi_done = tok_full + 2;       // [2] the epilogue is through with them
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + misc_off);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + misc_off + 4);
-    // per token: scale, sum of the codes, zero point, and as a float what the epilogue takes from the raw sum (p.fast: 1.5 * 2^23 +
-    // sum of the codes) or what meets mu (otherwise: sum of the codes less K zero points)
+    // per token: scale, sum of the codes, zero point, and the bits of the float 1.5 * 2^23 less the sum of the codes (p.fast) or,
+    // as a float, what meets mu (the sum of the codes less K zero points)
     auto tok_scale = [&](int buf) { return reinterpret_cast<float*>(smem + tok_off + buf * 16 * kTok); };
     auto tok_qsum = [&](int buf) { return reinterpret_cast<int32_t*>(smem + tok_off + buf * 16 * kTok + 4 * kTok); };
     auto tok_zp = [&](int buf) { return reinterpret_cast<int32_t*>(smem + tok_off + buf * 16 * kTok + 8 * kTok); };
@@ -129,10 +131,10 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         *abort_flag = 0;
         for (int i = 0; i < WS; ++i) { mbar_init(&w_full[i], 1); mbar_init(&w_empty[i], 4 * EW); }
         for (int i = 0; i < AS; ++i) { mbar_init(&s_full[i], 5); mbar_init(&s_empty[i], 1); }      // four expander warps and the copy
-        mbar_init(d_full, 1); mbar_init(acc_free, 4);
-        mbar_init(u_full, 4); mbar_init(u_empty, 1);
+        mbar_init(d_full, 1); mbar_init(acc_free, 8);
+        mbar_init(u_full, 8); mbar_init(u_empty, 1);
         mbar_init(t_full, 1); mbar_init(t_empty, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(&tok_full[i], 1); mbar_init(&epi_done[i], 4); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&tok_full[i], 1); mbar_init(&epi_done[i], 8); }
         fence_barrier_init();
         fence_proxy_async();
     }
@@ -170,7 +172,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             if (*abort_flag) for (int i = 0; i < 500; ++i) __nanosleep(100);
         }
     } else if (warp == 1) {
-        // ---------------- per-token scalars, codes and T ----------------
+        // ---------------- codes and T ----------------
         griddep_wait();
         if (lane == 0) {
             tma_prefetch_desc(&b_map);
@@ -178,28 +180,11 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             if (p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) *abort_flag = 1;   // the call already failed
         }
         __syncwarp();
-        int bs = 0; uint32_t bph = 0;
-        bool ok = true;
-        for (int i = 0; i < my_tiles && ok && !*abort_flag; ++i) {
-            const int t0 = tile_t0(i), buf = i & 1;
-            if (i >= 2 && !warp_wait(&epi_done[buf], (uint32_t)(((i >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x120); ok = false; break; }
-            for (int j = lane; j < kTok; j += 32) {
-                const int t = t0 + j;
-                tok_scale(buf)[j] = t < p.M ? p.scales[t] : 0.f;
-                int32_t qs = 0;
-                if (t < p.M) {
-                    const int4* parts = reinterpret_cast<const int4*>(p.qsum + (size_t)t * kQsumParts);
-                    const int4 a = parts[0], b = parts[1];
-                    qs = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
-                }
-                tok_qsum(buf)[j] = qs;
-                const int32_t zp = (p.zp && t < p.M) ? p.zp[t] : 0;
-                tok_zp(buf)[j] = zp;
-                tok_corr(buf)[j] = p.fast ? 12582912.f + (float)qs : (float)(qs - p.K * zp);
-            }
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&tok_full[buf]);
+        if (lane == 0) {
+            int bs = 0; uint32_t bph = 0;
+            bool ok = true;
+            for (int i = 0; i < my_tiles && ok && !*abort_flag; ++i) {
+                const int t0 = tile_t0(i);
                 int kb = u0 * (kUnitK / kBlockK);
                 for (int c = 0; c < kblocks; ++c) {
                     if (!wait_or_abort(&s_empty[bs], bph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x121); ok = false; break; }
@@ -217,9 +202,32 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                     }
                 }
             }
-            ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+            if (*abort_flag) for (int i = 0; i < 500; ++i) __nanosleep(100);
         }
-        if (lane == 0 && *abort_flag) for (int i = 0; i < 500; ++i) __nanosleep(100);
+    } else if (warp == 3) {
+        // ---------------- per-token scalars (a warp of its own: in the codes' warp their load latency, 2 us a tile, held up the
+        // codes of the tile) ----------------
+        griddep_wait();
+        for (int i = 0; i < my_tiles && !*abort_flag; ++i) {
+            const int t0 = tile_t0(i), buf = i & 1;
+            if (i >= 2 && !warp_wait(&epi_done[buf], (uint32_t)(((i >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x120); break; }
+            for (int j = lane; j < kTok; j += 32) {
+                const int t = t0 + j;
+                tok_scale(buf)[j] = t < p.M ? p.scales[t] : 0.f;
+                int32_t qs = 0;
+                if (t < p.M) {
+                    const int4* parts = reinterpret_cast<const int4*>(p.qsum + (size_t)t * kQsumParts);
+                    const int4 a = parts[0], b = parts[1];
+                    qs = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
+                }
+                tok_qsum(buf)[j] = qs;
+                const int32_t zp = (p.zp && t < p.M) ? p.zp[t] : 0;
+                tok_zp(buf)[j] = zp;
+                tok_corr(buf)[j] = p.fast ? __int_as_float(0x4B400000 - qs) : (float)(qs - p.K * zp);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tok_full[buf]);
+        }
     } else if (warp == 2) {
         // ---------------- MMA issue ----------------
         if (elect_one()) {
@@ -276,10 +284,11 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 tc_commit(d_full);
             }
         }
-    } else if (warp >= 4 && warp < 8) {
+    } else if (warp >= 4 && warp < 12) {
         // ---------------- epilogue ----------------
         const int q = warp & 3;
-        const int e = threadIdx.x - kEpiFirst;        // 0..127: output row of the tile
+        const int e = (threadIdx.x - kEpiFirst) & 127;        // output row of the tile
+        const int half = (warp - 4) >> 2;             // of the tile's tokens
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         bool ok = true;
         for (int i = 0; i < my_tiles; ++i) {
@@ -295,8 +304,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 if (ok) {
                     const bool vec = (p.r % 8 == 0) && ((reinterpret_cast<uintptr_t>(p.U) & 15) == 0);
 #pragma unroll
-                    for (int it = 0; it < 8; ++it) {
-                        const int idx = it * 128 + e;
+                    for (int it = 0; it < 4; ++it) {
+                        const int idx = it * 256 + half * 128 + e;
                         const int ur = idx >> 3, ch = idx & 7;
                         uint4 v = make_uint4(0u, 0u, 0u, 0u);
                         const int un = n0 + ur;
@@ -329,8 +338,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 const int4* zp_s = reinterpret_cast<const int4*>(tok_zp(buf));
                 // Finished values go straight to global memory: a lane has one row and two tokens in a word, its neighbour the
                 // other row of the pair; they swap halves, and a store instruction writes 64 bytes of each token's outputs.
-                // (Through a shared-memory tile, one 16-bit store a value, with three scalar loads and two conversions beside
-                // it, the epilogue took 10.8 us a tile, longer than the K loop of 5120 it runs under.)
+                // (Through a shared-memory tile, one 16-bit store a value with three scalar loads and two conversions beside
+                // it, four warps took 10.8 us a tile.)
                 const int odd = lane & 1;
                 const uint32_t sel = odd ? 0x3276u : 0x5410u;
                 const int n_pair = n & ~1;
@@ -348,12 +357,12 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                     }
                 };
 #pragma unroll 1
-                for (int c = 0; c < kTok / 16; ++c) {
+                for (int c = half * (kTok / 32); c < (half + 1) * (kTok / 32); ++c) {
                     uint32_t v[16], l[16];
                     tmem_ld_32x16(acc_addr + 16 * c, v);
                     if (lowrank) tmem_ld_32x16(tmem_base + lane_addr + LR_COL + 16 * c, l);
                     tc_wait_ld();
-                    if (c == kTok / 16 - 1) {
+                    if (c == (half + 1) * (kTok / 32) - 1) {
                         // both accumulators are in registers: the next tile's MMAs may start
                         tc_fence_before();
                         __syncwarp();
@@ -361,8 +370,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                     }
                     if (t0 + 16 * c >= p.M) continue;            // warp-uniform; nothing of this chunk is stored
                     if (p.fast) {
-                        // the raw sum is -2^7 times the sum over the set bits; 2^23 * 1.5 + integer is a float by its bits, and
-                        // the difference to (2^23 * 1.5 + sum of the codes) is exact
+                        // the raw sum is -2^7 times the sum over the set bits; 1.5 * 2^23 + integer (below 2^22) is a float by its
+                        // bits, and taking 1.5 * 2^23 off again is exact
 #pragma unroll
                         for (int j = 0; j < 16; j += 4) {
                             const float4 sc = sc_s[4 * c + (j >> 2)], co = co_s[4 * c + (j >> 2)];
@@ -370,7 +379,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                             float y[4];
 #pragma unroll
                             for (int h = 0; h < 4; ++h) {
-                                const float acc = __int_as_float(0x4B400000 - ((int32_t)v[j + h] >> 6)) - cos[h];
+                                const float acc = __int_as_float(__float_as_int(cos[h]) - ((int32_t)v[j + h] >> 6)) - 12582912.f;
                                 y[h] = __fmul_rn(__fmul_rn(alpha_n, scs[h]), acc) + (lowrank ? __uint_as_float(l[j + h]) : 0.f);
                             }
                             put(pack_bf16x2(y[0], y[1]), 16 * c + j);
@@ -403,10 +412,10 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             __syncwarp();
             if (lane == 0) mbar_arrive(&epi_done[buf]);
         }
-    } else if (warp >= 8) {
+    } else if (warp >= 12) {
         // ---------------- expansion of sign bits into the operand ring (tile boundaries do not matter here) ----------------
         const int q = warp & 3;
-        const int part = (warp - 8) >> 2;             // which of the EW warps of the lane quarter
+        const int part = (warp - 12) >> 2;             // which of the EW warps of the lane quarter
         const int row = q * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         // A warp's words of a unit (two blocks of eight) go to registers, a unit ahead, and the stage is let go at once: the copies
