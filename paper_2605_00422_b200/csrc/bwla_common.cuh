@@ -197,6 +197,12 @@ int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void*
 // stored zero point z - 2^(b-1) + code_bias; a code minus the zero point times the scale is the value it stands for.
 int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream);
+// The same for many tokens, on the tcgen05 tensor cores (rot_umma.cu); x in 16-byte pieces.  launch_rot goes there by itself.
+bool rot_umma_supports(const RotGeom& g, int64_t M, int n_problems, const RotProblem* problems);
+int launch_rot_umma(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
+                    const RotProblem* problems, uint32_t* status, cudaStream_t stream);
+// how many clusters of a kernel the device holds at once
+int resident_clusters(const void* kernel, int dc, int threads, size_t smem);
 // Rows of weights (fp32 or bf16): packed signs, scale and shift of every row.
 int launch_rot_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status,
                         cudaStream_t stream);

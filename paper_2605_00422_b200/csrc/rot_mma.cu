@@ -906,18 +906,18 @@ static RotKernel pick_kernel(const RotGeom& g) {
 }
 
 // How many clusters of the kernel the device holds at once (asked once per kernel, size and thread).
-static int resident_clusters(RotKernel k, int dc, int threads, size_t smem) {
-    struct Known { RotKernel k; int dc, threads, dev, n; size_t smem; };
+int resident_clusters(const void* k, int dc, int threads, size_t smem) {
+    struct Known { const void* k; int dc, threads, dev, n; size_t smem; };
     static thread_local Known known[16];
     static thread_local int used = 0;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
     for (int i = 0; i < 16 && i < used; ++i)
         if (known[i].k == k && known[i].dc == dc && known[i].threads == threads && known[i].dev == dev && known[i].smem == smem) return known[i].n;
-    if (cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRotMaxSmem) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRotMaxSmem) != cudaSuccess) { cudaGetLastError(); return 0; }
     int n = 0;
     if (dc == 1) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, (const void*)k, threads, smem) != cudaSuccess) { cudaGetLastError(); return 0; }
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) { cudaGetLastError(); return 0; }
         n *= sm_count();
     } else {
         cudaLaunchConfig_t cfg{};
@@ -928,7 +928,7 @@ static int resident_clusters(RotKernel k, int dc, int threads, size_t smem) {
         a[0].id = cudaLaunchAttributeClusterDimension;
         a[0].val.clusterDim.x = (unsigned)dc; a[0].val.clusterDim.y = 1; a[0].val.clusterDim.z = 1;
         cfg.attrs = a; cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n, (const void*)k, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+        if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     }
     known[used % 16] = Known{k, dc, threads, dev, n, smem};
     ++used;
@@ -944,7 +944,7 @@ static int choose_groups(const RotGeom& g, int64_t M, int n_problems) {
 static int launch_rot_kernel(RotKernel k, const RotGeom& g, RotKernelParams& p, size_t smem, int lr_total, cudaStream_t stream) {
     const int threads = 32 * g.warps * p.groups;
     smem = std::max(smem, (size_t)(g.group_off + p.groups * g.group_bytes));
-    const int room = resident_clusters(k, g.dc, threads, smem) / p.n_problems;
+    const int room = resident_clusters((const void*)k, g.dc, threads, smem) / p.n_problems;
     if (room < 1) return cuda_fail(cudaErrorInvalidConfiguration);
     p.clusters_per_problem = (int)std::min<int64_t>((p.M + p.groups - 1) / p.groups, room);
     p.rot_ctas = p.n_problems * p.clusters_per_problem * g.dc;
@@ -1028,6 +1028,8 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
         }
     }
     for (int i = n_problems; i <= kRotMaxProblems; ++i) p.lr_begin[i] = lr_total;
+    if (lr_total == 0 && p.x_vec && rot_umma_supports(base, M, n_problems, problems))
+        return launch_rot_umma(base, x, M, ldx, bits, asym, n_problems, problems, status, stream);
     RotKernel k = problems[0].yhat ? pick_kernel<kRotBf16, false>(g) : problems[0].digits ? pick_kernel<kRotDigits, false>(g) : pick_kernel<kRotQuant, false>(g);
     return launch_rot_kernel(k, g, p, smem, lr_total, stream);
 }

@@ -1,0 +1,561 @@
+// Online OKT (Sec. 3.1) for many tokens on the tcgen05 tensor cores, with the per-token quantiser (Sec. 4.1) or the bf16
+// rounding of the weight-only operating point fused in.  The warp-level kernel (rot_mma.cu) serves fewer tokens, every other
+// mode, and the factor sizes this one does not take.
+//
+//   X = reshape(x_t, n1 x n2) (row-major),   Z^T = P2^T X^T  [d][a],   Y^T = Z^T P1  [d][c]
+//
+// The same sums of products as there: x against the three bf16 terms of P2, then two fp16 terms of Z against two of P1 (three
+// products), small products first.  Z is scaled by a power of two per row d (its largest magnitude goes to [2^14, 2^15)), which
+// leaves exactly, row by row, with the scale of P1.
+//
+// What bounds it: 160 x 160 takes 60 MMAs of 128 x 160 x 16 a token and CTA (2400 cycles), and every value of Z and Y passes
+// through registers once (about 450 instructions a warp, 4 warps a scheduler: 1800 cycles); the warp-level kernel needs 9600
+// cycles of its MMAs alone, with operands re-read from shared memory as fast as it delivers, and one token's barriers stand
+// open.  So the two run side by side, three steps deep:
+//   MMA thread    Z(0), Z(1), Y(0), Z(2), Y(1), ...    Z(i) and Y(i) share one of two accumulators
+//   16 ALU warps  step i: Y(i-1) to registers, its largest magnitude published  (accumulator free: Z(i+1) may start)
+//                         Z(i) to two fp16 terms in tensor memory               (Y(i) may start)
+//                         Y(i-1) quantised and stored
+// A step is 1, 2 or 4 tokens, so that it fills up to 160 columns (64 x 80: 2 tokens).  Factors whose terms do not fit one CTA
+// (or with n2 > 128) are split by rows d over a cluster of two, which share nothing but the largest magnitudes.
+// 2048 tokens of 160 x 160: see kManyTokens below.
+//
+// Launched with programmatic stream serialisation: the factors are fetched before the preceding kernel of the stream has
+// finished; x is read, and everything is stored, after it.  Every wait is bounded (umma_wait.cuh).
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "bwla_common.cuh"
+#include "rot_mma.cuh"
+#include "tensor_map.cuh"
+#include "umma_ptx.cuh"
+#include "umma_wait.cuh"
+
+namespace bwla {
+
+namespace ru {
+constexpr int kAluWarps = 16;
+constexpr int kThreads = 128 + 32 * kAluWarps;
+constexpr int kPrepHeader = 256;          // of the prepared factors (rot_mma.cu)
+constexpr int kMaxSmem = 232448;
+struct Shared {
+    uint64_t x_full[2], x_empty[2];       // a step's x has landed; the MMAs that read it have completed
+    uint64_t z_full[2], y_full[2];        // accumulator i & 1 holds Z, Y
+    uint64_t d_free[2];                   // ... has been read
+    uint64_t a_ready;                     // the terms of Z are in tensor memory
+    uint64_t row_full[2][4];              // the exponents of a lane quarter's rows are there
+    uint64_t max_full[2];                 // all warps of the token (both CTAs) have left their maxima
+    uint32_t amax[2][32], vmin[2][32];    // [step parity][CTA][column part][lane quarter]
+    uint8_t zexp[2][4][32][4];            // biased exponents of the rows' largest |Z|: [step parity][quarter][lane][column part]
+    int qsum[2][4], count[2][4];          // code sums of the step's tokens, warps that have added theirs
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+constexpr int kSharedBytes = (int)((sizeof(Shared) + 127) / 128 * 128);
+}  // namespace ru
+
+struct RotUmmaGeom {
+    int n1, n2, K;
+    int nc;                 // columns of a token's Y: n1 rounded up to 16
+    int np;                 // columns of a token in the accumulators
+    int tps, ntot;          // tokens of a step, tps * np
+    int dc, dt;             // CTAs of a token, rows d of each
+    int atoms2, atoms1;     // K atoms of 32 elements over b / over a
+    int xb;                 // buffers of x
+    int p1_off, x_off, sh_off, total;
+    int s2, s1;             // row strides of the prepared factors
+};
+
+// False when the sizes are outside what the kernel takes: whole 16-byte pieces of the codes' order (n2 a multiple of 16), three
+// times n1 columns of tensor memory, at most 128 rows and the factors' terms in the shared memory of one CTA or of two.
+static bool rot_umma_geometry(const RotGeom& g, RotUmmaGeom* out) {
+    if (g.n2 % 16 != 0 || g.n2 < 16 || g.n1 > 160) return false;
+    RotUmmaGeom u{};
+    u.n1 = g.n1; u.n2 = g.n2; u.K = g.K; u.s2 = g.s2; u.s1 = g.s1;
+    u.nc = g.na * 8;
+    u.tps = u.nc <= 32 ? 4 : u.nc <= 80 ? 2 : 1;
+    u.np = u.tps == 1 ? (u.nc + 31) / 32 * 32 : u.nc;
+    u.ntot = u.tps * u.np;
+    u.atoms2 = (g.n2 + 31) / 32; u.atoms1 = (u.nc + 31) / 32;
+    for (u.dc = 1; u.dc <= 2; ++u.dc) {
+        u.dt = u.dc == 1 ? g.n2 : (g.n2 / 2 + 15) / 16 * 16;
+        if (u.dt > 128) continue;
+        for (u.xb = 2; u.xb >= 1; --u.xb) {
+            u.p1_off = 3 * u.atoms2 * u.dt * 64;
+            u.x_off = u.p1_off + 2 * u.atoms1 * u.nc * 64;
+            u.sh_off = u.x_off + u.xb * u.atoms2 * u.ntot * 64;
+            u.total = u.sh_off + ru::kSharedBytes;
+            // (an MMA reads 128 rows from the first row of any block of P2's terms)
+            if (u.total <= ru::kMaxSmem && u.p1_off - u.dt * 64 + 128 * 64 <= u.total) { *out = u; return true; }
+        }
+    }
+    return false;
+}
+
+struct RotUmmaParams {
+    RotUmmaGeom g;
+    int64_t M;
+    int bits, asym;
+    int n_problems, clusters_per_problem;
+    RotProblem prob[kRotMaxProblems];
+    uint32_t* status;
+};
+
+namespace {
+__device__ __forceinline__ void tmem_ld_32x8(uint32_t taddr, uint32_t* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_st_32x4(uint32_t taddr, const uint32_t (&v)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                 ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ bool warp_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+    for (uint32_t i = 0; i < kWaitLimit; ++i) {
+        const bool done = mbar_try_wait_cluster(bar, parity, kParkNs);
+        if (__all_sync(0xFFFFFFFFu, done)) return true;
+        if (*abort_flag) return false;
+    }
+    return false;
+}
+}  // namespace
+
+// NC: 8-column chunks of a step one ALU warp owns, at most.  BF16: the weight-only operating point.
+template <int NC, bool BF16>
+__global__ void __launch_bounds__(ru::kThreads, 1)
+rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ RotUmmaParams p) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const RotUmmaGeom& g = p.g;
+    ru::Shared& sh = *reinterpret_cast<ru::Shared*>(smem + g.sh_off);
+    volatile int* abort_flag = &sh.abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = g.dc > 1 ? (int)cluster_ctarank() : 0;
+    const int cl = (int)blockIdx.x / g.dc;
+    const int prob_i = cl / p.clusters_per_problem;
+    const RotProblem& pr = p.prob[prob_i];
+    const int64_t first = cl - (int64_t)prob_i * p.clusters_per_problem;      // steps first, first + clusters, ...
+    const int64_t steps_all = (p.M + g.tps - 1) / g.tps;
+    int n = first < steps_all ? (int)((steps_all - first + p.clusters_per_problem - 1) / p.clusters_per_problem) : 0;
+    const int rows = min(g.dt, g.n2 - rank * g.dt);
+
+    // ---- the layer's factors (they do not depend on the preceding kernel): rows of 64 bytes, swizzled ----
+    const uint8_t* t2 = pr.prepared + ru::kPrepHeader;
+    const size_t all2 = (size_t)g.n2 * g.s2;
+    const uint8_t* t1 = t2 + 3 * all2;
+    {
+        const int cpr2 = g.n2 >> 3;
+        for (int i = threadIdx.x; i < 3 * rows * cpr2; i += ru::kThreads) {
+            const int rr = i / cpr2, ch = i - rr * cpr2, term = rr / rows, r = rr - term * rows;
+            uint8_t* dst = smem + ((term * g.atoms2 + (ch >> 2)) * g.dt + r) * 64 + (((ch ^ (r >> 1)) & 3) << 4);
+            cp_async16(smem_u32(dst), t2 + term * all2 + (size_t)(rank * g.dt + r) * g.s2 + 16 * ch);
+        }
+        const int cpr1 = g.nc >> 3;
+        for (int i = threadIdx.x; i < 2 * g.nc * cpr1; i += ru::kThreads) {
+            const int rr = i / cpr1, ch = i - rr * cpr1, term = rr / g.nc, r = rr - term * g.nc;
+            uint8_t* dst = smem + g.p1_off + ((term * g.atoms1 + (ch >> 2)) * g.nc + r) * 64 + (((ch ^ (r >> 1)) & 3) << 4);
+            cp_async16(smem_u32(dst), t1 + (size_t)term * g.nc * g.s1 + (size_t)r * g.s1 + 16 * ch);
+        }
+    }
+    const int e1 = __ldg(reinterpret_cast<const int*>(pr.prepared) + 1);
+    if (threadIdx.x == 0) {
+        sh.abort_flag = 0;
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sh.x_full[i], 1); mbar_init(&sh.x_empty[i], 1);
+            mbar_init(&sh.z_full[i], 1); mbar_init(&sh.y_full[i], 1);
+            mbar_init(&sh.d_free[i], ru::kAluWarps); mbar_init(&sh.max_full[i], ru::kAluWarps * g.dc);
+            for (int j = 0; j < 4; ++j) { sh.qsum[i][j] = sh.count[i][j] = 0; mbar_init(&sh.row_full[i][j], 4); }
+        }
+        mbar_init(&sh.a_ready, ru::kAluWarps);
+        fence_barrier_init();
+    }
+    if (warp == 2) {
+        tmem_alloc(&sh.tmem_slot, 512);
+        tmem_relinquish();
+    }
+    cp_async_wait_all();
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    if (g.dc > 1) { cluster_arrive_release(); cluster_wait_acquire(); }       // the other CTA's barriers stand
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&sh.tmem_slot);
+    griddep_launch_dependents();
+    griddep_wait();                                   // x may be the output of the preceding kernel
+    if (p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) n = 0;      // the call already failed
+
+    if (warp == 0) {
+        // ---------------- x ----------------
+        if (elect_one()) {
+            tma_prefetch_desc(&x_map);
+            const int atom_bytes = g.ntot * 64;
+            for (int i = 0; i < n; ++i) {
+                const int b = g.xb == 2 ? i & 1 : 0;
+                const uint32_t use = (uint32_t)(g.xb == 2 ? i >> 1 : i);
+                if (!wait_or_abort(&sh.x_empty[b], (use & 1u) ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x210); break; }
+                const int t0 = (int)((first + (int64_t)i * p.clusters_per_problem) * g.tps);
+                uint8_t* dst = smem + g.x_off + b * g.atoms2 * atom_bytes;
+                mbar_expect_tx(&sh.x_full[b], (uint32_t)(g.atoms2 * atom_bytes));
+                for (int a = 0; a < g.atoms2; ++a) tma_load_3d(dst + a * atom_bytes, &x_map, 32 * a, 0, t0, &sh.x_full[b]);
+            }
+            if (*abort_flag) for (int i = 0; i < 500; ++i) __nanosleep(100);
+        }
+    } else if (warp == 1) {
+        // ---------------- MMAs ----------------
+        if (elect_one()) {
+            const uint32_t idesc_a = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.ntot >> 3) << 17) | ((128u >> 4) << 24);
+            const uint32_t idesc_c = (1u << 4) | ((uint32_t)(g.nc >> 3) << 17) | ((128u >> 4) << 24);
+            const uint64_t d_p2 = smem_desc_kmajor(smem_u32(smem), 64), d_p1 = smem_desc_kmajor(smem_u32(smem + g.p1_off), 64);
+            const uint64_t d_x = smem_desc_kmajor(smem_u32(smem + g.x_off), 64);
+            const uint32_t blk2 = (uint32_t)(g.dt * 64) >> 4, blkx = (uint32_t)(g.ntot * 64) >> 4, blk1 = (uint32_t)(g.nc * 64) >> 4;
+            const int ks2 = g.n2 >> 4, ks1 = g.nc >> 4;
+            auto put_z = [&](int i) -> bool {
+                const int b = g.xb == 2 ? i & 1 : 0;
+                const uint32_t use = (uint32_t)(g.xb == 2 ? i >> 1 : i);
+                if (!wait_or_abort(&sh.x_full[b], use & 1u, abort_flag)) { give_up(p.status, abort_flag, 0x220); return false; }
+                if (i >= 2 && !wait_or_abort(&sh.d_free[i & 1], (uint32_t)(((i >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x221); return false; }
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)((i & 1) * g.ntot);
+                const uint64_t xd = d_x + (uint64_t)((uint32_t)(b * g.atoms2) * blkx);
+                uint32_t acc = 0u;
+                for (int term = 2; term >= 0; --term)
+                    for (int k = 0; k < ks2; ++k) {
+                        mma_f16_ss(d, d_p2 + (uint64_t)((uint32_t)(term * g.atoms2 + (k >> 1)) * blk2 + 2u * (k & 1)),
+                                   xd + (uint64_t)((uint32_t)(k >> 1) * blkx + 2u * (k & 1)), idesc_a, acc);
+                        acc = 1u;
+                    }
+                tc_commit(&sh.x_empty[b]);
+                tc_commit(&sh.z_full[i & 1]);
+                return true;
+            };
+            bool ok = n > 0 ? put_z(0) : false;
+            for (int i = 0; i < n && ok; ++i) {
+                if (i + 1 < n && !put_z(i + 1)) break;
+                if (!wait_or_abort(&sh.a_ready, (uint32_t)(i & 1), abort_flag)) { give_up(p.status, abort_flag, 0x222); break; }
+                tc_fence_after();
+                for (int tk = 0; tk < g.tps; ++tk) {
+                    const uint32_t d = tmem + (uint32_t)((i & 1) * g.ntot + tk * g.np);
+                    const uint32_t a = tmem + (uint32_t)(2 * g.ntot + tk * (g.np >> 1));
+                    // lo hi, hi lo, hi hi
+#pragma unroll 1
+                    for (int q = 0; q < 3; ++q)
+                        for (int k = 0; k < ks1; ++k)
+                            mma_f16_ts(d, a + (q == 0 ? (uint32_t)(g.ntot >> 1) : 0u) + 8u * k,
+                                       d_p1 + (uint64_t)((uint32_t)((q == 1 ? g.atoms1 : 0) + (k >> 1)) * blk1 + 2u * (k & 1)), idesc_c,
+                                       (q | k) ? 1u : 0u);
+                }
+                tc_commit(&sh.y_full[i & 1]);
+            }
+        }
+    } else if (warp >= 4) {
+        // ---------------- everything between and behind the MMAs ----------------
+        const int w = warp - 4, q = w & 3, wc = w >> 2;
+        const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
+        const int cw = g.ntot >> 2;                   // columns of the step this warp owns
+        const int tk = wc * g.tps >> 2;               // their token
+        const int c_base = wc * cw - tk * g.np;       // first of them within the token
+        const bool some = q * 32 < rows, valid = q * 32 + lane < rows;        // (16 lanes at a time)
+        const int d = rank * g.dt + q * 32 + lane;
+        const int qmax = (1 << (p.bits - 1)) - 1;
+        const bool asym = p.asym != 0;
+        const int parts = 4 / g.tps;                  // warps of a token in a lane quarter
+        float y[NC * 8];
+        int z_exp = 0;
+        bool ok = true;
+#pragma unroll 1
+        for (int i = 0; i <= n && ok; ++i) {
+            const int pi = (i - 1) & 1;
+            const int64_t t = (first + (int64_t)(i - 1) * p.clusters_per_problem) * g.tps + tk;
+            float amax = 0.f, vmin = 0.f;
+            if (i > 0) {
+                // ---- Y of the step before to registers, at true scale; its extremes to the token's other warps
+                if (!warp_wait(&sh.y_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x230); ok = false; break; }
+                tc_fence_after();
+                if (some) {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+                        if (8 * j < cw) tmem_ld_32x8(tmem + lane_addr + (uint32_t)(pi * g.ntot + wc * cw + 8 * j), reinterpret_cast<uint32_t*>(y) + 8 * j);
+                    tc_wait_ld();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.d_free[pi]);
+                const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
+                const float f1 = pow2f(ey1), f2 = pow2f(ey2);
+                const bool far = __any_sync(0xFFFFFFFFu, ey2 != 0);
+#pragma unroll
+                for (int j = 0; j < NC; ++j) {
+                    // (columns beyond P1's rows and rows beyond P2's hold anything)
+                    const bool keep = valid && 8 * j < cw && c_base + 8 * j < g.nc;
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        float &a = y[8 * j + e], &b = y[8 * j + e + 1];
+                        mul2(a, b, f1);
+                        if (far) mul2(a, b, f2);
+                        if (!keep) a = b = 0.f;
+                        if (!BF16) {
+                            if (!asym) amax = fmaxf(amax, fmaxf(fabsf(a), fabsf(b)));
+                            else { amax = fmaxf(amax, fmaxf(a, b)); vmin = fminf(vmin, fminf(a, b)); }
+                        }
+                    }
+                }
+                if (!BF16) {
+                    // non-negative (NaNs aside), so their bit patterns order like the values
+                    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));
+                    const uint32_t v = asym ? __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(-vmin, 0.f))) : 0u;
+                    uint32_t* slot = &sh.amax[pi][rank * 16 + w];
+                    uint32_t* slot_v = &sh.vmin[pi][rank * 16 + w];
+                    if (g.dc == 1) {
+                        if (lane == 0) { *slot = m; *slot_v = v; mbar_arrive(&sh.max_full[pi]); }
+                    } else if (lane < 2) {
+                        st_shared_cluster_u32(map_shared_rank(smem_u32(slot), (uint32_t)lane), m);
+                        if (asym) st_shared_cluster_u32(map_shared_rank(smem_u32(slot_v), (uint32_t)lane), v);
+                        mbar_arrive_remote(map_shared_rank(smem_u32(&sh.max_full[pi]), (uint32_t)lane));
+                    }
+                }
+            }
+            if (i < n) {
+                // ---- Z of this step: the power of two of every row, then its two fp16 terms, in place of the step before's (whose
+                // MMAs have completed: this warp has seen Y above)
+                const int zi = i & 1;
+                if (!warp_wait(&sh.z_full[zi], (uint32_t)((i >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x231); ok = false; break; }
+                tc_fence_after();
+                const uint32_t src = tmem + lane_addr + (uint32_t)(zi * g.ntot + wc * cw);
+                if (some) {
+                    uint32_t m = 0u;
+#pragma unroll
+                    for (int j = 0; j < NC; j += 2) {
+                        uint32_t v[16];
+                        if (8 * j < cw) tmem_ld_32x8(src + 8 * j, v);
+                        if (j + 1 < NC && 8 * (j + 1) < cw) tmem_ld_32x8(src + 8 * (j + 1), v + 8);
+                        tc_wait_ld();
+                        if (8 * j < cw)
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) m = max(m, v[e] & 0x7FFFFFFFu);
+                        if (j + 1 < NC && 8 * (j + 1) < cw)
+#pragma unroll
+                            for (int e = 8; e < 16; ++e) m = max(m, v[e] & 0x7FFFFFFFu);
+                    }
+                    sh.zexp[zi][q][lane][wc] = (uint8_t)(m >> 23);
+                }
+                __syncwarp();
+                if (parts > 1) {
+                    if (lane == 0) mbar_arrive(&sh.row_full[zi][q]);
+                    if (!warp_wait(&sh.row_full[zi][q], (uint32_t)((i >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x233); ok = false; break; }
+                }
+                if (some) {
+                    const uint32_t ex4 = *reinterpret_cast<const volatile uint32_t*>(&sh.zexp[zi][q][lane][0]);
+                    uint32_t ex = 0u;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if ((j * g.tps >> 2) == tk) ex = max(ex, (ex4 >> (8 * j)) & 0xFFu);
+                    z_exp = max(-126, min(126, 14 + 127 - (int)ex));
+                    const float z_scale = pow2f(z_exp);
+                    const uint32_t dst = tmem + lane_addr + (uint32_t)(2 * g.ntot + (wc * cw >> 1));
+#pragma unroll
+                    for (int j = 0; j < NC; ++j) {
+                        if (8 * j < cw) {
+                            uint32_t v[8], h[4], l[4];
+                            tmem_ld_32x8(src + 8 * j, v);
+                            tc_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                float a = __uint_as_float(v[2 * e]), b = __uint_as_float(v[2 * e + 1]);
+                                mul2(a, b, z_scale);
+                                split2_pair(a, b, h[e], l[e]);
+                            }
+                            tmem_st_32x4(dst + 4 * j, h);
+                            tmem_st_32x4(dst + (uint32_t)(g.ntot >> 1) + 4 * j, l);
+                        }
+                    }
+                    tc_wait_st();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.a_ready);
+            }
+            if (i == 0) continue;
+            // ---- the step before: codes, scale and code sum, or bf16 values
+            if (BF16) {
+                if (t < p.M && valid) {
+                    // layout 1: inside each group of 32, position 2 (k % 16) + (k % 32) / 16
+                    __nv_bfloat16* yt = pr.yhat + t * (int64_t)g.K;
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const int c = c_base + 8 * j + e;
+                            if (8 * j < cw && c < g.n1) {
+                                const int k = c * g.n2 + d;
+                                yt[pr.codes_layout ? (k & ~31) + 2 * (k & 15) + ((k >> 4) & 1) : k] = __float2bfloat16_rn(y[8 * j + e]);
+                            }
+                        }
+                }
+                continue;
+            }
+            if (g.dc == 1 ? !warp_wait(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)
+                          : !warp_wait_cluster(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)) {
+                give_up(p.status, abort_flag, 0x232); ok = false; break;
+            }
+            {
+                const bool mine = lane < 16 * g.dc && (((lane & 15) >> 2) * g.tps >> 2) == tk;
+                amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, mine ? *reinterpret_cast<volatile uint32_t*>(&sh.amax[pi][lane]) : 0u));
+                if (asym) vmin = -__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, mine ? *reinterpret_cast<volatile uint32_t*>(&sh.vmin[pi][lane]) : 0u));
+            }
+            if (t < p.M) {
+                // The quantiser of rot_mma.cu, word for word the same roundings: fl(v + 1.5 * 2^23 + shift) leaves rne(v) + shift in
+                // the low mantissa bits, the low byte is stored, the patterns are summed.
+                float inv = 0.f, scale = 1.f, zero_f = 0.f, half_f = 0.f, levels = 0.f;
+                if (!asym) {
+                    if (amax != 0.f) { inv = __fdiv_rn((float)qmax, amax); scale = __fdiv_rn(amax, (float)qmax); }
+                } else {
+                    levels = (float)((1 << p.bits) - 1);
+                    const float range = __fsub_rn(amax, vmin);
+                    if (range != 0.f) { inv = __fdiv_rn(levels, range); scale = __fdiv_rn(range, levels); }
+                    const float tz = __fmul_rn(-vmin, inv);
+                    zero_f = fminf(fmaxf(__fadd_rn(__fadd_rn(tz, 12582912.f), -12582912.f), 0.f), levels);
+                    half_f = (float)(1 << (p.bits - 1));
+                }
+                const float store_shift = (float)pr.code_bias - half_f;
+                const int shift_i = (int)(zero_f + store_shift);
+                const uint32_t odd = (uint32_t)(shift_i & 1);
+                const float bias_even = 12582912.f + (float)(shift_i - (int)odd);
+                const float lo_b = 12582912.f + store_shift - (float)odd, hi_b = lo_b + levels;
+                int8_t* ct = pr.codes + t * (int64_t)g.K;
+                // Two columns at a time: lanes 8 apart have neighbouring bytes of a column in the contraction's order, so one
+                // of the two stores both lanes' codes of the first column, the other those of the second.
+                const int hb = (lane >> 3) & 1;
+                const uint32_t sel = hb ? 0x0004u : 0x0040u;
+                const int k0 = (c_base + hb) * g.n2 + (d & ~8);
+                int8_t* at = ct + (k0 & ~31) + 4 * (k0 & 7) + ((k0 & 31) >> 3);
+                int8_t* at_plain = ct + c_base * g.n2 + d;
+                uint32_t usum = 0u;
+                int counted = 0;
+                if (some) {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j) {
+                        if (8 * j < cw && c_base + 8 * j < g.n1) {
+#pragma unroll
+                            for (int e = 0; e < 8; e += 2) {
+                                const int c = c_base + 8 * j + e;
+                                float v0 = __fmul_rn(y[8 * j + e], inv), v1 = __fmul_rn(y[8 * j + e + 1], inv);
+                                add2(v0, v1, bias_even, bias_even);
+                                uint32_t w0 = __float_as_uint(v0), w1 = __float_as_uint(v1);
+                                if (asym) {
+                                    w0 = __float_as_uint(fminf(fmaxf(v0, lo_b), hi_b)) + odd;
+                                    w1 = __float_as_uint(fminf(fmaxf(v1, lo_b), hi_b)) + odd;
+                                }
+                                if (c < g.n1) { usum += w0; ++counted; }
+                                if (c + 1 < g.n1) { usum += w1; ++counted; }
+                                if (pr.codes_layout) {
+                                    const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, hb ? w0 : w1, 8);
+                                    if (valid && c + hb < g.n1) *reinterpret_cast<uint16_t*>(at) = (uint16_t)__byte_perm(hb ? w1 : w0, other, sel);
+                                    at += 2 * g.n2;
+                                } else {
+                                    if (valid && c < g.n1) at_plain[0] = (int8_t)w0;
+                                    if (valid && c + 1 < g.n1) at_plain[g.n2] = (int8_t)w1;
+                                    at_plain += 2 * g.n2;
+                                }
+                            }
+                        }
+                    }
+                }
+                if (pr.y && valid) {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (8 * j < cw && c_base + 8 * j + e < g.n1) pr.y[t * (int64_t)g.K + (c_base + 8 * j + e) * g.n2 + d] = y[8 * j + e];
+                }
+                if (pr.qsum) {
+                    // the token's last warp of this CTA to add its sum leaves the CTA's part; the consumer adds the parts
+                    int local = valid ? (int)(usum - (uint32_t)counted * (0x4B400000u + (uint32_t)pr.code_bias)) : 0;
+                    local = __reduce_add_sync(0xFFFFFFFFu, local);
+                    int last = 0, sum = 0;
+                    if (lane == 0) {
+                        if (local != 0) atomicAdd(&sh.qsum[pi][tk], local);
+                        __threadfence_block();
+                        last = atomicAdd(&sh.count[pi][tk], 1) == 4 * parts - 1;
+                        if (last) {
+                            __threadfence_block();
+                            sum = atomicExch(&sh.qsum[pi][tk], 0);
+                            sh.count[pi][tk] = 0;
+                        }
+                    }
+                    last = __shfl_sync(0xFFFFFFFFu, last, 0);
+                    sum = __shfl_sync(0xFFFFFFFFu, sum, 0);
+                    if (last && lane < kQsumParts && (lane == rank || (rank == 0 && lane >= g.dc)))
+                        pr.qsum[t * kQsumParts + lane] = lane == rank ? sum : 0;
+                }
+                if (lane == 0 && rank == 0 && q == 0 && c_base == 0) {
+                    pr.scales[t] = scale;
+                    if (pr.zp) pr.zp[t] = shift_i;
+                }
+            }
+        }
+        if (!ok) *abort_flag = 1;
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 2) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+    // nobody leaves while the other CTA may still store into its shared memory
+    if (g.dc > 1) { cluster_arrive_release(); cluster_wait_acquire(); }
+}
+
+bool rot_umma_supports(const RotGeom& base, int64_t M, int n_problems, const RotProblem* problems) {
+    // more tokens than rot_mma.cu spreads over the SMs one by one
+    if (M * n_problems <= sm_count()) return false;
+    for (int i = 0; i < n_problems; ++i)
+        if (!problems[i].prepared || problems[i].digits || problems[i].ysum || problems[i].packed) return false;
+    RotUmmaGeom u;
+    return rot_umma_geometry(base, &u);
+}
+
+int launch_rot_umma(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
+                    const RotProblem* problems, uint32_t* status, cudaStream_t stream) {
+    RotUmmaParams p{};
+    if (!rot_umma_geometry(base, &p.g)) return BWLA_ERR_INVALID_ARG;
+    const RotUmmaGeom& g = p.g;
+    p.M = M; p.bits = bits; p.asym = asym; p.n_problems = n_problems; p.status = status;
+    for (int i = 0; i < n_problems; ++i) p.prob[i] = problems[i];
+    CUtensorMap xm;
+    {
+        const uint64_t dims[3] = {(uint64_t)g.n2, (uint64_t)g.n1, (uint64_t)M};
+        const uint64_t strides[2] = {(uint64_t)g.n2 * 2, (uint64_t)ldx * 2};
+        const uint32_t box[3] = {32, (uint32_t)g.np, (uint32_t)g.tps};
+        const int st = make_map(&xm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, x, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B,
+                                CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+        if (st != BWLA_OK) return st;
+    }
+    const bool bf16 = problems[0].yhat != nullptr;
+    typedef void (*Kernel)(const CUtensorMap, const RotUmmaParams);
+    const Kernel k = g.ntot <= 128 ? (bf16 ? (Kernel)rot_umma_kernel<4, true> : (Kernel)rot_umma_kernel<4, false>)
+                                   : (bf16 ? (Kernel)rot_umma_kernel<5, true> : (Kernel)rot_umma_kernel<5, false>);
+    const int room = resident_clusters((const void*)k, g.dc, ru::kThreads, (size_t)g.total) / n_problems;
+    if (room < 1) return cuda_fail(cudaErrorInvalidConfiguration);
+    p.clusters_per_problem = (int)std::min<int64_t>((M + g.tps - 1) / g.tps, room);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(n_problems * p.clusters_per_problem * g.dc), 1, 1);
+    cfg.blockDim = dim3(ru::kThreads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)g.total;
+    cfg.stream = stream;
+    cudaLaunchAttribute attrs[2];
+    attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    // clusters that stay are placed on an empty device (see rot_mma.cu)
+    attrs[0].val.programmaticStreamSerializationAllowed = g.dc > 1 ? 0u : launch_overlap_allowed();
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = (unsigned)g.dc; attrs[1].val.clusterDim.y = 1; attrs[1].val.clusterDim.z = 1;
+    cfg.attrs = attrs;
+    cfg.numAttrs = g.dc > 1 ? 2 : 1;
+    ProfScope prof(kProfRotateQuant, stream);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, xm, p);
+    if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e); }
+    return after_launch();
+}
+
+}  // namespace bwla
