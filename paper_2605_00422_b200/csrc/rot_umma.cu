@@ -16,6 +16,9 @@
 //   16 ALU warps  step i: Y(i-1) to registers, its largest magnitude published  (accumulator free: Z(i+1) may start)
 //                         Z(i) to two fp16 terms in tensor memory               (Y(i) may start)
 //                         Y(i-1) quantised and stored
+// The tensor core truncates when it adds to its accumulator, so more than 128 values a contraction are summed in two chains, one
+// in each accumulator, and added with a rounded addition (160 x 160: 9.9e-7 of a token's full scale in one chain).  Both
+// accumulators then belong to one step, and the ALU warps quantise under the MMAs of Z.
 // A step is 1, 2 or 4 tokens, so that it fills up to 160 columns (64 x 80: 2 tokens).  Factors whose terms do not fit one CTA
 // (or with n2 > 128) are split by rows d over a cluster of two, which share nothing but the largest magnitudes.
 // 2048 tokens of 160 x 160: see kManyTokens below.
@@ -63,6 +66,7 @@ struct RotUmmaGeom {
     int dc, dt;             // CTAs of a token, rows d of each
     int atoms2, atoms1;     // K atoms of 32 elements over b / over a
     int xb;                 // buffers of x
+    int two;                // two chains of sums
     int p1_off, x_off, sh_off, total;
     int s2, s1;             // row strides of the prepared factors
 };
@@ -77,6 +81,8 @@ static bool rot_umma_geometry(const RotGeom& g, RotUmmaGeom* out) {
     u.tps = u.nc <= 32 ? 4 : u.nc <= 80 ? 2 : 1;
     u.np = u.tps == 1 ? (u.nc + 31) / 32 * 32 : u.nc;
     u.ntot = u.tps * u.np;
+    u.two = g.n2 > 128 || u.nc > 128;
+    if (u.two && u.nc < 32) return false;                     // (a chain without a step)
     u.atoms2 = (g.n2 + 31) / 32; u.atoms1 = (u.nc + 31) / 32;
     for (u.dc = 1; u.dc <= 2; ++u.dc) {
         u.dt = u.dc == 1 ? g.n2 : (g.n2 / 2 + 15) / 16 * 16;
@@ -122,8 +128,9 @@ __device__ __forceinline__ bool warp_wait_cluster(uint64_t* bar, uint32_t parity
 }
 }  // namespace
 
-// NC: 8-column chunks of a step one ALU warp owns, at most.  BF16: the weight-only operating point.
-template <int NC, bool BF16>
+// NC: 8-column chunks of a step one ALU warp owns, at most.  BF16: the weight-only operating point.  TWO: two chains of sums, one in
+// each accumulator.
+template <int NC, bool BF16, bool TWO>
 __global__ void __launch_bounds__(ru::kThreads, 1)
 rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ RotUmmaParams p) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -185,6 +192,9 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     griddep_wait();                                   // x may be the output of the preceding kernel
     if (p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) n = 0;      // the call already failed
 
+    // barrier and phase of step i's accumulator
+    auto acc_of = [](int i) { return TWO ? 0 : i & 1; };
+    auto phase_of = [](int i) { return (uint32_t)((TWO ? i : i >> 1) & 1); };
     if (warp == 0) {
         // ---------------- x ----------------
         if (elect_one()) {
@@ -209,43 +219,45 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             const uint64_t d_p2 = smem_desc_kmajor(smem_u32(smem), 64), d_p1 = smem_desc_kmajor(smem_u32(smem + g.p1_off), 64);
             const uint64_t d_x = smem_desc_kmajor(smem_u32(smem + g.x_off), 64);
             const uint32_t blk2 = (uint32_t)(g.dt * 64) >> 4, blkx = (uint32_t)(g.ntot * 64) >> 4, blk1 = (uint32_t)(g.nc * 64) >> 4;
-            const int ks2 = g.n2 >> 4, ks1 = g.nc >> 4;
+            const int ks2 = g.n2 >> 4, ks1 = g.nc >> 4, half2 = (ks2 + 1) >> 1, half1 = (ks1 + 1) >> 1;
             auto put_z = [&](int i) -> bool {
                 const int b = g.xb == 2 ? i & 1 : 0;
                 const uint32_t use = (uint32_t)(g.xb == 2 ? i >> 1 : i);
                 if (!wait_or_abort(&sh.x_full[b], use & 1u, abort_flag)) { give_up(p.status, abort_flag, 0x220); return false; }
-                if (i >= 2 && !wait_or_abort(&sh.d_free[i & 1], (uint32_t)(((i >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x221); return false; }
+                if (i >= (TWO ? 1 : 2) && !wait_or_abort(&sh.d_free[acc_of(i)], phase_of(i) ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x221); return false; }
                 tc_fence_after();
-                const uint32_t d = tmem + (uint32_t)((i & 1) * g.ntot);
                 const uint64_t xd = d_x + (uint64_t)((uint32_t)(b * g.atoms2) * blkx);
-                uint32_t acc = 0u;
                 for (int term = 2; term >= 0; --term)
                     for (int k = 0; k < ks2; ++k) {
+                        const int h = TWO ? k >= half2 : i & 1;
+                        const uint32_t d = tmem + (uint32_t)(h * g.ntot);
+                        const uint32_t acc = (term == 2 && (k == 0 || (TWO && k == half2))) ? 0u : 1u;
                         mma_f16_ss(d, d_p2 + (uint64_t)((uint32_t)(term * g.atoms2 + (k >> 1)) * blk2 + 2u * (k & 1)),
                                    xd + (uint64_t)((uint32_t)(k >> 1) * blkx + 2u * (k & 1)), idesc_a, acc);
-                        acc = 1u;
                     }
                 tc_commit(&sh.x_empty[b]);
-                tc_commit(&sh.z_full[i & 1]);
+                tc_commit(&sh.z_full[acc_of(i)]);
                 return true;
             };
-            bool ok = n > 0 ? put_z(0) : false;
+            bool ok = n > 0 && (TWO || put_z(0));
             for (int i = 0; i < n && ok; ++i) {
-                if (i + 1 < n && !put_z(i + 1)) break;
+                if (TWO ? !put_z(i) : i + 1 < n && !put_z(i + 1)) break;
                 if (!wait_or_abort(&sh.a_ready, (uint32_t)(i & 1), abort_flag)) { give_up(p.status, abort_flag, 0x222); break; }
                 tc_fence_after();
                 for (int tk = 0; tk < g.tps; ++tk) {
-                    const uint32_t d = tmem + (uint32_t)((i & 1) * g.ntot + tk * g.np);
                     const uint32_t a = tmem + (uint32_t)(2 * g.ntot + tk * (g.np >> 1));
                     // lo hi, hi lo, hi hi
 #pragma unroll 1
                     for (int q = 0; q < 3; ++q)
-                        for (int k = 0; k < ks1; ++k)
+                        for (int k = 0; k < ks1; ++k) {
+                            const int h = TWO ? k >= half1 : i & 1;
+                            const uint32_t d = tmem + (uint32_t)(h * g.ntot + tk * g.np);
                             mma_f16_ts(d, a + (q == 0 ? (uint32_t)(g.ntot >> 1) : 0u) + 8u * k,
                                        d_p1 + (uint64_t)((uint32_t)((q == 1 ? g.atoms1 : 0) + (k >> 1)) * blk1 + 2u * (k & 1)), idesc_c,
-                                       (q | k) ? 1u : 0u);
+                                       (q == 0 && (k == 0 || (TWO && k == half1))) ? 0u : 1u);
+                        }
                 }
-                tc_commit(&sh.y_full[i & 1]);
+                tc_commit(&sh.y_full[acc_of(i)]);
             }
         }
     } else if (warp >= 4) {
@@ -270,17 +282,27 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             float amax = 0.f, vmin = 0.f;
             if (i > 0) {
                 // ---- Y of the step before to registers, at true scale; its extremes to the token's other warps
-                if (!warp_wait(&sh.y_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x230); ok = false; break; }
+                if (!warp_wait(&sh.y_full[acc_of(i - 1)], phase_of(i - 1), abort_flag)) { give_up(p.status, abort_flag, 0x230); ok = false; break; }
                 tc_fence_after();
                 if (some) {
 #pragma unroll
                     for (int j = 0; j < NC; ++j)
-                        if (8 * j < cw) tmem_ld_32x8(tmem + lane_addr + (uint32_t)(pi * g.ntot + wc * cw + 8 * j), reinterpret_cast<uint32_t*>(y) + 8 * j);
+                        if (8 * j < cw) tmem_ld_32x8(tmem + lane_addr + (uint32_t)(acc_of(i - 1) * g.ntot + wc * cw + 8 * j), reinterpret_cast<uint32_t*>(y) + 8 * j);
                     tc_wait_ld();
+                    if (TWO)
+#pragma unroll
+                        for (int j = 0; j < NC; ++j)
+                            if (8 * j < cw) {
+                                uint32_t v[8];
+                                tmem_ld_32x8(tmem + lane_addr + (uint32_t)(g.ntot + wc * cw + 8 * j), v);
+                                tc_wait_ld();
+#pragma unroll
+                                for (int e = 0; e < 8; e += 2) add2(y[8 * j + e], y[8 * j + e + 1], __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+                            }
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&sh.d_free[pi]);
+                if (lane == 0) mbar_arrive(&sh.d_free[acc_of(i - 1)]);
                 const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
                 const float f1 = pow2f(ey1), f2 = pow2f(ey2);
                 const bool far = __any_sync(0xFFFFFFFFu, ey2 != 0);
@@ -315,34 +337,40 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     }
                 }
             }
-            if (i < n) {
+            auto convert = [&]() -> bool {
                 // ---- Z of this step: the power of two of every row, then its two fp16 terms, in place of the step before's (whose
                 // MMAs have completed: this warp has seen Y above)
                 const int zi = i & 1;
-                if (!warp_wait(&sh.z_full[zi], (uint32_t)((i >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x231); ok = false; break; }
+                if (!warp_wait(&sh.z_full[acc_of(i)], phase_of(i), abort_flag)) { give_up(p.status, abort_flag, 0x231); return false; }
                 tc_fence_after();
-                const uint32_t src = tmem + lane_addr + (uint32_t)(zi * g.ntot + wc * cw);
+                const uint32_t src = tmem + lane_addr + (uint32_t)(acc_of(i) * g.ntot + wc * cw);
+                auto load_z = [&](int j, float (&z)[8]) {
+                    uint32_t v[8], u[8];
+                    tmem_ld_32x8(src + 8 * j, v);
+                    if (TWO) tmem_ld_32x8(src + (uint32_t)g.ntot + 8 * j, u);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        z[e] = __uint_as_float(v[e]); z[e + 1] = __uint_as_float(v[e + 1]);
+                        if (TWO) add2(z[e], z[e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
+                    }
+                };
                 if (some) {
                     uint32_t m = 0u;
 #pragma unroll
-                    for (int j = 0; j < NC; j += 2) {
-                        uint32_t v[16];
-                        if (8 * j < cw) tmem_ld_32x8(src + 8 * j, v);
-                        if (j + 1 < NC && 8 * (j + 1) < cw) tmem_ld_32x8(src + 8 * (j + 1), v + 8);
-                        tc_wait_ld();
-                        if (8 * j < cw)
+                    for (int j = 0; j < NC; ++j)
+                        if (8 * j < cw) {
+                            float z[8];
+                            load_z(j, z);
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) m = max(m, v[e] & 0x7FFFFFFFu);
-                        if (j + 1 < NC && 8 * (j + 1) < cw)
-#pragma unroll
-                            for (int e = 8; e < 16; ++e) m = max(m, v[e] & 0x7FFFFFFFu);
-                    }
+                            for (int e = 0; e < 8; ++e) m = max(m, __float_as_uint(z[e]) & 0x7FFFFFFFu);
+                        }
                     sh.zexp[zi][q][lane][wc] = (uint8_t)(m >> 23);
                 }
                 __syncwarp();
                 if (parts > 1) {
                     if (lane == 0) mbar_arrive(&sh.row_full[zi][q]);
-                    if (!warp_wait(&sh.row_full[zi][q], (uint32_t)((i >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x233); ok = false; break; }
+                    if (!warp_wait(&sh.row_full[zi][q], (uint32_t)((i >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x233); return false; }
                 }
                 if (some) {
                     const uint32_t ex4 = *reinterpret_cast<const volatile uint32_t*>(&sh.zexp[zi][q][lane][0]);
@@ -356,14 +384,13 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
 #pragma unroll
                     for (int j = 0; j < NC; ++j) {
                         if (8 * j < cw) {
-                            uint32_t v[8], h[4], l[4];
-                            tmem_ld_32x8(src + 8 * j, v);
-                            tc_wait_ld();
+                            float z[8];
+                            uint32_t h[4], l[4];
+                            load_z(j, z);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
-                                float a = __uint_as_float(v[2 * e]), b = __uint_as_float(v[2 * e + 1]);
-                                mul2(a, b, z_scale);
-                                split2_pair(a, b, h[e], l[e]);
+                                mul2(z[2 * e], z[2 * e + 1], z_scale);
+                                split2_pair(z[2 * e], z[2 * e + 1], h[e], l[e]);
                             }
                             tmem_st_32x4(dst + 4 * j, h);
                             tmem_st_32x4(dst + (uint32_t)(g.ntot >> 1) + 4 * j, l);
@@ -374,8 +401,10 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh.a_ready);
-            }
-            if (i == 0) continue;
+                return true;
+            };
+            if (!TWO && i < n && !convert()) { ok = false; break; }
+            auto finish = [&]() -> bool {
             // ---- the step before: codes, scale and code sum, or bf16 values
             if (BF16) {
                 if (t < p.M && valid) {
@@ -392,11 +421,11 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                             }
                         }
                 }
-                continue;
+                return true;
             }
             if (g.dc == 1 ? !warp_wait(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)
                           : !warp_wait_cluster(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)) {
-                give_up(p.status, abort_flag, 0x232); ok = false; break;
+                give_up(p.status, abort_flag, 0x232); return false;
             }
             {
                 const bool mine = lane < 16 * g.dc && (((lane & 15) >> 2) * g.tps >> 2) == tk;
@@ -493,6 +522,10 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     if (pr.zp) pr.zp[t] = shift_i;
                 }
             }
+            return true;
+            };
+            if (i > 0 && !finish()) { ok = false; break; }
+            if (TWO && i < n && !convert()) { ok = false; break; }
         }
         if (!ok) *abort_flag = 1;
     }
@@ -534,8 +567,9 @@ int launch_rot_umma(const RotGeom& base, const void* x, int64_t M, int64_t ldx, 
     }
     const bool bf16 = problems[0].yhat != nullptr;
     typedef void (*Kernel)(const CUtensorMap, const RotUmmaParams);
-    const Kernel k = g.ntot <= 128 ? (bf16 ? (Kernel)rot_umma_kernel<4, true> : (Kernel)rot_umma_kernel<4, false>)
-                                   : (bf16 ? (Kernel)rot_umma_kernel<5, true> : (Kernel)rot_umma_kernel<5, false>);
+    const Kernel k = g.two ? (bf16 ? (Kernel)rot_umma_kernel<5, true, true> : (Kernel)rot_umma_kernel<5, false, true>)
+                   : g.ntot <= 128 ? (bf16 ? (Kernel)rot_umma_kernel<4, true, false> : (Kernel)rot_umma_kernel<4, false, false>)
+                                   : (bf16 ? (Kernel)rot_umma_kernel<5, true, false> : (Kernel)rot_umma_kernel<5, false, false>);
     const int room = resident_clusters((const void*)k, g.dc, ru::kThreads, (size_t)g.total) / n_problems;
     if (room < 1) return cuda_fail(cudaErrorInvalidConfiguration);
     p.clusters_per_problem = (int)std::min<int64_t>((M + g.tps - 1) / g.tps, room);
