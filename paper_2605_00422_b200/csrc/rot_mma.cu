@@ -120,65 +120,6 @@ size_t rot_prepared_bytes(const RotGeom& g) {
     return kRotHeader + (size_t)3 * g.n2p * g.s2 + (size_t)2 * g.na * 8 * g.s1;
 }
 
-// Exponent by which P1 is scaled: its largest magnitude goes to [2^13, 2^14).
-__device__ __forceinline__ int factor_exponent(float amax) { return min(13 - exponent_of(amax), 126); }
-
-// Largest |v| of n floats (v 16-byte aligned), over the threads of the block; `red` has a word per warp.
-__device__ __forceinline__ float block_absmax(const float* __restrict__ v, int n, uint32_t* red) {
-    uint32_t m = 0u;
-    const float4* v4 = reinterpret_cast<const float4*>(v);
-#pragma unroll 4
-    for (int i = threadIdx.x; i < (n >> 2); i += blockDim.x) {
-        const float4 f = __ldg(v4 + i);
-        m = max(m, max(max(__float_as_uint(f.x) & 0x7FFFFFFFu, __float_as_uint(f.y) & 0x7FFFFFFFu),
-                       max(__float_as_uint(f.z) & 0x7FFFFFFFu, __float_as_uint(f.w) & 0x7FFFFFFFu)));
-    }
-    if ((int)threadIdx.x < (n & 3)) m = max(m, __float_as_uint(__ldg(v + (n & ~3) + threadIdx.x)) & 0x7FFFFFFFu);
-    m = __reduce_max_sync(0xFFFFFFFFu, m);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, red[w]);
-    return __uint_as_float(m);
-}
-
-// The terms of rows [r0, r0 + rows) of factor^T (element (r, k) = P[k][r], times scale), zero outside n x n: blocks of `block`
-// bytes, one per term, with rows of `stride` bytes and kp columns.  Threads run along r, so the reads of P are coalesced.
-template <bool F16>
-__device__ __forceinline__ void split_factor(const float* __restrict__ P, int n, int r0, int rows, int kp, int stride, float scale,
-                                             uint8_t* dst, size_t block, int tid, int nthreads) {
-    const int pairs = rows * (kp >> 1);
-    constexpr int U = 4;
-    for (int i0 = tid; i0 < pairs; i0 += U * nthreads) {
-        float a[U], b[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * nthreads, k2 = i / rows, r = i - k2 * rows, k = 2 * k2;
-            const bool ok = i < pairs && r0 + r < n;
-            a[u] = ok && k < n ? __ldg(P + (size_t)k * n + r0 + r) : 0.f;
-            b[u] = ok && k + 1 < n ? __ldg(P + (size_t)(k + 1) * n + r0 + r) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * nthreads, k2 = i / rows, r = i - k2 * rows;
-            if (i < pairs) {
-                uint8_t* at = dst + (size_t)r * stride + 4 * k2;
-                uint32_t h, m, l;
-                if (F16) {
-                    split2_pair(a[u] * scale, b[u] * scale, h, l);
-                    *reinterpret_cast<uint32_t*>(at) = h;
-                    *reinterpret_cast<uint32_t*>(at + block) = l;
-                } else {
-                    split3_pair(a[u], b[u], h, m, l);
-                    *reinterpret_cast<uint32_t*>(at) = h;
-                    *reinterpret_cast<uint32_t*>(at + block) = m;
-                    *reinterpret_cast<uint32_t*>(at + 2 * block) = l;
-                }
-            }
-        }
-    }
-}
-
 // once per layer: P1, P2 (fp32) -> exponents (of max|P2|; by which P1 is scaled), the bf16 terms of P2^T and the fp16 terms of
 // P1^T, rows as they lie in shared memory
 __global__ void __launch_bounds__(256) prepare_rot_kernel(RotGeom g, const float* __restrict__ P1, const float* __restrict__ P2,
@@ -190,8 +131,8 @@ __global__ void __launch_bounds__(256) prepare_rot_kernel(RotGeom g, const float
     uint8_t* t2 = prepared + kRotHeader;
     uint8_t* t1 = t2 + (size_t)3 * rows2 * g.s2;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    split_factor<false>(P2, g.n2, 0, rows2, g.n2p, g.s2, 1.f, t2, (size_t)rows2 * g.s2, tid, nt);
-    split_factor<true>(P1, g.n1, 0, rows1, rows1, g.s1, pow2f(e1), t1, (size_t)rows1 * g.s1, tid, nt);
+    split_factor<false>(P2, g.n2, 0, rows2, g.n2p, 1.f, [&](int r, int k2) { return t2 + (size_t)r * g.s2 + 4 * k2; }, (size_t)rows2 * g.s2, tid, nt);
+    split_factor<true>(P1, g.n1, 0, rows1, rows1, pow2f(e1), [&](int r, int k2) { return t1 + (size_t)r * g.s1 + 4 * k2; }, (size_t)rows1 * g.s1, tid, nt);
 }
 
 int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void* prepared, cudaStream_t stream) {
@@ -279,8 +220,8 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         e2 = exponent_of(block_absmax(pr.P2, g.n2 * g.n2, red));
         e1 = factor_exponent(block_absmax(pr.P1, g.n1 * g.n1, red));
         __syncthreads();                              // (the words of `red` are cleared below)
-        split_factor<false>(pr.P2, g.n2, rank * rows2, rows2, g.n2p, g.s2, 1.f, p2s, part2, threadIdx.x, blockDim.x);
-        split_factor<true>(pr.P1, g.n1, 0, rows1, rows1, g.s1, pow2f(e1), p1s, part1, threadIdx.x, blockDim.x);
+        split_factor<false>(pr.P2, g.n2, rank * rows2, rows2, g.n2p, 1.f, [&](int r, int k2) { return p2s + r * g.s2 + 4 * k2; }, part2, threadIdx.x, blockDim.x);
+        split_factor<true>(pr.P1, g.n1, 0, rows1, rows1, pow2f(e1), [&](int r, int k2) { return p1s + r * g.s1 + 4 * k2; }, part1, threadIdx.x, blockDim.x);
     }
     const int cpr = g.n2 >> 3, chunks = g.n1 * cpr;   // 16-byte chunks (of bf16) per row of X, and in all
     auto zero_padding = [&]() {                       // what the contractions read of X beyond n1 x n2

@@ -85,4 +85,64 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 // floor(log2 v) of a non-negative finite v (subnormals and zero: -127)
 __device__ __forceinline__ int exponent_of(float v) { return (int)((__float_as_uint(v) >> 23) & 0xFFu) - 127; }
 
+// Exponent by which P1 is scaled: its largest magnitude goes to [2^13, 2^14).
+__device__ __forceinline__ int factor_exponent(float amax) { return min(13 - exponent_of(amax), 126); }
+
+// Largest |v| of n floats (v 16-byte aligned), over the threads of the block; `red` has a word per warp.
+__device__ __forceinline__ float block_absmax(const float* __restrict__ v, int n, uint32_t* red) {
+    uint32_t m = 0u;
+    const float4* v4 = reinterpret_cast<const float4*>(v);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < (n >> 2); i += blockDim.x) {
+        const float4 f = __ldg(v4 + i);
+        m = max(m, max(max(__float_as_uint(f.x) & 0x7FFFFFFFu, __float_as_uint(f.y) & 0x7FFFFFFFu),
+                       max(__float_as_uint(f.z) & 0x7FFFFFFFu, __float_as_uint(f.w) & 0x7FFFFFFFu)));
+    }
+    if ((int)threadIdx.x < (n & 3)) m = max(m, __float_as_uint(__ldg(v + (n & ~3) + threadIdx.x)) & 0x7FFFFFFFu);
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, red[w]);
+    return __uint_as_float(m);
+}
+
+// The terms of rows [r0, r0 + rows) of factor^T (element (r, k) = P[k][r], times scale), zero outside n x n: blocks of `block`
+// bytes, one per term, kp columns; columns 2 k2, 2 k2 + 1 of row r (counted from r0) go to place(r, k2).  Threads run along r, so
+// the reads of P are coalesced.
+template <bool F16, typename Place>
+__device__ __forceinline__ void split_factor(const float* __restrict__ P, int n, int r0, int rows, int kp, float scale, Place place,
+                                             size_t block, int tid, int nthreads) {
+    const int pairs = rows * (kp >> 1);
+    constexpr int U = 4;
+    for (int i0 = tid; i0 < pairs; i0 += U * nthreads) {
+        float a[U], b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * nthreads, k2 = i / rows, r = i - k2 * rows, k = 2 * k2;
+            const bool ok = i < pairs && r0 + r < n;
+            a[u] = ok && k < n ? __ldg(P + (size_t)k * n + r0 + r) : 0.f;
+            b[u] = ok && k + 1 < n ? __ldg(P + (size_t)(k + 1) * n + r0 + r) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * nthreads, k2 = i / rows, r = i - k2 * rows;
+            if (i < pairs) {
+                uint8_t* at = place(r, k2);
+                uint32_t h, m, l;
+                if (F16) {
+                    split2_pair(a[u] * scale, b[u] * scale, h, l);
+                    *reinterpret_cast<uint32_t*>(at) = h;
+                    *reinterpret_cast<uint32_t*>(at + block) = l;
+                } else {
+                    split3_pair(a[u], b[u], h, m, l);
+                    *reinterpret_cast<uint32_t*>(at) = h;
+                    *reinterpret_cast<uint32_t*>(at + block) = m;
+                    *reinterpret_cast<uint32_t*>(at + 2 * block) = l;
+                }
+            }
+        }
+    }
+}
+
 }  // namespace bwla

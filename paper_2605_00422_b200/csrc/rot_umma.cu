@@ -148,10 +148,12 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     const int rows = min(g.dt, g.n2 - rank * g.dt);
 
     // ---- the layer's factors (they do not depend on the preceding kernel): rows of 64 bytes, swizzled ----
-    const uint8_t* t2 = pr.prepared + ru::kPrepHeader;
-    const size_t all2 = (size_t)g.n2 * g.s2;
-    const uint8_t* t1 = t2 + 3 * all2;
-    {
+    int e1;
+    if (pr.prepared) {
+        const uint8_t* t2 = pr.prepared + ru::kPrepHeader;
+        const size_t all2 = (size_t)g.n2 * g.s2;
+        const uint8_t* t1 = t2 + 3 * all2;
+        e1 = __ldg(reinterpret_cast<const int*>(pr.prepared) + 1);
         const int cpr2 = g.n2 >> 3;
         for (int i = threadIdx.x; i < 3 * rows * cpr2; i += ru::kThreads) {
             const int rr = i / cpr2, ch = i - rr * cpr2, term = rr / rows, r = rr - term * rows;
@@ -165,7 +167,15 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             cp_async16(smem_u32(dst), t1 + (size_t)term * g.nc * g.s1 + (size_t)r * g.s1 + 16 * ch);
         }
     }
-    const int e1 = __ldg(reinterpret_cast<const int*>(pr.prepared) + 1);
+    else {
+        e1 = factor_exponent(block_absmax(pr.P1, g.n1 * g.n1, sh.amax[0]));
+        split_factor<false>(pr.P2, g.n2, rank * g.dt, rows, g.n2, 1.f, [&](int r, int k2) {
+            return smem + ((k2 >> 4) * g.dt + r) * 64 + ((((k2 >> 2) ^ (r >> 1)) & 3) << 4) + 4 * (k2 & 3);
+        }, (size_t)g.atoms2 * g.dt * 64, threadIdx.x, ru::kThreads);
+        split_factor<true>(pr.P1, g.n1, 0, g.nc, g.nc, pow2f(e1), [&](int r, int k2) {
+            return smem + g.p1_off + ((k2 >> 4) * g.nc + r) * 64 + ((((k2 >> 2) ^ (r >> 1)) & 3) << 4) + 4 * (k2 & 3);
+        }, (size_t)g.atoms1 * g.nc * 64, threadIdx.x, ru::kThreads);
+    }
     if (threadIdx.x == 0) {
         sh.abort_flag = 0;
         for (int i = 0; i < 2; ++i) {
@@ -322,19 +332,33 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                         }
                     }
                 }
-                if (!BF16) {
-                    // non-negative (NaNs aside), so their bit patterns order like the values
-                    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));
-                    const uint32_t v = asym ? __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(-vmin, 0.f))) : 0u;
+                auto publish = [&](uint32_t m, uint32_t v) {
                     uint32_t* slot = &sh.amax[pi][rank * 16 + w];
                     uint32_t* slot_v = &sh.vmin[pi][rank * 16 + w];
                     if (g.dc == 1) {
                         if (lane == 0) { *slot = m; *slot_v = v; mbar_arrive(&sh.max_full[pi]); }
                     } else if (lane < 2) {
                         st_shared_cluster_u32(map_shared_rank(smem_u32(slot), (uint32_t)lane), m);
-                        if (asym) st_shared_cluster_u32(map_shared_rank(smem_u32(slot_v), (uint32_t)lane), v);
+                        if (asym || BF16) st_shared_cluster_u32(map_shared_rank(smem_u32(slot_v), (uint32_t)lane), v);
                         mbar_arrive_remote(map_shared_rank(smem_u32(&sh.max_full[pi]), (uint32_t)lane));
                     }
+                };
+                if (BF16 && pr.ysum) {
+                    // the sum of the rounded values goes where the quantiser's two extremes go
+                    double s = 0.0;
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) s += (double)__bfloat162float(__float2bfloat16_rn(y[8 * j + e]));
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                    const unsigned long long bits = (unsigned long long)__double_as_longlong(s);
+                    publish((uint32_t)bits, (uint32_t)(bits >> 32));
+                }
+                if (!BF16) {
+                    // non-negative (NaNs aside), so their bit patterns order like the values
+                    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));
+                    const uint32_t v = asym ? __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(-vmin, 0.f))) : 0u;
+                    publish(m, v);
                 }
             }
             auto convert = [&]() -> bool {
@@ -421,14 +445,23 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                             }
                         }
                 }
-                return true;
+                if (!pr.ysum) return true;
             }
             if (g.dc == 1 ? !warp_wait(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)
                           : !warp_wait_cluster(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)) {
                 give_up(p.status, abort_flag, 0x232); return false;
             }
+            const bool mine = lane < 16 * g.dc && (((lane & 15) >> 2) * g.tps >> 2) == tk;
+            if (BF16) {
+                if (t < p.M && rank == 0 && q == 0 && c_base == 0) {
+                    double s = 0.0;
+                    if (mine) s = __hiloint2double((int)*reinterpret_cast<volatile uint32_t*>(&sh.vmin[pi][lane]), (int)*reinterpret_cast<volatile uint32_t*>(&sh.amax[pi][lane]));
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                    if (lane == 0) pr.ysum[t] = (float)s;
+                }
+                return true;
+            }
             {
-                const bool mine = lane < 16 * g.dc && (((lane & 15) >> 2) * g.tps >> 2) == tk;
                 amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, mine ? *reinterpret_cast<volatile uint32_t*>(&sh.amax[pi][lane]) : 0u));
                 if (asym) vmin = -__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, mine ? *reinterpret_cast<volatile uint32_t*>(&sh.vmin[pi][lane]) : 0u));
             }
@@ -544,7 +577,7 @@ bool rot_umma_supports(const RotGeom& base, int64_t M, int n_problems, const Rot
     // more tokens than rot_mma.cu spreads over the SMs one by one
     if (M * n_problems <= sm_count()) return false;
     for (int i = 0; i < n_problems; ++i)
-        if (!problems[i].prepared || problems[i].digits || problems[i].ysum || problems[i].packed) return false;
+        if (problems[i].digits || problems[i].packed) return false;
     RotUmmaGeom u;
     return rot_umma_geometry(base, &u);
 }
