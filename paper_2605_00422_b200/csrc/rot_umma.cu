@@ -102,7 +102,7 @@ static bool rot_umma_geometry(const RotGeom& g, RotUmmaGeom* out) {
 struct RotUmmaParams {
     RotUmmaGeom g;
     int64_t M;
-    int bits, asym;
+    int bits;
     int n_problems, clusters_per_problem;
     RotProblem prob[kRotMaxProblems];
     uint32_t* status;
@@ -126,11 +126,33 @@ __device__ __forceinline__ bool warp_wait_cluster(uint64_t* bar, uint32_t parity
     }
     return false;
 }
+// The warp's columns of an accumulator (TWO: the sum of two, `other` columns apart).
+template <int NC, bool TWO>
+__device__ __forceinline__ void load_sums(uint32_t src, uint32_t other, int cw, float (&v)[NC * 8]) {
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+        if (8 * j < cw) tmem_ld_32x8(src + 8 * j, reinterpret_cast<uint32_t*>(v) + 8 * j);
+    if (TWO) {
+#pragma unroll
+        for (int j = 0; j < NC; j += 2) {
+            uint32_t u[16];
+            if (8 * j < cw) tmem_ld_32x8(src + other + 8 * j, u);
+            if (j + 1 < NC && 8 * (j + 1) < cw) tmem_ld_32x8(src + other + 8 * (j + 1), u + 8);
+            tc_wait_ld();
+#pragma unroll
+            for (int e = 0; e < (j + 1 < NC ? 16 : 8); e += 2)
+                add2(v[8 * j + e], v[8 * j + e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
+        }
+    } else {
+        tc_wait_ld();
+    }
+}
 }  // namespace
 
-// NC: 8-column chunks of a step one ALU warp owns, at most.  BF16: the weight-only operating point.  TWO: two chains of sums, one in
-// each accumulator.
-template <int NC, bool BF16, bool TWO>
+// NC: 8-column chunks of a step one ALU warp owns, at most.  MODE: the symmetric or the asymmetric quantiser, or the weight-only
+// operating point.  TWO: two chains of sums, one in each accumulator.
+enum { kSym = 0, kAsym = 1, kBf16 = 2 };
+template <int NC, int MODE, bool TWO>
 __global__ void __launch_bounds__(ru::kThreads, 1)
 rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ RotUmmaParams p) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -272,6 +294,9 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         }
     } else if (warp >= 4) {
         // ---------------- everything between and behind the MMAs ----------------
+        // A warp issues an instruction about every six cycles here (four warps a scheduler), so instructions a value are what
+        // counts: no scaling pass over Y (a row's power of two goes into the quantiser's factor), one read of Z, no
+        // conditions on single values where whole chunks exist, two columns a store.
         const int w = warp - 4, q = w & 3, wc = w >> 2;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         const int cw = g.ntot >> 2;                   // columns of the step this warp owns
@@ -279,10 +304,11 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         const int c_base = wc * cw - tk * g.np;       // first of them within the token
         const bool some = q * 32 < rows, valid = q * 32 + lane < rows;        // (16 lanes at a time)
         const int d = rank * g.dt + q * 32 + lane;
-        const int qmax = (1 << (p.bits - 1)) - 1;
-        const bool asym = p.asym != 0;
         const int parts = 4 / g.tps;                  // warps of a token in a lane quarter
+        const int have = some ? min(cw, g.nc - c_base) : 0;                   // columns that hold sums (a multiple of 8), and
+        const int exist = some ? min(cw, g.n1 - c_base) : 0;                  // that are outputs (either may be negative)
         float y[NC * 8];
+        float f1 = 1.f;                               // power of two that brings this lane's row of y to true scale
         int z_exp = 0;
         bool ok = true;
 #pragma unroll 1
@@ -291,46 +317,21 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             const int64_t t = (first + (int64_t)(i - 1) * p.clusters_per_problem) * g.tps + tk;
             float amax = 0.f, vmin = 0.f;
             if (i > 0) {
-                // ---- Y of the step before to registers, at true scale; its extremes to the token's other warps
+                // ---- Y of the step before to registers; its extremes to the token's other warps
                 if (!warp_wait(&sh.y_full[acc_of(i - 1)], phase_of(i - 1), abort_flag)) { give_up(p.status, abort_flag, 0x230); ok = false; break; }
                 tc_fence_after();
-                if (some) {
-#pragma unroll
-                    for (int j = 0; j < NC; ++j)
-                        if (8 * j < cw) tmem_ld_32x8(tmem + lane_addr + (uint32_t)(acc_of(i - 1) * g.ntot + wc * cw + 8 * j), reinterpret_cast<uint32_t*>(y) + 8 * j);
-                    tc_wait_ld();
-                    if (TWO)
-#pragma unroll
-                        for (int j = 0; j < NC; ++j)
-                            if (8 * j < cw) {
-                                uint32_t v[8];
-                                tmem_ld_32x8(tmem + lane_addr + (uint32_t)(g.ntot + wc * cw + 8 * j), v);
-                                tc_wait_ld();
-#pragma unroll
-                                for (int e = 0; e < 8; e += 2) add2(y[8 * j + e], y[8 * j + e + 1], __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
-                            }
-                }
+                const uint32_t src = tmem + lane_addr + (uint32_t)(acc_of(i - 1) * g.ntot + wc * cw);
+                if (some) load_sums<NC, TWO>(src, (uint32_t)g.ntot, cw, y);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh.d_free[acc_of(i - 1)]);
                 const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
-                const float f1 = pow2f(ey1), f2 = pow2f(ey2);
-                const bool far = __any_sync(0xFFFFFFFFu, ey2 != 0);
+                f1 = pow2f(ey1);
+                if (__any_sync(0xFFFFFFFFu, ey2 != 0)) {          // scales at the ends of fp32's range
+                    const float f2 = pow2f(ey2);
 #pragma unroll
-                for (int j = 0; j < NC; ++j) {
-                    // (columns beyond P1's rows and rows beyond P2's hold anything)
-                    const bool keep = valid && 8 * j < cw && c_base + 8 * j < g.nc;
-#pragma unroll
-                    for (int e = 0; e < 8; e += 2) {
-                        float &a = y[8 * j + e], &b = y[8 * j + e + 1];
-                        mul2(a, b, f1);
-                        if (far) mul2(a, b, f2);
-                        if (!keep) a = b = 0.f;
-                        if (!BF16) {
-                            if (!asym) amax = fmaxf(amax, fmaxf(fabsf(a), fabsf(b)));
-                            else { amax = fmaxf(amax, fmaxf(a, b)); vmin = fminf(vmin, fminf(a, b)); }
-                        }
-                    }
+                    for (int j = 0; j < NC * 8; ++j) y[j] = y[j] * f1 * f2;
+                    f1 = 1.f;
                 }
                 auto publish = [&](uint32_t m, uint32_t v) {
                     uint32_t* slot = &sh.amax[pi][rank * 16 + w];
@@ -339,26 +340,37 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                         if (lane == 0) { *slot = m; *slot_v = v; mbar_arrive(&sh.max_full[pi]); }
                     } else if (lane < 2) {
                         st_shared_cluster_u32(map_shared_rank(smem_u32(slot), (uint32_t)lane), m);
-                        if (asym || BF16) st_shared_cluster_u32(map_shared_rank(smem_u32(slot_v), (uint32_t)lane), v);
+                        if (MODE != kSym) st_shared_cluster_u32(map_shared_rank(smem_u32(slot_v), (uint32_t)lane), v);
                         mbar_arrive_remote(map_shared_rank(smem_u32(&sh.max_full[pi]), (uint32_t)lane));
                     }
                 };
-                if (BF16 && pr.ysum) {
-                    // the sum of the rounded values goes where the quantiser's two extremes go
-                    double s = 0.0;
+                if (MODE == kBf16) {
+                    if (pr.ysum) {
+                        // the sum of the rounded values goes where the quantiser's two extremes go
+                        double s = 0.0;
+#pragma unroll
+                        for (int j = 0; j < NC; ++j)
+                            if (valid && 8 * j < have)
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) s += (double)__bfloat162float(__float2bfloat16_rn(y[8 * j + e] * f1));
+                        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                        const unsigned long long bits = (unsigned long long)__double_as_longlong(s);
+                        publish((uint32_t)bits, (uint32_t)(bits >> 32));
+                    }
+                } else {
 #pragma unroll
                     for (int j = 0; j < NC; ++j)
+                        if (8 * j < have)
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) s += (double)__bfloat162float(__float2bfloat16_rn(y[8 * j + e]));
-                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                    const unsigned long long bits = (unsigned long long)__double_as_longlong(s);
-                    publish((uint32_t)bits, (uint32_t)(bits >> 32));
-                }
-                if (!BF16) {
+                            for (int e = 0; e < 8; e += 2) {
+                                const float a = y[8 * j + e], b = y[8 * j + e + 1];
+                                if (MODE == kSym) amax = fmaxf(amax, fmaxf(fabsf(a), fabsf(b)));
+                                else { amax = fmaxf(amax, fmaxf(a, b)); vmin = fminf(vmin, fminf(a, b)); }
+                            }
+                    if (!valid) amax = vmin = 0.f;                // (rows beyond P2's hold anything)
                     // non-negative (NaNs aside), so their bit patterns order like the values
-                    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax));
-                    const uint32_t v = asym ? __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(-vmin, 0.f))) : 0u;
-                    publish(m, v);
+                    publish(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax * f1)),
+                            MODE == kAsym ? __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(-vmin * f1, 0.f))) : 0u);
                 }
             }
             auto convert = [&]() -> bool {
@@ -368,28 +380,16 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (!warp_wait(&sh.z_full[acc_of(i)], phase_of(i), abort_flag)) { give_up(p.status, abort_flag, 0x231); return false; }
                 tc_fence_after();
                 const uint32_t src = tmem + lane_addr + (uint32_t)(acc_of(i) * g.ntot + wc * cw);
-                auto load_z = [&](int j, float (&z)[8]) {
-                    uint32_t v[8], u[8];
-                    tmem_ld_32x8(src + 8 * j, v);
-                    if (TWO) tmem_ld_32x8(src + (uint32_t)g.ntot + 8 * j, u);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < 8; e += 2) {
-                        z[e] = __uint_as_float(v[e]); z[e + 1] = __uint_as_float(v[e + 1]);
-                        if (TWO) add2(z[e], z[e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
-                    }
-                };
+                float z[NC * 8];
                 if (some) {
-                    uint32_t m = 0u;
+                    load_sums<NC, TWO>(src, (uint32_t)g.ntot, cw, z);
+                    float m = 0.f;
 #pragma unroll
                     for (int j = 0; j < NC; ++j)
-                        if (8 * j < cw) {
-                            float z[8];
-                            load_z(j, z);
+                        if (8 * j < cw)
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) m = max(m, __float_as_uint(z[e]) & 0x7FFFFFFFu);
-                        }
-                    sh.zexp[zi][q][lane][wc] = (uint8_t)(m >> 23);
+                            for (int e = 0; e < 8; e += 2) m = fmaxf(m, fmaxf(fabsf(z[8 * j + e]), fabsf(z[8 * j + e + 1])));
+                    sh.zexp[zi][q][lane][wc] = (uint8_t)(__float_as_uint(m) >> 23);
                 }
                 __syncwarp();
                 if (parts > 1) {
@@ -408,13 +408,11 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
 #pragma unroll
                     for (int j = 0; j < NC; ++j) {
                         if (8 * j < cw) {
-                            float z[8];
                             uint32_t h[4], l[4];
-                            load_z(j, z);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
-                                mul2(z[2 * e], z[2 * e + 1], z_scale);
-                                split2_pair(z[2 * e], z[2 * e + 1], h[e], l[e]);
+                                mul2(z[8 * j + 2 * e], z[8 * j + 2 * e + 1], z_scale);
+                                split2_pair(z[8 * j + 2 * e], z[8 * j + 2 * e + 1], h[e], l[e]);
                             }
                             tmem_st_32x4(dst + 4 * j, h);
                             tmem_st_32x4(dst + (uint32_t)(g.ntot >> 1) + 4 * j, l);
@@ -427,54 +425,49 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (lane == 0) mbar_arrive(&sh.a_ready);
                 return true;
             };
-            if (!TWO && i < n && !convert()) { ok = false; break; }
-            auto finish = [&]() -> bool {
             // ---- the step before: codes, scale and code sum, or bf16 values
-            if (BF16) {
-                if (t < p.M && valid) {
-                    // layout 1: inside each group of 32, position 2 (k % 16) + (k % 32) / 16
-                    __nv_bfloat16* yt = pr.yhat + t * (int64_t)g.K;
+            auto finish = [&]() -> bool {
+                if (MODE == kBf16) {
+                    if (t < p.M && valid) {
+                        // layout 1: inside each group of 32, position 2 (k % 16) + (k % 32) / 16
+                        __nv_bfloat16* yt = pr.yhat + t * (int64_t)g.K;
 #pragma unroll
-                    for (int j = 0; j < NC; ++j)
+                        for (int j = 0; j < NC; ++j)
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const int c = c_base + 8 * j + e;
-                            if (8 * j < cw && c < g.n1) {
-                                const int k = c * g.n2 + d;
-                                yt[pr.codes_layout ? (k & ~31) + 2 * (k & 15) + ((k >> 4) & 1) : k] = __float2bfloat16_rn(y[8 * j + e]);
-                            }
-                        }
+                            for (int e = 0; e < 8; ++e)
+                                if (8 * j + e < exist) {
+                                    const int k = (c_base + 8 * j + e) * g.n2 + d;
+                                    yt[pr.codes_layout ? (k & ~31) + 2 * (k & 15) + ((k >> 4) & 1) : k] = __float2bfloat16_rn(y[8 * j + e] * f1);
+                                }
+                    }
+                    if (!pr.ysum) return true;
                 }
-                if (!pr.ysum) return true;
-            }
-            if (g.dc == 1 ? !warp_wait(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)
-                          : !warp_wait_cluster(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)) {
-                give_up(p.status, abort_flag, 0x232); return false;
-            }
-            const bool mine = lane < 16 * g.dc && (((lane & 15) >> 2) * g.tps >> 2) == tk;
-            if (BF16) {
-                if (t < p.M && rank == 0 && q == 0 && c_base == 0) {
-                    double s = 0.0;
-                    if (mine) s = __hiloint2double((int)*reinterpret_cast<volatile uint32_t*>(&sh.vmin[pi][lane]), (int)*reinterpret_cast<volatile uint32_t*>(&sh.amax[pi][lane]));
-                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                    if (lane == 0) pr.ysum[t] = (float)s;
+                if (g.dc == 1 ? !warp_wait(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)
+                              : !warp_wait_cluster(&sh.max_full[pi], (uint32_t)(((i - 1) >> 1) & 1), abort_flag)) {
+                    give_up(p.status, abort_flag, 0x232); return false;
                 }
-                return true;
-            }
-            {
-                amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, mine ? *reinterpret_cast<volatile uint32_t*>(&sh.amax[pi][lane]) : 0u));
-                if (asym) vmin = -__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, mine ? *reinterpret_cast<volatile uint32_t*>(&sh.vmin[pi][lane]) : 0u));
-            }
-            if (t < p.M) {
-                // The quantiser of rot_mma.cu, word for word the same roundings: fl(v + 1.5 * 2^23 + shift) leaves rne(v) + shift in
-                // the low mantissa bits, the low byte is stored, the patterns are summed.
-                float inv = 0.f, scale = 1.f, zero_f = 0.f, half_f = 0.f, levels = 0.f;
-                if (!asym) {
-                    if (amax != 0.f) { inv = __fdiv_rn((float)qmax, amax); scale = __fdiv_rn(amax, (float)qmax); }
-                } else {
-                    levels = (float)((1 << p.bits) - 1);
-                    const float range = __fsub_rn(amax, vmin);
-                    if (range != 0.f) { inv = __fdiv_rn(levels, range); scale = __fdiv_rn(range, levels); }
+                const bool mine = lane < 16 * g.dc && (((lane & 15) >> 2) * g.tps >> 2) == tk;
+                const bool writer = rank == 0 && q == 0 && c_base == 0;       // of the token's scalars
+                const uint32_t s0 = mine ? *reinterpret_cast<volatile uint32_t*>(&sh.amax[pi][lane]) : 0u;
+                const uint32_t s1 = mine && MODE != kSym ? *reinterpret_cast<volatile uint32_t*>(&sh.vmin[pi][lane]) : 0u;
+                if (t >= p.M) return true;
+                if (MODE == kBf16) {
+                    if (writer) {
+                        double s = __hiloint2double((int)s1, (int)s0);
+                        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                        if (lane == 0) pr.ysum[t] = (float)s;
+                    }
+                    return true;
+                }
+                amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, s0));
+                if (MODE == kAsym) vmin = -__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, s1));
+                // The quantiser of rot_mma.cu with the same roundings: fl(v + 1.5 * 2^23 + shift) leaves rne(v) + shift in the low
+                // mantissa bits, the low byte is stored, the patterns are summed.
+                const float levels = MODE == kSym ? (float)((1 << (p.bits - 1)) - 1) : (float)((1 << p.bits) - 1);
+                const float range = MODE == kSym ? amax : __fsub_rn(amax, vmin);
+                const float inv = range != 0.f ? __fdiv_rn(levels, range) : 0.f;
+                float zero_f = 0.f, half_f = 0.f;
+                if (MODE == kAsym) {
                     const float tz = __fmul_rn(-vmin, inv);
                     zero_f = fminf(fmaxf(__fadd_rn(__fadd_rn(tz, 12582912.f), -12582912.f), 0.f), levels);
                     half_f = (float)(1 << (p.bits - 1));
@@ -484,55 +477,81 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 const uint32_t odd = (uint32_t)(shift_i & 1);
                 const float bias_even = 12582912.f + (float)(shift_i - (int)odd);
                 const float lo_b = 12582912.f + store_shift - (float)odd, hi_b = lo_b + levels;
-                int8_t* ct = pr.codes + t * (int64_t)g.K;
-                // Two columns at a time: lanes 8 apart have neighbouring bytes of a column in the contraction's order, so one
-                // of the two stores both lanes' codes of the first column, the other those of the second.
-                const int hb = (lane >> 3) & 1;
-                const uint32_t sel = hb ? 0x0004u : 0x0040u;
-                const int k0 = (c_base + hb) * g.n2 + (d & ~8);
-                int8_t* at = ct + (k0 & ~31) + 4 * (k0 & 7) + ((k0 & 31) >> 3);
-                int8_t* at_plain = ct + c_base * g.n2 + d;
-                uint32_t usum = 0u;
-                int counted = 0;
-                if (some) {
-#pragma unroll
-                    for (int j = 0; j < NC; ++j) {
-                        if (8 * j < cw && c_base + 8 * j < g.n1) {
-#pragma unroll
-                            for (int e = 0; e < 8; e += 2) {
-                                const int c = c_base + 8 * j + e;
-                                float v0 = __fmul_rn(y[8 * j + e], inv), v1 = __fmul_rn(y[8 * j + e + 1], inv);
-                                add2(v0, v1, bias_even, bias_even);
-                                uint32_t w0 = __float_as_uint(v0), w1 = __float_as_uint(v1);
-                                if (asym) {
-                                    w0 = __float_as_uint(fminf(fmaxf(v0, lo_b), hi_b)) + odd;
-                                    w1 = __float_as_uint(fminf(fmaxf(v1, lo_b), hi_b)) + odd;
-                                }
-                                if (c < g.n1) { usum += w0; ++counted; }
-                                if (c + 1 < g.n1) { usum += w1; ++counted; }
-                                if (pr.codes_layout) {
-                                    const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, hb ? w0 : w1, 8);
-                                    if (valid && c + hb < g.n1) *reinterpret_cast<uint16_t*>(at) = (uint16_t)__byte_perm(hb ? w1 : w0, other, sel);
-                                    at += 2 * g.n2;
-                                } else {
-                                    if (valid && c < g.n1) at_plain[0] = (int8_t)w0;
-                                    if (valid && c + 1 < g.n1) at_plain[g.n2] = (int8_t)w1;
-                                    at_plain += 2 * g.n2;
-                                }
-                            }
-                        }
-                    }
+                if (writer && lane == 0) {
+                    pr.scales[t] = range != 0.f ? __fdiv_rn(range, levels) : 1.f;
+                    if (pr.zp) pr.zp[t] = shift_i;
                 }
                 if (pr.y && valid) {
 #pragma unroll
-                    for (int j = 0; j < NC; ++j)
+                    for (int j = 0; j < NC * 8; ++j)
+                        if (j < exist) pr.y[t * (int64_t)g.K + (c_base + j) * g.n2 + d] = y[j] * f1;
+                }
+                // fl(y inv) = fl(y_row_scaled (f inv)): f is a power of two, and where f inv leaves fp32's normal range the row is too
+                // small against the token's largest value for any code but zero
+                const float f_inv = inv * f1;
+                int8_t* const ct = pr.codes + t * (int64_t)g.K;
+                uint32_t usum = 0u;
+                auto words = [&](int j, uint32_t& w0, uint32_t& w1) {
+                    float v0 = __fmul_rn(y[j], f_inv), v1 = __fmul_rn(y[j + 1], f_inv);
+                    add2(v0, v1, bias_even, bias_even);
+                    if (MODE == kAsym) {
+                        w0 = __float_as_uint(fminf(fmaxf(v0, lo_b), hi_b)) + odd;
+                        w1 = __float_as_uint(fminf(fmaxf(v1, lo_b), hi_b)) + odd;
+                    } else {
+                        w0 = __float_as_uint(v0); w1 = __float_as_uint(v1);
+                    }
+                };
+                if (pr.codes_layout) {
+                    // Four columns at a time: lanes 8 apart have neighbouring bytes of a column in the contraction's order, so one
+                    // of the two stores both lanes' codes of the first two columns, the other those of the last two.
+                    const int hb = (lane >> 3) & 1;
+                    const uint32_t sel = hb ? 0x1504u : 0x5140u;
+                    const int k0 = (c_base + 2 * hb) * g.n2 + (d & ~8);
+                    // (a column further is n2 further in k, a multiple of 16: every other column has the same place in its group of 32)
+                    const int k1 = k0 + g.n2;
+                    int8_t* at0 = ct + (k0 & ~31) + 4 * (k0 & 7) + ((k0 & 31) >> 3);
+                    int8_t* at1 = ct + (k1 & ~31) + 4 * (k1 & 7) + ((k1 & 31) >> 3);
+                    const int step = 4 * g.n2, mine_first = 2 * hb;
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (8 * j < cw && c_base + 8 * j + e < g.n1) pr.y[t * (int64_t)g.K + (c_base + 8 * j + e) * g.n2 + d] = y[8 * j + e];
+                    for (int j = 0; j < NC * 8; j += 4) {
+                        if ((j & ~7) < exist) {
+                            uint32_t w0, w1, w2, w3;
+                            words(j, w0, w1);
+                            words(j + 2, w2, w3);
+                            const uint32_t p01 = __byte_perm(w0, w1, 0x0040), p23 = __byte_perm(w2, w3, 0x0040);
+                            const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, hb ? p01 : p23, 8);
+                            const uint32_t both = __byte_perm(hb ? p23 : p01, other, sel);
+                            if (j + 4 <= exist) {
+                                usum += w0 + w1;
+                                usum += w2 + w3;
+                                if (valid) {
+                                    *reinterpret_cast<uint16_t*>(at0) = (uint16_t)both;
+                                    *reinterpret_cast<uint16_t*>(at1) = (uint16_t)(both >> 16);
+                                }
+                            } else {
+                                if (j < exist) usum += w0;
+                                if (j + 1 < exist) usum += w1;
+                                if (j + 2 < exist) usum += w2;
+                                if (valid && j + mine_first < exist) *reinterpret_cast<uint16_t*>(at0) = (uint16_t)both;
+                                if (valid && j + mine_first + 1 < exist) *reinterpret_cast<uint16_t*>(at1) = (uint16_t)(both >> 16);
+                            }
+                            at0 += step; at1 += step;
+                        }
+                    }
+                } else {
+                    int8_t* at = ct + c_base * g.n2 + d;
+#pragma unroll
+                    for (int j = 0; j < NC * 8; j += 2) {
+                        uint32_t w0, w1;
+                        words(j, w0, w1);
+                        if (j < exist) { usum += w0; if (valid) at[0] = (int8_t)w0; }
+                        if (j + 1 < exist) { usum += w1; if (valid) at[g.n2] = (int8_t)w1; }
+                        at += 2 * g.n2;
+                    }
                 }
                 if (pr.qsum) {
                     // the token's last warp of this CTA to add its sum leaves the CTA's part; the consumer adds the parts
-                    int local = valid ? (int)(usum - (uint32_t)counted * (0x4B400000u + (uint32_t)pr.code_bias)) : 0;
+                    int local = valid ? (int)(usum - (uint32_t)max(exist, 0) * (0x4B400000u + (uint32_t)pr.code_bias)) : 0;
                     local = __reduce_add_sync(0xFFFFFFFFu, local);
                     int last = 0, sum = 0;
                     if (lane == 0) {
@@ -550,13 +569,9 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     if (last && lane < kQsumParts && (lane == rank || (rank == 0 && lane >= g.dc)))
                         pr.qsum[t * kQsumParts + lane] = lane == rank ? sum : 0;
                 }
-                if (lane == 0 && rank == 0 && q == 0 && c_base == 0) {
-                    pr.scales[t] = scale;
-                    if (pr.zp) pr.zp[t] = shift_i;
-                }
-            }
-            return true;
+                return true;
             };
+            if (!TWO && i < n && !convert()) { ok = false; break; }
             if (i > 0 && !finish()) { ok = false; break; }
             if (TWO && i < n && !convert()) { ok = false; break; }
         }
@@ -573,6 +588,12 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     if (g.dc > 1) { cluster_arrive_release(); cluster_wait_acquire(); }
 }
 
+typedef void (*Kernel)(const CUtensorMap, const RotUmmaParams);
+template <int MODE>
+static Kernel pick_rot_umma(const RotUmmaGeom& g) {
+    return g.two ? rot_umma_kernel<5, MODE, true> : g.ntot <= 128 ? rot_umma_kernel<4, MODE, false> : rot_umma_kernel<5, MODE, false>;
+}
+
 bool rot_umma_supports(const RotGeom& base, int64_t M, int n_problems, const RotProblem* problems) {
     // more tokens than rot_mma.cu spreads over the SMs one by one
     if (M * n_problems <= sm_count()) return false;
@@ -587,7 +608,7 @@ int launch_rot_umma(const RotGeom& base, const void* x, int64_t M, int64_t ldx, 
     RotUmmaParams p{};
     if (!rot_umma_geometry(base, &p.g)) return BWLA_ERR_INVALID_ARG;
     const RotUmmaGeom& g = p.g;
-    p.M = M; p.bits = bits; p.asym = asym; p.n_problems = n_problems; p.status = status;
+    p.M = M; p.bits = bits; p.n_problems = n_problems; p.status = status;
     for (int i = 0; i < n_problems; ++i) p.prob[i] = problems[i];
     CUtensorMap xm;
     {
@@ -598,11 +619,8 @@ int launch_rot_umma(const RotGeom& base, const void* x, int64_t M, int64_t ldx, 
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
         if (st != BWLA_OK) return st;
     }
-    const bool bf16 = problems[0].yhat != nullptr;
-    typedef void (*Kernel)(const CUtensorMap, const RotUmmaParams);
-    const Kernel k = g.two ? (bf16 ? (Kernel)rot_umma_kernel<5, true, true> : (Kernel)rot_umma_kernel<5, false, true>)
-                   : g.ntot <= 128 ? (bf16 ? (Kernel)rot_umma_kernel<4, true, false> : (Kernel)rot_umma_kernel<4, false, false>)
-                                   : (bf16 ? (Kernel)rot_umma_kernel<5, true, false> : (Kernel)rot_umma_kernel<5, false, false>);
+    const int mode = problems[0].yhat ? kBf16 : asym ? kAsym : kSym;
+    const Kernel k = mode == kSym ? pick_rot_umma<kSym>(g) : mode == kAsym ? pick_rot_umma<kAsym>(g) : pick_rot_umma<kBf16>(g);
     const int room = resident_clusters((const void*)k, g.dc, ru::kThreads, (size_t)g.total) / n_problems;
     if (room < 1) return cuda_fail(cudaErrorInvalidConfiguration);
     p.clusters_per_problem = (int)std::min<int64_t>((M + g.tps - 1) / g.tps, room);
