@@ -307,7 +307,6 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         const int parts = 4 / g.tps;                  // warps of a token in a lane quarter
         const int have = some ? min(cw, g.nc - c_base) : 0;                   // columns that hold sums (a multiple of 8), and
         const int exist = some ? min(cw, g.n1 - c_base) : 0;                  // that are outputs (either may be negative)
-        float y[NC * 8];
         float f1 = 1.f;                               // power of two that brings this lane's row of y to true scale
         int z_exp = 0;
         bool ok = true;
@@ -316,6 +315,7 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             const int pi = (i - 1) & 1;
             const int64_t t = (first + (int64_t)(i - 1) * p.clusters_per_problem) * g.tps + tk;
             float amax = 0.f, vmin = 0.f;
+            float y[NC * 8];
             if (i > 0) {
                 // ---- Y of the step before to registers; its extremes to the token's other warps
                 if (!warp_wait(&sh.y_full[acc_of(i - 1)], phase_of(i - 1), abort_flag)) { give_up(p.status, abort_flag, 0x230); ok = false; break; }
@@ -380,15 +380,35 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (!warp_wait(&sh.z_full[acc_of(i)], phase_of(i), abort_flag)) { give_up(p.status, abort_flag, 0x231); return false; }
                 tc_fence_after();
                 const uint32_t src = tmem + lane_addr + (uint32_t)(acc_of(i) * g.ntot + wc * cw);
-                float z[NC * 8];
+                // TWO: Z stays in registers over the exchange.  Otherwise the step before's Y is there, and Z is read twice.
+                constexpr int ZR = TWO ? NC * 8 : 16;
+                float z[ZR];
+                auto load_two = [&](int j) {                  // chunks j and j + 1, without a second chain
+                    uint32_t v[16];
+                    if (8 * j < cw) tmem_ld_32x8(src + 8 * j, v);
+                    if (8 * (j + 1) < cw) tmem_ld_32x8(src + 8 * (j + 1), v + 8);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) z[e % ZR] = __uint_as_float(v[e]);
+                };
                 if (some) {
-                    load_sums<NC, TWO>(src, (uint32_t)g.ntot, cw, z);
                     float m = 0.f;
+                    if constexpr (TWO) {
+                        load_sums<NC, true>(src, (uint32_t)g.ntot, cw, z);
 #pragma unroll
-                    for (int j = 0; j < NC; ++j)
-                        if (8 * j < cw)
+                        for (int j = 0; j < NC; ++j)
+                            if (8 * j < cw)
 #pragma unroll
-                            for (int e = 0; e < 8; e += 2) m = fmaxf(m, fmaxf(fabsf(z[8 * j + e]), fabsf(z[8 * j + e + 1])));
+                                for (int e = 0; e < 8; e += 2) m = fmaxf(m, fmaxf(fabsf(z[8 * j + e]), fabsf(z[8 * j + e + 1])));
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < NC; j += 2) {
+                            load_two(j);
+#pragma unroll
+                            for (int e = 0; e < 16; e += 2)
+                                if (8 * j + e < cw) m = fmaxf(m, fmaxf(fabsf(z[e]), fabsf(z[e + 1])));
+                        }
+                    }
                     sh.zexp[zi][q][lane][wc] = (uint8_t)(__float_as_uint(m) >> 23);
                 }
                 __syncwarp();
@@ -407,12 +427,14 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     const uint32_t dst = tmem + lane_addr + (uint32_t)(2 * g.ntot + (wc * cw >> 1));
 #pragma unroll
                     for (int j = 0; j < NC; ++j) {
+                        if (!TWO && j % 2 == 0) load_two(j);
                         if (8 * j < cw) {
                             uint32_t h[4], l[4];
+                            const int at = TWO ? 8 * j : 8 * (j & 1);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
-                                mul2(z[8 * j + 2 * e], z[8 * j + 2 * e + 1], z_scale);
-                                split2_pair(z[8 * j + 2 * e], z[8 * j + 2 * e + 1], h[e], l[e]);
+                                mul2(z[at + 2 * e], z[at + 2 * e + 1], z_scale);
+                                split2_pair(z[at + 2 * e], z[at + 2 * e + 1], h[e], l[e]);
                             }
                             tmem_st_32x4(dst + 4 * j, h);
                             tmem_st_32x4(dst + (uint32_t)(g.ntot >> 1) + 4 * j, l);
