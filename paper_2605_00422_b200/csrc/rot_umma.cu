@@ -380,34 +380,17 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (!warp_wait(&sh.z_full[acc_of(i)], phase_of(i), abort_flag)) { give_up(p.status, abort_flag, 0x231); return false; }
                 tc_fence_after();
                 const uint32_t src = tmem + lane_addr + (uint32_t)(acc_of(i) * g.ntot + wc * cw);
-                // TWO: Z stays in registers over the exchange.  Otherwise the step before's Y is there, and Z is read twice.
-                constexpr int ZR = TWO ? NC * 8 : 16;
-                float z[ZR];
-                auto load_two = [&](int j) {                  // chunks j and j + 1, without a second chain
-                    uint32_t v[16];
-                    if (8 * j < cw) tmem_ld_32x8(src + 8 * j, v);
-                    if (8 * (j + 1) < cw) tmem_ld_32x8(src + 8 * (j + 1), v + 8);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) z[e % ZR] = __uint_as_float(v[e]);
-                };
+                // (read twice, two chunks at a time: with all of Z in registers over the exchange they do not suffice)
+                float z[16];
+                auto load_two = [&](int j) { load_sums<2, TWO>(src + 8 * j, (uint32_t)g.ntot, cw - 8 * j, z); };
                 if (some) {
                     float m = 0.f;
-                    if constexpr (TWO) {
-                        load_sums<NC, true>(src, (uint32_t)g.ntot, cw, z);
 #pragma unroll
-                        for (int j = 0; j < NC; ++j)
-                            if (8 * j < cw)
+                    for (int j = 0; j < NC; j += 2) {
+                        load_two(j);
 #pragma unroll
-                                for (int e = 0; e < 8; e += 2) m = fmaxf(m, fmaxf(fabsf(z[8 * j + e]), fabsf(z[8 * j + e + 1])));
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < NC; j += 2) {
-                            load_two(j);
-#pragma unroll
-                            for (int e = 0; e < 16; e += 2)
-                                if (8 * j + e < cw) m = fmaxf(m, fmaxf(fabsf(z[e]), fabsf(z[e + 1])));
-                        }
+                        for (int e = 0; e < 16; e += 2)
+                            if (8 * j + e < cw) m = fmaxf(m, fmaxf(fabsf(z[e]), fabsf(z[e + 1])));
                     }
                     sh.zexp[zi][q][lane][wc] = (uint8_t)(__float_as_uint(m) >> 23);
                 }
@@ -427,10 +410,10 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     const uint32_t dst = tmem + lane_addr + (uint32_t)(2 * g.ntot + (wc * cw >> 1));
 #pragma unroll
                     for (int j = 0; j < NC; ++j) {
-                        if (!TWO && j % 2 == 0) load_two(j);
+                        if (j % 2 == 0) load_two(j);
                         if (8 * j < cw) {
                             uint32_t h[4], l[4];
-                            const int at = TWO ? 8 * j : 8 * (j & 1);
+                            const int at = 8 * (j & 1);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 mul2(z[at + 2 * e], z[at + 2 * e + 1], z_scale);
