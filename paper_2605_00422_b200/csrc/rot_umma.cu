@@ -48,10 +48,11 @@ struct Shared {
     uint64_t d_free[2];                   // ... has been read
     uint64_t a_ready;                     // the terms of Z are in tensor memory
     uint64_t row_full[2][4];              // the exponents of a lane quarter's rows are there
+    uint64_t out_full[2], out_free[2];    // the step's outputs and code sums are staged; have left
     uint64_t max_full[2];                 // all warps of the token (both CTAs) have left their maxima
     uint32_t amax[2][32], vmin[2][32];    // [step parity][CTA][column part][lane quarter]
     uint8_t zexp[2][4][32][4];            // biased exponents of the rows' largest |Z|: [step parity][quarter][lane][column part]
-    int qsum[2][4], count[2][4];          // code sums of the step's tokens, warps that have added theirs
+    int qsum[2][4];                       // code sums of the step's tokens
     uint32_t tmem_slot;
     int abort_flag;
 };
@@ -67,13 +68,15 @@ struct RotUmmaGeom {
     int atoms2, atoms1;     // K atoms of 32 elements over b / over a
     int xb;                 // buffers of x
     int two;                // two chains of sums
-    int p1_off, x_off, sh_off, total;
+    int staged;             // outputs of a step go through shared memory (two buffers of out_bytes)
+    int out_bytes;
+    int p1_off, x_off, st_off, sh_off, total;
     int s2, s1;             // row strides of the prepared factors
 };
 
 // False when the sizes are outside what the kernel takes: whole 16-byte pieces of the codes' order (n2 a multiple of 16), three
 // times n1 columns of tensor memory, at most 128 rows and the factors' terms in the shared memory of one CTA or of two.
-static bool rot_umma_geometry(const RotGeom& g, RotUmmaGeom* out) {
+static bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) {
     if (g.n2 % 16 != 0 || g.n2 < 16 || g.n1 > 160) return false;
     RotUmmaGeom u{};
     u.n1 = g.n1; u.n2 = g.n2; u.K = g.K; u.s2 = g.s2; u.s1 = g.s1;
@@ -87,10 +90,16 @@ static bool rot_umma_geometry(const RotGeom& g, RotUmmaGeom* out) {
     for (u.dc = 1; u.dc <= 2; ++u.dc) {
         u.dt = u.dc == 1 ? g.n2 : (g.n2 / 2 + 15) / 16 * 16;
         if (u.dt > 128) continue;
-        for (u.xb = 2; u.xb >= 1; --u.xb) {
+        // Outputs of whole tokens are contiguous: they are staged where two buffers fit, at the price of the second x if need
+        // be (stored from registers, a sector of 32 bytes is written in two or four pieces: 64 x 80, 4096 tokens 54 us).
+        for (int option = u.dc == 1 ? 0 : 2; option < 4; ++option) {
+            u.xb = 2 - (option & 1);
+            u.staged = option < 2;
+            u.out_bytes = u.tps * u.K * out_size;
             u.p1_off = 3 * u.atoms2 * u.dt * 64;
             u.x_off = u.p1_off + 2 * u.atoms1 * u.nc * 64;
-            u.sh_off = u.x_off + u.xb * u.atoms2 * u.ntot * 64;
+            u.st_off = u.x_off + u.xb * u.atoms2 * u.ntot * 64;
+            u.sh_off = (u.st_off + (u.staged ? 2 * u.out_bytes : 0) + 127) / 128 * 128;
             u.total = u.sh_off + ru::kSharedBytes;
             // (an MMA reads 128 rows from the first row of any block of P2's terms)
             if (u.total <= ru::kMaxSmem && u.p1_off - u.dt * 64 + 128 * 64 <= u.total) { *out = u; return true; }
@@ -118,6 +127,12 @@ __device__ __forceinline__ void tmem_st_32x4(uint32_t taddr, const uint32_t (&v)
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
                  ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;"
+                 ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ bool warp_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
     for (uint32_t i = 0; i < kWaitLimit; ++i) {
         const bool done = mbar_try_wait_cluster(bar, parity, kParkNs);
@@ -134,14 +149,15 @@ __device__ __forceinline__ void load_sums(uint32_t src, uint32_t other, int cw, 
         if (8 * j < cw) tmem_ld_32x8(src + 8 * j, reinterpret_cast<uint32_t*>(v) + 8 * j);
     if (TWO) {
 #pragma unroll
-        for (int j = 0; j < NC; j += 2) {
-            uint32_t u[16];
-            if (8 * j < cw) tmem_ld_32x8(src + other + 8 * j, u);
-            if (j + 1 < NC && 8 * (j + 1) < cw) tmem_ld_32x8(src + other + 8 * (j + 1), u + 8);
-            tc_wait_ld();
+        for (int j = 0; j < NC; ++j) {
+            uint32_t u[8];
+            if (8 * j < cw) {
+                tmem_ld_32x8(src + other + 8 * j, u);
+                tc_wait_ld();
 #pragma unroll
-            for (int e = 0; e < (j + 1 < NC ? 16 : 8); e += 2)
-                add2(v[8 * j + e], v[8 * j + e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
+                for (int e = 0; e < 8; e += 2)
+                    add2(v[8 * j + e], v[8 * j + e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
+            }
         }
     } else {
         tc_wait_ld();
@@ -204,7 +220,8 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             mbar_init(&sh.x_full[i], 1); mbar_init(&sh.x_empty[i], 1);
             mbar_init(&sh.z_full[i], 1); mbar_init(&sh.y_full[i], 1);
             mbar_init(&sh.d_free[i], ru::kAluWarps); mbar_init(&sh.max_full[i], ru::kAluWarps * g.dc);
-            for (int j = 0; j < 4; ++j) { sh.qsum[i][j] = sh.count[i][j] = 0; mbar_init(&sh.row_full[i][j], 4); }
+            mbar_init(&sh.out_full[i], ru::kAluWarps); mbar_init(&sh.out_free[i], 1);
+            for (int j = 0; j < 4; ++j) { sh.qsum[i][j] = 0; mbar_init(&sh.row_full[i][j], 4); }
         }
         mbar_init(&sh.a_ready, ru::kAluWarps);
         fence_barrier_init();
@@ -292,6 +309,32 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 tc_commit(&sh.y_full[acc_of(i)]);
             }
         }
+    } else if (warp == 3) {
+        // ---------------- code sums and staged outputs of a step ----------------
+        for (int i = 0; i < n; ++i) {
+            const int par = i & 1;
+            if (!warp_wait(&sh.out_full[par], (uint32_t)((i >> 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x240); break; }
+            const int64_t t0 = (first + (int64_t)i * p.clusters_per_problem) * g.tps;
+            const int tokens = (int)min((int64_t)g.tps, p.M - t0);
+            if (g.staged && lane == 0) {
+                const int size = g.out_bytes / g.tps;
+                uint8_t* dst = MODE == kBf16 ? reinterpret_cast<uint8_t*>(pr.yhat) : reinterpret_cast<uint8_t*>(pr.codes);
+                bulk_s2g(dst + t0 * size, smem + g.st_off + par * g.out_bytes, (uint32_t)(tokens * size));
+            }
+            if (MODE != kBf16 && pr.qsum) {
+                // every CTA of the cluster leaves its own part of the sum; the consumer adds the parts
+                const int tk = lane >> 3, part = lane & 7;
+                static_assert(kQsumParts == 8, "a lane per part");
+                const int sum = sh.qsum[par][tk];
+                __syncwarp();
+                if (part == 0) sh.qsum[par][tk] = 0;
+                if (tk < tokens && (part == rank || (rank == 0 && part >= g.dc))) pr.qsum[(t0 + tk) * kQsumParts + part] = part == rank ? sum : 0;
+            }
+            if (g.staged && lane == 0) bulk_wait_read();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.out_free[par]);
+        }
+        if (g.staged && lane == 0) bulk_wait_all();
     } else if (warp >= 4) {
         // ---------------- everything between and behind the MMAs ----------------
         // A warp issues an instruction about every six cycles here (four warps a scheduler), so instructions a value are what
@@ -432,10 +475,12 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             };
             // ---- the step before: codes, scale and code sum, or bf16 values
             auto finish = [&]() -> bool {
+                if (i >= 3 && !warp_wait(&sh.out_free[pi], (uint32_t)((((i - 1) >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x234); return false; }
+                uint8_t* const stage = smem + g.st_off + pi * g.out_bytes + tk * (g.out_bytes / g.tps);
                 if (MODE == kBf16) {
                     if (t < p.M && valid) {
                         // layout 1: inside each group of 32, position 2 (k % 16) + (k % 32) / 16
-                        __nv_bfloat16* yt = pr.yhat + t * (int64_t)g.K;
+                        __nv_bfloat16* yt = g.staged ? reinterpret_cast<__nv_bfloat16*>(stage) : pr.yhat + t * (int64_t)g.K;
 #pragma unroll
                         for (int j = 0; j < NC; ++j)
 #pragma unroll
@@ -494,7 +539,7 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 // fl(y inv) = fl(y_row_scaled (f inv)): f is a power of two, and where f inv leaves fp32's normal range the row is too
                 // small against the token's largest value for any code but zero
                 const float f_inv = inv * f1;
-                int8_t* const ct = pr.codes + t * (int64_t)g.K;
+                int8_t* const ct = g.staged ? reinterpret_cast<int8_t*>(stage) : pr.codes + t * (int64_t)g.K;
                 uint32_t usum = 0u;
                 auto words = [&](int j, uint32_t& w0, uint32_t& w1) {
                     float v0 = __fmul_rn(y[j], f_inv), v1 = __fmul_rn(y[j + 1], f_inv);
@@ -555,29 +600,19 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     }
                 }
                 if (pr.qsum) {
-                    // the token's last warp of this CTA to add its sum leaves the CTA's part; the consumer adds the parts
                     int local = valid ? (int)(usum - (uint32_t)max(exist, 0) * (0x4B400000u + (uint32_t)pr.code_bias)) : 0;
                     local = __reduce_add_sync(0xFFFFFFFFu, local);
-                    int last = 0, sum = 0;
-                    if (lane == 0) {
-                        if (local != 0) atomicAdd(&sh.qsum[pi][tk], local);
-                        __threadfence_block();
-                        last = atomicAdd(&sh.count[pi][tk], 1) == 4 * parts - 1;
-                        if (last) {
-                            __threadfence_block();
-                            sum = atomicExch(&sh.qsum[pi][tk], 0);
-                            sh.count[pi][tk] = 0;
-                        }
-                    }
-                    last = __shfl_sync(0xFFFFFFFFu, last, 0);
-                    sum = __shfl_sync(0xFFFFFFFFu, sum, 0);
-                    if (last && lane < kQsumParts && (lane == rank || (rank == 0 && lane >= g.dc)))
-                        pr.qsum[t * kQsumParts + lane] = lane == rank ? sum : 0;
+                    if (lane == 0 && local != 0) atomicAdd(&sh.qsum[pi][tk], local);
                 }
                 return true;
             };
             if (!TWO && i < n && !convert()) { ok = false; break; }
-            if (i > 0 && !finish()) { ok = false; break; }
+            if (i > 0) {
+                if (!finish()) { ok = false; break; }
+                if (g.staged) fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.out_full[pi]);
+            }
             if (TWO && i < n && !convert()) { ok = false; break; }
         }
         if (!ok) *abort_flag = 1;
@@ -605,13 +640,13 @@ bool rot_umma_supports(const RotGeom& base, int64_t M, int n_problems, const Rot
     for (int i = 0; i < n_problems; ++i)
         if (problems[i].digits || problems[i].packed) return false;
     RotUmmaGeom u;
-    return rot_umma_geometry(base, &u);
+    return rot_umma_geometry(base, problems[0].yhat ? 2 : 1, &u);
 }
 
 int launch_rot_umma(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                     const RotProblem* problems, uint32_t* status, cudaStream_t stream) {
     RotUmmaParams p{};
-    if (!rot_umma_geometry(base, &p.g)) return BWLA_ERR_INVALID_ARG;
+    if (!rot_umma_geometry(base, problems[0].yhat ? 2 : 1, &p.g)) return BWLA_ERR_INVALID_ARG;
     const RotUmmaGeom& g = p.g;
     p.M = M; p.bits = bits; p.n_problems = n_problems; p.status = status;
     for (int i = 0; i < n_problems; ++i) p.prob[i] = problems[i];
