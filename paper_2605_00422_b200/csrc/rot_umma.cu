@@ -127,6 +127,9 @@ __device__ __forceinline__ void tmem_st_32x4(uint32_t taddr, const uint32_t (&v)
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
                  ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
+__device__ __forceinline__ void st_shared_u16(uint32_t at, uint32_t v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)v) : "memory");
+}
 __device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;"
                  ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
@@ -539,69 +542,77 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 // fl(y inv) = fl(y_row_scaled (f inv)): f is a power of two, and where f inv leaves fp32's normal range the row is too
                 // small against the token's largest value for any code but zero
                 const float f_inv = inv * f1;
-                int8_t* const ct = g.staged ? reinterpret_cast<int8_t*>(stage) : pr.codes + t * (int64_t)g.K;
-                uint32_t usum = 0u;
-                auto words = [&](int j, uint32_t& w0, uint32_t& w1) {
-                    float v0 = __fmul_rn(y[j], f_inv), v1 = __fmul_rn(y[j + 1], f_inv);
-                    add2(v0, v1, bias_even, bias_even);
-                    if (MODE == kAsym) {
-                        w0 = __float_as_uint(fminf(fmaxf(v0, lo_b), hi_b)) + odd;
-                        w1 = __float_as_uint(fminf(fmaxf(v1, lo_b), hi_b)) + odd;
-                    } else {
-                        w0 = __float_as_uint(v0); w1 = __float_as_uint(v1);
-                    }
-                };
-                if (pr.codes_layout) {
-                    // Four columns at a time: lanes 8 apart have neighbouring bytes of a column in the contraction's order, so one
-                    // of the two stores both lanes' codes of the first two columns, the other those of the last two.
+                int code_sum = 0;                                 // of the stored codes less their bias
+                const int whole = pr.codes_layout ? max(exist, 0) & ~7 : 0;
+                if (whole > 0) {
+                    // The usual case: whole chunks of outputs, in the contraction's order.  Four codes of a lane make a
+                    // word by multiply-adds, every code shifted to c + 128 >= 0 (the bits of 1.5 * 2^23 below bit 16 are zero, so
+                    // nothing carries from one byte into the next).  Lanes 8 apart have neighbouring bytes of a column: they swap
+                    // words, and one of the two stores both lanes' codes of the first two columns, the other of the last two.
+                    // (Conditions a column, selects and packing one by one took 31 half-rate instructions for four columns, 250
+                    // cycles a scheduler.)
                     const int hb = (lane >> 3) & 1;
-                    const uint32_t sel = hb ? 0x1504u : 0x5140u;
-                    const int k0 = (c_base + 2 * hb) * g.n2 + (d & ~8);
-                    // (a column further is n2 further in k, a multiple of 16: every other column has the same place in its group of 32)
-                    const int k1 = k0 + g.n2;
-                    int8_t* at0 = ct + (k0 & ~31) + 4 * (k0 & 7) + ((k0 & 31) >> 3);
-                    int8_t* at1 = ct + (k1 & ~31) + 4 * (k1 & 7) + ((k1 & 31) >> 3);
-                    const int step = 4 * g.n2, mine_first = 2 * hb;
+                    const uint32_t sel = hb ? 0x3726u : 0x5140u;
+                    const int k0 = (c_base + 2 * hb) * g.n2 + (d & ~8), k1 = k0 + g.n2;
+                    const int off0 = (k0 & ~31) + 4 * (k0 & 7) + ((k0 & 31) >> 3), off1 = (k1 & ~31) + 4 * (k1 & 7) + ((k1 & 31) >> 3);
+                    const float b = bias_even + 128.f, lo = lo_b + 128.f, hi = hi_b + 128.f;
+                    // w0 + 2^8 w1 has 0x8B40 above its two bytes; that of the lower pair is taken off the upper one
+                    const uint32_t top = MODE == kAsym ? 0x74C00000u + 0x01010101u * odd : 0x74C00000u;
+                    uint32_t sum = 0u;
+                    auto all = [&](auto store) {
 #pragma unroll
-                    for (int j = 0; j < NC * 8; j += 4) {
-                        if ((j & ~7) < exist) {
-                            uint32_t w0, w1, w2, w3;
-                            words(j, w0, w1);
-                            words(j + 2, w2, w3);
-                            const uint32_t p01 = __byte_perm(w0, w1, 0x0040), p23 = __byte_perm(w2, w3, 0x0040);
-                            const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, hb ? p01 : p23, 8);
-                            const uint32_t both = __byte_perm(hb ? p23 : p01, other, sel);
-                            if (j + 4 <= exist) {
-                                usum += w0 + w1;
-                                usum += w2 + w3;
-                                if (valid) {
-                                    *reinterpret_cast<uint16_t*>(at0) = (uint16_t)both;
-                                    *reinterpret_cast<uint16_t*>(at1) = (uint16_t)(both >> 16);
-                                }
-                            } else {
-                                if (j < exist) usum += w0;
-                                if (j + 1 < exist) usum += w1;
-                                if (j + 2 < exist) usum += w2;
-                                if (valid && j + mine_first < exist) *reinterpret_cast<uint16_t*>(at0) = (uint16_t)both;
-                                if (valid && j + mine_first + 1 < exist) *reinterpret_cast<uint16_t*>(at1) = (uint16_t)(both >> 16);
-                            }
-                            at0 += step; at1 += step;
+                        for (int j = 0; j < NC * 8; j += 4) {
+                            if ((j & ~7) >= whole) break;
+                            float v[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) v[e] = __fmul_rn(y[j + e], f_inv);
+                            add2(v[0], v[1], b, b);
+                            add2(v[2], v[3], b, b);
+                            if (MODE == kAsym)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) v[e] = fminf(fmaxf(v[e], lo), hi);
+                            const uint32_t p01 = __float_as_uint(v[1]) * 256u + __float_as_uint(v[0]);
+                            const uint32_t p23 = __float_as_uint(v[3]) * 256u + __float_as_uint(v[2]);
+                            const uint32_t word = p23 * 65536u + (p01 + top);
+                            sum = __dp4a(word, 0x01010101u, sum);
+                            const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 8);
+                            const uint32_t both = __byte_perm(word, other, sel) ^ 0x80808080u;
+                            store(j, both);
                         }
+                    };
+                    if (g.staged) {
+                        uint32_t at0 = smem_u32(stage) + off0, at1 = smem_u32(stage) + off1;
+                        const uint32_t step = 4 * g.n2;
+                        all([&](int, uint32_t both) {
+                            if (valid) { st_shared_u16(at0, both); st_shared_u16(at1, both >> 16); }
+                            at0 += step; at1 += step;
+                        });
+                    } else {
+                        int8_t* at0 = pr.codes + t * (int64_t)g.K + off0;
+                        const int delta = off1 - off0, step = 4 * g.n2;
+                        all([&](int, uint32_t both) {
+                            if (valid) { *reinterpret_cast<uint16_t*>(at0) = (uint16_t)both; *reinterpret_cast<uint16_t*>(at0 + delta) = (uint16_t)(both >> 16); }
+                            at0 += step;
+                        });
                     }
-                } else {
-                    int8_t* at = ct + c_base * g.n2 + d;
+                    code_sum = (int)sum - whole * (128 + pr.code_bias);
+                }
+                if (whole < exist) {
+                    int8_t* const ct = g.staged ? reinterpret_cast<int8_t*>(stage) : pr.codes + t * (int64_t)g.K;
 #pragma unroll
-                    for (int j = 0; j < NC * 8; j += 2) {
-                        uint32_t w0, w1;
-                        words(j, w0, w1);
-                        if (j < exist) { usum += w0; if (valid) at[0] = (int8_t)w0; }
-                        if (j + 1 < exist) { usum += w1; if (valid) at[g.n2] = (int8_t)w1; }
-                        at += 2 * g.n2;
+                    for (int j = 0; j < NC * 8; ++j) {
+                        if (j >= whole && j < exist) {
+                            const float v = __fadd_rn(__fmul_rn(y[j], f_inv), bias_even);
+                            uint32_t word = __float_as_uint(v);
+                            if (MODE == kAsym) word = __float_as_uint(fminf(fmaxf(v, lo_b), hi_b)) + odd;
+                            code_sum += (int)(word - (0x4B400000u + (uint32_t)pr.code_bias));
+                            const int k = (c_base + j) * g.n2 + d;
+                            if (valid) ct[pr.codes_layout ? (k & ~31) + 4 * (k & 7) + ((k & 31) >> 3) : k] = (int8_t)word;
+                        }
                     }
                 }
                 if (pr.qsum) {
-                    int local = valid ? (int)(usum - (uint32_t)max(exist, 0) * (0x4B400000u + (uint32_t)pr.code_bias)) : 0;
-                    local = __reduce_add_sync(0xFFFFFFFFu, local);
+                    const int local = __reduce_add_sync(0xFFFFFFFFu, valid ? code_sum : 0);
                     if (lane == 0 && local != 0) atomicAdd(&sh.qsum[pi][tk], local);
                 }
                 return true;
