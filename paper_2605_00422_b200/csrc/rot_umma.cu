@@ -8,10 +8,11 @@
 // products), small products first.  Z is scaled by a power of two per row d (its largest magnitude goes to [2^14, 2^15)), which
 // leaves exactly, row by row, with the scale of P1.
 //
-// What bounds it: 160 x 160 takes 60 MMAs of 128 x 160 x 16 a token and CTA (2400 cycles), and every value of Z and Y passes
-// through registers once (about 450 instructions a warp, 4 warps a scheduler: 1800 cycles); the warp-level kernel needs 9600
-// cycles of its MMAs alone, with operands re-read from shared memory as fast as it delivers, and one token's barriers stand
-// open.  So the two run side by side, three steps deep:
+// What bounds it: 160 x 160 takes 60 MMAs of 128 x 160 x 16 a token and CTA (80 cycles each, 80 of the 128 rows in use); what the
+// ALU warps do with every value of Z and Y, in lock step and with five barriers a step, takes about twice that.  The warp-level
+// kernel needs 9600 cycles of its MMAs alone, with operands re-read from shared memory as fast as it delivers, and the barriers of
+// its one token stand open: 2048 tokens of 160 x 160 505 -> 231 us, 4096 of 64 x 80 77 -> 62 us.
+// MMAs and the work around them run side by side, three steps deep:
 //   MMA thread    Z(0), Z(1), Y(0), Z(2), Y(1), ...    Z(i) and Y(i) share one of two accumulators
 //   16 ALU warps  step i: Y(i-1) to registers, its largest magnitude published  (accumulator free: Z(i+1) may start)
 //                         Z(i) to two fp16 terms in tensor memory               (Y(i) may start)
@@ -21,7 +22,6 @@
 // accumulators then belong to one step, and the ALU warps quantise under the MMAs of Z.
 // A step is 1, 2 or 4 tokens, so that it fills up to 160 columns (64 x 80: 2 tokens).  Factors whose terms do not fit one CTA
 // (or with n2 > 128) are split by rows d over a cluster of two, which share nothing but the largest magnitudes.
-// 2048 tokens of 160 x 160: see kManyTokens below.
 //
 // Launched with programmatic stream serialisation: the factors are fetched before the preceding kernel of the stream has
 // finished; x is read, and everything is stored, after it.  Every wait is bounded (umma_wait.cuh).
@@ -646,7 +646,7 @@ static Kernel pick_rot_umma(const RotUmmaGeom& g) {
 }
 
 bool rot_umma_supports(const RotGeom& base, int64_t M, int n_problems, const RotProblem* problems) {
-    // more tokens than rot_mma.cu spreads over the SMs one by one
+    // More tokens than SMs: fewer are spread over warps and CTAs one by one (rot_mma.cu), which is the shorter way for one token.
     if (M * n_problems <= sm_count()) return false;
     for (int i = 0; i < n_problems; ++i)
         if (problems[i].digits || problems[i].packed) return false;

@@ -1,0 +1,49 @@
+"""The many-token tcgen05 rotation at the edges of its work split: 1, 2 and 4 tokens a step with a ragged last step, columns that do
+not fill a warp's chunks, rows that do not fill a lane quarter, factors in one CTA and in two, one chain of sums and two, outputs
+staged in shared memory and stored directly.
+
+Y is held to 9e-7 of the token's full scale (the bound of tests/test_rotation_umma_gpu.py), codes and scales must follow from the
+kernel's own Y exactly.  A linear's outputs must be those of the contraction on the codes that the same kernel returns in natural
+order: that covers the order and the sums that the contraction reads."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2605_00422_b200 import inputs as gen
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n1,n2,M,prepared", [
+    (1, 32, 597, True), (20, 32, 331, False), (32, 16, 150, True), (64, 80, 299, True), (64, 80, 299, False), (73, 64, 301, True),
+    (86, 128, 149, True), (108, 128, 160, False), (128, 128, 151, True), (140, 96, 150, True), (64, 160, 153, False),
+    (160, 160, 150, True), (160, 160, 150, False),
+])
+def test_edges(n1, n2, M, prepared):
+    from paper_2605_00422_b200 import bwla
+    K, N, bits = n1 * n2, 40, 6
+    rng = np.random.default_rng([n1, n2, M])
+    P1, P2 = gen.orthogonal_f32(n1, rng), gen.orthogonal_f32(n2, rng)
+    x = rng.standard_t(3, size=(M, K)).astype(np.float32)
+    x[0, 0] = 300.0
+    xb = gen.bf16_bits_from_f32(x)
+    packed = torch.from_numpy(rng.integers(-2 ** 31, 2 ** 31, size=(N, K // 32), dtype=np.int64).astype(np.int32)).cuda()
+    alpha, mu = torch.rand(N, device="cuda") + 0.5, 0.01 * torch.randn(N, device="cuda")
+    dP1, dP2, dx = H.f32_to_dev(P1), H.f32_to_dev(P2), H.bf16_to_dev(xb)
+    if prepared:
+        L = bwla.Layer(dP1, dP2, bits, packed, alpha, None, None, mu)
+        codes, scales, y = bwla.bwla_layer_rotate_quant(L, dx, want_y=True)
+        y = y.cpu().numpy().astype(np.float64)
+        Y = oracle.rotate(xb, P1, P2)
+        assert float((np.abs(y - Y) / np.abs(Y).max(axis=1, keepdims=True)).max()) <= 9e-7
+        q = oracle.quantize(y, bits, "f32")
+        assert np.array_equal(q["codes"], codes.cpu().numpy()) and np.array_equal(q["scales"], scales.cpu().numpy())
+        out = bwla.bwla_w1ax_linear_group([L], dx)[0]
+    else:
+        codes, scales = bwla.bwla_rotate_quant_act(dx, dP1, dP2, bits)
+        out = bwla.bwla_w1ax_linear(dx, dP1, dP2, bits, packed, alpha, None, None, mu)
+    again = bwla.bwla_w1a_gemm_codes(codes, scales, bits, packed, alpha, mu=mu)
+    again = again[0] if isinstance(again, tuple) else again
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
