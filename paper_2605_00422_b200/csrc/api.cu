@@ -421,8 +421,13 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
     }
     RotProblem pr{};
     pr.prepared = L->prepared; pr.yhat = (__nv_bfloat16*)(base + w.yhat); pr.ysum = L->mu ? (float*)(base + w.ysum) : nullptr;
+    const bool persistent = a16_persistent_supports(L->K);
+    pr.codes_layout = persistent ? 1 : 0;
     st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
     if (st != BWLA_OK) return st;
+    if (persistent)
+        return launch_a16_persistent(base + w.yhat, pr.ysum, M, L->K, L->N, L->packed, L->alpha, L->mu, L->U, L->r,
+                                     L->r > 0 ? base + w.T : nullptr, out_bf16, ldo, status, s);
     return launch_gemm_a16(base + w.yhat, pr.ysum, M, L->K, L->N, L->packed, L->alpha, L->mu, L->U, L->r,
                            L->r > 0 ? base + w.T : nullptr, out_bf16, ldo, status, s);
 }

@@ -240,6 +240,11 @@ enum { kDepChain = 0, kDepHead = 1, kDepSibling = 2 };
 
 // W1A16, the weight-only operating point (gemm_a16.cu): the bf16 contraction against the packed signs with the fused
 // epilogue.  Thl as for the int8 contractions (NULL when r == 0).
+// The same in persistent CTAs, yhat in the interleaved order (RotProblem::codes_layout 1)
+bool a16_persistent_supports(int64_t K);
+int launch_a16_persistent(const void* yhat, const float* ysum, int64_t M, int64_t K, int64_t N, const uint32_t* packed,
+                          const float* alpha, const float* mu, const void* U, int r, const void* Thl, void* out, int64_t ldo,
+                          uint32_t* status, cudaStream_t stream);
 bool a16_supports(int64_t M, int64_t K, int64_t N, int r);
 int launch_gemm_a16(const void* yhat, const float* ysum, int64_t M, int64_t K, int64_t N, const uint32_t* packed, const float* alpha,
                     const float* mu, const void* U, int r, const void* Thl, void* out, int64_t ldo, uint32_t* status,
