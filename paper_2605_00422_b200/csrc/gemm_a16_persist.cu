@@ -15,7 +15,7 @@
 // warps add it into running sums in registers, with rounded additions, while the next 512 go to the second accumulator.
 //
 // Warps 0..3: sign words, yhat and T, MMA issue, per-token sums.  4..11: epilogue, two per lane quarter, 64 tokens each; their running
-// sums take registers that the other warps give away.  12..19: expansion, two per lane quarter, every other stage each.
+// sums take registers that the other warps give away.  12..27: expansion, four per lane quarter, every fourth stage each.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -33,12 +33,12 @@ constexpr int kTok = 128;                 // tokens per tile
 constexpr int kUnitK = 1024;              // weights per row in one sign-word stage
 constexpr int kBlockK = 64;               // K per stage
 constexpr int kFlush = 8;                 // stages per accumulator
-constexpr int WS = 3, AS = 4, EW = 2;
+constexpr int WS = 3, AS = 4, EW = 4;
 static_assert(AS % EW == 0, "an operand stage must keep one owner among the expander parts");
 constexpr int kEpiFirst = 128, kExpFirst = 384;
-constexpr int kThreads = kExpFirst + 128 * EW;       // 640
-// registers: 96 a thread at launch (640 x 96 = 61440); 128 x 72 + 256 x 120 + 256 x 80 = 60416 after the split
-constexpr int kRegsControl = 72, kRegsEpilogue = 120, kRegsExpand = 80;
+constexpr int kThreads = kExpFirst + 128 * EW;       // 896
+// registers: 72 a thread at launch (896 x 72 = 64512); 128 x 56 + 256 x 112 + 512 x 56 = 64512 after the split
+constexpr int kRegsControl = 56, kRegsEpilogue = 112, kRegsExpand = 56;
 constexpr int w_bytes = kRows * 128, b_bytes = kTok * 128;
 constexpr int u_off = WS * w_bytes + AS * b_bytes;
 constexpr int t_off = u_off + kRows * 128;
@@ -73,6 +73,13 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
+}
+__device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+        : "memory");
 }
 __device__ __forceinline__ uint2 lds_words(const uint8_t* p) {
     uint2 v;
@@ -345,6 +352,9 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                 const uint32_t sel = odd ? 0x3276u : 0x5410u;
                 const int n_pair = n & ~1;
                 const bool pair_ok = ((reinterpret_cast<uintptr_t>(p.out) & 3) == 0) && (p.ldo & 1) == 0 && n_pair + 1 < p.N;
+                const bool whole = __all_sync(0xFFFFFFFFu, pair_ok) && t0 + kTok <= p.M;
+                __nv_bfloat16* at = p.out + (int64_t)(t0 + 64 * half + odd) * p.ldo + n_pair;
+                const int64_t step = 2 * p.ldo;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     uint32_t l[16];
@@ -372,7 +382,10 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                             const uint32_t word = pack_bf16x2(y[h], y[h + 1]);      // two tokens of this lane's row
                             const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 1);
                             const int t = t0 + tok0 + j + h;
-                            if (pair_ok) {
+                            if (whole) {
+                                *reinterpret_cast<uint32_t*>(at) = __byte_perm(word, other, sel);
+                                at += step;
+                            } else if (pair_ok) {
                                 if (t + odd < p.M) *reinterpret_cast<uint32_t*>(p.out + (int64_t)(t + odd) * p.ldo + n_pair) = __byte_perm(word, other, sel);
                             } else if (valid_row) {
                                 if (t < p.M) p.out[(int64_t)t * p.ldo + n] = __ushort_as_bfloat16((unsigned short)word);
@@ -436,12 +449,6 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
             for (int q = 0; q < PER; ++q) {
                 if (c == i + 1 && c < total && __all_sync(0xFFFFFFFFu, mbar_test_wait(&w_full[ws], wph))) take();
                 if (first + EW * q < ns && ok) {
-                    uint32_t v[32];
-                    const uint32_t w[2] = {~cur[q].x, ~cur[q].y};     // a set bit now means -1
-#pragma unroll
-                    for (int k = 0; k < 2; ++k)
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) v[16 * k + j] = ((w[k] << (15 - j)) & 0x80008000u) | 0x3F803F80u;
                     const int as = (g + EW * q) % AS;
                     const uint32_t aph = (uint32_t)(((g + EW * q) / AS) & 1);
                     if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(&s_empty[as], aph ^ 1u))) {
@@ -450,7 +457,14 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                     }
                     if (ok) {
                         tc_fence_after();
-                        tmem_st_32x32(tmem_base + lane_addr + A_COL + 32 * as, v);
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            const uint32_t w = ~(k == 0 ? cur[q].x : cur[q].y);       // a set bit now means -1
+                            uint32_t v[16];
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) v[j] = ((w << (15 - j)) & 0x80008000u) | 0x3F803F80u;
+                            tmem_st_32x16(tmem_base + lane_addr + A_COL + 32 * as + 16 * k, v);
+                        }
                         tc_wait_st();
                         tc_fence_before();
                         __syncwarp();
