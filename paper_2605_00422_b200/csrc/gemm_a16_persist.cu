@@ -153,9 +153,8 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
     const uint32_t tmem_base = *tmem_slot;
     griddep_launch_dependents();
 
-    if (warp < 4) set_regs_dec<kRegsControl>();
-    else if (warp < 12) set_regs_inc<kRegsEpilogue>();
-    else set_regs_dec<kRegsExpand>();
+    if (warp < 4) {
+    set_regs_dec<kRegsControl>();
     if (warp == 0) {
         // ---------------- packed sign words (independent of the preceding kernel) ----------------
         if (elect_one()) {
@@ -276,7 +275,9 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                 }
             }
         }
-    } else if (warp >= 4 && warp < 12) {
+    }
+    } else if (warp < 12) {
+        set_regs_inc<kRegsEpilogue>();
         // ---------------- epilogue ----------------
         const int q = warp & 3;
         const int e = (threadIdx.x - kEpiFirst) & 127;        // output row of the tile
@@ -327,18 +328,17 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                 tc_fence_after();
                 const uint32_t d_addr = tmem_base + lane_addr + D_COL + (uint32_t)(f & 1) * kTok + 64 * half;
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t v[2][16];
-                    tmem_ld_32x16(d_addr + 32 * c, v[0]);
-                    tmem_ld_32x16(d_addr + 32 * c + 16, v[1]);
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t v[16];
+                    tmem_ld_32x16(d_addr + 16 * c, v);
                     tc_wait_ld();
-                    if (c == 1) {
+                    if (c == 3) {
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&acc_free[f & 1]);
                     }
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) run[32 * c + j] += __uint_as_float(v[j >> 4][j & 15]);
+                    for (int j = 0; j < 16; ++j) run[16 * c + j] += __uint_as_float(v[j]);
                 }
             }
             if (i == 0) griddep_wait();                       // nothing is stored before the preceding kernel has completed
@@ -400,7 +400,8 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
             __syncwarp();
             if (lane == 0) mbar_arrive(&epi_done[buf]);
         }
-    } else if (warp >= 12) {
+    } else {
+        set_regs_dec<kRegsExpand>();
         // ---------------- expansion of sign bits into the operand ring (tile boundaries do not matter here) ----------------
         const int q = warp & 3;
         const int part = (warp - 12) >> 2;             // which of the EW warps of the lane quarter
