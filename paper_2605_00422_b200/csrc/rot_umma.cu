@@ -136,6 +136,10 @@ __device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t by
 }
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+// A word into the shared memory of a CTA of the cluster, counted (4 bytes) on a barrier of that CTA.
+__device__ __forceinline__ void st_async_u32(uint32_t cluster_addr, uint32_t v, uint32_t cluster_bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(cluster_addr), "r"(v), "r"(cluster_bar) : "memory");
+}
 __device__ __forceinline__ bool warp_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
     for (uint32_t i = 0; i < kWaitLimit; ++i) {
         const bool done = mbar_try_wait_cluster(bar, parity, kParkNs);
@@ -152,14 +156,20 @@ __device__ __forceinline__ void load_sums(uint32_t src, uint32_t other, int cw, 
         if (8 * j < cw) tmem_ld_32x8(src + 8 * j, reinterpret_cast<uint32_t*>(v) + 8 * j);
     if (TWO) {
 #pragma unroll
-        for (int j = 0; j < NC; ++j) {
-            uint32_t u[8];
+        for (int j = 0; j < NC; j += 2) {
             if (8 * j < cw) {
+                const bool both = j + 1 < NC && 8 * (j + 1) < cw;
+                uint32_t u[16] = {};
                 tmem_ld_32x8(src + other + 8 * j, u);
+                if (both) tmem_ld_32x8(src + other + 8 * (j + 1), u + 8);
                 tc_wait_ld();
 #pragma unroll
                 for (int e = 0; e < 8; e += 2)
                     add2(v[8 * j + e], v[8 * j + e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
+                if (both && j + 1 < NC)
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2)
+                        add2(v[8 * (j + 1 < NC ? j + 1 : j) + e], v[8 * (j + 1 < NC ? j + 1 : j) + e + 1], __uint_as_float(u[8 + e]), __uint_as_float(u[9 + e]));
             }
         }
     } else {
@@ -222,7 +232,7 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sh.x_full[i], 1); mbar_init(&sh.x_empty[i], 1);
             mbar_init(&sh.z_full[i], 1); mbar_init(&sh.y_full[i], 1);
-            mbar_init(&sh.d_free[i], ru::kAluWarps); mbar_init(&sh.max_full[i], ru::kAluWarps * g.dc);
+            mbar_init(&sh.d_free[i], ru::kAluWarps); mbar_init(&sh.max_full[i], g.dc == 1 ? ru::kAluWarps : 1);
             mbar_init(&sh.out_full[i], ru::kAluWarps); mbar_init(&sh.out_free[i], 1);
             for (int j = 0; j < 4; ++j) { sh.qsum[i][j] = 0; mbar_init(&sh.row_full[i][j], 4); }
         }
@@ -384,10 +394,16 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     uint32_t* slot_v = &sh.vmin[pi][rank * 16 + w];
                     if (g.dc == 1) {
                         if (lane == 0) { *slot = m; *slot_v = v; mbar_arrive(&sh.max_full[pi]); }
-                    } else if (lane < 2) {
-                        st_shared_cluster_u32(map_shared_rank(smem_u32(slot), (uint32_t)lane), m);
-                        if (MODE != kSym) st_shared_cluster_u32(map_shared_rank(smem_u32(slot_v), (uint32_t)lane), v);
-                        mbar_arrive_remote(map_shared_rank(smem_u32(&sh.max_full[pi]), (uint32_t)lane));
+                    } else {
+                        // (asynchronous stores that count on the barrier: an arrival with release at cluster scope waits for this
+                        // warp's codes of the step before to reach global memory, about 1000 cycles)
+                        constexpr uint32_t each = MODE == kSym ? 4u : 8u;
+                        if (w == 0 && lane == 0) mbar_expect_tx(&sh.max_full[pi], 2u * ru::kAluWarps * each);
+                        if (lane < 2) {
+                            const uint32_t bar = map_shared_rank(smem_u32(&sh.max_full[pi]), (uint32_t)lane);
+                            st_async_u32(map_shared_rank(smem_u32(slot), (uint32_t)lane), m, bar);
+                            if (MODE != kSym) st_async_u32(map_shared_rank(smem_u32(slot_v), (uint32_t)lane), v, bar);
+                        }
                     }
                 };
                 if (MODE == kBf16) {
@@ -482,16 +498,27 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 uint8_t* const stage = smem + g.st_off + pi * g.out_bytes + tk * (g.out_bytes / g.tps);
                 if (MODE == kBf16) {
                     if (t < p.M && valid) {
-                        // layout 1: inside each group of 32, position 2 (k % 16) + (k % 32) / 16
+                        // layout 1: inside each group of 32, position 2 (k % 16) + (k % 32) / 16; every other column has the same
+                        // place in its group (2 n2 is a multiple of 32)
                         __nv_bfloat16* yt = g.staged ? reinterpret_cast<__nv_bfloat16*>(stage) : pr.yhat + t * (int64_t)g.K;
+                        const int k0 = c_base * g.n2 + d, k1 = k0 + g.n2;
+                        __nv_bfloat16* at0 = yt + (pr.codes_layout ? (k0 & ~31) + 2 * (k0 & 15) + ((k0 >> 4) & 1) : k0);
+                        __nv_bfloat16* at1 = yt + (pr.codes_layout ? (k1 & ~31) + 2 * (k1 & 15) + ((k1 >> 4) & 1) : k1);
+                        const int step = 2 * g.n2;
+                        if (exist == NC * 8) {
 #pragma unroll
-                        for (int j = 0; j < NC; ++j)
+                            for (int j = 0; j < NC * 8; j += 2) {
+                                *at0 = __float2bfloat16_rn(y[j] * f1); *at1 = __float2bfloat16_rn(y[j + 1] * f1);
+                                at0 += step; at1 += step;
+                            }
+                        } else {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                if (8 * j + e < exist) {
-                                    const int k = (c_base + 8 * j + e) * g.n2 + d;
-                                    yt[pr.codes_layout ? (k & ~31) + 2 * (k & 15) + ((k >> 4) & 1) : k] = __float2bfloat16_rn(y[8 * j + e] * f1);
-                                }
+                            for (int j = 0; j < NC * 8; j += 2) {
+                                if (j < exist) *at0 = __float2bfloat16_rn(y[j] * f1);
+                                if (j + 1 < exist) *at1 = __float2bfloat16_rn(y[j + 1] * f1);
+                                at0 += step; at1 += step;
+                            }
+                        }
                     }
                     if (!pr.ysum) return true;
                 }
