@@ -345,15 +345,9 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 const int n_pair = n & ~1;
                 const bool pair_ok = ((reinterpret_cast<uintptr_t>(p.out) & 3) == 0) && (p.ldo & 1) == 0 && n_pair + 1 < p.N;
                 const uint32_t acc_addr = tmem_base + lane_addr + D_COL + (uint32_t)(i & 1) * kTok;
-                const bool whole = __all_sync(0xFFFFFFFFu, pair_ok) && t0 + kTok <= p.M;
-                __nv_bfloat16* at = p.out + (int64_t)(t0 + (kTok / 2) * half + odd) * p.ldo + n_pair;
-                const int64_t step = 2 * p.ldo;
                 auto put = [&](uint32_t word, int tok) {          // word: tokens tok (low half) and tok + 1 of this lane's row
                     const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 1);
-                    if (whole) {
-                        *reinterpret_cast<uint32_t*>(at) = __byte_perm(word, other, sel);
-                        at += step;
-                    } else if (pair_ok) {
+                    if (pair_ok) {
                         const int t = t0 + tok + odd;
                         if (t < p.M) *reinterpret_cast<uint32_t*>(p.out + (int64_t)t * p.ldo + n_pair) = __byte_perm(word, other, sel);
                     } else if (valid_row) {
