@@ -11,7 +11,7 @@
 // What bounds it: 160 x 160 takes 60 MMAs of 128 x 160 x 16 a token and CTA (80 cycles each, 80 of the 128 rows in use); what the
 // ALU warps do with every value of Z and Y, in lock step and with five barriers a step, takes about twice that.  The warp-level
 // kernel needs 9600 cycles of its MMAs alone, with operands re-read from shared memory as fast as it delivers, and the barriers of
-// its one token stand open: 2048 tokens of 160 x 160 505 -> 231 us, 4096 of 64 x 80 77 -> 62 us.
+// its one token stand open: 2048 tokens of 160 x 160 505 -> 209 us, 4096 of 64 x 80 77 -> 60 us.
 // MMAs and the work around them run side by side, three steps deep:
 //   MMA thread    Z(0), Z(1), Y(0), Z(2), Y(1), ...    Z(i) and Y(i) share one of two accumulators
 //   16 ALU warps  step i: Y(i-1) to registers, its largest magnitude published  (accumulator free: Z(i+1) may start)
@@ -39,7 +39,10 @@ namespace bwla {
 
 namespace ru {
 constexpr int kAluWarps = 16;
-constexpr int kThreads = 128 + 32 * kAluWarps;
+constexpr int kThreads = 128 + 32 * kAluWarps;       // 640
+// registers: 96 a thread at launch (640 x 96 = 61440); 128 x 56 + 512 x 104 = 60416 after the split (without it the two-chain
+// variant keeps values in local memory: 2048 tokens of 160 x 160 236 -> 209 us)
+constexpr int kRegsControl = 56, kRegsAlu = 104;
 constexpr int kPrepHeader = 256;          // of the prepared factors (rot_mma.cu)
 constexpr int kMaxSmem = 232448;
 struct Shared {
@@ -118,6 +121,10 @@ struct RotUmmaParams {
 };
 
 namespace {
+template <int N>
+__device__ __forceinline__ void set_regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void set_regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 __device__ __forceinline__ void tmem_ld_32x8(uint32_t taddr, uint32_t* v) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
@@ -257,6 +264,8 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     // barrier and phase of step i's accumulator
     auto acc_of = [](int i) { return TWO ? 0 : i & 1; };
     auto phase_of = [](int i) { return (uint32_t)((TWO ? i : i >> 1) & 1); };
+    if (warp < 4) {
+    set_regs_dec<ru::kRegsControl>();
     if (warp == 0) {
         // ---------------- x ----------------
         if (elect_one()) {
@@ -348,7 +357,9 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             if (lane == 0) mbar_arrive(&sh.out_free[par]);
         }
         if (g.staged && lane == 0) bulk_wait_all();
-    } else if (warp >= 4) {
+    }
+    } else {
+        set_regs_inc<ru::kRegsAlu>();
         // ---------------- everything between and behind the MMAs ----------------
         // A warp issues an instruction about every six cycles here (four warps a scheduler), so instructions a value are what
         // counts: no scaling pass over Y (a row's power of two goes into the quantiser's factor), one read of Z, no
