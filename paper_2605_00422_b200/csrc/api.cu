@@ -524,6 +524,12 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         st = launch_gemm_small(ga, count, 1, &taken, s);
         if (taken) return st;
     }
+    // More than 64 tokens: the tiles of all linears are walked by one launch, so that a last wave is left half empty once instead of
+    // once a linear, and one set-up is paid (333 tokens of q/k/v, 4096 -> 3 x 4096: 96 tiles each for 148 SMs).
+    bool together = all_i8 && count > 1;
+    for (int i = 0; i < count; ++i)
+        together = together && umma_persistent_supports(M, layers[i]->K, layers[i]->N, layers[i]->r) && (layers[i]->r > 0) == (L0->r > 0);
+    if (together) return launch_gemm_umma_persistent(ga, count, s);
     // Several contractions that all go to the small-batch tcgen05 kernel run beside one another (GemmArgs::dep_mode); each
     // plans for its share of the SMs (by row tiles) when all of them fit the device at once
     const bool siblings = count > 1 && M <= 64 && all_i8;

@@ -268,6 +268,7 @@ bool umma_supports(int64_t M, int64_t K, int64_t N, int r, int bits);
 int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream);
 // More than 64 tokens: the same contraction in CTAs that stay on their SM and take tiles of 128 rows x 128 tokens in turn.
 bool umma_persistent_supports(int64_t M, int64_t K, int64_t N, int r);
-int launch_gemm_umma_persistent(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream);
+// n linears with the same M and K, all of them or none with a low-rank branch; codes in the interleaved order
+int launch_gemm_umma_persistent(const GemmArgs* a, int n, cudaStream_t stream);
 
 }  // namespace bwla

@@ -626,7 +626,11 @@ static int choose_wide_splits(int tiles, int units, int narrow_splits, int sms) 
 // codes_interleaved: int8 [M][K] in the interleaved order.  a.Thl: bf16 [3][M][64], T = hi + mid + lo.
 int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream) {
     const int M = (int)a.M, N = (int)a.N, K = (int)a.K;
-    if (umma_persistent_supports(a.M, a.K, a.N, a.r)) return launch_gemm_umma_persistent(a, codes_interleaved, stream);
+    if (umma_persistent_supports(a.M, a.K, a.N, a.r)) {
+        GemmArgs one = a;
+        one.codes = codes_interleaved;
+        return launch_gemm_umma_persistent(&one, 1, stream);
+    }
     if (M > 64) return BWLA_ERR_UNSUPPORTED;                  // (every such problem this path takes went to the persistent kernel)
     const int n_tok = M <= 16 ? 16 : M <= 32 ? 32 : 64;
     const int row_tiles = (N + kRowsPerCta - 1) / kRowsPerCta;

@@ -57,18 +57,24 @@ static_assert(A_COL + 32 * AS <= TMEM_COLS, "tensor memory");
 static_assert(total <= 232448, "shared memory");
 }  // namespace persist
 
-struct PersistParams {
-    int M, N, K;
-    int row_tiles, tok_tiles;
-    int r;
+// One linear of a launch (linears of a group have M, K and the presence of a low-rank branch in common).
+struct PersistProblem {
+    int N, row_tiles, r;
+    int fast;                    // no zero points, no row shift, no accumulators wanted, sums below 2^22: the short epilogue
     const float* scales; const int32_t* qsum; const int32_t* zp;
     const float* alpha; const float* mu; const int32_t* rowsum;
     const __nv_bfloat16* U;
     __nv_bfloat16* out; int64_t ldo;
     int32_t* acc_debug;
-    int fast;                    // no zero points, no row shift, no accumulators wanted, sums below 2^22: the short epilogue
+};
+struct PersistParams {
+    int M, K, tok_tiles, n;
+    int lowrank;
+    int tile_begin[kRotMaxProblems + 1];     // tiles of problem i: [tile_begin[i], tile_begin[i + 1])
+    PersistProblem prob[kRotMaxProblems];
     uint32_t* status;
 };
+struct PersistMaps { CUtensorMap w[kRotMaxProblems], b[kRotMaxProblems], t[kRotMaxProblems]; };
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     uint32_t r;
@@ -82,8 +88,7 @@ __device__ __forceinline__ uint4 lds_words(const uint8_t* p) {
 }
 
 __global__ void __launch_bounds__(persist::kThreads, 1)
-umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap b_map,
-                           const __grid_constant__ CUtensorMap t_map, PersistParams p) {
+umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps maps, const __grid_constant__ PersistParams p) {
     using namespace persist;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -114,7 +119,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     auto tok_corr = [&](int buf) { return reinterpret_cast<float*>(smem + tok_off + buf * 16 * kTok + 12 * kTok); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles = p.row_tiles * p.tok_tiles;
+    const int tiles = p.tile_begin[p.n];
     const int my_tiles = (int)blockIdx.x < tiles ? (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int units = (p.K + kUnitK - 1) / kUnitK;
     const int kblocks = p.K / kBlockK;
@@ -122,10 +127,17 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     // integers, the order does not matter), so that they do not all ask the same slices of the L2 at the same time.
     const int u0 = (int)(((int64_t)blockIdx.x * units) / gridDim.x);
     auto unit_at = [&](int j) { const int u = u0 + j; return u < units ? u : u - units; };
-    const bool lowrank = p.r > 0;
-    // tile i of this CTA: row tiles fastest, so that the CTAs working at the same time share a token tile's codes in the L2
-    auto tile_n0 = [&](int i) { return (((int)blockIdx.x + i * (int)gridDim.x) % p.row_tiles) * kRows; };
-    auto tile_t0 = [&](int i) { return (((int)blockIdx.x + i * (int)gridDim.x) / p.row_tiles) * kTok; };
+    const bool lowrank = p.lowrank != 0;
+    // tile i of this CTA: one problem after the other, row tiles fastest, so that the CTAs working at the same time share a token
+    // tile's codes in the L2
+    struct Tile { int pi, n0, t0; };
+    auto tile_at = [&](int i) -> Tile {
+        int g = (int)blockIdx.x + i * (int)gridDim.x, pi = 0;
+        while (pi + 1 < p.n && g >= p.tile_begin[pi + 1]) ++pi;
+        g -= p.tile_begin[pi];
+        const int rows = p.prob[pi].row_tiles;
+        return Tile{pi, (g % rows) * kRows, (g / rows) * kTok};
+    };
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
@@ -151,21 +163,22 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     if (warp == 0) {
         // ---------------- packed sign words (independent of the preceding kernel) ----------------
         if (elect_one()) {
-            tma_prefetch_desc(&w_map);
+            for (int i = 0; i < p.n; ++i) tma_prefetch_desc(&maps.w[i]);
             // one token tile: every word is read once; more: once per token tile, so they may stay
             const uint64_t stream_once = l2_policy_evict_first();
             const bool once = p.tok_tiles == 1;
             int ws = 0; uint32_t wph = 0;
             for (int i = 0; i < my_tiles && !*abort_flag; ++i) {
-                const int n0 = tile_n0(i);
+                const Tile at = tile_at(i);
+                const int n0 = at.n0;
                 for (int u = 0; u < units && !*abort_flag; ++u) {
                     if (!mbar_test_wait(&w_empty[ws], wph ^ 1)) {
                         griddep_wait();
                         if (!wait_or_abort(&w_empty[ws], wph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x110); break; }
                     }
                     mbar_expect_tx(&w_full[ws], w_bytes);
-                    if (once) tma_load_2d_hint(wbuf + ws * w_bytes, &w_map, unit_at(u) * (kUnitK / 32), n0, &w_full[ws], stream_once);
-                    else tma_load_2d(wbuf + ws * w_bytes, &w_map, unit_at(u) * (kUnitK / 32), n0, &w_full[ws]);
+                    if (once) tma_load_2d_hint(wbuf + ws * w_bytes, &maps.w[at.pi], unit_at(u) * (kUnitK / 32), n0, &w_full[ws], stream_once);
+                    else tma_load_2d(wbuf + ws * w_bytes, &maps.w[at.pi], unit_at(u) * (kUnitK / 32), n0, &w_full[ws]);
                     if (++ws == WS) { ws = 0; wph ^= 1; }
                 }
             }
@@ -175,8 +188,10 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         // ---------------- codes and T ----------------
         griddep_wait();
         if (lane == 0) {
-            tma_prefetch_desc(&b_map);
-            if (lowrank) tma_prefetch_desc(&t_map);
+            for (int i = 0; i < p.n; ++i) {
+                tma_prefetch_desc(&maps.b[i]);
+                if (lowrank) tma_prefetch_desc(&maps.t[i]);
+            }
             if (p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) *abort_flag = 1;   // the call already failed
         }
         __syncwarp();
@@ -184,12 +199,13 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             int bs = 0; uint32_t bph = 0;
             bool ok = true;
             for (int i = 0; i < my_tiles && ok && !*abort_flag; ++i) {
-                const int t0 = tile_t0(i);
+                const Tile at = tile_at(i);
+                const int t0 = at.t0;
                 int kb = u0 * (kUnitK / kBlockK);
                 for (int c = 0; c < kblocks; ++c) {
                     if (!wait_or_abort(&s_empty[bs], bph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x121); ok = false; break; }
                     mbar_expect_tx(&s_full[bs], b_bytes);
-                    tma_load_2d(bbuf + bs * b_bytes, &b_map, kb * kBlockK, t0, &s_full[bs]);
+                    tma_load_2d(bbuf + bs * b_bytes, &maps.b[at.pi], kb * kBlockK, t0, &s_full[bs]);
                     if (++bs == AS) { bs = 0; bph ^= 1; }
                     if (++kb == kblocks) kb = 0;
                 }
@@ -198,7 +214,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                     if (i >= 1 && !wait_or_abort(t_empty, (uint32_t)((i - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x122); ok = false; }
                     if (ok) {
                         mbar_expect_tx(t_full, 3 * b_bytes);
-                        for (int h = 0; h < 3; ++h) tma_load_3d(tbuf + h * b_bytes, &t_map, 0, t0, h, t_full);
+                        for (int h = 0; h < 3; ++h) tma_load_3d(tbuf + h * b_bytes, &maps.t[at.pi], 0, t0, h, t_full);
                     }
                 }
             }
@@ -209,21 +225,23 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         // codes of the tile) ----------------
         griddep_wait();
         for (int i = 0; i < my_tiles && !*abort_flag; ++i) {
-            const int t0 = tile_t0(i), buf = i & 1;
+            const Tile at = tile_at(i);
+            const PersistProblem& pr = p.prob[at.pi];
+            const int t0 = at.t0, buf = i & 1;
             if (i >= 2 && !warp_wait(&epi_done[buf], (uint32_t)(((i >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x120); break; }
             for (int j = lane; j < kTok; j += 32) {
                 const int t = t0 + j;
-                tok_scale(buf)[j] = t < p.M ? p.scales[t] : 0.f;
+                tok_scale(buf)[j] = t < p.M ? pr.scales[t] : 0.f;
                 int32_t qs = 0;
                 if (t < p.M) {
-                    const int4* parts = reinterpret_cast<const int4*>(p.qsum + (size_t)t * kQsumParts);
+                    const int4* parts = reinterpret_cast<const int4*>(pr.qsum + (size_t)t * kQsumParts);
                     const int4 a = parts[0], b = parts[1];
                     qs = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
                 }
                 tok_qsum(buf)[j] = qs;
-                const int32_t zp = (p.zp && t < p.M) ? p.zp[t] : 0;
+                const int32_t zp = (pr.zp && t < p.M) ? pr.zp[t] : 0;
                 tok_zp(buf)[j] = zp;
-                tok_corr(buf)[j] = p.fast ? __int_as_float(0x4B400000 - qs) : (float)(qs - p.K * zp);
+                tok_corr(buf)[j] = pr.fast ? __int_as_float(0x4B400000 - qs) : (float)(qs - p.K * zp);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&tok_full[buf]);
@@ -292,30 +310,32 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         bool ok = true;
         for (int i = 0; i < my_tiles; ++i) {
-            const int n0 = tile_n0(i), t0 = tile_t0(i), buf = i & 1;
+            const Tile at = tile_at(i);
+            const PersistProblem& pr = p.prob[at.pi];
+            const int n0 = at.n0, t0 = at.t0, buf = i & 1;
             const int n = n0 + e;
-            const bool valid_row = n < p.N;
-            const float alpha_n = valid_row ? __ldg(p.alpha + n) : 0.f;
-            const float mu_n = (p.mu && valid_row) ? __ldg(p.mu + n) : 0.f;
-            const int32_t rs_n = (p.zp && valid_row) ? __ldg(p.rowsum + n) : 0;
+            const bool valid_row = n < pr.N;
+            const float alpha_n = valid_row ? __ldg(pr.alpha + n) : 0.f;
+            const float mu_n = (pr.mu && valid_row) ? __ldg(pr.mu + n) : 0.f;
+            const int32_t rs_n = (pr.zp && valid_row) ? __ldg(pr.rowsum + n) : 0;
             if (lowrank) {
                 // this tile's rows of U: 128 rows x 8 chunks of 16 bytes, 128B-swizzled K-major, zero beyond N and r
                 if (ok && i >= 1 && !warp_wait(u_empty, (uint32_t)((i - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x140); ok = false; }
                 if (ok) {
-                    const bool vec = (p.r % 8 == 0) && ((reinterpret_cast<uintptr_t>(p.U) & 15) == 0);
+                    const bool vec = (pr.r % 8 == 0) && ((reinterpret_cast<uintptr_t>(pr.U) & 15) == 0);
 #pragma unroll
                     for (int it = 0; it < 4; ++it) {
                         const int idx = it * 256 + half * 128 + e;
                         const int ur = idx >> 3, ch = idx & 7;
                         uint4 v = make_uint4(0u, 0u, 0u, 0u);
                         const int un = n0 + ur;
-                        if (un < p.N && ch * 8 < p.r) {
-                            const __nv_bfloat16* src = p.U + (int64_t)un * p.r + ch * 8;
+                        if (un < pr.N && ch * 8 < pr.r) {
+                            const __nv_bfloat16* src = pr.U + (int64_t)un * pr.r + ch * 8;
                             if (vec) {
                                 v = __ldg(reinterpret_cast<const uint4*>(src));
                             } else {
                                 uint32_t w[4] = {0u, 0u, 0u, 0u};
-                                for (int c = 0; c < 8 && ch * 8 + c < p.r; ++c)
+                                for (int c = 0; c < 8 && ch * 8 + c < pr.r; ++c)
                                     w[c >> 1] |= (uint32_t)__bfloat16_as_ushort(src[c]) << (16 * (c & 1));
                                 v = make_uint4(w[0], w[1], w[2], w[3]);
                             }
@@ -343,17 +363,17 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 const int odd = lane & 1;
                 const uint32_t sel = odd ? 0x3276u : 0x5410u;
                 const int n_pair = n & ~1;
-                const bool pair_ok = ((reinterpret_cast<uintptr_t>(p.out) & 3) == 0) && (p.ldo & 1) == 0 && n_pair + 1 < p.N;
+                const bool pair_ok = ((reinterpret_cast<uintptr_t>(pr.out) & 3) == 0) && (pr.ldo & 1) == 0 && n_pair + 1 < pr.N;
                 const uint32_t acc_addr = tmem_base + lane_addr + D_COL + (uint32_t)(i & 1) * kTok;
                 auto put = [&](uint32_t word, int tok) {          // word: tokens tok (low half) and tok + 1 of this lane's row
                     const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 1);
                     if (pair_ok) {
                         const int t = t0 + tok + odd;
-                        if (t < p.M) *reinterpret_cast<uint32_t*>(p.out + (int64_t)t * p.ldo + n_pair) = __byte_perm(word, other, sel);
+                        if (t < p.M) *reinterpret_cast<uint32_t*>(pr.out + (int64_t)t * pr.ldo + n_pair) = __byte_perm(word, other, sel);
                     } else if (valid_row) {
 #pragma unroll
                         for (int h = 0; h < 2; ++h)
-                            if (t0 + tok + h < p.M) p.out[(int64_t)(t0 + tok + h) * p.ldo + n] = __ushort_as_bfloat16((unsigned short)(word >> (16 * h)));
+                            if (t0 + tok + h < p.M) pr.out[(int64_t)(t0 + tok + h) * pr.ldo + n] = __ushort_as_bfloat16((unsigned short)(word >> (16 * h)));
                     }
                 };
 #pragma unroll 1
@@ -369,7 +389,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                         if (lane == 0) mbar_arrive(acc_free);
                     }
                     if (t0 + 16 * c >= p.M) continue;            // warp-uniform; nothing of this chunk is stored
-                    if (p.fast) {
+                    if (pr.fast) {
                         // the raw sum is -2^7 times the sum over the set bits; 1.5 * 2^23 + integer (below 2^22) is a float by its
                         // bits, and taking 1.5 * 2^23 off again is exact
 #pragma unroll
@@ -396,10 +416,10 @@ umma_w1a_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
 #pragma unroll
                             for (int h = 0; h < 4; ++h) {
                                 const int32_t acc = -((int32_t)v[j + h] >> 6) - qss[h] - zps[h] * rs_n;
-                                if (p.acc_debug && valid_row && t0 + 16 * c + j + h < p.M) p.acc_debug[(int64_t)(t0 + 16 * c + j + h) * p.N + n] = acc;
+                                if (pr.acc_debug && valid_row && t0 + 16 * c + j + h < p.M) pr.acc_debug[(int64_t)(t0 + 16 * c + j + h) * pr.N + n] = acc;
                                 y[h] = fmaf(__fmul_rn(mu_n, scs[h]), cos[h], __fmul_rn(__fmul_rn(alpha_n, scs[h]), (float)acc) + (lowrank ? __uint_as_float(l[j + h]) : 0.f));
                             }
-                            if (p.out) {
+                            if (pr.out) {
                                 put(pack_bf16x2(y[0], y[1]), 16 * c + j);
                                 put(pack_bf16x2(y[2], y[3]), 16 * c + j + 2);
                             }
@@ -503,44 +523,52 @@ bool umma_persistent_supports(int64_t M, int64_t K, int64_t N, int r) {
     return M > 64 && K % 128 == 0 && r <= kLowrankPad && N > 0;
 }
 
-int launch_gemm_umma_persistent(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream) {
+int launch_gemm_umma_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
     using namespace persist;
-    const int M = (int)a.M, N = (int)a.N, K = (int)a.K;
+    if (n < 1 || n > kRotMaxProblems) return BWLA_ERR_INVALID_ARG;
+    const int M = (int)a[0].M, K = (int)a[0].K;
     const int sms = sm_count();
     if (sms <= 0) return BWLA_ERR_CUDA;
-    CUtensorMap wm, bm, tm;
-    {
-        const uint64_t dims[2] = {(uint64_t)K / 32, (uint64_t)N};
-        const uint64_t strides[1] = {(uint64_t)K / 8};
-        const uint32_t box[2] = {32, kRows};
-        int st = make_map(&wm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, a.packed, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-        if (st != BWLA_OK) return st;
-    }
-    {
-        const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
-        const uint64_t strides[1] = {(uint64_t)K};
-        const uint32_t box[2] = {kBlockK, kTok};
-        int st = make_map(&bm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, codes_interleaved, dims, strides, box,
-                          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-        if (st != BWLA_OK) return st;
-    }
-    if (a.r > 0) {
-        const uint64_t dims[3] = {(uint64_t)kLowrankPad, (uint64_t)M, 3};
-        const uint64_t strides[2] = {(uint64_t)kLowrankPad * 2, (uint64_t)M * kLowrankPad * 2};
-        const uint32_t box[3] = {(uint32_t)kLowrankPad, kTok, 1};
-        int st = make_map(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, a.Thl, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-        if (st != BWLA_OK) return st;
-    } else {
-        tm = bm;   // never dereferenced
-    }
+    PersistMaps maps;
     PersistParams p{};
-    p.M = M; p.N = N; p.K = K; p.row_tiles = (N + kRows - 1) / kRows; p.tok_tiles = (M + kTok - 1) / kTok; p.r = a.r;
-    p.scales = a.scales; p.qsum = a.qsum; p.zp = a.zp; p.alpha = a.alpha; p.mu = a.mu; p.rowsum = a.rowsum;
-    p.U = (const __nv_bfloat16*)a.U; p.out = (__nv_bfloat16*)a.out; p.ldo = a.ldo; p.acc_debug = a.acc_debug; p.status = a.status;
-    p.fast = !a.zp && !a.mu && !a.acc_debug && a.out && (int64_t)K << (a.bits - 1) < (int64_t)1 << 22;
-    const int tiles = p.row_tiles * p.tok_tiles;
+    p.M = M; p.K = K; p.tok_tiles = (M + kTok - 1) / kTok; p.n = n; p.lowrank = a[0].r > 0; p.status = a[0].status;
+    for (int i = 0; i < n; ++i) {
+        const GemmArgs& g = a[i];
+        const int N = (int)g.N;
+        {
+            const uint64_t dims[2] = {(uint64_t)K / 32, (uint64_t)N};
+            const uint64_t strides[1] = {(uint64_t)K / 8};
+            const uint32_t box[2] = {32, kRows};
+            int st = make_map(&maps.w[i], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, g.packed, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+            if (st != BWLA_OK) return st;
+        }
+        {
+            const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
+            const uint64_t strides[1] = {(uint64_t)K};
+            const uint32_t box[2] = {kBlockK, kTok};
+            int st = make_map(&maps.b[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, g.codes, dims, strides, box,
+                              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+            if (st != BWLA_OK) return st;
+        }
+        if (g.r > 0) {
+            const uint64_t dims[3] = {(uint64_t)kLowrankPad, (uint64_t)M, 3};
+            const uint64_t strides[2] = {(uint64_t)kLowrankPad * 2, (uint64_t)M * kLowrankPad * 2};
+            const uint32_t box[3] = {(uint32_t)kLowrankPad, kTok, 1};
+            int st = make_map(&maps.t[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, g.Thl, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+            if (st != BWLA_OK) return st;
+        } else {
+            maps.t[i] = maps.b[i];   // never dereferenced
+        }
+        PersistProblem& pr = p.prob[i];
+        pr.N = N; pr.row_tiles = (N + kRows - 1) / kRows; pr.r = g.r;
+        pr.scales = g.scales; pr.qsum = g.qsum; pr.zp = g.zp; pr.alpha = g.alpha; pr.mu = g.mu; pr.rowsum = g.rowsum;
+        pr.U = (const __nv_bfloat16*)g.U; pr.out = (__nv_bfloat16*)g.out; pr.ldo = g.ldo; pr.acc_debug = g.acc_debug;
+        pr.fast = !g.zp && !g.mu && !g.acc_debug && g.out && (int64_t)K << (g.bits - 1) < (int64_t)1 << 22;
+        p.tile_begin[i + 1] = p.tile_begin[i] + pr.row_tiles * p.tok_tiles;
+    }
+    for (int i = n; i < kRotMaxProblems; ++i) { maps.w[i] = maps.w[0]; maps.b[i] = maps.b[0]; maps.t[i] = maps.t[0]; p.tile_begin[i + 1] = p.tile_begin[n]; }
 
     static thread_local int configured = -1;
     int dev = 0;
@@ -550,7 +578,7 @@ int launch_gemm_umma_persistent(const GemmArgs& a, const int8_t* codes_interleav
         configured = dev;
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)std::min(tiles, sms), 1, 1);
+    cfg.gridDim = dim3((unsigned)std::min(p.tile_begin[n], sms), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = total;
     cfg.stream = stream;
@@ -560,7 +588,7 @@ int launch_gemm_umma_persistent(const GemmArgs& a, const int8_t* codes_interleav
     cfg.attrs = attrs;
     cfg.numAttrs = 1;
     ProfScope prof(kProfContraction, stream);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, umma_w1a_persistent_kernel, wm, bm, tm, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, umma_w1a_persistent_kernel, maps, p);
     if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e); }
     return after_launch();
 }
