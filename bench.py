@@ -10,7 +10,7 @@ larger than L2, so every step streams them from DRAM again).
 
 Prints ONE JSON line (rank 0).  `value` is the decode figure (algorithmic HBM bytes of the whole stack per second
 at --decode-m tokens); `prefill` holds the INT8 TOPS figure at --prefill-m tokens; `roofline` is for the dominant
-kernel (the tcgen05 contraction) timed with CUDA events around each of its launches.
+kernel (the contraction) timed with CUDA events around each of its launches.
 """
 from __future__ import annotations
 
@@ -60,7 +60,7 @@ def contraction_kernel_bytes(sh: gen.LinearShape, M: int) -> int:
 
 def kernel_source_hash() -> str:
     import hashlib
-    with open(os.path.join(ROOT, "paper_2605_00422_b200", "csrc", "gemm_umma.cu"), "rb") as f:
+    with open(os.path.join(ROOT, "paper_2605_00422_b200", "csrc", "gemm_small.cu"), "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()
 
 
@@ -544,7 +544,7 @@ def run_ours(args):
     k_ms, k_n = prof.get("contraction", (0.0, 0))
     k_bytes = args.layers * sum(contraction_kernel_bytes(sh, M) for sh in shapes)
     achieved = k_bytes / (k_ms * 1e-3) / 1e9 if k_ms > 0 else None
-    roofline = {"bound": "hbm", "kernel": "umma_w1a_kernel (tcgen05 kind::i8 contraction), decode stack",
+    roofline = {"bound": "hbm", "kernel": "gemm_small_kernel (mma.sync int8 contraction), decode stack",
                 "achieved": achieved, "peak": peaks["hbm_gbs"], "peak_source": peaks["source"], "unit": "GB/s",
                 "frac": (achieved / peaks["hbm_gbs"]) if achieved else None,
                 "traffic": measured_traffic("decode", k_bytes / k_n) if k_n else None,
