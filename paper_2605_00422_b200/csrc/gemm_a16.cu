@@ -5,6 +5,9 @@
 //   yhat = bf16(Y)                                      (rot_mma.cu; also sum_k yhat for the row-shift term)
 //   out[t][n] = bf16( alpha[n] * sum_k s[n][k] * yhat[t][k] + U[n,:] . T[t,:] + mu[n] * sum_k yhat[t][k] )
 //
+// This kernel serves K that is not a multiple of 128 (and more than 32 tokens); gemm_a16_persist.cu and the digits of gemm_small.cu
+// serve the rest.
+//
 // Tile of one CTA: 128 tokens (the accumulator's lanes) x 128 weight rows (its columns) x all of K.
 //   A operand: yhat, K-major, by TMA (64 values of k = one 128-byte swizzle atom per stage);
 //   B operand: the signs of 128 rows expanded to +-1 in bf16 by four warps (each owns one stage and takes every fourth
