@@ -67,14 +67,17 @@ struct PersistProblem {
     __nv_bfloat16* out; int64_t ldo;
     int32_t* acc_debug;
 };
+// NP: 1, or up to kRotMaxProblems (a lone linear launched with the parameters of four starts 1 us later)
+template <int NP>
 struct PersistParams {
     int M, K, tok_tiles, n;
     int lowrank;
-    int tile_begin[kRotMaxProblems + 1];     // tiles of problem i: [tile_begin[i], tile_begin[i + 1])
-    PersistProblem prob[kRotMaxProblems];
+    int tile_begin[NP + 1];     // tiles of problem i: [tile_begin[i], tile_begin[i + 1])
+    PersistProblem prob[NP];
     uint32_t* status;
 };
-struct PersistMaps { CUtensorMap w[kRotMaxProblems], b[kRotMaxProblems], t[kRotMaxProblems]; };
+template <int NP>
+struct PersistMaps { CUtensorMap w[NP], b[NP], t[NP]; };
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     uint32_t r;
@@ -87,8 +90,9 @@ __device__ __forceinline__ uint4 lds_words(const uint8_t* p) {
     return v;
 }
 
+template <int NP>
 __global__ void __launch_bounds__(persist::kThreads, 1)
-umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps maps, const __grid_constant__ PersistParams p) {
+umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const __grid_constant__ PersistParams<NP> p) {
     using namespace persist;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -133,7 +137,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps maps, const __gri
     struct Tile { int pi, n0, t0; };
     auto tile_at = [&](int i) -> Tile {
         int g = (int)blockIdx.x + i * (int)gridDim.x, pi = 0;
-        while (pi + 1 < p.n && g >= p.tile_begin[pi + 1]) ++pi;
+        if (NP > 1)
+            while (pi + 1 < p.n && g >= p.tile_begin[pi + 1]) ++pi;
         g -= p.tile_begin[pi];
         const int rows = p.prob[pi].row_tiles;
         return Tile{pi, (g % rows) * kRows, (g / rows) * kTok};
@@ -523,14 +528,14 @@ bool umma_persistent_supports(int64_t M, int64_t K, int64_t N, int r) {
     return M > 64 && K % 128 == 0 && r <= kLowrankPad && N > 0;
 }
 
-int launch_gemm_umma_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
+template <int NP>
+static int launch_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
     using namespace persist;
-    if (n < 1 || n > kRotMaxProblems) return BWLA_ERR_INVALID_ARG;
     const int M = (int)a[0].M, K = (int)a[0].K;
     const int sms = sm_count();
     if (sms <= 0) return BWLA_ERR_CUDA;
-    PersistMaps maps;
-    PersistParams p{};
+    PersistMaps<NP> maps;
+    PersistParams<NP> p{};
     p.M = M; p.K = K; p.tok_tiles = (M + kTok - 1) / kTok; p.n = n; p.lowrank = a[0].r > 0; p.status = a[0].status;
     for (int i = 0; i < n; ++i) {
         const GemmArgs& g = a[i];
@@ -568,13 +573,13 @@ int launch_gemm_umma_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
         pr.fast = !g.zp && !g.mu && !g.acc_debug && g.out && (int64_t)K << (g.bits - 1) < (int64_t)1 << 22;
         p.tile_begin[i + 1] = p.tile_begin[i] + pr.row_tiles * p.tok_tiles;
     }
-    for (int i = n; i < kRotMaxProblems; ++i) { maps.w[i] = maps.w[0]; maps.b[i] = maps.b[0]; maps.t[i] = maps.t[0]; p.tile_begin[i + 1] = p.tile_begin[n]; }
+    for (int i = n; i < NP; ++i) { maps.w[i] = maps.w[0]; maps.b[i] = maps.b[0]; maps.t[i] = maps.t[0]; p.tile_begin[i + 1] = p.tile_begin[n]; }
 
     static thread_local int configured = -1;
     int dev = 0;
     BWLA_CUDA_TRY(cudaGetDevice(&dev));
     if (configured != dev) {
-        BWLA_CUDA_TRY(cudaFuncSetAttribute(umma_w1a_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, total));
+        BWLA_CUDA_TRY(cudaFuncSetAttribute(umma_w1a_persistent_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, total));
         configured = dev;
     }
     cudaLaunchConfig_t cfg{};
@@ -588,9 +593,14 @@ int launch_gemm_umma_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
     cfg.attrs = attrs;
     cfg.numAttrs = 1;
     ProfScope prof(kProfContraction, stream);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, umma_w1a_persistent_kernel, maps, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, umma_w1a_persistent_kernel<NP>, maps, p);
     if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e); }
     return after_launch();
+}
+
+int launch_gemm_umma_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
+    if (n < 1 || n > kRotMaxProblems) return BWLA_ERR_INVALID_ARG;
+    return n == 1 ? launch_persistent<1>(a, n, stream) : launch_persistent<kRotMaxProblems>(a, n, stream);
 }
 
 }  // namespace bwla
