@@ -524,11 +524,16 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         st = launch_gemm_small(ga, count, 1, &taken, s);
         if (taken) return st;
     }
-    // More than 64 tokens: the tiles of all linears are walked by one launch, so that a last wave is left half empty once instead of
-    // once a linear, and one set-up is paid (333 tokens of q/k/v, 4096 -> 3 x 4096: 96 tiles each for 148 SMs).
+    // More than 64 tokens and few tiles: the tiles of all linears are walked by one launch, so that a last wave is left half empty
+    // once instead of once a linear, and one set-up is paid (333 tokens of 4096 -> 3 x 4096: 96 tiles each for 148 SMs; the block
+    // 250 -> 229 us).  A tile then costs 1 % more (it looks its linear up), which 24 waves of tiles make up for one set-up.
     bool together = all_i8 && count > 1;
-    for (int i = 0; i < count; ++i)
+    int64_t tiles_m = 0;
+    for (int i = 0; i < count; ++i) {
         together = together && umma_persistent_supports(M, layers[i]->K, layers[i]->N, layers[i]->r) && (layers[i]->r > 0) == (L0->r > 0);
+        tiles_m += (layers[i]->N + 127) / 128 * ((M + 127) / 128);
+    }
+    together = together && tiles_m <= 24 * (int64_t)sm_count();
     if (together) return launch_gemm_umma_persistent(ga, count, s);
     // Several contractions that all go to the small-batch tcgen05 kernel run beside one another (GemmArgs::dep_mode); each
     // plans for its share of the SMs (by row tiles) when all of them fit the device at once

@@ -70,7 +70,7 @@ struct PersistProblem {
 // NP: 1, or up to kRotMaxProblems (a lone linear launched with the parameters of four starts 1 us later)
 template <int NP>
 struct PersistParams {
-    int M, K, tok_tiles, n;
+    int M, K, tok_tiles;
     int lowrank;
     int tile_begin[NP + 1];     // tiles of problem i: [tile_begin[i], tile_begin[i + 1])
     PersistProblem prob[NP];
@@ -123,7 +123,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
     auto tok_corr = [&](int buf) { return reinterpret_cast<float*>(smem + tok_off + buf * 16 * kTok + 12 * kTok); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles = p.tile_begin[p.n];
+    const int tiles = p.tile_begin[NP];
     const int my_tiles = (int)blockIdx.x < tiles ? (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int units = (p.K + kUnitK - 1) / kUnitK;
     const int kblocks = p.K / kBlockK;
@@ -138,7 +138,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
     auto tile_at = [&](int i) -> Tile {
         int g = (int)blockIdx.x + i * (int)gridDim.x, pi = 0;
         if (NP > 1)
-            while (pi + 1 < p.n && g >= p.tile_begin[pi + 1]) ++pi;
+            while (pi + 1 < NP && g >= p.tile_begin[pi + 1]) ++pi;
         g -= p.tile_begin[pi];
         const int rows = p.prob[pi].row_tiles;
         return Tile{pi, (g % rows) * kRows, (g / rows) * kTok};
@@ -168,7 +168,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
     if (warp == 0) {
         // ---------------- packed sign words (independent of the preceding kernel) ----------------
         if (elect_one()) {
-            for (int i = 0; i < p.n; ++i) tma_prefetch_desc(&maps.w[i]);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) tma_prefetch_desc(&maps.w[i]);
             // one token tile: every word is read once; more: once per token tile, so they may stay
             const uint64_t stream_once = l2_policy_evict_first();
             const bool once = p.tok_tiles == 1;
@@ -193,7 +194,8 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
         // ---------------- codes and T ----------------
         griddep_wait();
         if (lane == 0) {
-            for (int i = 0; i < p.n; ++i) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
                 tma_prefetch_desc(&maps.b[i]);
                 if (lowrank) tma_prefetch_desc(&maps.t[i]);
             }
@@ -536,7 +538,7 @@ static int launch_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
     if (sms <= 0) return BWLA_ERR_CUDA;
     PersistMaps<NP> maps;
     PersistParams<NP> p{};
-    p.M = M; p.K = K; p.tok_tiles = (M + kTok - 1) / kTok; p.n = n; p.lowrank = a[0].r > 0; p.status = a[0].status;
+    p.M = M; p.K = K; p.tok_tiles = (M + kTok - 1) / kTok; p.lowrank = a[0].r > 0; p.status = a[0].status;
     for (int i = 0; i < n; ++i) {
         const GemmArgs& g = a[i];
         const int N = (int)g.N;
