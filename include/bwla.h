@@ -50,8 +50,8 @@ enum {
                                  shapes the other two do not take */
     BWLA_PATH_BITPLANE = 2,   /* up to four tokens: two's-complement bit-planes of the codes against the packed sign
                                  words with and + popc on the integer pipes; the weights are never expanded */
-    BWLA_PATH_I8 = 3          /* sign words expanded to int8 in tensor memory, tcgen05 kind::i8 with int32 accumulators
-                                 in tensor memory; needs K % 128 == 0 and r <= 64 */
+    BWLA_PATH_I8 = 3          /* sign words expanded to int8 for the int8 tensor cores, int32 accumulators: in registers
+                                 (mma.sync) up to 16 tokens, in tensor memory (tcgen05) above; K % 128 == 0, r <= 64 */
 };
 
 #define BWLA_DTYPE_F32 0
@@ -210,7 +210,7 @@ int bwla_layer_set_activation_quant(bwla_layer* layer, int mode);
  * a bf16 contraction on the tensor cores with fp32 accumulation (partial sums of 128 values of k are added in rounded
  * fp32).  The layer's activation bit width and quantiser mode are not used.
  *   x_bf16 device, bf16 [M][ldx], 16-byte aligned, ldx >= K and a multiple of 8; out_bf16 device, bf16 [M][ldo], ldo >= N
- *   workspace: 256-byte aligned device scratch of bwla_w1a16_workspace_bytes(layer, M) bytes (about 7 bytes per
+ *   workspace: 256-byte aligned device scratch of bwla_w1a16_workspace_bytes(layer, M) bytes (2 to 3 bytes per
  *     activation value); its first 256 bytes must be zero before the first call; bwla_check_status reads it.
  * Needs K % 64 == 0, r <= 64 and factor sizes the tensor-core rotation takes, else BWLA_ERR_UNSUPPORTED.  M == 0 is a
  * no-op.  Asynchronous on `stream`.
@@ -280,7 +280,7 @@ int bwla_force_path(int path);
 
 /* The same for the kernel that evaluates the online OKT + quantiser: BWLA_ROT_AUTO (per shape), BWLA_ROT_SIMT (the
  * kernel with fp32 FMA tiles, P1/P2 staged in shared memory and warp-shuffle reductions; takes every shape) or
- * BWLA_ROT_UMMA (the tcgen05 kernel; shapes it does not take still go to the other one). */
+ * BWLA_ROT_UMMA (the tensor-core kernels; shapes they do not take still go to the other one). */
 enum { BWLA_ROT_AUTO = 0, BWLA_ROT_SIMT = 1, BWLA_ROT_UMMA = 2 };
 int bwla_force_rotation(int which);
 
