@@ -244,7 +244,9 @@ static int lowrank_umma_parts(int64_t M, int64_t K) {
 }
 
 bool lowrank_umma_supports(int64_t M, int64_t K, int r) {
-    return M > 64 && r > 0 && r <= lru::kCols && lowrank_cols(r) == lru::kCols && K % lru::kBlockK == 0 && K >= lru::kBlockK;
+    // (from 50 tokens where the rotation of a token takes a cluster of three, 160 x 160: it goes to rot_umma.cu then, which has no
+    // blocks for T beside it)
+    return (M > 64 || (K > 128 * 128 && 3 * M > 148)) && r > 0 && r <= lru::kCols && lowrank_cols(r) == lru::kCols && K % lru::kBlockK == 0 && K >= lru::kBlockK;
 }
 
 size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r) {

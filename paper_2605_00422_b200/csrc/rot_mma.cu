@@ -969,8 +969,8 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
         }
     }
     for (int i = n_problems; i <= kRotMaxProblems; ++i) p.lr_begin[i] = lr_total;
-    if (lr_total == 0 && p.x_vec && rot_umma_supports(base, M, n_problems, problems))
-        return launch_rot_umma(base, x, M, ldx, bits, asym, n_problems, problems, status, stream);
+    if (lr_total == 0 && p.x_vec && rot_umma_supports(g, M, n_problems, problems))
+        return launch_rot_umma(g, x, M, ldx, bits, asym, n_problems, problems, status, stream);
     RotKernel k = problems[0].yhat ? pick_kernel<kRotBf16, false>(g) : problems[0].digits ? pick_kernel<kRotDigits, false>(g) : pick_kernel<kRotQuant, false>(g);
     return launch_rot_kernel(k, g, p, smem, lr_total, stream);
 }

@@ -684,8 +684,9 @@ static Kernel pick_rot_umma(const RotUmmaGeom& g) {
 }
 
 bool rot_umma_supports(const RotGeom& base, int64_t M, int n_problems, const RotProblem* problems) {
-    // More tokens than SMs: fewer are spread over warps and CTAs one by one (rot_mma.cu), which is the shorter way for one token.
-    if (M * n_problems <= sm_count()) return false;
+    // More CTAs than SMs: fewer tokens are spread over warps and CTAs one by one (rot_mma.cu), which is the shorter way for one token
+    // as long as every CTA has an SM of its own.
+    if (M * n_problems * base.dc <= sm_count()) return false;
     for (int i = 0; i < n_problems; ++i)
         if (problems[i].digits || problems[i].packed) return false;
     RotUmmaGeom u;

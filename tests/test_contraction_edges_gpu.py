@@ -37,7 +37,7 @@ def test_few_tokens_accumulate_exactly(M, K, N, bits):
 
 
 @pytest.mark.parametrize("K,N,n1,n2,r,M", [(1280, 200, 20, 64, 13, 17), (1024, 129, 32, 32, 0, 32), (1280, 129, 20, 64, 13, 33), (1152, 257, 18, 64, 0, 150),
-                                           (128, 19300, 8, 16, 4, 260)])
+                                           (128, 19300, 8, 16, 4, 260), (25600, 40, 160, 160, 13, 52)])
 def test_weight_only(K, N, n1, n2, r, M):
     from paper_2605_00422_b200 import bwla
     sh = gen.small_shape(K, N, n1, n2, r, shape_id=K + N + M)
