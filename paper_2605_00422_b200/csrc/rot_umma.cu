@@ -88,7 +88,7 @@ static bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) 
     u.np = u.tps == 1 ? (u.nc + 31) / 32 * 32 : u.nc;
     u.ntot = u.tps * u.np;
     u.two = g.n2 > 128 || u.nc > 128;
-    if (u.two && u.nc < 32) return false;                     // (a chain without a step)
+    if (u.two && (u.nc < 32 || g.n2 < 32)) return false;      // (one step of 16 values: the second chain of that contraction would have none)
     u.atoms2 = (g.n2 + 31) / 32; u.atoms1 = (u.nc + 31) / 32;
     for (u.dc = 1; u.dc <= 2; ++u.dc) {
         u.dt = u.dc == 1 ? g.n2 : (g.n2 / 2 + 15) / 16 * 16;

@@ -20,6 +20,7 @@ pytestmark = pytest.mark.gpu
     (1, 32, 597, True), (20, 32, 331, False), (32, 16, 150, True), (64, 80, 299, True), (64, 80, 299, False), (73, 64, 301, True),
     (86, 128, 149, True), (108, 128, 160, False), (128, 128, 151, True), (140, 96, 150, True), (64, 160, 153, False),
     (160, 160, 150, True), (160, 160, 150, False), (160, 160, 50, True), (160, 160, 61, False),
+    (160, 16, 150, True), (144, 16, 150, False), (132, 16, 160, True),      # two chains over a, a single step over b
 ])
 def test_edges(n1, n2, M, prepared):
     from paper_2605_00422_b200 import bwla
