@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "bwla.h"
+#include "host_plans.h"
 
 namespace bwla {
 
@@ -73,19 +74,11 @@ struct ProfScope {
 // workspace layout (byte offsets into the caller's scratch buffer; every section 256-byte aligned)
 // ---------------------------------------------------------------------------------------------
 constexpr int kStatusBytes = 256;        // word 0: status; words 1..: where a bounded wait gave up
-constexpr int kLowrankPad = 64;          // T is kept as bf16 [3][M][64] (T = hi + mid + lo), zero beyond r <= 64
-
 // The code sum of a token is kept as kQsumParts partial sums (one per CTA of the prologue cluster that quantised a slab
 // of the token; unused parts are zero): the consumer adds them, the producers need no exchange.
 constexpr int kQsumParts = 8;
 
-// With few tokens V is read by several blocks that each take a part of K; their partial sums of T meet in the workspace and
-// the last block to arrive adds them in a fixed order (counters: status words 4..11, one per tile of T).
-constexpr int kLrKSplitMax = 16;
-constexpr int kLrSplitTiles = 8;
-constexpr int kLrCounterWord = 4;
-
-__host__ __device__ inline int lowrank_cols(int r) { return r > kLowrankPad ? (r + 1) / 2 * 2 : kLowrankPad; }
+constexpr int kLrCounterWord = 4;        // first of the arrival counters of split tiles of T among the status words
 
 // T = V x for many tokens on the tensor cores (lowrank_umma.cu): whether it takes the problem, the bytes of partial sums
 // it needs in the workspace (0: none), and the launch for the problems of one group (all share x, M, K; every entry of
@@ -96,11 +89,10 @@ size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r);
 int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_problems, const OktLowrank* lowrank,
                         uint32_t* status, cudaStream_t stream);
 
-// Bytes of partial sums of T: up to 64 tokens fp32 [tiles][parts][tile], beyond that what the tcgen05 kernel leaves.
+// Bytes of partial sums of T, whichever kernel leaves them.
 inline size_t lowrank_part_bytes(int64_t M, int64_t K, int r) {
     if (r <= 0) return 0;
-    const size_t few = M <= 64 ? (size_t)((M + 15) / 16) * kLrKSplitMax * 16 * (size_t)lowrank_cols(r) * 4 : 0;
-    return align_up(std::max(few, lowrank_umma_part_bytes(M, K, r)), 256);
+    return align_up(std::max(lowrank_split_bytes(M, lowrank_cols(r)), lowrank_umma_part_bytes(M, K, r)), 256);
 }
 
 struct Workspace {

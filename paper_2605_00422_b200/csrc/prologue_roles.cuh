@@ -427,19 +427,14 @@ inline int plan_lowrank(PrologueParams& p, float* lr_part, uint32_t* lr_count, i
     const bool rows16 = ((reinterpret_cast<uintptr_t>(p.x) | reinterpret_cast<uintptr_t>(p.V)) & 15) == 0 && p.ldx % 8 == 0 &&
                         K % 32 == 0 && p.lr_cols % 8 == 0;
     // (the wide tiles read x once but need enough token tiles to fill the device: 16 tokens x 64 columns per block)
-    p.lr_wide = rows16 ? ((M >= 1024 && p.lr_cols == 64) ? 3 : M > 32 ? 4 : 2) : ((M >= 64 && p.lr_cols % 8 == 0) ? 1 : 0);
-    const int cols = p.lr_wide == 4 ? 32 : 16;                // of one lr_wide 2 / 4 block
-    const int64_t tiles = ((p.lr_cols + cols - 1) / cols) * ((M + 15) / 16);
+    p.lr_wide = rows16 ? ((M >= 1024 && p.lr_cols == 64) ? 3 : lowrank_tile_cols(M) == 32 ? 4 : 2) : ((M >= 64 && p.lr_cols % 8 == 0) ? 1 : 0);
+    const int cols = lowrank_tile_cols(M);                    // of one lr_wide 2 / 4 block
     int blocks = p.lr_wide == 1 ? (p.lr_cols / 8) * (int)((M + 7) / 8)
-               : p.lr_wide == 2 || p.lr_wide == 4 ? (int)tiles
+               : p.lr_wide == 2 || p.lr_wide == 4 ? (int)lowrank_tiles(M, p.lr_cols)
                : p.lr_wide == 3 ? (int)((M + 15) / 16) : (p.lr_cols / 2) * (int)((M + 15) / 16);
-    // A block of few tokens that read all of V alone would stream it (cold: from HBM) through one SM and become the longest
-    // part of the launch; instead K is split so that a warp has about as many chunks as it can request at once.  There are as
-    // many arrival counters as eight tiles need (64 tokens of up to 64 columns).
     p.lr_ks = 1; p.lr_part = lr_part; p.lr_count = lr_count;
-    const int per = warps * (p.lr_wide == 4 ? 2 : 4);         // chunks a block has in registers at once
-    if ((p.lr_wide == 2 || p.lr_wide == 4) && tiles <= kLrSplitTiles && lr_part && lr_count) {
-        p.lr_ks = (int)std::min<int64_t>(kLrKSplitMax, std::max(1, (K / 32 + per / 2) / per));
+    if ((p.lr_wide == 2 || p.lr_wide == 4) && lr_part && lr_count) {
+        p.lr_ks = lowrank_ksplit(M, K, p.lr_cols, warps);
         blocks *= p.lr_ks;
     }
     // shared memory of a low-rank block: per-warp partial sums, and its rows of V when those are staged (few tokens)

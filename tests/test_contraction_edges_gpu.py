@@ -77,3 +77,11 @@ def test_a_group_equals_its_linears(M, r, asym):
         else:
             a, b = out.double(), alone.double()
             assert torch.all((a - b).abs() <= 2.0 ** -7 * a.abs() + 1e-4 * a.abs().max())
+
+
+@pytest.mark.parametrize("r,M", [(72, 5), (120, 16), (65, 1)])
+def test_ranks_above_64_whose_columns_do_not_fill_a_tile(r, M):
+    """16 x 256: two warps a CTA, so K is split sixteen ways; the partial sums of the last tile of columns lie in front of the codes."""
+    from paper_2605_00422_b200 import bwla
+    from tests.test_parity_gpu import _run_layer_case
+    _run_layer_case(bwla, 0, gen.small_shape(4096, 40, 16, 256, r, shape_id=r), M, 6)

@@ -1,0 +1,40 @@
+"""Sizes and splits the host decides (csrc/host_plans.h), walked over every size the entry points accept: no GPU.
+
+The header is compiled with g++ into a small program per property; a line of its output is a violation."""
+import os
+import subprocess
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def violations(tmp_path, body: str) -> str:
+    src, exe = tmp_path / "walk.cpp", tmp_path / "walk"
+    src.write_text('#include "host_plans.h"\n#include <cstdio>\nusing namespace bwla;\nint main() {\n' + body + "\n}\n")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2605_00422_b200", "csrc"), "-o", str(exe), str(src)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout[:2000]
+
+
+def test_partial_sums_of_the_low_rank_term_fit_their_section(tmp_path):
+    """What the blocks that split K write ([tile][part][16][columns], whole tiles) against what the workspace holds for it; ranks
+    above 64 whose padded columns do not fill the last tile are the narrow case."""
+    assert violations(tmp_path, """
+    for (int r = 1; r <= 256; ++r)
+        for (int M = 1; M <= 80; ++M)
+            for (int K = 32; K <= 25600; K += 32)
+                for (int warps = 1; warps <= 16; ++warps) {
+                    const int cols = lowrank_cols(r), ks = lowrank_ksplit(M, K, cols, warps);
+                    const size_t wrote = ks > 1 ? (size_t)lowrank_tiles(M, cols) * ks * 16 * lowrank_tile_cols(M) * 4 : 0;
+                    if (wrote > lowrank_split_bytes(M, cols)) { std::printf("r %d M %d K %d warps %d\\n", r, M, K, warps); return 0; }
+                }""") == ""
+
+
+def test_the_workspace_has_that_room(tmp_path):
+    from paper_2605_00422_b200 import bwla
+    rows = violations(tmp_path, """
+    for (int r : {64, 65, 72, 88, 104, 120, 128, 136, 256})
+        for (int M : {1, 8, 16, 17, 32, 33, 64}) std::printf("%d %d %zu\\n", r, M, lowrank_split_bytes(M, lowrank_cols(r)));""")
+    for line in rows.splitlines():
+        r, M, need = map(int, line.split())
+        off_T, n_T = bwla.bwla_workspace_section(M, 4096, 64, r, 6, bwla.BWLA_WS_T)
+        off_codes, _ = bwla.bwla_workspace_section(M, 4096, 64, r, 6, bwla.BWLA_WS_CODES)
+        assert off_codes - (off_T + n_T) >= need, f"r {r}, {M} tokens"
