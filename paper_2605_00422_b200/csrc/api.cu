@@ -222,7 +222,7 @@ int bwla_w1ax_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, cons
         // layer has that done once)
         RotProblem pr{};
         pr.P1 = P1; pr.P2 = P2; pr.codes = codes; pr.codes_layout = path == BWLA_PATH_I8 ? 1 : 0; pr.scales = scales; pr.qsum = qsum;
-        OktLowrank lr{V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status) + kLrCounterWord};
+        OktLowrank lr{V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status) + kLrCounterWord, (float*)codes};
         st = launch_rot(geom, x_bf16, M, ldx, bits, 0, 1, &pr, &lr, (uint32_t*)(base + ws.status), s);
     } else {
         st = launch_prologue(x_bf16, M, K, ldx, P1, n1, P2, n2, bits, codes, path == BWLA_PATH_I8 ? 1 : 0, scales, qsum,
@@ -367,19 +367,17 @@ int bwla_layer_rotate_quant(const bwla_layer* L, const void* x_bf16, int64_t M, 
                            nullptr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
-// Up to how many tokens the weight-only operating point runs on three int8 digits per value (gemm_small.cu)
-constexpr int kDigitTokens = 32;
 struct A16Workspace { size_t status, yhat, ysum, scales, T, lr_part, total; };
 static A16Workspace a16_layout(const bwla_layer* L, int64_t M) {
     A16Workspace w{};
     size_t off = 0;
     w.status = off; off += kStatusBytes;
-    w.yhat = off;   off += align_up((size_t)M * (size_t)L->K * (M <= kDigitTokens ? 3 : 2), 256);       // bf16, or three digits
-    w.ysum = off;   off += align_up((size_t)M * (M <= kDigitTokens ? 3 * kQsumParts * 4 : 4), 256);      // sums of either
+    w.yhat = off;   off += align_up(a16_value_bytes(M, L->K), 256);          // (first the partial sums of T from lowrank_umma.cu)
+    w.ysum = off;   off += align_up(a16_sum_bytes(M), 256);
     w.scales = off; off += align_up((size_t)M * 4, 256);
     const size_t lr_cols = (size_t)lowrank_cols(L->r);
     w.T = off;      off += align_up((size_t)M * lr_cols * 6, 256);
-    w.lr_part = off; off += lowrank_part_bytes(M, L->K, L->r);
+    w.lr_part = off; off += L->r > 0 ? lowrank_split_bytes(M, lowrank_cols(L->r)) : 0;
     w.total = off;
     return w;
 }
@@ -403,7 +401,7 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
     const A16Workspace w = a16_layout(L, M);
     char* base = (char*)workspace;
     uint32_t* status = (uint32_t*)(base + w.status);
-    OktLowrank lr{L->V, L->r, base + w.T, L->r > 0 ? (float*)(base + w.lr_part) : nullptr, status + kLrCounterWord};
+    OktLowrank lr{L->V, L->r, base + w.T, L->r > 0 ? (float*)(base + w.lr_part) : nullptr, status + kLrCounterWord, (float*)(base + w.yhat)};
     if (M <= kDigitTokens) {
         GemmArgs g{};
         g.codes = (const int8_t*)(base + w.yhat); g.scales = (const float*)(base + w.scales); g.qsum = (const int32_t*)(base + w.ysum);
@@ -491,7 +489,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
             pr[i].zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr;
             pr[i].scales = (float*)(wbase[i] + ws[i].scales); pr[i].qsum = (int32_t*)(wbase[i] + ws[i].qsum);
             lr[i] = OktLowrank{L->V, L->r, wbase[i] + ws[i].T, L->r > 0 ? (float*)(wbase[i] + ws[i].lr_part) : nullptr,
-                               status + 8 * i + kLrCounterWord};
+                               status + 8 * i + kLrCounterWord, (float*)(wbase[i] + ws[i].codes)};
         }
         st = launch_rot(L0->geom, x_bf16, M, ldx, L0->bits, L0->asym, count, pr, lr, status, s);
         if (st != BWLA_OK) return st;

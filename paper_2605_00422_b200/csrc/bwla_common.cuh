@@ -74,26 +74,16 @@ struct ProfScope {
 // workspace layout (byte offsets into the caller's scratch buffer; every section 256-byte aligned)
 // ---------------------------------------------------------------------------------------------
 constexpr int kStatusBytes = 256;        // word 0: status; words 1..: where a bounded wait gave up
-// The code sum of a token is kept as kQsumParts partial sums (one per CTA of the prologue cluster that quantised a slab
+// The code sum of a token is kept as kQsumParts partial sums (host_plans.h; one per CTA of the prologue cluster that quantised a slab
 // of the token; unused parts are zero): the consumer adds them, the producers need no exchange.
-constexpr int kQsumParts = 8;
 
 constexpr int kLrCounterWord = 4;        // first of the arrival counters of split tiles of T among the status words
 
-// T = V x for many tokens on the tensor cores (lowrank_umma.cu): whether it takes the problem, the bytes of partial sums
-// it needs in the workspace (0: none), and the launch for the problems of one group (all share x, M, K; every entry of
-// `lowrank` has V, Thl and, where partial sums are needed, lr_part set).
+// T = V x for many tokens on the tensor cores (lowrank_umma.cu), for the problems of one group (all share x, M, K; every entry of
+// `lowrank` has V, Thl and, where partial sums are needed, umma_part set).
 struct OktLowrank;
-bool lowrank_umma_supports(int64_t M, int64_t K, int r);
-size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r);
 int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_problems, const OktLowrank* lowrank,
                         uint32_t* status, cudaStream_t stream);
-
-// Bytes of partial sums of T, whichever kernel leaves them.
-inline size_t lowrank_part_bytes(int64_t M, int64_t K, int r) {
-    if (r <= 0) return 0;
-    return align_up(std::max(lowrank_split_bytes(M, lowrank_cols(r)), lowrank_umma_part_bytes(M, K, r)), 256);
-}
 
 struct Workspace {
     size_t status, scales, zp, qsum, T, lr_part, codes, total;
@@ -108,8 +98,9 @@ inline Workspace workspace_layout(int64_t M, int64_t K, int64_t N, int r, int bi
     w.qsum = off;   off += align_up((size_t)M * 4 * kQsumParts, 256);
     const size_t lr_cols = (size_t)lowrank_cols(r);
     w.T = off;      off += align_up((size_t)M * lr_cols * 6, 256);     // bf16 [3][M][cols]
-    w.lr_part = off; off += lowrank_part_bytes(M, K, r);
-    w.codes = off;  off += align_up((size_t)M * (size_t)K, 256);
+    w.lr_part = off; off += r > 0 ? lowrank_split_bytes(M, lowrank_cols(r)) : 0;
+    // (the tcgen05 kernel for T leaves its partial sums where the rotation behind it puts the codes)
+    w.codes = off;  off += align_up(std::max((size_t)M * (size_t)K, lowrank_umma_part_bytes(M, K, r)), 256);
     (void)N; (void)bits;
     w.total = off;
     return w;
@@ -175,7 +166,8 @@ struct RotProblem {
     // final binarisation
     uint32_t* packed; float *alpha, *mu;
 };
-struct OktLowrank { const void* V; int r; void* Thl; float* lr_part; uint32_t* lr_count; };   // V == NULL: no T = V x blocks
+// V == NULL: no T = V x.  lr_part, lr_count: of the blocks beside the rotation; umma_part: of lowrank_umma.cu, may overlap the codes.
+struct OktLowrank { const void* V; int r; void* Thl; float* lr_part; uint32_t* lr_count; float* umma_part; };
 // false when the factor sizes are outside what the kernel takes (n2 a multiple of 8 up to 256, n1 up to 192)
 bool rot_geometry(int n1, int n2, RotGeom* out);
 // rows of x that start on 16 bytes (others are read element by element, and the tcgen05 V x kernel does not take them)

@@ -26,9 +26,8 @@
 namespace bwla {
 
 namespace lru {
-constexpr int kTok = 128;                 // tokens per tile
-constexpr int kCols = 64;                 // columns of T (r padded)
-constexpr int kBlockK = 64;               // values of k per stage: one 128-byte swizzle atom of bf16
+constexpr int kTok = kLruTok, kCols = kLruCols;      // tokens per tile, columns of T (r padded)
+constexpr int kBlockK = kLruBlockK;       // values of k per stage: one 128-byte swizzle atom of bf16
 constexpr int kFlushBlocks = 2;           // stages per accumulator: 128 values of k
 constexpr int kStages = 4;
 constexpr int kThreads = 192;
@@ -36,8 +35,6 @@ constexpr int x_bytes = kTok * kBlockK * 2, v_bytes = kCols * kBlockK * 2, stage
 constexpr int bars_off = kStages * stage_bytes;
 constexpr int smem_bytes = bars_off + 256 + 1024;
 constexpr int kTmemCols = 2 * kCols;
-constexpr int kMaxParts = 16;             // parts of K per token tile
-constexpr int kTargetCtas = 160;          // parts are chosen so that tiles x parts comes near this
 }  // namespace lru
 
 struct LrUmmaParams {
@@ -234,29 +231,6 @@ __global__ void __launch_bounds__(lru::kTok) lowrank_reduce_kernel(const LrUmmaP
 // ---------------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------------
-// Parts of K for M tokens: enough CTAs to fill the device while every part keeps at least eight stages.
-static int lowrank_umma_parts(int64_t M, int64_t K) {
-    const int64_t tiles = (M + lru::kTok - 1) / lru::kTok;
-    int64_t ks = std::max<int64_t>(1, lru::kTargetCtas / tiles);
-    ks = std::min<int64_t>(ks, lru::kMaxParts);
-    ks = std::min<int64_t>(ks, std::max<int64_t>(1, K / (8 * lru::kBlockK)));
-    return (int)ks;
-}
-
-bool lowrank_umma_supports(int64_t M, int64_t K, int r) {
-    // (from 50 tokens where the rotation of a token takes a cluster of three, 160 x 160: it goes to rot_umma.cu then, which has no
-    // blocks for T beside it)
-    return (M > 64 || (K > 128 * 128 && 3 * M > 148)) && r > 0 && r <= lru::kCols && lowrank_cols(r) == lru::kCols && K % lru::kBlockK == 0 && K >= lru::kBlockK;
-}
-
-size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r) {
-    if (!lowrank_umma_supports(M, K, r)) return 0;
-    const int ks = lowrank_umma_parts(M, K);
-    if (ks == 1) return 0;
-    const int64_t tiles = (M + lru::kTok - 1) / lru::kTok;
-    return (size_t)tiles * ks * lru::kCols * lru::kTok * 4;
-}
-
 int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_problems, const OktLowrank* lowrank,
                         uint32_t* status, cudaStream_t stream) {
     using namespace lru;
@@ -275,14 +249,14 @@ int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_
         if (st != BWLA_OK) return st;
     }
     for (int i = 0; i < n_problems; ++i) {
-        if (!lowrank[i].V || !lowrank[i].Thl || (p.ks > 1 && !lowrank[i].lr_part)) return BWLA_ERR_INVALID_ARG;
+        if (!lowrank[i].V || !lowrank[i].Thl || (p.ks > 1 && !lowrank[i].umma_part)) return BWLA_ERR_INVALID_ARG;
         const uint64_t dims[2] = {(uint64_t)K, (uint64_t)lowrank[i].r};       // rows beyond r read as zero
         const uint64_t strides[1] = {(uint64_t)K * 2};
         const uint32_t box[2] = {kBlockK, kCols};
         int st = make_map(&maps.v[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lowrank[i].V, dims, strides, box,
                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
         if (st != BWLA_OK) return st;
-        p.part[i] = lowrank[i].lr_part;
+        p.part[i] = lowrank[i].umma_part;
         p.Thl[i] = (__nv_bfloat16*)lowrank[i].Thl;
     }
     static thread_local int configured_device = -1;

@@ -935,7 +935,7 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
         for (int i = 0; i < n_problems; ++i)
             if (lowrank[i].V && lowrank[i].r > 0 && lowrank[i].Thl && lowrank_umma_supports(M, g.K, lowrank[i].r) && p.x_vec &&
                 (reinterpret_cast<uintptr_t>(lowrank[i].V) & 15) == 0 &&
-                (lowrank[i].lr_part || lowrank_umma_part_bytes(M, g.K, lowrank[i].r) == 0)) {
+                (lowrank[i].umma_part || lowrank_umma_part_bytes(M, g.K, lowrank[i].r) == 0)) {
                 batch[nb++] = lowrank[i];
                 lr_done[i] = true;
             }

@@ -85,3 +85,15 @@ def test_ranks_above_64_whose_columns_do_not_fill_a_tile(r, M):
     from paper_2605_00422_b200 import bwla
     from tests.test_parity_gpu import _run_layer_case
     _run_layer_case(bwla, 0, gen.small_shape(4096, 40, 16, 256, r, shape_id=r), M, 6)
+
+
+def test_one_weight_only_workspace_serves_smaller_batches():
+    from paper_2605_00422_b200 import bwla
+    sh = gen.small_shape(1024, 64, 32, 32, 16, shape_id=9)
+    dl = H.DeviceLayer(gen.make_layer(0, sh, 8), bwla)
+    layer = bwla.Layer(dl.P1, dl.P2, 8, dl.packed, dl.alpha, dl.U, dl.V)
+    sizes = [bwla.bwla_w1a16_workspace_bytes(layer, M) for M in range(1, 200)]
+    assert sizes == sorted(sizes)
+    ws = torch.zeros(bwla.bwla_w1a16_workspace_bytes(layer, 40), dtype=torch.uint8, device="cuda")
+    bwla.bwla_layer_w1a16_linear(layer, H.bf16_to_dev(gen.make_activations(0, sh, 32)), workspace=ws)
+    assert bwla.bwla_check_status(ws) == 0

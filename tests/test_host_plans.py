@@ -38,3 +38,46 @@ def test_the_workspace_has_that_room(tmp_path):
         off_T, n_T = bwla.bwla_workspace_section(M, 4096, 64, r, 6, bwla.BWLA_WS_T)
         off_codes, _ = bwla.bwla_workspace_section(M, 4096, 64, r, 6, bwla.BWLA_WS_CODES)
         assert off_codes - (off_T + n_T) >= need, f"r {r}, {M} tokens"
+
+
+SIZES = (32, 128, 512, 1152, 4096, 5120, 8192, 11008, 13824, 16384, 16416, 20480, 25600)
+RANKS = (0, 1, 32, 64, 65, 72, 128, 256)
+
+
+def test_a_workspace_for_many_tokens_serves_fewer():
+    """A program that allocates for its largest batch calls with every smaller one."""
+    from paper_2605_00422_b200 import bwla
+    for K in SIZES:
+        for r in RANKS:
+            sizes = [bwla.bwla_workspace_bytes(M, K, 4096, r, 6) for M in range(1, 700)]
+            drops = [M for M, (a, b) in enumerate(zip(sizes, sizes[1:]), 2) if b < a]
+            assert not drops, f"K {K}, rank {r}: {drops[:5]} tokens need less than one token fewer"
+
+
+def test_a_weight_only_workspace_for_many_tokens_serves_fewer(tmp_path):
+    assert violations(tmp_path, """
+    for (long K = 64; K <= 25600; K += 64)
+        for (long M = 1; M <= 200; ++M)
+            if (a16_value_bytes(M + 1, K) < a16_value_bytes(M, K) || a16_sum_bytes(M + 1) < a16_sum_bytes(M) || a16_value_bytes(M, K) < (size_t)(2 * M * K) ||
+                (M <= kDigitTokens && (a16_value_bytes(M, K) < (size_t)(3 * M * K) || a16_sum_bytes(M) < (size_t)(96 * M)))) { std::printf("%ld tokens, K %ld\\n", M, K); return 0; }""") == ""
+
+
+def test_problems_of_the_built_in_scratch():
+    """bwla_w1ax_linear_static: 4 MiB hold the codes and at most 688 KiB of everything that does not grow with the tokens."""
+    from paper_2605_00422_b200 import bwla
+    for M, K in ((64, 25600), (134, 25600), (167, 20480), (246, 13824), (512, 5120)):
+        for r in (0, 16, 64):
+            assert bwla.bwla_workspace_bytes(M, K, 4096, r, 6) <= bwla.BWLA_STATIC_SCRATCH_BYTES, (M, K, r)
+    for K in SIZES:
+        for r in RANKS:
+            for M in range(1, 256):
+                per_token = K + 40 + 6 * max(64, r + r % 2)
+                assert bwla.bwla_workspace_bytes(M, K, 4096, r, 6) <= M * per_token + 688 * 1024 + 256 * 6, (M, K, r)
+
+
+def test_partial_sums_of_many_tokens_fit_where_the_codes_go(tmp_path):
+    assert violations(tmp_path, """
+    for (int r : {1, 64})
+        for (long M = 1; M <= 5000; ++M)
+            for (long K = 64; K <= 25600; K += 64)
+                if (lowrank_umma_part_bytes(M, K, r) > (size_t)(M * K)) { std::printf("%ld tokens, K %ld\\n", M, K); return 0; }""") == ""
