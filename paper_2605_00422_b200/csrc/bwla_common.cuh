@@ -130,22 +130,7 @@ int launch_prologue(const void* x, int64_t M, int64_t K, int64_t ldx, const floa
                     int bits, int8_t* codes, int codes_layout, float* scales, int32_t* qsum, const void* V, int r,
                     void* Thl, float* lr_part, uint32_t* status, cudaStream_t stream);
 
-// ---- rotation + quantiser on the warp-level tensor-core path (rot_mma.cu) ----
-// Geometry of the kernel for one pair of Kronecker factor sizes; computed on the host, passed to the kernels by value.
-struct RotGeom {
-    int n1, n2, K;
-    int n2p;                // n2 rounded up to 16
-    int na;                 // 8-column tiles of a and c: n1 rounded up to 16, in eighths
-    int cw, ntw;            // warps the column tiles are dealt to (1, 2 or 4), tiles per warp
-    int dtc, dc;            // 16-row tiles of d per CTA, CTAs per token (cluster size, up to 8)
-    int warps;              // warps of one token in a CTA: a group
-    int max_groups;         // groups a CTA can hold
-    int s2, s1;             // bytes per row of operands contracted over b / over a
-    int p1_off, group_off, group_bytes;     // shared memory: P2^T terms at 0, P1^T terms, then per group
-    int z_rel, red_rel;                     // ... x at 0, Z^T, RotShared
-    int alias_z;            // Z^T takes the place of x
-    int pad;                // bytes added to every row against bank conflicts
-};
+// ---- rotation + quantiser on the warp-level tensor-core path (rot_mma.cu; its geometry: host_plans.h) ----
 constexpr int kRotMaxProblems = 4;          // linears that share one x and are rotated by one launch
 struct RotProblem {
     const uint8_t* prepared;    // terms of P2^T and P1^T (launch_prepare_rot), or NULL: P1 and P2 are split by every CTA
@@ -168,11 +153,8 @@ struct RotProblem {
 };
 // V == NULL: no T = V x.  lr_part, lr_count: of the blocks beside the rotation; umma_part: of lowrank_umma.cu, may overlap the codes.
 struct OktLowrank { const void* V; int r; void* Thl; float* lr_part; uint32_t* lr_count; float* umma_part; };
-// false when the factor sizes are outside what the kernel takes (n2 a multiple of 8 up to 256, n1 up to 192)
-bool rot_geometry(int n1, int n2, RotGeom* out);
 // rows of x that start on 16 bytes (others are read element by element, and the tcgen05 V x kernel does not take them)
 bool rot_accepts_x(const void* x, int64_t ldx);
-size_t rot_prepared_bytes(const RotGeom& g);
 int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void* prepared, cudaStream_t stream);
 // One launch for up to kRotMaxProblems linears that read the same x: rotation + quantiser for each, and the T = V x
 // blocks of those with a low-rank branch.

@@ -71,6 +71,146 @@ inline size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r) {
     return ks > 1 ? (size_t)lowrank_umma_tiles(M) * ks * kLruCols * kLruTok * 4 : 0;
 }
 
+// ---- rotation + quantiser on mma.sync (rot_mma.cu) ----
+constexpr int kRotMaxWarps = 16;          // per CTA
+constexpr int kRotMaxSmem = 232448 - 128; // the 227 KB a block may have, less the static shared memory of the roles
+constexpr int kRotHeader = 256;           // prepared factors: exponents, then the terms
+constexpr int kRotRedBytes = 3072;        // per group: RotShared
+
+// Geometry of the kernel for one pair of Kronecker factor sizes; computed on the host, passed to the kernels by value.
+struct RotGeom {
+    int n1, n2, K;
+    int n2p;                // n2 rounded up to 16
+    int na;                 // 8-column tiles of a and c: n1 rounded up to 16, in eighths
+    int cw, ntw;            // warps the column tiles are dealt to (1, 2 or 4), tiles per warp
+    int dtc, dc;            // 16-row tiles of d per CTA, CTAs per token (cluster size, up to 8)
+    int warps;              // warps of one token in a CTA: a group
+    int max_groups;         // groups a CTA can hold
+    int s2, s1;             // bytes per row of operands contracted over b / over a
+    int p1_off, group_off, group_bytes;     // shared memory: P2^T terms at 0, P1^T terms, then per group
+    int z_rel, red_rel;                     // ... x at 0, Z^T, RotShared
+    int alias_z;            // Z^T takes the place of x
+    int pad;                // bytes added to every row against bank conflicts
+};
+inline int round_to(int v, int m) { return (v + m - 1) / m * m; }
+
+// A warp may have ntw column tiles at most; `alias`: Z^T takes the place of x, which is dead by then (the next token's x then
+// arrives late, which costs about a fifth).  Fills in what follows from dc and alias; false when it does not fit.
+inline bool rot_layout(RotGeom& g, int dc, int alias, int pad) {
+    const int tiles = g.n2p / 16;
+    g.dtc = (tiles + dc - 1) / dc;
+    g.warps = g.dtc * g.cw;
+    if (g.warps > kRotMaxWarps || (dc - 1) * g.dtc >= tiles || dc * g.warps > 64) return false;
+    // Rows of an odd number of 16-byte chunks (pad 16): the eight rows of an ldmatrix then fall into different banks.  The
+    // largest factors only fit without that padding, and without the rows of x beyond n1.
+    g.pad = pad;
+    g.s2 = g.n2p * 2 + pad; g.s1 = g.na * 16 + pad;
+    const int x = (pad ? g.cw * g.ntw * 8 : g.n1) * g.s2, z = g.cw > 1 ? 2 * g.dtc * 16 * g.s1 : 0;
+    g.dc = dc; g.alias_z = alias;
+    g.p1_off = 3 * g.dtc * 16 * g.s2;
+    g.group_off = g.p1_off + 2 * g.na * 8 * g.s1;
+    // (a warp's column tiles beyond n1 are read all the same and dropped: they must lie inside the block, 180 x 136)
+    g.group_bytes = std::max((alias ? std::max(x, z) : x + z) + kRotRedBytes, g.cw * g.ntw * 8 * g.s2);
+    g.z_rel = alias ? 0 : x; g.red_rel = g.group_bytes - kRotRedBytes;
+    if (g.group_off + g.group_bytes > kRotMaxSmem) return false;
+    g.max_groups = dc == 1 ? std::min(std::min(kRotMaxWarps / g.warps, 8), (kRotMaxSmem - g.group_off) / g.group_bytes) : 1;   // (barriers 1..8)
+    return true;
+}
+
+// Chooses the split of a token over warps and CTAs: the one that keeps most warps busy on an SM (16 is what the registers
+// allow), counting that the last CTA of a cluster may have fewer rows.
+inline bool rot_geometry(int n1, int n2, RotGeom* out) {
+    if (n1 < 1 || n2 < 8 || n2 % 8 != 0 || n2 > 256 || n1 > 192) return false;
+    RotGeom g{};
+    g.n1 = n1; g.n2 = n2; g.K = n1 * n2;
+    g.n2p = round_to(n2, 16); g.na = round_to(n1, 16) / 8;
+    g.cw = g.na <= 8 ? 1 : g.na <= 16 ? 2 : 4;
+    g.ntw = (g.na + g.cw - 1) / g.cw;                         // (the last warp may have tiles beyond na, which it ignores)
+    double best = 0.0;
+    for (int pad = 16; pad >= 0 && best == 0.0; pad -= 16)
+        for (int dc = 1; dc <= 8; ++dc)
+            for (int alias = 0; alias <= (g.cw > 1 ? 1 : 0); ++alias) {
+                RotGeom t = g;
+                if (!rot_layout(t, dc, alias, pad)) continue;
+                const int ctas = dc == 1 ? 1 : std::min(kRotMaxWarps / t.warps, (kRotMaxSmem + 1024) / (t.group_off + t.group_bytes + 1024));
+                const double score = (double)(g.n2p / 16) * g.cw / dc * t.max_groups * ctas * (alias ? 0.8 : 1.0);
+                if (score > best * 1.001) { best = score; *out = t; }
+            }
+    return best != 0.0;
+}
+
+// Few tokens: what counts is the time of one token, so it is spread over more warps (up to 64 columns: two warps instead of
+// one) and, while every cluster finds SMs of its own, over more CTAs: MMAs of a CTA at 2 cycles each, against about 5000
+// cycles for the cluster's barriers and its later start (64 x 128, one token: 6.7 us on eight CTAs, 5.2 on one).
+inline RotGeom few_tokens_geometry(const RotGeom& base, int64_t clusters, int sms) {
+    RotGeom best = base;
+    double best_cost = 0.0;
+    const int ksteps = base.n2p / 16 + base.na / 2;
+    for (int dc = 1; dc <= 8 && clusters * dc <= sms; ++dc) {
+        RotGeom t = base;
+        if (t.na > 4 && t.na <= 8) { t.cw = 2; t.ntw = 4; }
+        if (!rot_layout(t, dc, 0, base.pad) && (t.cw == 1 || !rot_layout(t, dc, 1, base.pad))) continue;
+        const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 5000.0 + 300.0 * dc : 0.0);
+        if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = t; }
+    }
+    return best;
+}
+
+inline size_t rot_prepared_bytes(const RotGeom& g) {
+    return kRotHeader + (size_t)3 * g.n2p * g.s2 + (size_t)2 * g.na * 8 * g.s1;
+}
+
+// ---- rotation of many tokens on tcgen05 (rot_umma.cu) ----
+constexpr int kRotUmmaSharedBytes = 1792;      // its barriers and small per-CTA state
+struct RotUmmaGeom {
+    int n1, n2, K;
+    int nc;                 // columns of a token's Y: n1 rounded up to 16
+    int np;                 // columns of a token in the accumulators
+    int tps, ntot;          // tokens of a step, tps * np
+    int dc, dt;             // CTAs of a token, rows d of each
+    int atoms2, atoms1;     // K atoms of 32 elements over b / over a
+    int xb;                 // buffers of x
+    int two;                // two chains of sums
+    int staged;             // outputs of a step go through shared memory (two buffers of out_bytes)
+    int out_bytes;
+    int p1_off, x_off, st_off, sh_off, total;
+    int s2, s1;             // row strides of the prepared factors
+};
+
+// False when the sizes are outside what the kernel takes: whole 16-byte pieces of the codes' order (n2 a multiple of 16), three
+// times n1 columns of tensor memory, at most 128 rows and the factors' terms in the shared memory of one CTA or of two.
+inline bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) {
+    if (g.n2 % 16 != 0 || g.n2 < 16 || g.n1 > 160) return false;
+    RotUmmaGeom u{};
+    u.n1 = g.n1; u.n2 = g.n2; u.K = g.K; u.s2 = g.s2; u.s1 = g.s1;
+    u.nc = g.na * 8;
+    u.tps = u.nc <= 32 ? 4 : u.nc <= 80 ? 2 : 1;
+    u.np = u.tps == 1 ? (u.nc + 31) / 32 * 32 : u.nc;
+    u.ntot = u.tps * u.np;
+    u.two = g.n2 > 128 || u.nc > 128;
+    if (u.two && (u.nc < 32 || g.n2 < 32)) return false;      // (one step of 16 values: the second chain of that contraction would have none)
+    u.atoms2 = (g.n2 + 31) / 32; u.atoms1 = (u.nc + 31) / 32;
+    for (u.dc = 1; u.dc <= 2; ++u.dc) {
+        u.dt = u.dc == 1 ? g.n2 : (g.n2 / 2 + 15) / 16 * 16;
+        if (u.dt > 128) continue;
+        // Outputs of whole tokens are contiguous: they are staged where two buffers fit, at the price of the second x if need
+        // be (stored from registers, a sector of 32 bytes is written in two or four pieces: 64 x 80, 4096 tokens 54 us).
+        for (int option = u.dc == 1 ? 0 : 2; option < 4; ++option) {
+            u.xb = 2 - (option & 1);
+            u.staged = option < 2;
+            u.out_bytes = u.tps * u.K * out_size;
+            u.p1_off = 3 * u.atoms2 * u.dt * 64;
+            u.x_off = u.p1_off + 2 * u.atoms1 * u.nc * 64;
+            u.st_off = u.x_off + u.xb * u.atoms2 * u.ntot * 64;
+            u.sh_off = (u.st_off + (u.staged ? 2 * u.out_bytes : 0) + 127) / 128 * 128;
+            u.total = u.sh_off + kRotUmmaSharedBytes;
+            // (an MMA reads 128 rows from the first row of any block of P2's terms)
+            if (u.total <= kRotMaxSmem && u.p1_off - u.dt * 64 + 128 * 64 <= u.total) { *out = u; return true; }
+        }
+    }
+    return false;
+}
+
 // ---- the weight-only operating point ----
 // Up to how many tokens it runs on three int8 digits per value (gemm_small.cu)
 constexpr int kDigitTokens = 32;

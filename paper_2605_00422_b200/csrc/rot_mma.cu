@@ -38,11 +38,6 @@ namespace bwla {
 
 enum { kRotQuant = 0, kRotBf16 = 1, kRotBinarize = 2, kRotDigits = 3 };
 
-constexpr int kRotMaxWarps = 16;          // per CTA
-constexpr int kRotMaxSmem = 232448 - 128; // the 227 KB a block may have, less the static shared memory of the roles
-constexpr int kRotHeader = 256;           // prepared factors: exponents, then the terms
-constexpr int kRotRedBytes = 3072;        // per group (and room for an ldmatrix that reads eight rows past x)
-
 // What the warps and CTAs of a token exchange: one per group, behind its operand tiles.  [token parity][warp of the token]
 struct RotShared {
     uint32_t xmax[2][64];                 // bits of the largest |x|
@@ -52,73 +47,6 @@ struct RotShared {
     int qsum[2][3];
 };
 static_assert(sizeof(RotShared) <= kRotRedBytes, "RotShared");
-
-static int round_to(int v, int m) { return (v + m - 1) / m * m; }
-
-// A warp may have ntw column tiles at most; `alias`: Z^T takes the place of x, which is dead by then (the next token's x then
-// arrives late, which costs about a fifth).  Fills in what follows from dc and alias; false when it does not fit.
-static bool rot_layout(RotGeom& g, int dc, int alias, int pad) {
-    const int tiles = g.n2p / 16;
-    g.dtc = (tiles + dc - 1) / dc;
-    g.warps = g.dtc * g.cw;
-    if (g.warps > kRotMaxWarps || (dc - 1) * g.dtc >= tiles || dc * g.warps > 64) return false;
-    // Rows of an odd number of 16-byte chunks (pad 16): the eight rows of an ldmatrix then fall into different banks.  The
-    // largest factors only fit without that padding, and without the rows of x beyond n1.
-    g.pad = pad;
-    g.s2 = g.n2p * 2 + pad; g.s1 = g.na * 16 + pad;
-    const int x = (pad ? g.cw * g.ntw * 8 : g.n1) * g.s2, z = g.cw > 1 ? 2 * g.dtc * 16 * g.s1 : 0;
-    g.dc = dc; g.alias_z = alias;
-    g.p1_off = 3 * g.dtc * 16 * g.s2;
-    g.group_off = g.p1_off + 2 * g.na * 8 * g.s1;
-    g.group_bytes = (alias ? std::max(x, z) : x + z) + kRotRedBytes;
-    g.z_rel = alias ? 0 : x; g.red_rel = g.group_bytes - kRotRedBytes;
-    if (g.group_off + g.group_bytes > kRotMaxSmem) return false;
-    g.max_groups = dc == 1 ? std::min(std::min(kRotMaxWarps / g.warps, 8), (kRotMaxSmem - g.group_off) / g.group_bytes) : 1;   // (barriers 1..8)
-    return true;
-}
-
-// Chooses the split of a token over warps and CTAs: the one that keeps most warps busy on an SM (16 is what the registers
-// allow), counting that the last CTA of a cluster may have fewer rows.
-bool rot_geometry(int n1, int n2, RotGeom* out) {
-    if (n1 < 1 || n2 < 8 || n2 % 8 != 0 || n2 > 256 || n1 > 192) return false;
-    RotGeom g{};
-    g.n1 = n1; g.n2 = n2; g.K = n1 * n2;
-    g.n2p = round_to(n2, 16); g.na = round_to(n1, 16) / 8;
-    g.cw = g.na <= 8 ? 1 : g.na <= 16 ? 2 : 4;
-    g.ntw = (g.na + g.cw - 1) / g.cw;                         // (the last warp may have tiles beyond na, which it ignores)
-    double best = 0.0;
-    for (int pad = 16; pad >= 0 && best == 0.0; pad -= 16)
-        for (int dc = 1; dc <= 8; ++dc)
-            for (int alias = 0; alias <= (g.cw > 1 ? 1 : 0); ++alias) {
-                RotGeom t = g;
-                if (!rot_layout(t, dc, alias, pad)) continue;
-                const int ctas = dc == 1 ? 1 : std::min(kRotMaxWarps / t.warps, (kRotMaxSmem + 1024) / (t.group_off + t.group_bytes + 1024));
-                const double score = (double)(g.n2p / 16) * g.cw / dc * t.max_groups * ctas * (alias ? 0.8 : 1.0);
-                if (score > best * 1.001) { best = score; *out = t; }
-            }
-    return best != 0.0;
-}
-
-// Few tokens: what counts is the time of one token, so it is spread over more warps (up to 64 columns: two warps instead of
-// one) and, while every cluster finds SMs of its own, over more CTAs: MMAs of a CTA at 2 cycles each, against about 5000
-// cycles for the cluster's barriers and its later start (64 x 128, one token: 6.7 us on eight CTAs, 5.2 on one).
-static RotGeom few_tokens_geometry(const RotGeom& base, int64_t clusters, int sms) {
-    RotGeom best = base;
-    double best_cost = 0.0;
-    const int ksteps = base.n2p / 16 + base.na / 2;
-    for (int dc = 1; dc <= 8 && clusters * dc <= sms; ++dc) {
-        RotGeom t = base;
-        if (t.na > 4 && t.na <= 8) { t.cw = 2; t.ntw = 4; }
-        if (!rot_layout(t, dc, 0, base.pad) && (t.cw == 1 || !rot_layout(t, dc, 1, base.pad))) continue;
-        const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 5000.0 + 300.0 * dc : 0.0);
-        if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = t; }
-    }
-    return best;
-}
-
-size_t rot_prepared_bytes(const RotGeom& g) {
-    return kRotHeader + (size_t)3 * g.n2p * g.s2 + (size_t)2 * g.na * 8 * g.s1;
-}
 
 // once per layer: P1, P2 (fp32) -> exponents (of max|P2|; by which P1 is scaled), the bf16 terms of P2^T and the fp16 terms of
 // P1^T, rows as they lie in shared memory

@@ -43,8 +43,6 @@ constexpr int kThreads = 128 + 32 * kAluWarps;       // 640
 // registers: 96 a thread at launch (640 x 96 = 61440); 128 x 56 + 512 x 104 = 60416 after the split (without it the two-chain
 // variant keeps values in local memory: 2048 tokens of 160 x 160 236 -> 209 us)
 constexpr int kRegsControl = 56, kRegsAlu = 104;
-constexpr int kPrepHeader = 256;          // of the prepared factors (rot_mma.cu)
-constexpr int kMaxSmem = 232448;
 struct Shared {
     uint64_t x_full[2], x_empty[2];       // a step's x has landed; the MMAs that read it have completed
     uint64_t z_full[2], y_full[2];        // accumulator i & 1 holds Z, Y
@@ -59,57 +57,8 @@ struct Shared {
     uint32_t tmem_slot;
     int abort_flag;
 };
-constexpr int kSharedBytes = (int)((sizeof(Shared) + 127) / 128 * 128);
+static_assert(sizeof(Shared) <= kRotUmmaSharedBytes, "Shared");
 }  // namespace ru
-
-struct RotUmmaGeom {
-    int n1, n2, K;
-    int nc;                 // columns of a token's Y: n1 rounded up to 16
-    int np;                 // columns of a token in the accumulators
-    int tps, ntot;          // tokens of a step, tps * np
-    int dc, dt;             // CTAs of a token, rows d of each
-    int atoms2, atoms1;     // K atoms of 32 elements over b / over a
-    int xb;                 // buffers of x
-    int two;                // two chains of sums
-    int staged;             // outputs of a step go through shared memory (two buffers of out_bytes)
-    int out_bytes;
-    int p1_off, x_off, st_off, sh_off, total;
-    int s2, s1;             // row strides of the prepared factors
-};
-
-// False when the sizes are outside what the kernel takes: whole 16-byte pieces of the codes' order (n2 a multiple of 16), three
-// times n1 columns of tensor memory, at most 128 rows and the factors' terms in the shared memory of one CTA or of two.
-static bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) {
-    if (g.n2 % 16 != 0 || g.n2 < 16 || g.n1 > 160) return false;
-    RotUmmaGeom u{};
-    u.n1 = g.n1; u.n2 = g.n2; u.K = g.K; u.s2 = g.s2; u.s1 = g.s1;
-    u.nc = g.na * 8;
-    u.tps = u.nc <= 32 ? 4 : u.nc <= 80 ? 2 : 1;
-    u.np = u.tps == 1 ? (u.nc + 31) / 32 * 32 : u.nc;
-    u.ntot = u.tps * u.np;
-    u.two = g.n2 > 128 || u.nc > 128;
-    if (u.two && (u.nc < 32 || g.n2 < 32)) return false;      // (one step of 16 values: the second chain of that contraction would have none)
-    u.atoms2 = (g.n2 + 31) / 32; u.atoms1 = (u.nc + 31) / 32;
-    for (u.dc = 1; u.dc <= 2; ++u.dc) {
-        u.dt = u.dc == 1 ? g.n2 : (g.n2 / 2 + 15) / 16 * 16;
-        if (u.dt > 128) continue;
-        // Outputs of whole tokens are contiguous: they are staged where two buffers fit, at the price of the second x if need
-        // be (stored from registers, a sector of 32 bytes is written in two or four pieces: 64 x 80, 4096 tokens 54 us).
-        for (int option = u.dc == 1 ? 0 : 2; option < 4; ++option) {
-            u.xb = 2 - (option & 1);
-            u.staged = option < 2;
-            u.out_bytes = u.tps * u.K * out_size;
-            u.p1_off = 3 * u.atoms2 * u.dt * 64;
-            u.x_off = u.p1_off + 2 * u.atoms1 * u.nc * 64;
-            u.st_off = u.x_off + u.xb * u.atoms2 * u.ntot * 64;
-            u.sh_off = (u.st_off + (u.staged ? 2 * u.out_bytes : 0) + 127) / 128 * 128;
-            u.total = u.sh_off + ru::kSharedBytes;
-            // (an MMA reads 128 rows from the first row of any block of P2's terms)
-            if (u.total <= ru::kMaxSmem && u.p1_off - u.dt * 64 + 128 * 64 <= u.total) { *out = u; return true; }
-        }
-    }
-    return false;
-}
 
 struct RotUmmaParams {
     RotUmmaGeom g;
@@ -208,7 +157,7 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     // ---- the layer's factors (they do not depend on the preceding kernel): rows of 64 bytes, swizzled ----
     int e1;
     if (pr.prepared) {
-        const uint8_t* t2 = pr.prepared + ru::kPrepHeader;
+        const uint8_t* t2 = pr.prepared + kRotHeader;
         const size_t all2 = (size_t)g.n2 * g.s2;
         const uint8_t* t1 = t2 + 3 * all2;
         e1 = __ldg(reinterpret_cast<const int*>(pr.prepared) + 1);

@@ -81,3 +81,36 @@ def test_partial_sums_of_many_tokens_fit_where_the_codes_go(tmp_path):
         for (long M = 1; M <= 5000; ++M)
             for (long K = 64; K <= 25600; K += 64)
                 if (lowrank_umma_part_bytes(M, K, r) > (size_t)(M * K)) { std::printf("%ld tokens, K %ld\\n", M, K); return 0; }""") == ""
+
+
+def test_operands_of_the_rotations_lie_inside_the_block(tmp_path):
+    """Every pair of factor sizes, every number of tokens the few-token plan distinguishes: what ldmatrix reads of x and of P1's terms
+    (whole column tiles of every warp, also beyond n1), what an MMA reads of P2's (128 rows), and the chains of sums (none empty)."""
+    assert violations(tmp_path, """
+    long seen = 0;
+    auto check = [&](const RotGeom& g) {
+        const int total = g.group_off + g.group_bytes, rows = g.cw * g.ntw * 8;
+        const bool ok = total <= kRotMaxSmem && g.group_off + rows * g.s2 <= total && g.p1_off + (g.na * 8 + rows) * g.s1 <= total &&
+                        (g.alias_z ? 0 : rows * (g.pad ? g.s2 : 0)) <= g.red_rel && g.red_rel + kRotRedBytes <= g.group_bytes &&
+                        g.group_off + g.max_groups * g.group_bytes <= kRotMaxSmem &&
+                        (g.group_off | g.group_bytes | g.p1_off | g.z_rel | g.red_rel | g.s1 | g.s2) % 16 == 0 && g.dc * g.dtc * 16 >= g.n2;
+        if (!ok) std::printf("%d x %d: cluster %d, %d warps of %d tiles\\n", g.n1, g.n2, g.dc, g.cw, g.ntw);
+        return ok;
+    };
+    for (int n1 = 1; n1 <= 192; ++n1)
+        for (int n2 = 8; n2 <= 256; n2 += 8) {
+            RotGeom g{};
+            if (n1 * n2 % 32 || n1 * n2 > 25600 || !rot_geometry(n1, n2, &g)) continue;
+            ++seen;
+            if (!check(g)) return 0;
+            for (int clusters = 1; clusters <= 148; ++clusters)
+                if (!check(few_tokens_geometry(g, clusters, 148))) return 0;
+            for (int size = 1; size <= 2; ++size) {
+                RotUmmaGeom u{};
+                if (!rot_umma_geometry(g, size, &u)) continue;
+                const int ks2 = n2 / 16, ks1 = u.nc / 16;
+                if (u.total > kRotMaxSmem || u.p1_off - u.dt * 64 + 128 * 64 > u.total || 3 * u.ntot > 512 || u.dc * u.dt < n2 ||
+                    (u.two && ((ks2 + 1) / 2 >= ks2 || (ks1 + 1) / 2 >= ks1))) { std::printf("%d x %d on tcgen05\\n", n1, n2); return 0; }
+            }
+        }
+    if (seen < 2000) std::printf("only %ld pairs\\n", seen);""") == ""

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n1,n2,M,pad,scale", [
     (1, 32, 5, 0, 1.0), (4, 16, 700, 0, 1.0), (20, 32, 333, 0, 1.0), (48, 64, 449, 0, 1.0), (73, 64, 3, 0, 1.0),
-    (100, 128, 2, 0, 1.0), (112, 128, 150, 0, 1.0), (140, 96, 4, 0, 1.0), (172, 136, 3, 0, 1.0), (188, 136, 2, 0, 1.0), (64, 256, 5, 0, 1.0),
+    (100, 128, 2, 0, 1.0), (112, 128, 150, 0, 1.0), (140, 96, 4, 0, 1.0), (172, 136, 3, 0, 1.0), (180, 136, 3, 0, 1.0), (188, 136, 2, 0, 1.0), (64, 256, 5, 0, 1.0),
     (36, 248, 2, 0, 1.0), (64, 80, 7, 1, 1.0), (160, 160, 2, 3, 1.0), (64, 80, 3, 0, 2.0 ** 100), (64, 80, 3, 0, 2.0 ** -110),
 ])
 def test_edges(n1, n2, M, pad, scale):
