@@ -80,6 +80,8 @@ int bwla_pack_signs(const void* w, int dtype, int64_t N, int64_t K, int64_t ldw,
  * a row's largest rotated magnitude, so a sign can differ from the exact one only where |X - mu| is below that.
  * Factor sizes that kernel does not take (n2 % 8 != 0, n2 > 256, n1 > 192) return BWLA_ERR_UNSUPPORTED.
  * N == 0 is a no-op.  Asynchronous on `stream`; bwla_check_status(workspace, stream) reports a device-side timeout.
+ * The inputs may be what the preceding kernel of `stream` makes, and packed, alpha and mu may be constants of the next
+ * call on `stream` without a synchronisation, as bwla_pack_signs' words may: no call starts before these two have ended.
  */
 size_t bwla_binarize_workspace_bytes(int64_t K);
 int bwla_binarize_rows(const void* w_res, int dtype, int64_t N, int64_t K, int64_t ldw, const float* P1, int n1,

@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(256) pack_signs_vec_kernel(const T* __restrict
             }
         }
     }
+    __threadfence();       // (the next call may read the words as constants, before it waits for this kernel's end)
 }
 
 // Rows whose start is not 16-byte aligned.  One warp produces one 32-bit word per step: lane l looks at weight
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(256) pack_signs_kernel(const T* __restrict__ w
         const uint32_t word = __ballot_sync(0xFFFFFFFFu, pos);
         if (lane == 0) packed[i] = word;
     }
+    __threadfence();
 }
 
 // One warp per row: the number of +1 weights minus the number of -1 weights.

@@ -128,7 +128,9 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     uint8_t* const xs = gs;
     uint8_t* const zs = gs + g.z_rel;
 
-    // ---- the layer's constants (they do not depend on the preceding kernel), and the zeros around x ----
+    // ---- the layer's constants (they do not depend on the preceding kernel, except that the factors of a binarisation may be what it has
+    //      made), and the zeros around x ----
+    if (MODE == kRotBinarize) griddep_wait();
     int e2, e1;
     if (pr.prepared) {
         const uint8_t* t2 = pr.prepared + kRotHeader + (size_t)rank * part2;
@@ -168,7 +170,9 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     for (int i = tid; i < (int)(sizeof(RotShared) / 4); i += T) reinterpret_cast<uint32_t*>(&sh)[i] = 0u;
     __syncthreads();
     if (g.dc > 1) { cluster_arrive_release(); cluster_wait_acquire(); }   // every CTA of the cluster runs: its slots may be written
-    griddep_launch_dependents();
+    // (The signs, scales and shifts of a binarisation are constants of the calls behind it, which read constants before they wait: they
+    // start when this kernel has ended.)
+    if (MODE != kRotBinarize) griddep_launch_dependents();
     int ntok = tok0 < p.M ? (int)((p.M - tok0 + stride - 1) / stride) : 0;
     // this thread's chunks of X: tid, tid + T, ...; (row, column) advance without divisions
     const int ch_a0 = tid / cpr, ch_c0 = tid - ch_a0 * cpr, ch_da = T / cpr, ch_dc = T - ch_da * cpr;
@@ -753,6 +757,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         barrier();
         flush_qsum(tok0 + (int64_t)(ntok - 1) * stride, (ntok - 1) & 1);
     }
+    if (MODE == kRotBinarize) __threadfence();       // (see above: complete in memory, not only issued)
     // nobody leaves while a neighbour may still store into its shared memory
     if (g.dc > 1) { cluster_arrive_release(); cluster_wait_acquire(); }
 }

@@ -10,6 +10,7 @@ import torch
 
 import oracle
 from paper_2605_00422_b200 import inputs as gen
+from tests import helpers as H
 
 pytestmark = pytest.mark.gpu
 
@@ -79,3 +80,31 @@ def test_binarised_layer_reproduces_rows_that_are_binary_after_the_rotation(bwla
     want = x @ W.astype(np.float64).T
     got = out.float().cpu().numpy().astype(np.float64)
     assert np.linalg.norm(got - want) / np.linalg.norm(want) < 2e-2
+
+
+def test_a_linear_may_take_what_the_call_before_it_has_binarised():
+    """Rows, then a raw one-token linear with their signs, scales and shifts on the same stream, buffers made beforehand and holding other
+    values: the contraction fetches sign words before it waits for its predecessor, and must not see the old ones."""
+    import ctypes as C
+    from paper_2605_00422_b200 import bwla
+    n1, n2, N, K = 32, 64, 3000, 2048                    # (more rows than SMs have groups for: they end at different times)
+    rng = np.random.default_rng(5)
+    P1, P2 = H.f32_to_dev(gen.orthogonal_f32(n1, rng)), H.f32_to_dev(gen.orthogonal_f32(n2, rng))
+    x = H.bf16_to_dev(gen.bf16_bits_from_f32(rng.standard_normal((1, K)).astype(np.float32)))
+    packed = torch.empty((N, K // 32), dtype=torch.int32, device="cuda")
+    alpha, mu = torch.empty(N, device="cuda"), torch.empty(N, device="cuda")
+    ws_b = torch.zeros(bwla.bwla_binarize_workspace_bytes(K), dtype=torch.uint8, device="cuda")
+    ws, out = bwla.new_workspace(1, K, N, 0, 6), torch.empty((1, N), dtype=torch.bfloat16, device="cuda")
+    p = lambda t: C.c_void_p(t.data_ptr())
+    for rnd in range(6):
+        W = torch.from_numpy((rng.standard_normal((N, K)) * 0.02).astype(np.float32)).cuda()
+        want_words, want_alpha, want_mu = bwla.bwla_binarize_rows(W, P1, P2)
+        torch.cuda.synchronize()
+        want = bwla.bwla_w1ax_linear(x, P1, P2, 6, want_words, want_alpha, mu=want_mu).clone()
+        packed.fill_(-1); alpha.fill_(1.0); mu.fill_(7.0)
+        torch.cuda.synchronize()
+        st = bwla._lib.bwla_binarize_rows(p(W), 0, N, K, K, p(P1), n1, p(P2), n2, p(packed), p(alpha), p(mu), p(ws_b), ws_b.numel(), bwla._stream())
+        assert st == 0
+        bwla.bwla_w1ax_linear(x, P1, P2, 6, packed, alpha, mu=mu, out=out, workspace=ws)
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), want.view(torch.int16)), f"round {rnd}"
