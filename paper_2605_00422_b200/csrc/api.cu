@@ -101,6 +101,7 @@ struct bwla_layer {
     uint8_t* prepared;
     bool rot;                 // the tensor-core rotation takes these factor sizes
     RotGeom geom;
+    uint8_t* okt;             // the factors once more in okt_umma.cu's form, inside `prepared`, or NULL where that kernel is not chosen
     int asym;                 // activation quantiser: 0 symmetric, 1 asymmetric (per-token zero point)
     int32_t* rowsum;          // [N] sign sums of the rows, inside `prepared`
 };
@@ -287,11 +288,20 @@ int bwla_workspace_section(int64_t M, int64_t K, int64_t N, int r, int bits, int
 
 // ---- prepared layers -------------------------------------------------------------------------------------------
 
+struct PreparedLayout { bool rot; RotGeom geom; bool has_okt; OktGeom okt_geom; size_t okt, rowsum; };
+static PreparedLayout prepared_layout(int n1, int n2) {
+    PreparedLayout p{};
+    p.rot = rot_geometry(n1, n2, &p.geom);
+    p.okt = p.rot ? align_up(rot_prepared_bytes(p.geom), 256) : 256;
+    p.has_okt = p.rot && rot_okt_factors(p.geom) && okt_geometry(n1, n2, &p.okt_geom);
+    p.rowsum = p.okt + (p.has_okt ? align_up(okt_prepared_bytes(p.okt_geom), 256) : 0);
+    return p;
+}
+
 size_t bwla_layer_prepared_bytes(int64_t K, int64_t N, int n1, int n2, int r) {
     if (!valid_rotation_dims(K, n1, n2) || N < 0 || r < 0 || r > 256) return 0;
-    RotGeom g;
-    // the terms of the Kronecker factors for the tensor-core rotation, then the sign sums of the rows
-    return (rot_geometry(n1, n2, &g) ? align_up(rot_prepared_bytes(g), 256) : 256) + align_up((size_t)N * 4, 256);
+    // the terms of the Kronecker factors for the tensor-core rotations, then the sign sums of the rows
+    return prepared_layout(n1, n2).rowsum + align_up((size_t)N * 4, 256);
 }
 
 int bwla_layer_create(bwla_layer** layer, int64_t K, int64_t N, const float* P1, int n1, const float* P2, int n2, int bits,
@@ -312,11 +322,14 @@ int bwla_layer_create(bwla_layer** layer, int64_t K, int64_t N, const float* P1,
     L->K = K; L->N = N; L->n1 = n1; L->n2 = n2; L->bits = bits; L->r = r;
     L->P1 = P1; L->P2 = P2; L->packed = packed; L->alpha = alpha; L->mu = mu; L->U = U_bf16; L->V = V_bf16;
     L->prepared = (uint8_t*)prepared;
-    L->rot = rot_geometry(n1, n2, &L->geom);
+    const PreparedLayout lay = prepared_layout(n1, n2);
+    L->rot = lay.rot; L->geom = lay.geom;
+    L->okt = lay.has_okt ? L->prepared + lay.okt : nullptr;
     L->asym = 0;
-    L->rowsum = (int32_t*)((uint8_t*)prepared + (L->rot ? align_up(rot_prepared_bytes(L->geom), 256) : 256));
+    L->rowsum = (int32_t*)(L->prepared + lay.rowsum);
     if (L->rot) {
         st = launch_prepare_rot(L->geom, P1, P2, prepared, (cudaStream_t)stream);
+        if (st == BWLA_OK && L->okt) st = launch_prepare_okt(lay.okt_geom, P1, P2, L->okt, (cudaStream_t)stream);
         if (st != BWLA_OK) { free(L); return st; }
     }
     st = launch_row_sums(packed, N, K, L->rowsum, (cudaStream_t)stream);
@@ -345,7 +358,7 @@ int bwla_layer_rotate_quant_asym(const bwla_layer* L, const void* x_bf16, int64_
     if (!L->rot) return BWLA_ERR_UNSUPPORTED;
     // the kernel keeps u - 2^(b-1) so that codes fit int8; the bias puts u and the zero point back in [0, 2^b - 1]
     RotProblem pr{};
-    pr.prepared = L->prepared; pr.codes = (int8_t*)codes; pr.zp = zeros; pr.code_bias = 1 << (L->bits - 1); pr.scales = scales; pr.y = y_f32;
+    pr.prepared = L->prepared; pr.okt = L->okt; pr.codes = (int8_t*)codes; pr.zp = zeros; pr.code_bias = 1 << (L->bits - 1); pr.scales = scales; pr.y = y_f32;
     return launch_rot(L->geom, x_bf16, M, ldx, L->bits, 1, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
@@ -359,7 +372,7 @@ int bwla_layer_rotate_quant(const bwla_layer* L, const void* x_bf16, int64_t M, 
     if (st != BWLA_OK) return st;
     if (L->rot && g_forced_rotation != BWLA_ROT_SIMT) {
         RotProblem pr{};
-        pr.prepared = L->prepared; pr.codes = codes; pr.scales = scales; pr.y = y_f32;
+        pr.prepared = L->prepared; pr.okt = L->okt; pr.codes = codes; pr.scales = scales; pr.y = y_f32;
         return launch_rot(L->geom, x_bf16, M, ldx, L->bits, 0, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
     }
     if (y_f32) return BWLA_ERR_UNSUPPORTED;      // only the tensor-core kernel can hand out Y
@@ -485,7 +498,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         for (int i = 0; i < count; ++i) {
             const bwla_layer* L = layers[i];
             pr[i] = RotProblem{};
-            pr[i].prepared = L->prepared; pr[i].codes = (int8_t*)(wbase[i] + ws[i].codes); pr[i].codes_layout = path[i] == BWLA_PATH_I8 ? 1 : 0;
+            pr[i].prepared = L->prepared; pr[i].okt = L->okt; pr[i].codes = (int8_t*)(wbase[i] + ws[i].codes); pr[i].codes_layout = path[i] == BWLA_PATH_I8 ? 1 : 0;
             pr[i].zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr;
             pr[i].scales = (float*)(wbase[i] + ws[i].scales); pr[i].qsum = (int32_t*)(wbase[i] + ws[i].qsum);
             lr[i] = OktLowrank{L->V, L->r, wbase[i] + ws[i].T, L->r > 0 ? (float*)(wbase[i] + ws[i].lr_part) : nullptr,

@@ -135,6 +135,7 @@ constexpr int kRotMaxProblems = 4;          // linears that share one x and are 
 struct RotProblem {
     const uint8_t* prepared;    // terms of P2^T and P1^T (launch_prepare_rot), or NULL: P1 and P2 are split by every CTA
     const float *P1, *P2;       // read only when `prepared` is NULL
+    const uint8_t* okt;         // beside `prepared`: the terms in the layout of okt_umma.cu, or NULL where that kernel is not chosen
     // quantiser (yhat == NULL)
     int8_t* codes;              // [M][K]
     int codes_layout;           // 0: natural k order; 1: the interleaved order of the tensor-core contraction
@@ -164,11 +165,28 @@ int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void*
 int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream);
 // The same for many tokens, on the tcgen05 tensor cores (rot_umma.cu); x in 16-byte pieces.  launch_rot goes there by itself.
-bool rot_umma_supports(const RotGeom& g, int64_t M, int n_problems, const RotProblem* problems);
+bool rot_umma_supports(const RotGeom& g, int n_problems, const RotProblem* problems);
 int launch_rot_umma(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                     const RotProblem* problems, uint32_t* status, cudaStream_t stream);
 // how many clusters of a kernel the device holds at once
 int resident_clusters(const void* kernel, int dc, int threads, size_t smem);
+// ---- many tokens of factors up to 128 (okt_umma.cu; launch_rot goes there by itself) ----
+// Geometry of the kernel for one pair of factor sizes.
+struct OktGeom {
+    int n1, n2, K;
+    int n1p, n2p;           // n1, n2 rounded up to 16: columns of Z^T / Y^T, contraction depth of the first stage
+    int atom2, atom1;       // bytes of one K-atom row (the swizzle span) of operands contracted over b / over a
+    int dt_count, dt_rows;  // tiles of the rows d of P2^T (= tensor-memory lanes) and rows per tile (a multiple of 8)
+    int cs_count, cs_cols;  // slabs of the rows c of P1^T (= output columns) and columns per slab (a multiple of 16)
+    int p2t_bytes, p1t_bytes, x_bytes;      // one tile of P2^T terms, one slab of P1^T terms, one token's X tile
+    int p1t_off, x_off, bar_off;            // shared-memory offsets (P2^T tile at 0)
+    int tmem_cols, smem_bytes;
+};
+bool okt_geometry(int n1, int n2, OktGeom* out);
+size_t okt_prepared_bytes(const OktGeom& g);
+int launch_prepare_okt(const OktGeom& g, const float* P1, const float* P2, void* prepared, cudaStream_t stream);
+int launch_okt(const OktGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
+               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream);
 // Rows of weights (fp32 or bf16): packed signs, scale and shift of every row.
 int launch_rot_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status,
                         cudaStream_t stream);

@@ -58,10 +58,8 @@ inline int lowrank_umma_parts(int64_t M, int64_t K) {
     ks = std::min<int64_t>(ks, kLruMaxParts);
     return (int)std::min<int64_t>(ks, std::max<int64_t>(1, K / (8 * kLruBlockK)));
 }
-// (from 50 tokens where the rotation of a token takes a cluster of three, 160 x 160: it goes to rot_umma.cu then, which has no
-// blocks for T beside it)
 inline bool lowrank_umma_supports(int64_t M, int64_t K, int r) {
-    return (M > 64 || (K > 128 * 128 && 3 * M > 148)) && r > 0 && r <= kLruCols && K % kLruBlockK == 0;
+    return M > 64 && r > 0 && r <= kLruCols && K % kLruBlockK == 0;
 }
 // Bytes of its partial sums.  They lie where the rotation that follows it leaves the codes (or the rotated values) and are never
 // larger than those: 256 bytes a column of 128 tokens against 128 values of K / 512 parts at the least.
@@ -140,24 +138,43 @@ inline bool rot_geometry(int n1, int n2, RotGeom* out) {
 }
 
 // Few tokens: what counts is the time of one token, so it is spread over more warps (up to 64 columns: two warps instead of
-// one) and, while every cluster finds SMs of its own, over more CTAs: MMAs of a CTA at 2 cycles each, against about 5000
-// cycles for the cluster's barriers and its later start (64 x 128, one token: 6.7 us on eight CTAs, 5.2 on one).
-inline RotGeom few_tokens_geometry(const RotGeom& base, int64_t clusters, int sms) {
-    RotGeom best = base;
+// one) and over more CTAs: MMAs of a CTA at 2 cycles each, against about 5000 cycles for the cluster's barriers and its later start
+// (64 x 128, one token: 6.7 us on eight CTAs, 5.2 on one).  `resident(geometry)`: every token finds a cluster at once; false when no
+// split has that (a second round of clusters doubles the time: 128 x 128, 16 tokens in clusters of eight 23.6 us).
+template <typename Resident>
+inline bool few_tokens_geometry(const RotGeom& base, RotGeom* out, Resident resident) {
     double best_cost = 0.0;
     const int ksteps = base.n2p / 16 + base.na / 2;
-    for (int dc = 1; dc <= 8 && clusters * dc <= sms; ++dc) {
+    for (int dc = 1; dc <= 8; ++dc) {
         RotGeom t = base;
         if (t.na > 4 && t.na <= 8) { t.cw = 2; t.ntw = 4; }
         if (!rot_layout(t, dc, 0, base.pad) && (t.cw == 1 || !rot_layout(t, dc, 1, base.pad))) continue;
         const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 5000.0 + 300.0 * dc : 0.0);
-        if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = t; }
+        if ((best_cost == 0.0 || cost < best_cost) && resident(t)) { best_cost = cost; *out = t; }
     }
-    return best;
+    return best_cost != 0.0;
 }
 
 inline size_t rot_prepared_bytes(const RotGeom& g) {
     return kRotHeader + (size_t)3 * g.n2p * g.s2 + (size_t)2 * g.na * 8 * g.s1;
+}
+
+// ---- which kernel rotates many tokens (more than the device holds clusters for) ----
+// A call of one prepared linear of 32 outputs, us at 150, 1024 and 4096 (x 128: 2048) tokens, and the error of the rotation against 64
+// bits in 1e-7 of a row's 2-norm, on rot_mma.cu | okt_umma.cu | rot_umma.cu:
+//    64 x  64    21    31    64   1.4  |  26    43   103   1.7  |  22    38    88   1.4
+//    64 x  80    23    41    92   1.4  |  28    46   110   1.8  |  24    41    91   1.5
+//    64 x  88    27    50   121   1.5  |  29    47   111   2.0  |      -
+//    64 x 128    32    60   153   1.5  |  33    51   126   2.3  |  30    47   106   1.7
+//    86 x 128    46    94   288   1.5  |  39    61   152   2.5  |  45    80   230   1.9
+//   108 x 128    55   114   197   1.5  |  46    74   118   2.6  |  50    87   139   2.0
+//   128 x 128    66   155   273   1.5  |  50    78   125   2.7  |  50    79   126   2.0
+//   160 x 160   100   296     -   1.5  | 101   316     -   3.2  |  81   156     -   2.3
+// mma.sync wherever one warp holds all columns of a token and a CTA several tokens; rot_umma.cu (and for the bf16 values of the
+// weight-only operating point everywhere else); okt_umma.cu where a step of rot_umma.cu holds one token in half of its columns.
+inline bool rot_mma_always(const RotGeom& g) { return g.cw == 1 && g.n2p <= 80; }
+inline bool rot_okt_factors(const RotGeom& g) {
+    return !rot_mma_always(g) && g.na <= 16 && g.n2 <= 128 && (g.na > 10 || g.n2 % 16 != 0);
 }
 
 // ---- rotation of many tokens on tcgen05 (rot_umma.cu) ----
@@ -170,7 +187,6 @@ struct RotUmmaGeom {
     int dc, dt;             // CTAs of a token, rows d of each
     int atoms2, atoms1;     // K atoms of 32 elements over b / over a
     int xb;                 // buffers of x
-    int two;                // two chains of sums
     int staged;             // outputs of a step go through shared memory (two buffers of out_bytes)
     int out_bytes;
     int p1_off, x_off, st_off, sh_off, total;
@@ -178,17 +194,16 @@ struct RotUmmaGeom {
 };
 
 // False when the sizes are outside what the kernel takes: whole 16-byte pieces of the codes' order (n2 a multiple of 16), three
-// times n1 columns of tensor memory, at most 128 rows and the factors' terms in the shared memory of one CTA or of two.
+// times n1 columns of tensor memory, at most 128 rows and the factors' terms in the shared memory of one CTA or of two; both
+// contractions at least two steps of 16 values deep (the second chain of sums would have none).
 inline bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) {
-    if (g.n2 % 16 != 0 || g.n2 < 16 || g.n1 > 160) return false;
+    if (g.n2 % 16 != 0 || g.n2 < 32 || g.na < 4 || g.n1 > 160) return false;
     RotUmmaGeom u{};
     u.n1 = g.n1; u.n2 = g.n2; u.K = g.K; u.s2 = g.s2; u.s1 = g.s1;
     u.nc = g.na * 8;
     u.tps = u.nc <= 32 ? 4 : u.nc <= 80 ? 2 : 1;
     u.np = u.tps == 1 ? (u.nc + 31) / 32 * 32 : u.nc;
     u.ntot = u.tps * u.np;
-    u.two = g.n2 > 128 || u.nc > 128;
-    if (u.two && (u.nc < 32 || g.n2 < 32)) return false;      // (one step of 16 values: the second chain of that contraction would have none)
     u.atoms2 = (g.n2 + 31) / 32; u.atoms1 = (u.nc + 31) / 32;
     for (u.dc = 1; u.dc <= 2; ++u.dc) {
         u.dt = u.dc == 1 ? g.n2 : (g.n2 / 2 + 15) / 16 * 16;

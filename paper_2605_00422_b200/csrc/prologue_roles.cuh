@@ -445,4 +445,11 @@ inline int plan_lowrank(PrologueParams& p, float* lr_part, uint32_t* lr_count, i
     return blocks;
 }
 
+// The same for T of one linear beside a rotation.
+inline int plan_lowrank(PrologueParams& p, const void* x, int64_t M, int K, int64_t ldx, const OktLowrank& lr, int warps, size_t smem_limit, size_t* smem) {
+    p.x = (const __nv_bfloat16*)x; p.M = M; p.K = K; p.ldx = ldx;
+    p.V = (const __nv_bfloat16*)lr.V; p.r = lr.r; p.Thl = (__nv_bfloat16*)lr.Thl; p.lr_cols = lowrank_cols(lr.r);
+    return plan_lowrank(p, lr.lr_part, lr.lr_count, warps, smem_limit, smem);
+}
+
 }  // namespace bwla

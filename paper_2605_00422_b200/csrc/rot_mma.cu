@@ -782,11 +782,11 @@ static RotKernel pick_kernel(const RotGeom& g) {
 // How many clusters of the kernel the device holds at once (asked once per kernel, size and thread).
 int resident_clusters(const void* k, int dc, int threads, size_t smem) {
     struct Known { const void* k; int dc, threads, dev, n; size_t smem; };
-    static thread_local Known known[16];
+    static thread_local Known known[64];
     static thread_local int used = 0;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
-    for (int i = 0; i < 16 && i < used; ++i)
+    for (int i = 0; i < 64 && i < used; ++i)
         if (known[i].k == k && known[i].dc == dc && known[i].threads == threads && known[i].dev == dev && known[i].smem == smem) return known[i].n;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRotMaxSmem) != cudaSuccess) { cudaGetLastError(); return 0; }
     int n = 0;
@@ -804,7 +804,7 @@ int resident_clusters(const void* k, int dc, int threads, size_t smem) {
         cfg.attrs = a; cfg.numAttrs = 1;
         if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     }
-    known[used % 16] = Known{k, dc, threads, dev, n, smem};
+    known[used % 64] = Known{k, dc, threads, dev, n, smem};
     ++used;
     return n;
 }
@@ -848,64 +848,87 @@ static int launch_rot_kernel(RotKernel k, const RotGeom& g, RotKernelParams& p, 
     return after_launch();
 }
 
+static RotKernel rot_kernel_of(const RotGeom& g, const RotProblem& pr) {
+    return pr.yhat ? pick_kernel<kRotBf16, false>(g) : pr.digits ? pick_kernel<kRotDigits, false>(g) : pick_kernel<kRotQuant, false>(g);
+}
+
 int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream) {
     if (M == 0 || n_problems == 0) return BWLA_OK;
-    const RotGeom g = M * n_problems <= sm_count() ? few_tokens_geometry(base, M * n_problems, sm_count()) : base;
     if (n_problems > kRotMaxProblems || M >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
+    const bool vec = rot_accepts_x(x, ldx);
+    // ---- T = V x.  Many tokens: for all linears, as a launch of its own on the tcgen05 tensor cores.  Every kernel of the chain waits for
+    //      its predecessor before it ends, so the contraction still finds T complete. ----
+    OktLowrank beside[kRotMaxProblems] = {};          // what is left for blocks of the rotation's own launch
+    if (lowrank) {
+        OktLowrank batch[kRotMaxProblems];
+        int nb = 0;
+        for (int i = 0; i < n_problems; ++i) {
+            if (!lowrank[i].V || lowrank[i].r <= 0 || !lowrank[i].Thl) continue;
+            if (lowrank_umma_supports(M, base.K, lowrank[i].r) && vec && (reinterpret_cast<uintptr_t>(lowrank[i].V) & 15) == 0 &&
+                (lowrank[i].umma_part || lowrank_umma_part_bytes(M, base.K, lowrank[i].r) == 0))
+                batch[nb++] = lowrank[i];
+            else
+                beside[i] = lowrank[i];
+        }
+        if (nb > 0) {
+            const int st = launch_lowrank_umma(x, M, base.K, ldx, nb, batch, status, stream);
+            if (st != BWLA_OK) return st;
+        }
+    }
+    // T of linears without blocks beside the rotation, as a launch of its own: wide tiles (their registers do not fit), rows that do not
+    // start on 16 bytes (their blocks want more warps than a token has), or `all`
+    auto own_launch = [&](bool all) -> int {
+        for (int i = 0; i < n_problems; ++i) {
+            if (!beside[i].V) continue;
+            PrologueParams probe{};
+            size_t bytes = 0;
+            plan_lowrank(probe, x, M, base.K, ldx, beside[i], kRotMaxWarps, kRotMaxSmem, &bytes);
+            if (!all && (probe.lr_wide == 2 || probe.lr_wide == 4)) continue;
+            const int st = launch_prologue(x, M, base.K, ldx, nullptr, 0, nullptr, 0, bits, nullptr, 0, nullptr, nullptr, beside[i].V, beside[i].r,
+                                           beside[i].Thl, beside[i].lr_part, beside[i].lr_count ? beside[i].lr_count - kLrCounterWord : nullptr, stream);
+            if (st != BWLA_OK) return st;
+            beside[i] = OktLowrank{};
+        }
+        return BWLA_OK;
+    };
+    // ---- the kernel: while the device holds a cluster for every token, mma.sync, spread for the time of one token ----
+    RotGeom g = base;
+    const bool few = M * n_problems <= sm_count() && few_tokens_geometry(base, &g, [&](const RotGeom& t) {
+        return t.dc == 1 || M * n_problems <= resident_clusters((const void*)rot_kernel_of(t, problems[0]), t.dc, 32 * t.warps, (size_t)(t.group_off + t.group_bytes));
+    });
+    if (!few && vec) {
+        bool okt = rot_okt_factors(base) && !problems[0].yhat && !problems[0].digits;
+        for (int i = 0; i < n_problems; ++i) okt = okt && (problems[i].okt || !problems[i].prepared);
+        OktGeom og;
+        if (okt && okt_geometry(base.n1, base.n2, &og)) {
+            const int st = own_launch(false);
+            return st != BWLA_OK ? st : launch_okt(og, x, M, ldx, bits, asym, n_problems, problems, beside, status, stream);
+        }
+        if (rot_umma_supports(base, n_problems, problems)) {
+            const int st = own_launch(true);
+            return st != BWLA_OK ? st : launch_rot_umma(base, x, M, ldx, bits, asym, n_problems, problems, status, stream);
+        }
+    }
+    const int st = own_launch(false);
+    if (st != BWLA_OK) return st;
     RotKernelParams p{};
-    p.g = g; p.x = x; p.ldx = ldx; p.x_vec = rot_accepts_x(x, ldx); p.M = M; p.bits = bits; p.asym = asym; p.n_problems = n_problems;
+    p.g = g; p.x = x; p.ldx = ldx; p.x_vec = vec; p.M = M; p.bits = bits; p.asym = asym; p.n_problems = n_problems;
     p.status = status;
     p.groups = choose_groups(g, M, n_problems);
     size_t smem = 0;
     int lr_total = 0;
-    // Many tokens: T = V x of all problems goes first, as a launch of its own on the tensor cores.  Every kernel of the
-    // chain waits for its predecessor before it ends, so the contraction still finds T complete.
-    bool lr_done[kRotMaxProblems] = {};
-    if (lowrank) {
-        OktLowrank batch[kRotMaxProblems];
-        int nb = 0;
-        for (int i = 0; i < n_problems; ++i)
-            if (lowrank[i].V && lowrank[i].r > 0 && lowrank[i].Thl && lowrank_umma_supports(M, g.K, lowrank[i].r) && p.x_vec &&
-                (reinterpret_cast<uintptr_t>(lowrank[i].V) & 15) == 0 &&
-                (lowrank[i].umma_part || lowrank_umma_part_bytes(M, g.K, lowrank[i].r) == 0)) {
-                batch[nb++] = lowrank[i];
-                lr_done[i] = true;
-            }
-        if (nb > 0) {
-            int st = launch_lowrank_umma(x, M, g.K, ldx, nb, batch, status, stream);
-            if (st != BWLA_OK) return st;
-        }
-    }
     for (int i = 0; i < n_problems; ++i) {
         p.prob[i] = problems[i];
         p.lr_begin[i] = lr_total;
-        if (lowrank && !lr_done[i] && lowrank[i].V && lowrank[i].r > 0 && lowrank[i].Thl) {
-            PrologueParams& lp = p.lr[i];
-            lp.x = (const __nv_bfloat16*)x; lp.M = M; lp.K = g.K; lp.ldx = ldx;
-            lp.V = (const __nv_bfloat16*)lowrank[i].V; lp.r = lowrank[i].r; lp.Thl = (__nv_bfloat16*)lowrank[i].Thl;
-            lp.lr_cols = lowrank_cols(lowrank[i].r);
+        if (beside[i].V) {
             size_t lr_smem = 0;
-            const int blocks = plan_lowrank(lp, lowrank[i].lr_part, lowrank[i].lr_count, g.warps * p.groups, kRotMaxSmem, &lr_smem);
-            if (lp.lr_wide == 3) {
-                // Many tokens that the tcgen05 kernel does not take: wide tiles, as a launch of their own (their registers
-                // do not fit a block of this kernel)
-                int st = launch_prologue(x, M, g.K, ldx, nullptr, 0, nullptr, 0, bits, nullptr, 0, nullptr, nullptr, lowrank[i].V,
-                                         lowrank[i].r, lowrank[i].Thl, lowrank[i].lr_part,
-                                         lowrank[i].lr_count ? lowrank[i].lr_count - kLrCounterWord : nullptr, stream);
-                if (st != BWLA_OK) return st;
-                lp = PrologueParams{};
-            } else {
-                lr_total += blocks;
-                smem = std::max(smem, lr_smem);
-            }
+            lr_total += plan_lowrank(p.lr[i], x, M, g.K, ldx, beside[i], g.warps * p.groups, kRotMaxSmem, &lr_smem);
+            smem = std::max(smem, lr_smem);
         }
     }
     for (int i = n_problems; i <= kRotMaxProblems; ++i) p.lr_begin[i] = lr_total;
-    if (lr_total == 0 && p.x_vec && rot_umma_supports(g, M, n_problems, problems))
-        return launch_rot_umma(g, x, M, ldx, bits, asym, n_problems, problems, status, stream);
-    RotKernel k = problems[0].yhat ? pick_kernel<kRotBf16, false>(g) : problems[0].digits ? pick_kernel<kRotDigits, false>(g) : pick_kernel<kRotQuant, false>(g);
-    return launch_rot_kernel(k, g, p, smem, lr_total, stream);
+    return launch_rot_kernel(rot_kernel_of(g, problems[0]), g, p, smem, lr_total, stream);
 }
 
 int launch_rot_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status,

@@ -1,26 +1,27 @@
 // Online OKT (Sec. 3.1) for many tokens on the tcgen05 tensor cores, with the per-token quantiser (Sec. 4.1) or the bf16
-// rounding of the weight-only operating point fused in.  The warp-level kernel (rot_mma.cu) serves fewer tokens, every other
-// mode, and the factor sizes this one does not take.
+// rounding of the weight-only operating point fused in.  rot_mma.cu serves fewer tokens, every other mode and small factors, okt_umma.cu
+// those between (host_plans.h has the rule).
 //
 //   X = reshape(x_t, n1 x n2) (row-major),   Z^T = P2^T X^T  [d][a],   Y^T = Z^T P1  [d][c]
 //
-// The same sums of products as there: x against the three bf16 terms of P2, then two fp16 terms of Z against two of P1 (three
+// The same sums of products as in rot_mma.cu: x against the three bf16 terms of P2, then two fp16 terms of Z against two of P1 (three
 // products), small products first.  Z is scaled by a power of two per row d (its largest magnitude goes to [2^14, 2^15)), which
 // leaves exactly, row by row, with the scale of P1.
 //
+// The tensor core truncates when it adds to its accumulator, so each contraction is summed in two chains, one in each of two
+// accumulators, and added with a rounded addition.  (One chain, with the accumulators of two steps in turn, took 68 us for a call of
+// 64 x 80 and 4096 tokens instead of 91, but left 2.15e-7 of a row's 2-norm against 1.80e-7 of okt_umma.cu's six bf16 products and 1.50e-7
+// of two chains; 160 x 160: 9.9e-7 of a token's full scale.)
+//
 // What bounds it: 160 x 160 takes 60 MMAs of 128 x 160 x 16 a token and CTA (80 cycles each, 80 of the 128 rows in use); what the
-// ALU warps do with every value of Z and Y, in lock step and with five barriers a step, takes about twice that.  The warp-level
-// kernel needs 9600 cycles of its MMAs alone, with operands re-read from shared memory as fast as it delivers, and the barriers of
-// its one token stand open: 2048 tokens of 160 x 160 505 -> 209 us, 4096 of 64 x 80 77 -> 60 us.
-// MMAs and the work around them run side by side, three steps deep:
-//   MMA thread    Z(0), Z(1), Y(0), Z(2), Y(1), ...    Z(i) and Y(i) share one of two accumulators
-//   16 ALU warps  step i: Y(i-1) to registers, its largest magnitude published  (accumulator free: Z(i+1) may start)
-//                         Z(i) to two fp16 terms in tensor memory               (Y(i) may start)
+// ALU warps do with every value of Z and Y, in lock step and with five barriers a step, takes about twice that (2048 tokens of
+// 160 x 160: 209 us; on mma.sync 505, whose operands are re-read from shared memory as fast as it delivers).
+// MMAs and the work around them run side by side:
+//   MMA thread    Z(0), Y(0), Z(1), Y(1), ...          Z(i) and Y(i) share the accumulators
+//   16 ALU warps  step i: Y(i-1) to registers, its largest magnitude published  (accumulators free: Z(i) may start)
 //                         Y(i-1) quantised and stored
-// The tensor core truncates when it adds to its accumulator, so more than 128 values a contraction are summed in two chains, one
-// in each accumulator, and added with a rounded addition (160 x 160: 9.9e-7 of a token's full scale in one chain).  Both
-// accumulators then belong to one step, and the ALU warps quantise under the MMAs of Z.
-// A step is 1, 2 or 4 tokens, so that it fills up to 160 columns (64 x 80: 2 tokens).  Factors whose terms do not fit one CTA
+//                         Z(i) to two fp16 terms in tensor memory               (Y(i) may start)
+// A step is 1, 2 or 4 tokens, so that it fills up to 160 columns (64 x 128: 2 tokens).  Factors whose terms do not fit one CTA
 // (or with n2 > 128) are split by rows d over a cluster of two, which share nothing but the largest magnitudes.
 //
 // Launched with programmatic stream serialisation: the factors are fetched before the preceding kernel of the stream has
@@ -43,10 +44,11 @@ constexpr int kThreads = 128 + 32 * kAluWarps;       // 640
 // registers: 96 a thread at launch (640 x 96 = 61440); 128 x 56 + 512 x 104 = 60416 after the split (without it the two-chain
 // variant keeps values in local memory: 2048 tokens of 160 x 160 236 -> 209 us)
 constexpr int kRegsControl = 56, kRegsAlu = 104;
+constexpr int kChunks = 5;                // 8-column chunks of a step one ALU warp owns, at most
 struct Shared {
     uint64_t x_full[2], x_empty[2];       // a step's x has landed; the MMAs that read it have completed
-    uint64_t z_full[2], y_full[2];        // accumulator i & 1 holds Z, Y
-    uint64_t d_free[2];                   // ... has been read
+    uint64_t z_full, y_full;              // the accumulators hold Z, Y
+    uint64_t d_free;                      // ... have been read
     uint64_t a_ready;                     // the terms of Z are in tensor memory
     uint64_t row_full[2][4];              // the exponents of a lane quarter's rows are there
     uint64_t out_full[2], out_free[2];    // the step's outputs and code sums are staged; have left
@@ -104,43 +106,39 @@ __device__ __forceinline__ bool warp_wait_cluster(uint64_t* bar, uint32_t parity
     }
     return false;
 }
-// The warp's columns of an accumulator (TWO: the sum of two, `other` columns apart).
-template <int NC, bool TWO>
+// The warp's columns of the sum of both chains, whose accumulators are `other` columns apart.
+template <int NC>
 __device__ __forceinline__ void load_sums(uint32_t src, uint32_t other, int cw, float (&v)[NC * 8]) {
 #pragma unroll
     for (int j = 0; j < NC; ++j)
         if (8 * j < cw) tmem_ld_32x8(src + 8 * j, reinterpret_cast<uint32_t*>(v) + 8 * j);
-    if (TWO) {
 #pragma unroll
-        for (int j = 0; j < NC; j += 2) {
-            if (8 * j < cw) {
-                const bool both = j + 1 < NC && 8 * (j + 1) < cw;
-                uint32_t u[16] = {};
-                tmem_ld_32x8(src + other + 8 * j, u);
-                if (both) tmem_ld_32x8(src + other + 8 * (j + 1), u + 8);
-                tc_wait_ld();
+    for (int j = 0; j < NC; j += 2) {
+        if (8 * j < cw) {
+            const bool both = j + 1 < NC && 8 * (j + 1) < cw;
+            uint32_t u[16] = {};
+            tmem_ld_32x8(src + other + 8 * j, u);
+            if (both) tmem_ld_32x8(src + other + 8 * (j + 1), u + 8);
+            tc_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 8; e += 2)
+                add2(v[8 * j + e], v[8 * j + e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
+            if (both && j + 1 < NC)
 #pragma unroll
                 for (int e = 0; e < 8; e += 2)
-                    add2(v[8 * j + e], v[8 * j + e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
-                if (both && j + 1 < NC)
-#pragma unroll
-                    for (int e = 0; e < 8; e += 2)
-                        add2(v[8 * (j + 1 < NC ? j + 1 : j) + e], v[8 * (j + 1 < NC ? j + 1 : j) + e + 1], __uint_as_float(u[8 + e]), __uint_as_float(u[9 + e]));
-            }
+                    add2(v[8 * (j + 1 < NC ? j + 1 : j) + e], v[8 * (j + 1 < NC ? j + 1 : j) + e + 1], __uint_as_float(u[8 + e]), __uint_as_float(u[9 + e]));
         }
-    } else {
-        tc_wait_ld();
     }
 }
 }  // namespace
 
-// NC: 8-column chunks of a step one ALU warp owns, at most.  MODE: the symmetric or the asymmetric quantiser, or the weight-only
-// operating point.  TWO: two chains of sums, one in each accumulator.
+// MODE: the symmetric or the asymmetric quantiser, or the weight-only operating point.
 enum { kSym = 0, kAsym = 1, kBf16 = 2 };
-template <int NC, int MODE, bool TWO>
+template <int MODE>
 __global__ void __launch_bounds__(ru::kThreads, 1)
 rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ RotUmmaParams p) {
     extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr int NC = ru::kChunks;
     const RotUmmaGeom& g = p.g;
     ru::Shared& sh = *reinterpret_cast<ru::Shared*>(smem + g.sh_off);
     volatile int* abort_flag = &sh.abort_flag;
@@ -187,12 +185,12 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         sh.abort_flag = 0;
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sh.x_full[i], 1); mbar_init(&sh.x_empty[i], 1);
-            mbar_init(&sh.z_full[i], 1); mbar_init(&sh.y_full[i], 1);
-            mbar_init(&sh.d_free[i], ru::kAluWarps); mbar_init(&sh.max_full[i], g.dc == 1 ? ru::kAluWarps : 1);
+            mbar_init(&sh.max_full[i], g.dc == 1 ? ru::kAluWarps : 1);
             mbar_init(&sh.out_full[i], ru::kAluWarps); mbar_init(&sh.out_free[i], 1);
             for (int j = 0; j < 4; ++j) { sh.qsum[i][j] = 0; mbar_init(&sh.row_full[i][j], 4); }
         }
-        mbar_init(&sh.a_ready, ru::kAluWarps);
+        mbar_init(&sh.z_full, 1); mbar_init(&sh.y_full, 1);
+        mbar_init(&sh.d_free, ru::kAluWarps); mbar_init(&sh.a_ready, ru::kAluWarps);
         fence_barrier_init();
     }
     if (warp == 2) {
@@ -210,9 +208,8 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     griddep_wait();                                   // x may be the output of the preceding kernel
     if (p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0) n = 0;      // the call already failed
 
-    // barrier and phase of step i's accumulator
-    auto acc_of = [](int i) { return TWO ? 0 : i & 1; };
-    auto phase_of = [](int i) { return (uint32_t)((TWO ? i : i >> 1) & 1); };
+    // phase of step i's accumulators
+    auto phase_of = [](int i) { return (uint32_t)(i & 1); };
     if (warp < 4) {
     set_regs_dec<ru::kRegsControl>();
     if (warp == 0) {
@@ -244,24 +241,23 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 const int b = g.xb == 2 ? i & 1 : 0;
                 const uint32_t use = (uint32_t)(g.xb == 2 ? i >> 1 : i);
                 if (!wait_or_abort(&sh.x_full[b], use & 1u, abort_flag)) { give_up(p.status, abort_flag, 0x220); return false; }
-                if (i >= (TWO ? 1 : 2) && !wait_or_abort(&sh.d_free[acc_of(i)], phase_of(i) ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x221); return false; }
+                if (i >= 1 && !wait_or_abort(&sh.d_free, phase_of(i) ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x221); return false; }
                 tc_fence_after();
                 const uint64_t xd = d_x + (uint64_t)((uint32_t)(b * g.atoms2) * blkx);
                 for (int term = 2; term >= 0; --term)
                     for (int k = 0; k < ks2; ++k) {
-                        const int h = TWO ? k >= half2 : i & 1;
+                        const int h = k >= half2;
                         const uint32_t d = tmem + (uint32_t)(h * g.ntot);
-                        const uint32_t acc = (term == 2 && (k == 0 || (TWO && k == half2))) ? 0u : 1u;
+                        const uint32_t acc = (term == 2 && (k == 0 || k == half2)) ? 0u : 1u;
                         mma_f16_ss(d, d_p2 + (uint64_t)((uint32_t)(term * g.atoms2 + (k >> 1)) * blk2 + 2u * (k & 1)),
                                    xd + (uint64_t)((uint32_t)(k >> 1) * blkx + 2u * (k & 1)), idesc_a, acc);
                     }
                 tc_commit(&sh.x_empty[b]);
-                tc_commit(&sh.z_full[acc_of(i)]);
+                tc_commit(&sh.z_full);
                 return true;
             };
-            bool ok = n > 0 && (TWO || put_z(0));
-            for (int i = 0; i < n && ok; ++i) {
-                if (TWO ? !put_z(i) : i + 1 < n && !put_z(i + 1)) break;
+            for (int i = 0; i < n; ++i) {
+                if (!put_z(i)) break;
                 if (!wait_or_abort(&sh.a_ready, (uint32_t)(i & 1), abort_flag)) { give_up(p.status, abort_flag, 0x222); break; }
                 tc_fence_after();
                 for (int tk = 0; tk < g.tps; ++tk) {
@@ -270,14 +266,14 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
 #pragma unroll 1
                     for (int q = 0; q < 3; ++q)
                         for (int k = 0; k < ks1; ++k) {
-                            const int h = TWO ? k >= half1 : i & 1;
+                            const int h = k >= half1;
                             const uint32_t d = tmem + (uint32_t)(h * g.ntot + tk * g.np);
                             mma_f16_ts(d, a + (q == 0 ? (uint32_t)(g.ntot >> 1) : 0u) + 8u * k,
                                        d_p1 + (uint64_t)((uint32_t)((q == 1 ? g.atoms1 : 0) + (k >> 1)) * blk1 + 2u * (k & 1)), idesc_c,
-                                       (q == 0 && (k == 0 || (TWO && k == half1))) ? 0u : 1u);
+                                       (q == 0 && (k == 0 || k == half1)) ? 0u : 1u);
                         }
                 }
-                tc_commit(&sh.y_full[acc_of(i)]);
+                tc_commit(&sh.y_full);
             }
         }
     } else if (warp == 3) {
@@ -334,13 +330,13 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             float y[NC * 8];
             if (i > 0) {
                 // ---- Y of the step before to registers; its extremes to the token's other warps
-                if (!warp_wait(&sh.y_full[acc_of(i - 1)], phase_of(i - 1), abort_flag)) { give_up(p.status, abort_flag, 0x230); ok = false; break; }
+                if (!warp_wait(&sh.y_full, phase_of(i - 1), abort_flag)) { give_up(p.status, abort_flag, 0x230); ok = false; break; }
                 tc_fence_after();
-                const uint32_t src = tmem + lane_addr + (uint32_t)(acc_of(i - 1) * g.ntot + wc * cw);
-                if (some) load_sums<NC, TWO>(src, (uint32_t)g.ntot, cw, y);
+                const uint32_t src = tmem + lane_addr + (uint32_t)(wc * cw);
+                if (some) load_sums<NC>(src, (uint32_t)g.ntot, cw, y);
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&sh.d_free[acc_of(i - 1)]);
+                if (lane == 0) mbar_arrive(&sh.d_free);
                 const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
                 f1 = pow2f(ey1);
                 if (__any_sync(0xFFFFFFFFu, ey2 != 0)) {          // scales at the ends of fp32's range
@@ -399,12 +395,12 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 // ---- Z of this step: the power of two of every row, then its two fp16 terms, in place of the step before's (whose
                 // MMAs have completed: this warp has seen Y above)
                 const int zi = i & 1;
-                if (!warp_wait(&sh.z_full[acc_of(i)], phase_of(i), abort_flag)) { give_up(p.status, abort_flag, 0x231); return false; }
+                if (!warp_wait(&sh.z_full, phase_of(i), abort_flag)) { give_up(p.status, abort_flag, 0x231); return false; }
                 tc_fence_after();
-                const uint32_t src = tmem + lane_addr + (uint32_t)(acc_of(i) * g.ntot + wc * cw);
+                const uint32_t src = tmem + lane_addr + (uint32_t)(wc * cw);
                 // (read twice, two chunks at a time: with all of Z in registers over the exchange they do not suffice)
                 float z[16];
-                auto load_two = [&](int j) { load_sums<2, TWO>(src + 8 * j, (uint32_t)g.ntot, cw - 8 * j, z); };
+                auto load_two = [&](int j) { load_sums<2>(src + 8 * j, (uint32_t)g.ntot, cw - 8 * j, z); };
                 if (some) {
                     float m = 0.f;
 #pragma unroll
@@ -604,14 +600,13 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 }
                 return true;
             };
-            if (!TWO && i < n && !convert()) { ok = false; break; }
             if (i > 0) {
                 if (!finish()) { ok = false; break; }
                 if (g.staged) fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh.out_full[pi]);
             }
-            if (TWO && i < n && !convert()) { ok = false; break; }
+            if (i < n && !convert()) { ok = false; break; }
         }
         if (!ok) *abort_flag = 1;
     }
@@ -627,15 +622,8 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
 }
 
 typedef void (*Kernel)(const CUtensorMap, const RotUmmaParams);
-template <int MODE>
-static Kernel pick_rot_umma(const RotUmmaGeom& g) {
-    return g.two ? rot_umma_kernel<5, MODE, true> : g.ntot <= 128 ? rot_umma_kernel<4, MODE, false> : rot_umma_kernel<5, MODE, false>;
-}
-
-bool rot_umma_supports(const RotGeom& base, int64_t M, int n_problems, const RotProblem* problems) {
-    // More CTAs than SMs: fewer tokens are spread over warps and CTAs one by one (rot_mma.cu), which is the shorter way for one token
-    // as long as every CTA has an SM of its own.
-    if (M * n_problems * base.dc <= sm_count()) return false;
+bool rot_umma_supports(const RotGeom& base, int n_problems, const RotProblem* problems) {
+    if (rot_mma_always(base)) return false;
     for (int i = 0; i < n_problems; ++i)
         if (problems[i].digits || problems[i].packed) return false;
     RotUmmaGeom u;
@@ -659,7 +647,7 @@ int launch_rot_umma(const RotGeom& base, const void* x, int64_t M, int64_t ldx, 
         if (st != BWLA_OK) return st;
     }
     const int mode = problems[0].yhat ? kBf16 : asym ? kAsym : kSym;
-    const Kernel k = mode == kSym ? pick_rot_umma<kSym>(g) : mode == kAsym ? pick_rot_umma<kAsym>(g) : pick_rot_umma<kBf16>(g);
+    const Kernel k = mode == kSym ? rot_umma_kernel<kSym> : mode == kAsym ? rot_umma_kernel<kAsym> : rot_umma_kernel<kBf16>;
     const int room = resident_clusters((const void*)k, g.dc, ru::kThreads, (size_t)g.total) / n_problems;
     if (room < 1) return cuda_fail(cudaErrorInvalidConfiguration);
     p.clusters_per_problem = (int)std::min<int64_t>((M + g.tps - 1) / g.tps, room);

@@ -103,14 +103,17 @@ def test_operands_of_the_rotations_lie_inside_the_block(tmp_path):
             if (n1 * n2 % 32 || n1 * n2 > 25600 || !rot_geometry(n1, n2, &g)) continue;
             ++seen;
             if (!check(g)) return 0;
-            for (int clusters = 1; clusters <= 148; ++clusters)
-                if (!check(few_tokens_geometry(g, clusters, 148))) return 0;
+            for (int clusters = 1; clusters <= 148; ++clusters) {
+                RotGeom few = g;
+                if (few_tokens_geometry(g, &few, [&](const RotGeom& t) { return clusters * t.dc <= 148; }) && (clusters * few.dc > 148 || !check(few))) return 0;
+            }
+            if (rot_okt_factors(g) && (n1 > 128 || n2 > 128 || rot_mma_always(g))) { std::printf("%d x %d: okt_umma.cu does not take them\\n", n1, n2); return 0; }
             for (int size = 1; size <= 2; ++size) {
                 RotUmmaGeom u{};
                 if (!rot_umma_geometry(g, size, &u)) continue;
                 const int ks2 = n2 / 16, ks1 = u.nc / 16;
                 if (u.total > kRotMaxSmem || u.p1_off - u.dt * 64 + 128 * 64 > u.total || 3 * u.ntot > 512 || u.dc * u.dt < n2 ||
-                    (u.two && ((ks2 + 1) / 2 >= ks2 || (ks1 + 1) / 2 >= ks1))) { std::printf("%d x %d on tcgen05\\n", n1, n2); return 0; }
+                    (ks2 + 1) / 2 >= ks2 || (ks1 + 1) / 2 >= ks1) { std::printf("%d x %d on tcgen05\\n", n1, n2); return 0; }
             }
         }
     if (seen < 2000) std::printf("only %ld pairs\\n", seen);""") == ""
