@@ -304,6 +304,9 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
     };
     // acc += (one or two steps of 16 values of the contraction) A terms x B, in chains that start from zero with the smallest
     // products, two column tiles side by side.  `terms` lists (A term, B fragments) from small to large.
+    // Up to 32 columns the splits are a large part of the error: chains are 16 values long, the second contraction's small products have one
+    // of their own, with lo lo among them (32 x 32: 1.45e-7 -> 1.14e-7 of a row's 2-norm, six bf16 products 1.17e-7; one token 3.7 -> 3.8 us).
+    constexpr bool FINE = !EXCH && NTW <= 4;
     float acc[NTW][4];
     auto clear = [&]() {
 #pragma unroll
@@ -344,9 +347,12 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             }
         };
         int kk = 0;
+        if constexpr (!FINE) {
 #pragma unroll 1
-        for (; kk + 1 < ksteps2; kk += 2) step(kk, std::true_type{});
-        if (kk < ksteps2) step(kk, std::false_type{});
+            for (; kk + 1 < ksteps2; kk += 2) step(kk, std::true_type{});
+        }
+#pragma unroll 1
+        for (; kk < ksteps2; ++kk) step(kk, std::false_type{});
     };
     // acc += (terms of Z^T, one or two steps of 16 values of a) times the terms of P1: lo hi, hi lo, hi hi
     auto stage_c = [&](int kk, auto two_, const uint32_t (*zh)[4], const uint32_t (*zl)[4]) {
@@ -361,6 +367,19 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
                 load_b(fl[h], at + part1, j + 1 < NTW);
             }
             float t[2][4];
+            if constexpr (FINE) {
+                float u[2][4];
+#pragma unroll
+                for (int jj = 0; jj < 2; ++jj) {
+                    mma_16816<true>(u[jj], zl[0], fl[0][2 * jj], fl[0][2 * jj + 1], zero4);
+                    mma_16816<true>(u[jj], zl[0], fh[0][2 * jj], fh[0][2 * jj + 1], u[jj]);
+                    mma_16816<true>(u[jj], zh[0], fl[0][2 * jj], fl[0][2 * jj + 1], u[jj]);
+                    mma_16816<true>(t[jj], zh[0], fh[0][2 * jj], fh[0][2 * jj + 1], zero4);
+                    add4(t[jj], u[jj]);
+                    add4(acc[j + jj], t[jj]);
+                }
+                continue;
+            }
 #pragma unroll
             for (int q = 0; q < 3; ++q)
 #pragma unroll
@@ -469,8 +488,8 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         if (row_lo_ok) {
             if (!EXCH) {
 #pragma unroll
-                for (int kk = 0; kk < NTW / 2; kk += 2) {
-                    if (kk + 1 < NTW / 2) stage_c(kk, std::true_type{}, &zh[kk], &zl[kk]);
+                for (int kk = 0; kk < NTW / 2; kk += FINE ? 1 : 2) {
+                    if (!FINE && kk + 1 < NTW / 2) stage_c(kk, std::true_type{}, &zh[kk], &zl[kk]);
                     else stage_c(kk, std::false_type{}, &zh[kk], &zl[kk]);
                 }
             } else {

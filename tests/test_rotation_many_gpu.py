@@ -52,7 +52,7 @@ def test_edges(n1, n2, M, prepared):
     assert torch.equal(out.view(torch.int16), again.view(torch.int16))
 
 
-@pytest.mark.parametrize("n1,n2,most", [(48, 64, 1.60), (64, 64, 1.75), (64, 80, 1.80), (64, 88, 2.05), (64, 128, 2.40), (86, 128, 2.60),
+@pytest.mark.parametrize("n1,n2,most", [(32, 32, 1.17), (32, 64, 1.36), (48, 64, 1.60), (64, 64, 1.75), (64, 80, 1.80), (64, 88, 2.05), (64, 128, 2.40), (86, 128, 2.60),
                                         (96, 96, 2.25), (108, 128, 2.75), (112, 128, 2.75), (128, 128, 2.80), (160, 160, 3.20)])
 def test_error_against_64_bits(n1, n2, most):
     """Root mean square over 300 tokens of the error's 2-norm over the row's, in 1e-7: what the sums of six bf16 products, accumulated in one
