@@ -259,9 +259,16 @@ int bwla_w1a_gemm_codes(const int8_t* codes, const float* scales, int64_t M, int
     const int path = resolve_path(M, K, N, r, bits);
 
     int8_t* inter = (path == BWLA_PATH_I8) ? (int8_t*)(base + ws.codes) : nullptr;
+    // (T on tcgen05 goes first: its partial sums lie where the codes go)
+    const OktLowrank lr{V_bf16, r, Thl, nullptr, nullptr, (float*)(base + ws.codes)};
+    const bool many = r > 0 && M > 64 && lowrank_umma_takes(x_bf16, M, K, ldx, lr);
+    if (many) {
+        st = launch_lowrank_umma(x_bf16, M, K, ldx, 1, &lr, (uint32_t*)(base + ws.status), s);
+        if (st != BWLA_OK) return st;
+    }
     st = launch_prepare_codes(codes, M, K, inter, qsum, s);
     if (st != BWLA_OK) return st;
-    if (r > 0) {
+    if (r > 0 && !many) {
         st = launch_prologue(x_bf16, M, K, ldx, nullptr, 0, nullptr, 0, bits, nullptr, 0, nullptr, nullptr, V_bf16, r, Thl,
                              (float*)(base + ws.lr_part), (uint32_t*)(base + ws.status), s);
         if (st != BWLA_OK) return st;

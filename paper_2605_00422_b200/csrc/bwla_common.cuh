@@ -82,6 +82,7 @@ constexpr int kLrCounterWord = 4;        // first of the arrival counters of spl
 // T = V x for many tokens on the tensor cores (lowrank_umma.cu), for the problems of one group (all share x, M, K; every entry of
 // `lowrank` has V, Thl and, where partial sums are needed, umma_part set).
 struct OktLowrank;
+bool lowrank_umma_takes(const void* x, int64_t M, int64_t K, int64_t ldx, const OktLowrank& lowrank);
 int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_problems, const OktLowrank* lowrank,
                         uint32_t* status, cudaStream_t stream);
 
@@ -100,7 +101,7 @@ inline Workspace workspace_layout(int64_t M, int64_t K, int64_t N, int r, int bi
     w.T = off;      off += align_up((size_t)M * lr_cols * 6, 256);     // bf16 [3][M][cols]
     w.lr_part = off; off += r > 0 ? lowrank_split_bytes(M, lowrank_cols(r)) : 0;
     // (the tcgen05 kernel for T leaves its partial sums where the rotation behind it puts the codes)
-    w.codes = off;  off += align_up(std::max((size_t)M * (size_t)K, lowrank_umma_part_bytes(M, K, r)), 256);
+    w.codes = off;  off += align_up((size_t)M * (size_t)K, 256);
     (void)N; (void)bits;
     w.total = off;
     return w;

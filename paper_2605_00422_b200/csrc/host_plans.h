@@ -25,7 +25,8 @@ constexpr int kLrKSplitMax = 16;
 constexpr int kLrSplitTiles = 8;
 constexpr int kLrTileTok = 16;           // tokens of a tile
 
-inline int lowrank_tile_cols(int64_t M) { return M > 32 ? 32 : 16; }
+// (beyond 64 tokens K is not split, and narrow tiles fill more SMs)
+inline int lowrank_tile_cols(int64_t M) { return M > 32 && M <= 64 ? 32 : 16; }
 inline int64_t lowrank_tiles(int64_t M, int lr_cols) {
     const int cols = lowrank_tile_cols(M);
     return ((lr_cols + cols - 1) / cols) * ((M + kLrTileTok - 1) / kLrTileTok);
@@ -54,17 +55,16 @@ constexpr int kLruMaxParts = 16;         // parts of K per token tile
 constexpr int kLruTargetCtas = 160;      // parts are chosen so that tiles x parts comes near this, every part at least eight stages long
 inline int64_t lowrank_umma_tiles(int64_t M) { return (M + kLruTok - 1) / kLruTok; }
 inline int lowrank_umma_parts(int64_t M, int64_t K) {
-    int64_t ks = std::max<int64_t>(1, kLruTargetCtas / lowrank_umma_tiles(M));
-    ks = std::min<int64_t>(ks, kLruMaxParts);
-    return (int)std::min<int64_t>(ks, std::max<int64_t>(1, K / (8 * kLruBlockK)));
+    const int64_t tiles = lowrank_umma_tiles(M);
+    int64_t ks = std::min<int64_t>(std::max<int64_t>(1, kLruTargetCtas / tiles), kLruMaxParts);
+    ks = std::min<int64_t>(ks, std::max<int64_t>(1, K / (8 * kLruBlockK)));
+    return (int)std::min<int64_t>(ks, std::max<int64_t>(1, M * K / (tiles * kLruCols * kLruTok * 4)));      // (their room: below)
 }
-inline bool lowrank_umma_supports(int64_t M, int64_t K, int r) {
-    return M > 64 && r > 0 && r <= kLruCols && K % kLruBlockK == 0;
-}
+// Which problems it takes; which of them go to it, launch_rot decides.
+inline bool lowrank_umma_supports(int64_t K, int r) { return r > 0 && r <= kLruCols && K % kLruBlockK == 0; }
 // Bytes of its partial sums.  They lie where the rotation that follows it leaves the codes (or the rotated values) and are never
-// larger than those: 256 bytes a column of 128 tokens against 128 values of K / 512 parts at the least.
-inline size_t lowrank_umma_part_bytes(int64_t M, int64_t K, int r) {
-    if (!lowrank_umma_supports(M, K, r)) return 0;
+// larger than those.
+inline size_t lowrank_umma_part_bytes(int64_t M, int64_t K) {
     const int ks = lowrank_umma_parts(M, K);
     return ks > 1 ? (size_t)lowrank_umma_tiles(M) * ks * kLruCols * kLruTok * 4 : 0;
 }
@@ -140,16 +140,19 @@ inline bool rot_geometry(int n1, int n2, RotGeom* out) {
 // Few tokens: what counts is the time of one token, so it is spread over more warps (up to 64 columns: two warps instead of
 // one) and over more CTAs: MMAs of a CTA at 2 cycles each, against about 5000 cycles for the cluster's barriers and its later start
 // (64 x 128, one token: 6.7 us on eight CTAs, 5.2 on one).  `resident(geometry)`: every token finds a cluster at once; false when no
-// split has that (a second round of clusters doubles the time: 128 x 128, 16 tokens in clusters of eight 23.6 us).
+// split has that (a second round of clusters doubles the time: 128 x 128, 16 tokens in clusters of eight 23.6 us).  `raw`: every CTA
+// splits all of P1 and its rows of P2 first, a pair of values in about 220 cycles a thread (one token of 108 x 128: 23 us on two warps in
+// each of eight CTAs, 14 on sixteen warps in one).
 template <typename Resident>
-inline bool few_tokens_geometry(const RotGeom& base, RotGeom* out, Resident resident) {
+inline bool few_tokens_geometry(const RotGeom& base, bool raw, RotGeom* out, Resident resident) {
     double best_cost = 0.0;
     const int ksteps = base.n2p / 16 + base.na / 2;
     for (int dc = 1; dc <= 8; ++dc) {
         RotGeom t = base;
         if (t.na > 4 && t.na <= 8) { t.cw = 2; t.ntw = 4; }
         if (!rot_layout(t, dc, 0, base.pad) && (t.cw == 1 || !rot_layout(t, dc, 1, base.pad))) continue;
-        const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 5000.0 + 300.0 * dc : 0.0);
+        const int pairs = t.dtc * 8 * t.n2p + 32 * t.na * t.na;
+        const double cost = 2.0 * 3.0 * t.dtc * t.na * ksteps + (dc > 1 ? 5000.0 + 300.0 * dc : 0.0) + (raw ? 220.0 * pairs / (32 * t.warps) : 0.0);
         if ((best_cost == 0.0 || cost < best_cost) && resident(t)) { best_cost = cost; *out = t; }
     }
     return best_cost != 0.0;

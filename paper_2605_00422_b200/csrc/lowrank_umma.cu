@@ -231,6 +231,12 @@ __global__ void __launch_bounds__(lru::kTok) lowrank_reduce_kernel(const LrUmmaP
 // ---------------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------------
+// x and V in 16-byte pieces, and room for the partial sums where there are any
+bool lowrank_umma_takes(const void* x, int64_t M, int64_t K, int64_t ldx, const OktLowrank& l) {
+    return lowrank_umma_supports(K, l.r) && rot_accepts_x(x, ldx) && (reinterpret_cast<uintptr_t>(l.V) & 15) == 0 &&
+           (l.umma_part || lowrank_umma_part_bytes(M, K) == 0);
+}
+
 int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_problems, const OktLowrank* lowrank,
                         uint32_t* status, cudaStream_t stream) {
     using namespace lru;

@@ -320,9 +320,10 @@ okt_umma_kernel(const __grid_constant__ CUtensorMap x_map, const OktKernelParams
     if (!pr.okt) {
         // raw factors: every CTA splits what it needs of them, into the places where prepare_okt_kernel's terms would be copied
         auto place = [](uint8_t* at, int rows, int atom) {
+            const int sh = 31 - __clz(atom);
             return [=](int r, int k2) {
-                const int j = 4 * k2 / atom;
-                return at + (size_t)j * rows * atom + okt_swizzle((uint32_t)(r * atom + 4 * k2 - j * atom), atom);
+                const int j = (4 * k2) >> sh;
+                return at + ((j * rows) << sh) + okt_swizzle((uint32_t)(((r - j) << sh) + 4 * k2), atom);
             };
         };
         split_factor<false>(pr.P2, g.n2, d0, g.dt_rows, g.n2p, 1.f, place(p2t, g.dt_rows, g.atom2), (size_t)g.dt_rows * g.n2p * 2, threadIdx.x, kOktThreads);

@@ -876,34 +876,32 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
     if (M == 0 || n_problems == 0) return BWLA_OK;
     if (n_problems > kRotMaxProblems || M >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
     const bool vec = rot_accepts_x(x, ldx);
-    // ---- T = V x.  Many tokens: for all linears, as a launch of its own on the tcgen05 tensor cores.  Every kernel of the chain waits for
-    //      its predecessor before it ends, so the contraction still finds T complete. ----
+    // ---- T = V x: beside the rotation, or before it in launches of its own.  Every kernel of the chain waits for its predecessor before it
+    //      ends, so the contraction still finds T complete. ----
     OktLowrank beside[kRotMaxProblems] = {};          // what is left for blocks of the rotation's own launch
-    if (lowrank) {
+    bool any = false;
+    for (int i = 0; lowrank && i < n_problems; ++i)
+        if (lowrank[i].V && lowrank[i].r > 0 && lowrank[i].Thl) { beside[i] = lowrank[i]; any = true; }
+    // on the tcgen05 tensor cores, for all linears that it takes at once
+    auto on_tcgen05 = [&]() -> int {
         OktLowrank batch[kRotMaxProblems];
         int nb = 0;
+        any = false;
         for (int i = 0; i < n_problems; ++i) {
-            if (!lowrank[i].V || lowrank[i].r <= 0 || !lowrank[i].Thl) continue;
-            if (lowrank_umma_supports(M, base.K, lowrank[i].r) && vec && (reinterpret_cast<uintptr_t>(lowrank[i].V) & 15) == 0 &&
-                (lowrank[i].umma_part || lowrank_umma_part_bytes(M, base.K, lowrank[i].r) == 0))
-                batch[nb++] = lowrank[i];
-            else
-                beside[i] = lowrank[i];
+            if (!beside[i].V) continue;
+            if (lowrank_umma_takes(x, M, base.K, ldx, beside[i])) { batch[nb++] = beside[i]; beside[i] = OktLowrank{}; }
+            else any = true;
         }
-        if (nb > 0) {
-            const int st = launch_lowrank_umma(x, M, base.K, ldx, nb, batch, status, stream);
-            if (st != BWLA_OK) return st;
-        }
-    }
-    // T of linears without blocks beside the rotation, as a launch of its own: wide tiles (their registers do not fit), rows that do not
-    // start on 16 bytes (their blocks want more warps than a token has), or `all`
+        return nb > 0 ? launch_lowrank_umma(x, M, base.K, ldx, nb, batch, status, stream) : BWLA_OK;
+    };
+    // as blocks of a launch of their own: `all`, or the wide tiles, whose registers do not fit beside the rotation
     auto own_launch = [&](bool all) -> int {
         for (int i = 0; i < n_problems; ++i) {
             if (!beside[i].V) continue;
             PrologueParams probe{};
             size_t bytes = 0;
             plan_lowrank(probe, x, M, base.K, ldx, beside[i], kRotMaxWarps, kRotMaxSmem, &bytes);
-            if (!all && (probe.lr_wide == 2 || probe.lr_wide == 4)) continue;
+            if (!all && probe.lr_wide != 3) continue;
             const int st = launch_prologue(x, M, base.K, ldx, nullptr, 0, nullptr, 0, bits, nullptr, 0, nullptr, nullptr, beside[i].V, beside[i].r,
                                            beside[i].Thl, beside[i].lr_part, beside[i].lr_count ? beside[i].lr_count - kLrCounterWord : nullptr, stream);
             if (st != BWLA_OK) return st;
@@ -911,25 +909,32 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
         }
         return BWLA_OK;
     };
+    int st = M > 64 ? on_tcgen05() : BWLA_OK;
+    if (st != BWLA_OK) return st;
     // ---- the kernel: while the device holds a cluster for every token, mma.sync, spread for the time of one token ----
     RotGeom g = base;
-    const bool few = M * n_problems <= sm_count() && few_tokens_geometry(base, &g, [&](const RotGeom& t) {
-        return t.dc == 1 || M * n_problems <= resident_clusters((const void*)rot_kernel_of(t, problems[0]), t.dc, 32 * t.warps, (size_t)(t.group_off + t.group_bytes));
+    const bool few = M * n_problems <= sm_count() && few_tokens_geometry(base, !problems[0].prepared, &g, [&](const RotGeom& t) {
+        // (behind another kernel a cluster finds its place later than single CTAs do, where these are possible half of the SMs must be
+        // left: 32 tokens of 108 x 128 in clusters of four 36 us a call, in CTAs 28)
+        return t.dc == 1 || ((base.dc > 1 || 2 * M * n_problems * t.dc <= sm_count()) && M * n_problems <= resident_clusters((const void*)rot_kernel_of(t, problems[0]), t.dc, 32 * t.warps, (size_t)(t.group_off + t.group_bytes)));
     });
     if (!few && vec) {
         bool okt = rot_okt_factors(base) && !problems[0].yhat && !problems[0].digits;
         for (int i = 0; i < n_problems; ++i) okt = okt && (problems[i].okt || !problems[i].prepared);
         OktGeom og;
         if (okt && okt_geometry(base.n1, base.n2, &og)) {
-            const int st = own_launch(false);
+            st = own_launch(false);
             return st != BWLA_OK ? st : launch_okt(og, x, M, ldx, bits, asym, n_problems, problems, beside, status, stream);
         }
-        if (rot_umma_supports(base, n_problems, problems)) {
-            const int st = own_launch(true);
+        // (which has no blocks for T beside it: with those, up to 64 tokens, the rounds of mma.sync are shorter than two more launches unless a
+        // token takes a cluster; three linears with rank 64, 64 tokens: 64 x 128 39 | 52 us, 160 x 160 92 | 81)
+        if (rot_umma_supports(base, n_problems, problems) && !(any && base.dc == 1)) {
+            st = on_tcgen05();
+            if (st == BWLA_OK) st = own_launch(true);
             return st != BWLA_OK ? st : launch_rot_umma(base, x, M, ldx, bits, asym, n_problems, problems, status, stream);
         }
     }
-    const int st = own_launch(false);
+    st = own_launch(false);
     if (st != BWLA_OK) return st;
     RotKernelParams p{};
     p.g = g; p.x = x; p.ldx = ldx; p.x_vec = vec; p.M = M; p.bits = bits; p.asym = asym; p.n_problems = n_problems;
