@@ -97,3 +97,13 @@ def test_one_weight_only_workspace_serves_smaller_batches():
     ws = torch.zeros(bwla.bwla_w1a16_workspace_bytes(layer, 40), dtype=torch.uint8, device="cuda")
     bwla.bwla_layer_w1a16_linear(layer, H.bf16_to_dev(gen.make_activations(0, sh, 32)), workspace=ws)
     assert bwla.bwla_check_status(ws) == 0
+
+
+def test_sums_of_codes_beyond_their_bit_width():
+    """65536 codes of 127 declared as 4 bits: 8.3 million, beyond the short epilogue's 2^22."""
+    from paper_2605_00422_b200 import bwla
+    M, K, N = 65, 65536, 64
+    codes = torch.full((M, K), 127, dtype=torch.int8, device="cuda")
+    words = torch.full((N, K // 32), -1, dtype=torch.int32, device="cuda")
+    out, _ = bwla.bwla_w1a_gemm_codes(codes, torch.ones(M, device="cuda"), 4, words, torch.ones(N, device="cuda"))
+    assert torch.all(out.float() == torch.tensor(127.0 * K).bfloat16().float().item())
