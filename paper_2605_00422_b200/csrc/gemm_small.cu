@@ -259,7 +259,10 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                 qsf = fmaf((float)q2, 65536.f, (float)(256 * q1 + q0));
             }
             if (live && pr.out) {
-                const float y = fmaf(__fmul_rn(w.mu[h], sc), qsf, __fmul_rn(__fmul_rn(w.al[h], sc), accf) + (lr[0][i] + (lr[1][i] + lr[2][i])));
+                const float low = lr[0][i] + (lr[1][i] + lr[2][i]);
+                float y;
+                if constexpr (PL == 1) y = fmaf(__fmul_rn(w.mu[h], sc), qsf, __fmul_rn(__fmul_rn(w.al[h], sc), accf) + low);
+                else y = fmaf(w.mu[h], __fmul_rn(qsf, sc), __fmul_rn(w.al[h], __fmul_rn(accf, sc)) + low);      // (sc: a power of two, may be subnormal)
                 pr.out[(int64_t)t * pr.ldo + n] = __float2bfloat16_rn(y);
             }
         }

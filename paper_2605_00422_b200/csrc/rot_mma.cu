@@ -665,8 +665,8 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             // within 2^-23 of it: what an fp32 sum of the values would round away.  (A token with an infinity or a NaN in it
             // gets a NaN scale.)
             const uint32_t top = slots_max(sh.amax[par]);
-            const int es = min(21 - exponent_of(__uint_as_float(top)), 126);
-            const float mult = pow2f(es);
+            const int es = 21 - exponent_of(__uint_as_float(top)), es2 = max(es - 126, 0);      // (to 148: in two factors)
+            const float mult = pow2f(min(es, 126)), mult2 = pow2f(es2);
             const int64_t plane = p.M * (int64_t)g.K;
             int8_t* ct = pr.codes + t * (int64_t)g.K;
             const int tile_step = 8 * g.n2;
@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
                 int q0[4], q1[4], q2[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    q0[i] = __float_as_int(__fadd_rn(acc[j][i] * mult, 12582912.f)) - 0x4B400000;      // (the product is exact)
+                    q0[i] = __float_as_int(__fadd_rn(acc[j][i] * mult * mult2, 12582912.f)) - 0x4B400000;      // (the products are exact)
                     q1[i] = (q0[i] + 128) >> 8;
                     q2[i] = (q1[i] + 128) >> 8;
                 }
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
                 const int local = __reduce_add_sync(0xFFFFFFFFu, d[pl]);
                 if (lane == 0 && local != 0) atomicAdd(&sh.qsum[par][pl], local);
             }
-            if (tid == 0 && rank == 0) pr.scales[t] = top >= 0x7F800000u ? __uint_as_float(0x7FC00000u) : pow2f(-es);
+            if (tid == 0 && rank == 0) pr.scales[t] = top >= 0x7F800000u ? __uint_as_float(0x7FC00000u) : pow2f(es2 - es) * pow2f(-es2);
         } else if (MODE == kRotBf16) {
             // the weight-only operating point: bf16 values (layout 1: inside each group of 32, position 2 (k % 16) +
             // (k % 32) / 16), and where asked for their sum

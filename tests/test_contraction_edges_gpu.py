@@ -107,3 +107,20 @@ def test_sums_of_codes_beyond_their_bit_width():
     words = torch.full((N, K // 32), -1, dtype=torch.int32, device="cuda")
     out, _ = bwla.bwla_w1a_gemm_codes(codes, torch.ones(M, device="cuda"), 4, words, torch.ones(N, device="cuda"))
     assert torch.all(out.float() == torch.tensor(127.0 * K).bfloat16().float().item())
+
+
+@pytest.mark.parametrize("e", [-100, -118, -122])
+def test_weight_only_tokens_near_the_end_of_the_exponent_range(e):
+    """Tokens of 2^e (values stay normal numbers), scales of 2^60: the fixed-point digits keep their 23 bits; outputs to bf16's rounding."""
+    from paper_2605_00422_b200 import bwla
+    n1, n2, K, N, M = 32, 64, 2048, 64, 3
+    rng = np.random.default_rng(-e)
+    P1, P2 = H.f32_to_dev(gen.orthogonal_f32(n1, rng)), H.f32_to_dev(gen.orthogonal_f32(n2, rng))
+    x = (torch.from_numpy(rng.standard_normal((M, K)).astype(np.float32)).cuda().double() * 2.0 ** e).bfloat16()
+    words = torch.from_numpy(rng.integers(-2 ** 31, 2 ** 31, size=(N, K // 32), dtype=np.int64).astype(np.int32)).cuda()
+    layer = bwla.Layer(P1, P2, 8, words, torch.full((N,), 2.0 ** 60, device="cuda"))
+    out = bwla.bwla_layer_w1a16_linear(layer, x).double()
+    bits = (words.unsqueeze(-1) >> torch.arange(32, device="cuda", dtype=torch.int32)) & 1
+    Y = (P1.double().t() @ x.double().view(M, n1, n2) @ P2.double()).reshape(M, K)
+    want = (Y @ (2.0 * bits.reshape(N, K).double() - 1.0).t()) * 2.0 ** 60
+    assert float((out - want).norm() / want.norm()) <= 5e-3          # two roundings to bf16 (2^-9 each at most) and their sum over K
