@@ -76,7 +76,7 @@ int bwla_pack_signs(const void* w, int dtype, int64_t N, int64_t K, int64_t ldw,
  *   packed device, uint32 [N][K/32]; alpha, mu device, fp32 [N]; all written in full
  *   workspace: 256-byte aligned device scratch of bwla_binarize_workspace_bytes(K) bytes (0 for an invalid K); the call
  *     clears its status words itself.
- * The rotation runs on the tensor-core kernel (fp32 rows as three bf16 terms, three passes); its error is below 1e-6 of
+ * The rotation runs on the tensor-core kernel (fp32 rows as three bf16 terms); its error is below 1e-6 of
  * a row's largest rotated magnitude, so a sign can differ from the exact one only where |X - mu| is below that.
  * Factor sizes that kernel does not take (n2 % 8 != 0, n2 > 256, n1 > 192) return BWLA_ERR_UNSUPPORTED.
  * N == 0 is a no-op.  Asynchronous on `stream`; bwla_check_status(workspace, stream) reports a device-side timeout.
@@ -209,8 +209,10 @@ int bwla_layer_set_activation_quant(bwla_layer* layer, int mode);
  * The weight-only operating point, W1A16 (Table 1, upper half: binarised weights, 16-bit activations), on a prepared
  * layer: the rotated activation Y = P1^T X P2 (Sec. 3.1) is rounded to bf16 instead of being quantised to integer codes,
  *   out[t][n] = bf16( alpha[n] * sum_k sign[n][k] * bf16(Y[t][k]) + U (V x_t) [+ mu[n] * sum_k bf16(Y[t][k])] ),
- * a bf16 contraction on the tensor cores with fp32 accumulation (partial sums of 128 values of k are added in rounded
- * fp32).  The layer's activation bit width and quantiser mode are not used.
+ * Up to 32 tokens (K % 128 == 0) the rounded values are contracted exactly as integers, 23-bit fixed-point numbers in units of
+ * 2^-21 of the power of two below the token's largest: values below 2^-14 of it lose low bits, by at most 2^-22 of the largest; a token with
+ * an infinity or a NaN gives NaN throughout.  Otherwise a bf16 contraction on the tensor cores with fp32 accumulation (partial sums of 512
+ * values of k are added in rounded fp32).  The layer's activation bit width and quantiser mode are not used.
  *   x_bf16 device, bf16 [M][ldx], 16-byte aligned, ldx >= K and a multiple of 8; out_bf16 device, bf16 [M][ldo], ldo >= N
  *   workspace: 256-byte aligned device scratch of bwla_w1a16_workspace_bytes(layer, M) bytes (2 to 3 bytes per
  *     activation value); its first 256 bytes must be zero before the first call; bwla_check_status reads it.
@@ -221,7 +223,7 @@ size_t bwla_w1a16_workspace_bytes(const bwla_layer* layer, int64_t M);
 int bwla_layer_w1a16_linear(const bwla_layer* layer, const void* x_bf16, int64_t M, int64_t ldx, void* out_bf16,
                             int64_t ldo, void* workspace, size_t workspace_bytes, void* stream);
 
-/* The asymmetric quantiser alone: codes device uint8 [M][K] (u), scales device fp32 [M], zeros device int32 [M] (z),
+/* The asymmetric quantiser alone (x_bf16 16-byte aligned, ldx a multiple of 8): codes device uint8 [M][K] (u), scales device fp32 [M], zeros device int32 [M] (z),
  * y_f32 device fp32 [M][K] or NULL. */
 int bwla_layer_rotate_quant_asym(const bwla_layer* layer, const void* x_bf16, int64_t M, int64_t ldx,
                                  uint8_t* codes, float* scales, int32_t* zeros, float* y_f32, void* stream);
@@ -229,7 +231,11 @@ int bwla_layer_rotate_quant_asym(const bwla_layer* layer, const void* x_bf16, in
 /*
  * Several layers that read the same activations (q, k, v of an attention block; gate and up of an MLP) in one
  * call: x is rotated and quantised for every layer (each has its own P1, P2) by one launch, and the contractions
- * follow.  All layers must have the same K, n1, n2 and bits; count <= 4.
+ * follow.  All layers must have the same K, n1, n2 and bits; count <= 4.  With the asymmetric quantiser x must be 16-byte aligned and
+ * ldx a multiple of 8 (else BWLA_ERR_UNSUPPORTED).
+ * Which kernel rotates depends on the factors and on tokens x layers against the SMs, and how K is cut for T = V x and for the bf16
+ * contraction on those and on N.  A call repeats itself bit for bit; the same token in another batch or group may get the next
+ * code where its value is within 1e-6 of full scale of a rounding boundary, and fp32 sums in another order.
  *   outs  host array of `count` device pointers, bf16 [M][ldos[i]];  ldos host array, ldos[i] >= N_i
  *   workspace: 256-byte aligned device scratch of bwla_group_workspace_bytes; its first 256 bytes must be zero
  *   before the first call (status words, as for bwla_w1ax_linear; bwla_check_status applies to it)

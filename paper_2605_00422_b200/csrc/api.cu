@@ -55,7 +55,7 @@ static bool valid_rotation_dims(int64_t K, int n1, int n2) {
 }
 
 // Up to how many tokens the bit-plane kernel is chosen over the tcgen05 one (0: never).  Measured per launch with cold
-// weights on the Qwen3-32B and LLaMA-2-7B shapes (profiles/contraction_paths_small_m.md): at these sizes both kernels are
+// weights on the Qwen3-32B and LLaMA-2-7B shapes: at these sizes both kernels are
 // bound by fixed latencies rather than by the stream of sign words, the tensor-core kernel's are the shorter ones
 // (21 against 27 microseconds for 5120 -> 25600 at one token), and the bit-plane kernel's time grows with tokens x bits.
 // It is therefore only taken where the tensor-core kernel cannot run (K not a multiple of 128, rank above 64).
@@ -63,9 +63,6 @@ static int bitplane_max_tokens(int64_t K, int64_t N, int bits) {
     (void)N; (void)bits;
     return (K % 128 != 0) ? 4 : 0;
 }
-
-// Up to how many tokens the warp-level MMA kernel (gemm_small.cu) runs the contraction.
-constexpr int kSmallTokens = 16;
 
 // Which kernel family runs the contraction.  A forced family that cannot take the shape falls back to the simple one.
 static int resolve_path(int64_t M, int64_t K, int64_t N, int r, int bits) {
@@ -362,7 +359,7 @@ int bwla_layer_rotate_quant_asym(const bwla_layer* L, const void* x_bf16, int64_
     if (!x_bf16 || !codes || !scales || !zeros || ((uintptr_t)codes & 15)) return BWLA_ERR_INVALID_ARG;
     int st = check_device();
     if (st != BWLA_OK) return st;
-    if (!L->rot) return BWLA_ERR_UNSUPPORTED;
+    if (!L->rot || !rot_accepts_x(x_bf16, ldx)) return BWLA_ERR_UNSUPPORTED;
     // the kernel keeps u - 2^(b-1) so that codes fit int8; the bias puts u and the zero point back in [0, 2^b - 1]
     RotProblem pr{};
     pr.prepared = L->prepared; pr.okt = L->okt; pr.codes = (int8_t*)codes; pr.zp = zeros; pr.code_bias = 1 << (L->bits - 1); pr.scales = scales; pr.y = y_f32;
@@ -416,7 +413,7 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < bwla_w1a16_workspace_bytes(L, M)) return BWLA_ERR_WORKSPACE;
     int st = check_device();
     if (st != BWLA_OK) return st;
-    if (!L->rot || !a16_supports(M, L->K, L->N, L->r)) return BWLA_ERR_UNSUPPORTED;
+    if (!L->rot || !rot_accepts_x(x_bf16, ldx) || !a16_supports(M, L->K, L->N, L->r)) return BWLA_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
     const A16Workspace w = a16_layout(L, M);
     char* base = (char*)workspace;
@@ -498,7 +495,8 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         path[i] = resolve_path(M, layers[i]->K, layers[i]->N, layers[i]->r, layers[i]->bits);
     }
     const bool rot = L0->rot && g_forced_rotation != BWLA_ROT_SIMT;      // (the layers share n1 and n2)
-    if (L0->asym && !rot) return BWLA_ERR_UNSUPPORTED;     // the asymmetric quantiser lives in the tensor-core rotation
+    // the asymmetric quantiser lives in the tensor-core rotation
+    if (L0->asym && (!rot || !rot_accepts_x(x_bf16, ldx))) return BWLA_ERR_UNSUPPORTED;
     if (rot) {
         RotProblem pr[kRotMaxProblems];
         OktLowrank lr[kRotMaxProblems];

@@ -242,8 +242,8 @@ int launch_gemm_simple(const GemmArgs& a, cudaStream_t stream);
 bool bitplane_supports(int64_t M, int64_t K, int64_t N, int r, int bits);
 int launch_gemm_bitplane(const GemmArgs& a, cudaStream_t stream);
 
-// Up to 64 tokens: warp-level int8 MMAs, all linears of a group (same M, K, bits; a.codes in the interleaved order) in one
-// launch.  planes == 3: three digit planes per token (the weight-only operating point, up to 32 tokens).  *taken is false, and
+// Up to kSmallTokens tokens: warp-level int8 MMAs, all linears of a group (same M, K, bits; a.codes in the interleaved order) in one
+// launch.  planes == 3: three digit planes per token (the weight-only operating point, up to kDigitTokens).  *taken is false, and
 // nothing has been launched, for shapes whose codes do not fit shared memory: those go to the tcgen05 kernels.
 bool gemm_small_fits(const GemmArgs* a, int n, int planes);
 int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStream_t stream);

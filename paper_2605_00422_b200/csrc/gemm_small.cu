@@ -1,5 +1,5 @@
-// The binary-weight contraction for a decode batch (up to 64 tokens) on warp-level int8 MMAs, every linear of a group in one
-// launch.
+// The binary-weight contraction for a decode batch (up to 16 tokens, 32 as digits) on warp-level int8 MMAs, every linear of a group in
+// one launch.
 //
 //   tot[n][t] = sum_k bit(n,k) * q[t][k],   acc = 2 tot - sum_k q[t][k] - zp[t] * rowsum[n]            (sign = 2 bit - 1)
 //   out[t][n] = bf16(alpha[n] * s_t * acc + U[n,:] . T[t,:] [+ mu[n] * s_t * sum_k (q[t][k] - zp[t])])  (Eq. 4; Sec. 3.2)
@@ -42,7 +42,7 @@ namespace small_ {
 constexpr int kWarps = 16, kThreads = 32 * kWarps;
 constexpr int kUnit = 512, kSteps = 4;                        // k per item; code rows of 128 k in it
 constexpr int kSmemMax = 232448 - 256;
-// Sub-groups the tokens of a row group are dealt to: the accumulators of 64 tokens (12 tiles of digits) do not fit one warp's
+// Sub-groups the tokens of a row group are dealt to: the accumulators of 12 tiles (the digits of 32 tokens) do not fit one warp's
 // registers (each then expands the sign bits for itself, which its MMAs cover).
 __host__ __device__ constexpr int token_parts(int NT) { return NT >= 8 ? 2 : 1; }
 }  // namespace small_
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
 // ---------------------------------------------------------------------------------------------
 struct SmallPlan { int S, run, t_off, tok_off, acc_off, smem; int clusters[kRotMaxProblems]; };
 
-static int token_tiles(int64_t M) { return M <= 8 ? 1 : M <= 16 ? 2 : M <= 32 ? 4 : 8; }
+static int token_tiles(int64_t M) { return M <= 8 ? 1 : M <= 16 ? 2 : 4; }
 
 // How many clusters of S such CTAs the device holds at once.  (Clusters are placed inside a GPC, so this is less than SMs / S:
 // asked once per size and thread.)
@@ -488,7 +488,7 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     static thread_local Known known[16];
     static thread_local int used = 0;
     const int64_t M = a[0].M, K = a[0].K;
-    if (n < 1 || n > kRotMaxProblems || M < 1 || M > (planes == 3 ? 32 : 64) || K % 128 != 0 || (planes == 3 && K > 25600)) return false;
+    if (n < 1 || n > kRotMaxProblems || M < 1 || M > (planes == 3 ? kDigitTokens : kSmallTokens) || K % 128 != 0 || (planes == 3 && K > 25600)) return false;
     Key k{};
     for (int i = 0; i < n; ++i) {
         if (a[i].N < 1 || a[i].N > ((int64_t)1 << 30) || a[i].r > kLowrankPad || M * a[i].N >= (int64_t)1 << 31) return false;
@@ -580,12 +580,7 @@ int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStr
             default: return launch_small_nt<4, 3>(p, grid, pl.smem, stream);
         }
     }
-    switch (NTP) {
-        case 1: return launch_small_nt<1, 1>(p, grid, pl.smem, stream);
-        case 2: return launch_small_nt<2, 1>(p, grid, pl.smem, stream);
-        case 4: return launch_small_nt<4, 1>(p, grid, pl.smem, stream);
-        default: return launch_small_nt<8, 1>(p, grid, pl.smem, stream);
-    }
+    return NTP == 1 ? launch_small_nt<1, 1>(p, grid, pl.smem, stream) : launch_small_nt<2, 1>(p, grid, pl.smem, stream);
 }
 
 }  // namespace bwla

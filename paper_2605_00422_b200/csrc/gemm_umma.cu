@@ -679,7 +679,8 @@ int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStr
 
     dim3 grid((unsigned)row_tiles, (unsigned)tok_tiles, (unsigned)split);
     switch (n_tok) {
-                case 16: return wide_split ? launch_umma_t<16, 3, 2, 512, 2, 4>(wm, bm, tm, p, grid, stream)
+        // (up to 16 tokens only where the codes of a K above 100 thousand do not fit gemm_small.cu's shared memory)
+        case 16: return wide_split ? launch_umma_t<16, 3, 2, 512, 2, 4>(wm, bm, tm, p, grid, stream)
                                    : launch_umma_t<16, 3, 2, 256, 2, 2>(wm, bm, tm, p, grid, stream);
         case 32: return wide_split ? launch_umma_t<32, 3, 2, 512, 2, 4>(wm, bm, tm, p, grid, stream)
                                    : launch_umma_t<32, 3, 2, 256, 2, 2>(wm, bm, tm, p, grid, stream);

@@ -4,14 +4,14 @@
 //
 // One CTA per tile pays its set-up (barriers, tensor memory, the first loads from HBM) and its epilogue (read-back,
 // scaling, 32 KB of output) with the tensor core idle: at 128 tokens that was more than the tile's K loop.  Here the
-// producers, the expanders and the MMA issuer run on into the next tile while four epilogue warps finish the last one:
+// producers, the expanders and the MMA issuer run on into the next tile while eight epilogue warps finish the last one:
 //   warp 0        packed sign words by TMA (a unit of 1024 weights x 128 rows per stage), all tiles back to back
-//   warp 1        per tile: the tokens' scales / code sums / zero points into shared memory, the codes k-block by k-block
-//                 by TMA, then the three bf16 terms of T
+//   warp 1        per tile: the codes k-block by k-block by TMA, then the three bf16 terms of T
 //   warp 2        MMA issue: the tile's K loop into the int32 accumulator, then the low-rank MMAs, one commit per tile
-//   warps 4..7    epilogue: stage the tile's rows of U, read the accumulators back, scale, write bf16 through shared
-//                 memory with 128-bit stores; the accumulator is handed back as soon as it has been read
-//   warps 8..23   expansion of sign bits into the tensor-memory operand ring (as in gemm_umma.cu), tile boundaries unseen
+//   warp 3        per tile: the tokens' scales, code sums and zero points into shared memory
+//   warps 4..11   epilogue: stage the tile's rows of U, read the accumulators back (64 tokens each), scale, write bf16 straight from
+//                 registers; the accumulator is handed back as soon as it has been read
+//   warps 12..27  expansion of sign bits into the tensor-memory operand ring (as in gemm_umma.cu), tile boundaries unseen
 // Every wait is bounded (umma_wait.cuh).
 #include <cuda_bf16.h>
 

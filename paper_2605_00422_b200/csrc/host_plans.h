@@ -229,6 +229,9 @@ inline bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) 
     return false;
 }
 
+// Up to how many tokens the warp-level MMA kernel (gemm_small.cu) runs the int8 contraction.
+constexpr int kSmallTokens = 16;
+
 // ---- the weight-only operating point ----
 // Up to how many tokens it runs on three int8 digits per value (gemm_small.cu)
 constexpr int kDigitTokens = 32;

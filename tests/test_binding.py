@@ -99,3 +99,17 @@ def test_what_was_refused_is_refused_in_the_same_way():
         with pytest.raises(bwla.BwlaError) as e:
             call()
         assert e.value.status == bwla.BWLA_ERR_INVALID_ARG
+
+
+@pytest.mark.gpu
+def test_rows_off_16_bytes_where_the_header_asks_for_them():
+    from paper_2605_00422_b200 import bwla
+    layer = _layer(bwla)
+    x = torch.zeros((2, 1025), dtype=torch.bfloat16, device="cuda")[:, :1024]
+    assert bwla.bwla_w1ax_linear_group([layer], x)[0].shape == (2, 64)
+    bwla.bwla_layer_set_activation_quant(layer, bwla.BWLA_ACT_ASYMMETRIC)
+    for call in (lambda: bwla.bwla_w1ax_linear_group([layer], x), lambda: bwla.bwla_layer_w1a16_linear(layer, x),
+                 lambda: bwla.bwla_layer_rotate_quant_asym(layer, x)):
+        with pytest.raises(bwla.BwlaError) as e:
+            call()
+        assert e.value.status == bwla.BWLA_ERR_UNSUPPORTED
