@@ -1,18 +1,25 @@
 // The binary-weight contraction for many tokens: the arithmetic of gemm_umma.cu (sign words expanded into tensor memory
-// as the A operand of tcgen05.mma kind::i8, low-rank term as kind::f16 MMAs, fused epilogue) in CTAs that stay on their
-// SM and take tiles of 128 output rows x 128 tokens in turn.
+// as the A operand of tcgen05.mma kind::i8, low-rank term as kind::f16 MMAs, fused epilogue) in pairs of CTAs that stay on their
+// SMs and take tiles of 256 output rows x 128 tokens in turn.
+//
+// A pair (cta_group::2, clusters of two) is one tensor core to the MMAs: each CTA holds 128 of the rows, in its own tensor memory, and
+// half of the tokens' codes, in its own shared memory.  One CTA alone needs 16 KB of codes for the 256 cycles of a k-block's MMAs, 64
+// bytes a cycle and SM, which is what the L2 delivers; a CTA of a pair needs half of that.  4096 tokens of 25600 -> 5120: 469 us before,
+// 394 now (2730 TOP/s, about what the power limit leaves: twice the sustained bf16 rate of cuBLAS); 5120 -> 25600, where the epilogue of
+// a tile takes longer than its K loop: 462 and 455.
 //
 // One CTA per tile pays its set-up (barriers, tensor memory, the first loads from HBM) and its epilogue (read-back,
 // scaling, 32 KB of output) with the tensor core idle: at 128 tokens that was more than the tile's K loop.  Here the
 // producers, the expanders and the MMA issuer run on into the next tile while eight epilogue warps finish the last one:
 //   warp 0        packed sign words by TMA (a unit of 1024 weights x 128 rows per stage), all tiles back to back
-//   warp 1        per tile: the codes k-block by k-block by TMA, then the three bf16 terms of T
-//   warp 2        MMA issue: the tile's K loop into the int32 accumulator, then the low-rank MMAs, one commit per tile
+//   warp 1        per tile: the codes k-block by k-block by TMA, then the three bf16 terms of T (64 tokens of either)
+//   warp 2        in the even CTA, MMA issue: the tile's K loop into the int32 accumulator, then the low-rank MMAs, one commit per tile
 //   warp 3        per tile: the tokens' scales, code sums and zero points into shared memory
 //   warps 4..11   epilogue: stage the tile's rows of U, read the accumulators back (64 tokens each), scale, write bf16 straight from
 //                 registers; the accumulator is handed back as soon as it has been read
 //   warps 12..27  expansion of sign bits into the tensor-memory operand ring (as in gemm_umma.cu), tile boundaries unseen
-// Every wait is bounded (umma_wait.cuh).
+// What the issuer waits for arrives on barriers of the even CTA, from both; its commits arrive in both.  Every wait is bounded
+// (umma_wait.cuh).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -27,24 +34,27 @@ namespace bwla {
 using namespace ptx;
 
 namespace persist {
-constexpr int kRows = 128;                // output rows per tile
+constexpr int kRows = 128;                // output rows per tile and CTA (256 a pair)
 constexpr int kTok = 128;                 // tokens per tile
+constexpr int kHalfTok = kTok / 2;        // of which a CTA loads the codes and T
 constexpr int kUnitK = 1024;              // weights per row in one sign-word stage
 constexpr int kBlockK = 128;              // K per code stage and per operand stage
 // A stage is a k-block's codes in shared memory and its expanded signs in tensor memory, under one pair of barriers: the issuing
 // thread runs one wait and one commit per k-block.  (With a ring and barriers for each operand the loop took 590 cycles per
 // k-block, 500 of them also without any of the copies, stores and MMAs: the issuing thread's waits and commits were the bound.)
-constexpr int WS = 3, AS = 4, EW = 4;
-static_assert(AS % EW == 0, "an operand stage must keep one owner among the expander parts");
+constexpr int WS = 3, BS = 8, AS = 4, EW = 4;
+static_assert(AS % EW == 0 && BS % AS == 0, "an operand stage must keep one owner among the expander parts");
 // Two epilogue warps per lane quarter, 64 tokens each: one warp needs about eight cycles an instruction beside the expanders, and
 // with four warps the epilogue of a tile took 8 us, more than the K loop of 5120 it runs under.
 constexpr int kEpiFirst = 128, kExpFirst = 384;
 constexpr int kThreads = kExpFirst + 128 * EW;       // 896
-constexpr int w_bytes = kRows * 128, b_bytes = kTok * 128;
-constexpr int u_off = WS * w_bytes + AS * b_bytes;
+// registers: 72 a thread at launch (896 x 72 = 64512); 128 x 40 + 256 x 88 + 512 x 72 = 64512 after the split
+constexpr int kRegsControl = 40, kRegsEpilogue = 88;
+constexpr int w_bytes = kRows * 128, b_bytes = kHalfTok * 128;
+constexpr int u_off = WS * w_bytes + BS * b_bytes;
 constexpr int t_off = u_off + kRows * 128;
 constexpr int bars_off = t_off + 3 * b_bytes;
-constexpr int n_bars = 2 * WS + 2 * AS + 12;
+constexpr int n_bars = 2 * WS + 2 * BS + 12;
 constexpr int misc_off = bars_off + n_bars * 8;
 constexpr int tok_off = (misc_off + 31) / 16 * 16;   // [2][scales, code sums, zero points, corrections][kTok]
 constexpr int used = tok_off + 2 * 16 * kTok;
@@ -103,9 +113,9 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + bars_off);
     uint64_t* w_full = bars;                 // [WS]
     uint64_t* w_empty = w_full + WS;
-    uint64_t* s_full = w_empty + WS;         // [AS] codes landed and signs expanded
-    uint64_t* s_empty = s_full + AS;         // [AS] the MMAs that read both have completed
-    uint64_t* d_full = s_empty + AS;         // the tile's MMAs (low-rank ones included) have completed
+    uint64_t* s_full = w_empty + WS;         // [BS] codes landed and signs expanded, in both CTAs (the even CTA's are used)
+    uint64_t* s_empty = s_full + BS;         // [BS] the MMAs that read both have completed
+    uint64_t* d_full = s_empty + BS;         // the tile's MMAs (low-rank ones included) have completed
     uint64_t* acc_free = d_full + 1;         // the epilogue has read the tile's accumulators
     uint64_t* u_full = acc_free + 1;         // the tile's rows of U are staged
     uint64_t* u_empty = u_full + 1;          // the low-rank MMAs have read them
@@ -123,48 +133,55 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
     auto tok_corr = [&](int buf) { return reinterpret_cast<float*>(smem + tok_off + buf * 16 * kTok + 12 * kTok); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
     const int tiles = p.tile_begin[NP];
-    const int my_tiles = (int)blockIdx.x < tiles ? (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const int my_tiles = pair < tiles ? (tiles - pair + pairs - 1) / pairs : 0;
     const int units = (p.K + kUnitK - 1) / kUnitK;
     const int kblocks = p.K / kBlockK;
-    // CTAs that work on the same token tile read the same codes: each starts at a unit of its own and goes round (the sums are
+    // Pairs that work on the same token tile read the same codes: each starts at a unit of its own and goes round (the sums are
     // integers, the order does not matter), so that they do not all ask the same slices of the L2 at the same time.
-    const int u0 = (int)(((int64_t)blockIdx.x * units) / gridDim.x);
+    const int u0 = (int)(((int64_t)pair * units) / pairs);
     auto unit_at = [&](int j) { const int u = u0 + j; return u < units ? u : u - units; };
     const bool lowrank = p.lowrank != 0;
-    // tile i of this CTA: one problem after the other, row tiles fastest, so that the CTAs working at the same time share a token
+    // tile i of this pair: one problem after the other, row tiles fastest, so that the CTAs working at the same time share a token
     // tile's codes in the L2
     struct Tile { int pi, n0, t0; };
     auto tile_at = [&](int i) -> Tile {
-        int g = (int)blockIdx.x + i * (int)gridDim.x, pi = 0;
+        int g = pair + i * pairs, pi = 0;
         if (NP > 1)
             while (pi + 1 < NP && g >= p.tile_begin[pi + 1]) ++pi;
         g -= p.tile_begin[pi];
         const int rows = p.prob[pi].row_tiles;
-        return Tile{pi, (g % rows) * kRows, (g / rows) * kTok};
+        return Tile{pi, (g % rows) * 2 * kRows + rank * kRows, (g / rows) * kTok};
     };
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         for (int i = 0; i < WS; ++i) { mbar_init(&w_full[i], 1); mbar_init(&w_empty[i], 4 * EW); }
-        for (int i = 0; i < AS; ++i) { mbar_init(&s_full[i], 5); mbar_init(&s_empty[i], 1); }      // four expander warps and the copy
-        mbar_init(d_full, 1); mbar_init(acc_free, 8);
-        mbar_init(u_full, 8); mbar_init(u_empty, 1);
+        for (int i = 0; i < BS; ++i) { mbar_init(&s_full[i], 9); mbar_init(&s_empty[i], 1); }      // four expander warps a CTA, and the copies
+        mbar_init(d_full, 1); mbar_init(acc_free, 16);
+        mbar_init(u_full, 16); mbar_init(u_empty, 1);
         mbar_init(t_full, 1); mbar_init(t_empty, 1);
         for (int i = 0; i < 2; ++i) { mbar_init(&tok_full[i], 1); mbar_init(&epi_done[i], 8); }
         fence_barrier_init();
         fence_proxy_async();
     }
     if (warp == 2) {
-        tmem_alloc(tmem_slot, TMEM_COLS);
-        tmem_relinquish();
+        tmem_alloc_pair(tmem_slot, TMEM_COLS);
+        tmem_relinquish_pair();
     }
     tc_fence_before();
     __syncthreads();
+    cluster_arrive_release();                 // the other CTA's barriers stand
+    cluster_wait_acquire();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     griddep_launch_dependents();
+    // what the MMA thread, in the even CTA, waits for
+    auto issuer = [&](uint64_t* bar) { return map_shared_rank(smem_u32(bar), 0u); };
 
+    if (warp < 4) {
+    set_regs_dec<kRegsControl>();
     if (warp == 0) {
         // ---------------- packed sign words (independent of the preceding kernel) ----------------
         if (elect_one()) {
@@ -207,21 +224,21 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
             bool ok = true;
             for (int i = 0; i < my_tiles && ok && !*abort_flag; ++i) {
                 const Tile at = tile_at(i);
-                const int t0 = at.t0;
+                const int t0 = at.t0 + rank * kHalfTok;
                 int kb = u0 * (kUnitK / kBlockK);
                 for (int c = 0; c < kblocks; ++c) {
                     if (!wait_or_abort(&s_empty[bs], bph ^ 1, abort_flag)) { give_up(p.status, abort_flag, 0x121); ok = false; break; }
-                    mbar_expect_tx(&s_full[bs], b_bytes);
-                    tma_load_2d(bbuf + bs * b_bytes, &maps.b[at.pi], kb * kBlockK, t0, &s_full[bs]);
-                    if (++bs == AS) { bs = 0; bph ^= 1; }
+                    if (rank == 0) mbar_expect_tx(&s_full[bs], 2 * b_bytes);
+                    tma_load_2d_pair(bbuf + bs * b_bytes, &maps.b[at.pi], kb * kBlockK, t0, issuer(&s_full[bs]));
+                    if (++bs == BS) { bs = 0; bph ^= 1; }
                     if (++kb == kblocks) kb = 0;
                 }
                 // T is first needed when the K loop is over; the previous tile's low-rank MMAs have long read theirs
                 if (ok && lowrank) {
                     if (i >= 1 && !wait_or_abort(t_empty, (uint32_t)((i - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x122); ok = false; }
                     if (ok) {
-                        mbar_expect_tx(t_full, 3 * b_bytes);
-                        for (int h = 0; h < 3; ++h) tma_load_3d(tbuf + h * b_bytes, &maps.t[at.pi], 0, t0, h, t_full);
+                        if (rank == 0) mbar_expect_tx(t_full, 6 * b_bytes);
+                        for (int h = 0; h < 3; ++h) tma_load_3d_pair(tbuf + h * b_bytes, &maps.t[at.pi], 0, t0, h, issuer(t_full));
                     }
                 }
             }
@@ -254,14 +271,14 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
             if (lane == 0) mbar_arrive(&tok_full[buf]);
         }
     } else if (warp == 2) {
-        // ---------------- MMA issue ----------------
-        if (elect_one()) {
-            const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTok >> 3) << 17) | ((128u >> 4) << 24);
-            const uint32_t idesc_lr = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTok >> 3) << 17) | ((128u >> 4) << 24);
+        // ---------------- MMA issue, for both CTAs ----------------
+        if (rank == 0 && elect_one()) {
+            const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTok >> 3) << 17) | ((256u >> 4) << 24);
+            const uint32_t idesc_lr = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTok >> 3) << 17) | ((256u >> 4) << 24);
             const uint32_t a_base = tmem_base + A_COL;
             const uint64_t desc_hi = smem_desc_sw128(0u, 0u);
             const uint32_t b_lo0 = (smem_u32(bbuf) & 0x3FFFFu) >> 4;
-            int as = 0; uint32_t aph = 0;
+            int bs = 0; uint32_t bph = 0;
             bool ok = true;
             griddep_wait();                           // everything this thread waits for follows the preceding kernel
             for (int i = 0; i < my_tiles && ok; ++i) {
@@ -271,17 +288,17 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                 const uint32_t d_addr = tmem_base + D_COL + (uint32_t)(i & 1) * kTok;
                 uint32_t acc = 0;
                 for (int kb = 0; kb < kblocks && ok; ++kb) {
-                    if (!wait_or_abort(&s_full[as], aph, abort_flag)) { give_up(p.status, abort_flag, 0x132); ok = false; break; }
+                    if (!wait_or_abort(&s_full[bs], bph, abort_flag)) { give_up(p.status, abort_flag, 0x132); ok = false; break; }
                     tc_fence_after();
-                    const uint64_t desc = desc_hi | (uint64_t)(b_lo0 + (uint32_t)as * (b_bytes >> 4));
-                    const uint32_t a_addr = a_base + 32 * as;
+                    const uint64_t desc = desc_hi | (uint64_t)(b_lo0 + (uint32_t)bs * (b_bytes >> 4));
+                    const uint32_t a_addr = a_base + 32 * (bs % AS);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        mma_i8_ts(d_addr, a_addr + 8 * j, desc + 2 * j, idesc, acc);
+                        mma_i8_ts_pair(d_addr, a_addr + 8 * j, desc + 2 * j, idesc, acc);
                         acc = 1u;
                     }
-                    tc_commit(&s_empty[as]);
-                    if (++as == AS) { as = 0; aph ^= 1u; }
+                    tc_commit_pair(&s_empty[bs]);
+                    if (++bs == BS) { bs = 0; bph ^= 1u; }
                 }
                 // The epilogue of the tile before has had this tile's whole K loop to read its accumulators; it is waited for
                 // here, before this tile's MMAs are committed, so that completions of acc_free are seen strictly in order
@@ -299,17 +316,19 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                             const uint32_t t_addr = smem_u32(tbuf + h * b_bytes);
 #pragma unroll
                             for (int j = 0; j < 4; ++j)
-                                mma_f16_ss(tmem_base + LR_COL, smem_desc_sw128(u_addr, 32 * j), smem_desc_sw128(t_addr, 32 * j),
+                                mma_f16_ss_pair(tmem_base + LR_COL, smem_desc_sw128(u_addr, 32 * j), smem_desc_sw128(t_addr, 32 * j),
                                            idesc_lr, (h | j) ? 1u : 0u);
                         }
-                        tc_commit(u_empty);
-                        tc_commit(t_empty);
+                        tc_commit_pair(u_empty);
+                        tc_commit_pair(t_empty);
                     }
                 }
-                tc_commit(d_full);
+                tc_commit_pair(d_full);
             }
         }
-    } else if (warp >= 4 && warp < 12) {
+    }
+    } else if (warp < 12) {
+        set_regs_inc<kRegsEpilogue>();
         // ---------------- epilogue ----------------
         const int q = warp & 3;
         const int e = (threadIdx.x - kEpiFirst) & 127;        // output row of the tile
@@ -351,7 +370,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                     }
                     fence_proxy_async();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(u_full);
+                    if (lane == 0) mbar_arrive_pair(issuer(u_full));
                 }
             }
             if (i == 0) griddep_wait();                       // nothing is stored before the preceding kernel has completed
@@ -393,7 +412,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                         // both accumulators are in registers: the next tile's MMAs may start
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(acc_free);
+                        if (lane == 0) mbar_arrive_pair(issuer(acc_free));
                     }
                     if (t0 + 16 * c >= p.M) continue;            // warp-uniform; nothing of this chunk is stored
                     if (pr.fast) {
@@ -439,7 +458,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
             __syncwarp();
             if (lane == 0) mbar_arrive(&epi_done[buf]);
         }
-    } else if (warp >= 12) {
+    } else {
         // ---------------- expansion of sign bits into the operand ring (tile boundaries do not matter here) ----------------
         const int q = warp & 3;
         const int part = (warp - 12) >> 2;             // which of the EW warps of the lane quarter
@@ -453,6 +472,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
         // parity wait cannot tell a phase from the one two before it.  (The last unit of a row may hold fewer than eight
         // blocks, which is why neither follows from the position inside the unit.)
         constexpr int PER = kUnitK / kBlockK / EW;
+        const uint32_t filled = issuer(s_full);
         int ws = 0; uint32_t wph = 0;
         const int total = my_tiles * units;
         int c = 0, u_nxt = 0;                         // next unit to take: running number, position in its row
@@ -493,11 +513,14 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                     for (int k = 0; k < 4; ++k)
 #pragma unroll
                         for (int j = 0; j < 8; ++j) v[8 * k + j] = (w[k] << (7 - j)) & 0x80808080u;
-                    const int as = (g + EW * q) % AS;
-                    const uint32_t aph = (uint32_t)(((g + EW * q) / AS) & 1);
-                    if (!__all_sync(0xFFFFFFFFu, mbar_test_wait(&s_empty[as], aph ^ 1u))) {
+                    const int as = (g + EW * q) % AS, bs = (g + EW * q) % BS;
+                    // the block that used the operand stage before: AS blocks ago, under the barrier of its own code stage
+                    const int before = g + EW * q - AS;
+                    const int gone = before & (BS - 1);
+                    const uint32_t gone_ph = (uint32_t)((before / BS) & 1);
+                    if (before >= 0 && !__all_sync(0xFFFFFFFFu, mbar_test_wait(&s_empty[gone], gone_ph))) {
                         griddep_wait();
-                        if (!warp_wait(&s_empty[as], aph ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x151); ok = false; }
+                        if (!warp_wait(&s_empty[gone], gone_ph, abort_flag)) { give_up(p.status, abort_flag, 0x151); ok = false; }
                     }
                     if (ok) {
                         tc_fence_after();
@@ -505,7 +528,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                         tc_wait_st();
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(&s_full[as]);
+                        if (lane == 0) mbar_arrive_pair(filled + 8u * (uint32_t)bs);
                     }
                 }
             }
@@ -517,10 +540,12 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
     }
     tc_fence_before();
     __syncthreads();
+    cluster_arrive_release();                 // nobody leaves while the other CTA may still reach its memories
+    cluster_wait_acquire();
     if (warp == 2) {
         __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem_base, TMEM_COLS);
+        tmem_dealloc_pair(tmem_base, TMEM_COLS);
     }
 }
 
@@ -534,8 +559,6 @@ template <int NP>
 static int launch_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
     using namespace persist;
     const int M = (int)a[0].M, K = (int)a[0].K;
-    const int sms = sm_count();
-    if (sms <= 0) return BWLA_ERR_CUDA;
     PersistMaps<NP> maps;
     PersistParams<NP> p{};
     p.M = M; p.K = K; p.tok_tiles = (M + kTok - 1) / kTok; p.lowrank = a[0].r > 0; p.status = a[0].status;
@@ -553,7 +576,7 @@ static int launch_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
         {
             const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
             const uint64_t strides[1] = {(uint64_t)K};
-            const uint32_t box[2] = {kBlockK, kTok};
+            const uint32_t box[2] = {kBlockK, kHalfTok};
             int st = make_map(&maps.b[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, g.codes, dims, strides, box,
                               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
             if (st != BWLA_OK) return st;
@@ -561,7 +584,7 @@ static int launch_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
         if (g.r > 0) {
             const uint64_t dims[3] = {(uint64_t)kLowrankPad, (uint64_t)M, 3};
             const uint64_t strides[2] = {(uint64_t)kLowrankPad * 2, (uint64_t)M * kLowrankPad * 2};
-            const uint32_t box[3] = {(uint32_t)kLowrankPad, kTok, 1};
+            const uint32_t box[3] = {(uint32_t)kLowrankPad, kHalfTok, 1};
             int st = make_map(&maps.t[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, g.Thl, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
                               CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
             if (st != BWLA_OK) return st;
@@ -569,7 +592,7 @@ static int launch_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
             maps.t[i] = maps.b[i];   // never dereferenced
         }
         PersistProblem& pr = p.prob[i];
-        pr.N = N; pr.row_tiles = (N + kRows - 1) / kRows; pr.r = g.r;
+        pr.N = N; pr.row_tiles = (N + 2 * kRows - 1) / (2 * kRows); pr.r = g.r;
         pr.scales = g.scales; pr.qsum = g.qsum; pr.zp = g.zp; pr.alpha = g.alpha; pr.mu = g.mu; pr.rowsum = g.rowsum;
         pr.U = (const __nv_bfloat16*)g.U; pr.out = (__nv_bfloat16*)g.out; pr.ldo = g.ldo; pr.acc_debug = g.acc_debug;
         pr.fast = !g.zp && !g.mu && !g.acc_debug && g.out && (int64_t)K << 7 < (int64_t)1 << 22;      // (whatever the codes a caller hands over)
@@ -584,16 +607,20 @@ static int launch_persistent(const GemmArgs* a, int n, cudaStream_t stream) {
         BWLA_CUDA_TRY(cudaFuncSetAttribute(umma_w1a_persistent_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, total));
         configured = dev;
     }
+    const int pairs = resident_clusters((const void*)umma_w1a_persistent_kernel<NP>, 2, kThreads, total);
+    if (pairs < 1) return cuda_fail(cudaErrorInvalidConfiguration);
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)std::min(p.tile_begin[n], sms), 1, 1);
+    cfg.gridDim = dim3(2u * (unsigned)std::min(p.tile_begin[n], pairs), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = total;
     cfg.stream = stream;
-    cudaLaunchAttribute attrs[1];
+    cudaLaunchAttribute attrs[2];
     attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attrs[0].val.programmaticStreamSerializationAllowed = launch_overlap_allowed();
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = 2; attrs[1].val.clusterDim.y = 1; attrs[1].val.clusterDim.z = 1;
     cfg.attrs = attrs;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     ProfScope prof(kProfContraction, stream);
     cudaError_t e = cudaLaunchKernelEx(&cfg, umma_w1a_persistent_kernel<NP>, maps, p);
     if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e); }
