@@ -427,8 +427,11 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                 const int blk = first_nxt + EW * q;                   // 8 bytes of the row's 128
                 nxt[q] = lds_words(wrow + (((blk >> 1) ^ (row & 7)) << 4) + 8 * (blk & 1));
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&w_empty[ws]);
+            // (behind the loads' data: see release_stage)
+            uint32_t seen = 0u;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) seen ^= nxt[q].x ^ nxt[q].y;
+            release_stage(&w_empty[ws], seen);
             if (++ws == WS) { ws = 0; wph ^= 1u; }
             base_nxt += ns_nxt;
             if (++u_nxt == units) u_nxt = 0;

@@ -487,8 +487,11 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
             const uint8_t* wrow = wbuf + ws * w_bytes + row * 128;
 #pragma unroll
             for (int q = 0; q < PER; ++q) nxt[q] = lds_words(wrow + (((first_nxt + EW * q) ^ (row & 7)) << 4));
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&w_empty[ws]);
+            // (behind the loads' data: see release_stage)
+            uint32_t seen = 0u;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) seen ^= nxt[q].x ^ nxt[q].y ^ nxt[q].z ^ nxt[q].w;
+            release_stage(&w_empty[ws], seen);
             if (++ws == WS) { ws = 0; wph ^= 1u; }
             base_nxt += ns_nxt;
             if (++u_nxt == units) u_nxt = 0;

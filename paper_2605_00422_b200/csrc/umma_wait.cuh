@@ -47,4 +47,12 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
+// A warp hands a stage of shared memory back to the copies after reading it into registers.  An arrival may overtake loads whose data
+// nobody has asked for yet, and the next copy then overwrites words that have not been read; so the arriving lane follows from the data
+// (`seen`: a word that depends on everything this lane has loaded), which has to be there.
+__device__ __forceinline__ void release_stage(uint64_t* bar, uint32_t seen) {
+    const uint32_t vote = __ballot_sync(0xFFFFFFFFu, (seen & 1u) != 0u);
+    if ((threadIdx.x & 31u) == (vote & 31u)) mbar_arrive(bar);
+}
+
 }  // namespace bwla
