@@ -424,14 +424,15 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
         g.codes = (const int8_t*)(base + w.yhat); g.scales = (const float*)(base + w.scales); g.qsum = (const int32_t*)(base + w.ysum);
         g.M = M; g.K = L->K; g.N = L->N; g.bits = 8; g.packed = L->packed; g.alpha = L->alpha; g.mu = L->mu;
         g.Thl = L->r > 0 ? base + w.T : nullptr; g.U = L->U; g.r = L->r; g.out = out_bf16; g.ldo = ldo; g.status = status;
-        if (gemm_small_fits(&g, 1, 3)) {
+        const bool small = M <= kSmallDigitTokens && gemm_small_fits(&g, 1, 3);
+        if (small || umma_digits_supports(M, L->K, L->N, L->r)) {
             RotProblem pr{};
             pr.prepared = L->prepared; pr.digits = 1; pr.codes = (int8_t*)(base + w.yhat); pr.codes_layout = 1;
             pr.scales = (float*)(base + w.scales); pr.qsum = (int32_t*)(base + w.ysum);
             st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
             if (st != BWLA_OK) return st;
             bool taken = false;
-            return launch_gemm_small(&g, 1, 3, &taken, s);
+            return small ? launch_gemm_small(&g, 1, 3, &taken, s) : launch_gemm_umma_digits(g, s);
         }
     }
     RotProblem pr{};

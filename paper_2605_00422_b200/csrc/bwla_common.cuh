@@ -243,7 +243,7 @@ bool bitplane_supports(int64_t M, int64_t K, int64_t N, int r, int bits);
 int launch_gemm_bitplane(const GemmArgs& a, cudaStream_t stream);
 
 // Up to kSmallTokens tokens: warp-level int8 MMAs, all linears of a group (same M, K, bits; a.codes in the interleaved order) in one
-// launch.  planes == 3: three digit planes per token (the weight-only operating point, up to kDigitTokens).  *taken is false, and
+// launch.  planes == 3: three digit planes per token (the weight-only operating point, up to kSmallDigitTokens).  *taken is false, and
 // nothing has been launched, for shapes whose codes do not fit shared memory: those go to the tcgen05 kernels.
 bool gemm_small_fits(const GemmArgs* a, int n, int planes);
 int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStream_t stream);
@@ -251,6 +251,9 @@ int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStr
 // tcgen05 path with the fused epilogue.  codes_interleaved: int8 [M][K] in the interleaved order.
 bool umma_supports(int64_t M, int64_t K, int64_t N, int r, int bits);
 int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream);
+// The weight-only operating point for few tokens as three digit planes a value, a.codes int8 [3][M][K]: planes are tokens to the MMAs
+bool umma_digits_supports(int64_t M, int64_t K, int64_t N, int r);
+int launch_gemm_umma_digits(const GemmArgs& a, cudaStream_t stream);
 // More than 64 tokens: the same contraction in CTAs that stay on their SM and take tiles of 128 rows x 128 tokens in turn.
 bool umma_persistent_supports(int64_t M, int64_t K, int64_t N, int r);
 // n linears with the same M and K, all of them or none with a low-rank branch; codes in the interleaved order

@@ -1,4 +1,4 @@
-// The binary-weight contraction for a decode batch (up to 16 tokens, 32 as digits) on warp-level int8 MMAs, every linear of a group in
+// The binary-weight contraction for a decode batch (up to 16 tokens, 4 as digits) on warp-level int8 MMAs, every linear of a group in
 // one launch.
 //
 //   tot[n][t] = sum_k bit(n,k) * q[t][k],   acc = 2 tot - sum_k q[t][k] - zp[t] * rowsum[n]            (sign = 2 bit - 1)
@@ -23,7 +23,7 @@
 // memory (rows of 128 bytes, permuted so that every read is free of bank conflicts).  K is split over a cluster of S CTAs
 // where the codes would not fit or rows are few.  The epilogue, once per run, also evaluates U T (bf16 MMAs, three terms of T).
 //
-// PL = 3 is the weight-only operating point: an activation is a 23-bit fixed-point number of a power-of-two scale, kept as
+// PL = 3 is the weight-only operating point for up to 4 tokens whose codes fit one CTA (more: gemm_umma.cu): an activation is a 23-bit fixed-point number of a power-of-two scale, kept as
 // three signed base-256 digits (rot_mma.cu); the digits are contracted like three tokens' codes, exactly, and put together in
 // the epilogue.
 #include <cuda_bf16.h>
@@ -42,9 +42,6 @@ namespace small_ {
 constexpr int kWarps = 16, kThreads = 32 * kWarps;
 constexpr int kUnit = 512, kSteps = 4;                        // k per item; code rows of 128 k in it
 constexpr int kSmemMax = 232448 - 256;
-// Sub-groups the tokens of a row group are dealt to: the accumulators of 12 tiles (the digits of 32 tokens) do not fit one warp's
-// registers (each then expands the sign bits for itself, which its MMAs cover).
-__host__ __device__ constexpr int token_parts(int NT) { return NT >= 8 ? 2 : 1; }
 }  // namespace small_
 
 struct SmallProblem {
@@ -93,7 +90,7 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) 
 template <int NTP, int PL, bool SPLIT>
 __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const __grid_constant__ SmallParams p) {
     using namespace small_;
-    constexpr int NT = NTP * PL, TP = token_parts(NT), NTPW = NTP / TP, NTW = NT / TP;        // ... W: of one item
+    constexpr int NT = NTP * PL;
     constexpr bool AHEAD = NT == 1;                   // (registers: beyond that the rows of a fragment are fetched when its turn comes)
     constexpr int TOK = 8 * NT, SETS = NT == 1 ? 4 : NT <= 3 ? 2 : 1;
     extern __shared__ __align__(16) uint8_t smem[];
@@ -127,16 +124,16 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
             for (int i = 128 * tid; i < rows * pr.r * 2; i += 128 * kThreads) prefetch_l2_line(u + i);
         }
     }
-    // this warp's items of a run of `n` groups from `g`: [lo, hi) in the order (group, token part, unit)
+    // this warp's items of a run of `n` groups from `g`: [lo, hi) in the order (group, unit)
     int g = g_lo, n = min(p.run, g_hi - g_lo), it, it_end;
     auto share = [&]() {
-        const int all = n * TP * un;
+        const int all = n * un;
         it = all * warp / kWarps; it_end = all * (warp + 1) / kWarps;
     };
     share();
     auto load_w = [&](uint4 (&w)[4], int item) {
         const int sub = item / un, u = item - sub * un;
-        const int n0 = (g + sub / TP) * 32 + gq, k16 = (ub + u) * (kUnit / 128) + tq;            // 16-byte pieces of a row
+        const int n0 = (g + sub) * 32 + gq, k16 = (ub + u) * (kUnit / 128) + tq;            // 16-byte pieces of a row
         const uint8_t* at = reinterpret_cast<const uint8_t*>(pr.packed) + 16 * k16;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -270,7 +267,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
     const uint32_t b0 = smem_u32(smem) + (uint32_t)((tq * TOK + gq) * 128), b_swz = (uint32_t)((gq ^ (tq << 1)) << 4);
 #pragma unroll 1
     while (g < g_hi) {
-        int32_t acc[SETS][2][NTW][4];
+        int32_t acc[SETS][2][NT][4];
         int sub = it < it_end ? it / un : 0, u = it - sub * un;
         auto clear = [&]() {
 #pragma unroll
@@ -278,7 +275,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                    for (int nt = 0; nt < NTW; ++nt)
+                    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                         for (int e = 0; e < 4; ++e) acc[s][mt][nt][e] = 0;
         };
@@ -289,9 +286,8 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
 #pragma unroll
             for (int j = 0; j < 4; ++j) w[j] = wn[j];
             if (it + 1 < it_end) load_w(wn, it + 1);
-            const int part = TP > 1 ? sub % TP : 0;
-            // column tile j of the item: plane j / NTPW, token tile part * NTPW + j % NTPW
-            const uint32_t b_item = b0 + (uint32_t)((u * kSteps * TOK + 8 * NTPW * part) * 128);
+            // column tile j of the item: plane j / NTP, token tile j % NTP
+            const uint32_t b_item = b0 + (uint32_t)(u * kSteps * TOK * 128);
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
                 uint32_t a[2][4][4];
@@ -309,8 +305,8 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
                     }
                 }
 #pragma unroll
-                for (int nt = 0; nt < NTW; ++nt) {
-                    const uint32_t at = b_item + (uint32_t)(8 * ((nt / NTPW) * NTP + nt % NTPW) * 128);
+                for (int nt = 0; nt < NT; ++nt) {
+                    const uint32_t at = b_item + (uint32_t)(8 * nt * 128);
                     const uint4 c0 = lds128(at + ((uint32_t)(32 * x) ^ b_swz)), c1 = lds128(at + ((uint32_t)(32 * x + 16) ^ b_swz));
                     const uint32_t bl[4] = {c0.x, c0.y, c0.z, c0.w}, bh[4] = {c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
@@ -322,18 +318,17 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
             }
             if (++u == un || it + 1 == it_end) {
                 // the group (or the warp's share of it) is done: into the CTA's sums
-                const uint32_t at = smem_u32(accs) + (uint32_t)(((sub / TP) * 2 * NT * 128 + lane) * 4);
+                const uint32_t at = smem_u32(accs) + (uint32_t)((sub * 2 * NT * 128 + lane) * 4);
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                    for (int nt = 0; nt < NTW; ++nt)
+                    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             int32_t v = acc[0][mt][nt][e];
 #pragma unroll
                             for (int z = 1; z < SETS; ++z) v += acc[z][mt][nt][e] >> z;
-                            const int col = (nt / NTPW) * NTP + NTPW * part + nt % NTPW;
-                            red_shared_add(at + (uint32_t)(((mt * NT + col) * 4 + e) * 128), v);
+                            red_shared_add(at + (uint32_t)(((mt * NT + nt) * 4 + e) * 128), v);
                         }
                 clear();
                 u = 0; ++sub;
@@ -399,7 +394,7 @@ __global__ void __launch_bounds__(small_::kThreads, 1) gemm_small_kernel(const _
 // ---------------------------------------------------------------------------------------------
 struct SmallPlan { int S, run, t_off, tok_off, acc_off, smem; int clusters[kRotMaxProblems]; };
 
-static int token_tiles(int64_t M) { return M <= 8 ? 1 : M <= 16 ? 2 : 4; }
+static int token_tiles(int64_t M) { return M <= 8 ? 1 : 2; }
 
 // How many clusters of S such CTAs the device holds at once.  (Clusters are placed inside a GPC, so this is less than SMs / S:
 // asked once per size and thread.)
@@ -472,7 +467,7 @@ static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int 
         pl.smem = off + pl.run * group_bytes;
         const double step = NT == 1 ? 30.0 : 22.0 * NT + 8.0;     // cycles per SM and code row of an item
         const int runs = (longest + pl.run - 1) / pl.run;
-        auto items = [&](int g) { return (double)((g * token_parts(NT) * per_cta + kWarps - 1) / kWarps) * kWarps / token_parts(NT); };
+        auto items = [&](int g) { return (double)((g * per_cta + kWarps - 1) / kWarps) * kWarps; };
         const double cost = (runs - 1) * items(pl.run) * kSteps * step + items(longest - (runs - 1) * pl.run) * kSteps * step +
                             runs * (1500.0 + 60.0 * NT * pl.run / S) + per_cta * kSteps * tok * 128 / 40.0 + (S > 1 ? 1500.0 + 1000.0 * runs : 0.0);
         if (!found || cost < best_cost) { best_cost = cost; *best = pl; found = true; }
@@ -488,7 +483,7 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     static thread_local Known known[16];
     static thread_local int used = 0;
     const int64_t M = a[0].M, K = a[0].K;
-    if (n < 1 || n > kRotMaxProblems || M < 1 || M > (planes == 3 ? kDigitTokens : kSmallTokens) || K % 128 != 0 || (planes == 3 && K > 25600)) return false;
+    if (n < 1 || n > kRotMaxProblems || M < 1 || M > (planes == 3 ? kSmallDigitTokens : kSmallTokens) || K % 128 != 0 || (planes == 3 && K > 25600)) return false;
     Key k{};
     for (int i = 0; i < n; ++i) {
         if (a[i].N < 1 || a[i].N > ((int64_t)1 << 30) || a[i].r > kLowrankPad || M * a[i].N >= (int64_t)1 << 31) return false;
@@ -517,7 +512,7 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
 
 bool gemm_small_fits(const GemmArgs* a, int n, int planes) {
     SmallPlan pl;
-    return small_plan(a, n, planes, &pl);
+    return small_plan(a, n, planes, &pl) && (planes == 1 || pl.S == 1);
 }
 
 template <int NTP, int PL, bool SPLIT>
@@ -556,7 +551,7 @@ static int launch_small_nt(const SmallParams& p, int grid, int smem, cudaStream_
 // *taken is false where the shapes do not fit (nothing has been launched then).
 int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStream_t stream) {
     SmallPlan pl;
-    *taken = small_plan(a, n, planes, &pl);
+    *taken = small_plan(a, n, planes, &pl) && (planes == 1 || pl.S == 1);
     if (!*taken) return BWLA_OK;
     const int M = (int)a[0].M, K = (int)a[0].K, NTP = token_tiles(M);
     SmallParams p{};
@@ -573,13 +568,7 @@ int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStr
         begin += pl.clusters[i];
     }
     const int grid = begin * pl.S;
-    if (planes == 3) {
-        switch (NTP) {
-            case 1: return launch_small_nt<1, 3>(p, grid, pl.smem, stream);
-            case 2: return launch_small_nt<2, 3>(p, grid, pl.smem, stream);
-            default: return launch_small_nt<4, 3>(p, grid, pl.smem, stream);
-        }
-    }
+    if (planes == 3) return launch_small_t<1, 3, false>(p, grid, pl.smem, stream);
     return NTP == 1 ? launch_small_nt<1, 1>(p, grid, pl.smem, stream) : launch_small_nt<2, 1>(p, grid, pl.smem, stream);
 }
 

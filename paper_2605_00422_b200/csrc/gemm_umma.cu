@@ -51,10 +51,11 @@ constexpr int kBlockK = 128;             // K per code sub-block / per tensor-me
 constexpr int kFirstExpander = 192;      // warps 0, 1: TMA; warps 2..5: MMA issue; warps 6..: expand + epilogue
 struct UmmaParams {
     int M, N, K;
+    int rows;                    // of the codes: M, or 3 M of the digit planes [3][M] (the weight-only operating point, few tokens)
     int total_units, splits;
     int r;                       // low-rank width, 0..kLowrankPad
     const float* scales;         // [M]
-    const int32_t* qsum;         // [M][kQsumParts] partial sums
+    const int32_t* qsum;         // [rows][kQsumParts] partial sums
     const float* alpha;          // [N]
     const float* mu;             // [N] or NULL
     const int32_t* zp;           // [M] zero points of asymmetric codes, or NULL
@@ -111,7 +112,16 @@ __device__ __forceinline__ float finish_value(int32_t d, float l, float alpha_sc
     return fmaf(mu_sc, (float)(qs - kz), __fmul_rn(alpha_sc, (float)acc) + l);
 }
 
-template <int N_TOK, int WS, int BS, int TMEM_COLS, int NISS, int EW>
+// The same from the accumulators of a value's three base-256 digits (q: sums of the digits): the low two digits' sums together are still
+// exact in int32 (|sum of a digit| <= 128 K); sc is a power of two and may be subnormal.
+__device__ __forceinline__ float finish_digits(const int32_t (&d)[3], const int32_t (&q)[3], float l, float alpha, float mu, float sc) {
+    const int32_t a0 = -(d[0] >> 6) - q[0], a1 = -(d[1] >> 6) - q[1], a2 = -(d[2] >> 6) - q[2];
+    const float acc = fmaf((float)a2, 65536.f, (float)(256 * a1 + a0)), sum = fmaf((float)q[2], 65536.f, (float)(256 * q[1] + q[0]));
+    return fmaf(mu, __fmul_rn(sum, sc), __fmul_rn(alpha, __fmul_rn(acc, sc)) + l);
+}
+
+// PL: 1, or 3 digit planes: columns plane * M + t of the accumulators (M tokens in one tile)
+template <int N_TOK, int WS, int BS, int TMEM_COLS, int NISS, int EW, int PL>
 __global__ void __launch_bounds__(kFirstExpander + 128 * EW, TMEM_COLS == 256 ? 2 : 1)
 umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap b_map,
                 const __grid_constant__ CUtensorMap t_map, UmmaParams p) {
@@ -251,13 +261,13 @@ umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
                 const int t = t0 + i;
                 scale_s[i] = t < p.M ? p.scales[t] : 0.f;
                 int32_t qs = 0;
-                if (t < p.M) {
+                if (t < p.rows) {
                     const int4* parts = reinterpret_cast<const int4*>(p.qsum + (size_t)t * kQsumParts);
                     const int4 a = parts[0], b = parts[1];
                     qs = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
                 }
                 qsum_s[i] = qs;
-                zp_s[i] = (p.zp && t < p.M) ? p.zp[t] : 0;
+                zp_s[i] = (PL == 1 && p.zp && t < p.M) ? p.zp[t] : 0;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(s_full);
@@ -432,7 +442,7 @@ umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
             // the warps of a quarter take chunks of 16 tokens in turn
 #pragma unroll 1
             for (int c = part; c < N_TOK / 16; c += EW) {
-                if (t0 + 16 * c >= p.M) break;                 // warp-uniform
+                if (t0 + 16 * c >= p.rows) break;              // warp-uniform
                 uint32_t v[16], l[16];
                 tmem_ld_32x16(tmem_base + lane_addr + 16 * c, v);
                 if (lowrank_here) tmem_ld_32x16(tmem_base + lane_addr + L::D2_COL + 16 * c, l);
@@ -447,6 +457,15 @@ umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
                         for (int j = 0; j < 16; ++j) v[j] += v2[j];
                     }
                 }
+                if (PL == 3) {
+                    // digits of a value lie M columns apart: they meet behind the barrier, in shared memory
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        red_i[(16 * c + j) * kRowsPerCta + row] = (int32_t)v[j];
+                        if (lowrank_here && 16 * c < M_) red_f[(16 * c + j) * kRowsPerCta + row] = __uint_as_float(l[j]);
+                    }
+                }
+                if constexpr (PL == 1) {
                 // the chunk's scales and code sums go to registers first: the tile stores below may alias them as far as
                 // the compiler knows, and a load behind every store would serialise the loop
                 float sc[16]; int32_t qs[16], zp[16];
@@ -474,9 +493,22 @@ umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
                         if (lowrank_here) red_f[(16 * c + j) * kRowsPerCta + row] = __uint_as_float(l[j]);
                     }
                 }
+                }
             }
         }
-        if (p.splits == 1) {
+        if (PL == 3 && p.splits == 1) {
+            asm volatile("bar.sync 1, %0;" ::"r"(kExpanders) : "memory");
+            if (ok) {
+                // a thread finishes its row for every part-th token
+                const int n = n0 + row;
+                for (int t = part; t < p.M && n < p.N; t += EW) {
+                    const int32_t d[3] = {red_i[t * kRowsPerCta + row], red_i[(p.M + t) * kRowsPerCta + row], red_i[(2 * p.M + t) * kRowsPerCta + row]};
+                    const int32_t qs[3] = {qsum_s[t], qsum_s[p.M + t], qsum_s[2 * p.M + t]};
+                    const float l = lowrank ? red_f[t * kRowsPerCta + row] : 0.f;
+                    p.out[(int64_t)t * p.ldo + n] = __float2bfloat16_rn(finish_digits(d, qs, l, alpha_row, mu_row, scale_s[t]));
+                }
+            }
+        } else if (p.splits == 1) {
             asm volatile("bar.sync 1, %0;" ::"r"(kExpanders) : "memory");   // the output tile is complete (all expander warps, always)
             if (ok && p.out) {
                 // 16 threads move one token's 128 outputs (256 bytes) with 128-bit stores
@@ -511,23 +543,34 @@ umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
             for (int ti = e >> 5; ; ti += kExpanders / 32) {
                 const int tt = split + ti * p.splits;
                 if (tt >= N_TOK || t0 + tt >= p.M) break;
-                const uint32_t off_i = smem_u32(&red_i[tt * kRowsPerCta + r4]);
-                uint4 part[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (c < p.splits) part[c] = ld_shared_cluster_v4(map_shared_rank(off_i, c));
                 uint4 lf = make_uint4(0u, 0u, 0u, 0u);
                 if (lowrank) lf = ld_shared_cluster_v4(map_shared_rank(smem_u32(&red_f[tt * kRowsPerCta + r4]), 0));
-                int32_t d[4] = {0, 0, 0, 0};
+                int32_t ds[PL][4];
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (c < p.splits) { d[0] += (int32_t)part[c].x; d[1] += (int32_t)part[c].y; d[2] += (int32_t)part[c].z; d[3] += (int32_t)part[c].w; }
+                for (int pl = 0; pl < PL; ++pl) {
+                    const uint32_t off_i = smem_u32(&red_i[(pl * p.M + tt) * kRowsPerCta + r4]);
+                    uint4 part[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        if (c < p.splits) part[c] = ld_shared_cluster_v4(map_shared_rank(off_i, c));
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) ds[pl][j] = 0;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        if (c < p.splits) { ds[pl][0] += (int32_t)part[c].x; ds[pl][1] += (int32_t)part[c].y; ds[pl][2] += (int32_t)part[c].z; ds[pl][3] += (int32_t)part[c].w; }
+                }
+                const int32_t(&d)[4] = ds[0];
                 const float l4[4] = {__uint_as_float(lf.x), __uint_as_float(lf.y), __uint_as_float(lf.z), __uint_as_float(lf.w)};
                 __align__(8) __nv_bfloat16 y4[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     float y = 0.f;
-                    if (n + j < p.N) {
+                    if (PL == 3) {
+                        if (n + j < p.N) {
+                            const int32_t dd[3] = {ds[0][j], ds[PL / 2][j], ds[PL - 1][j]}, qs[3] = {qsum_s[tt], qsum_s[p.M + tt], qsum_s[2 * p.M + tt]};
+                            y = finish_digits(dd, qs, l4[j], p.alpha[n + j], p.mu ? p.mu[n + j] : 0.f, scale_s[tt]);
+                        }
+                    } else if (n + j < p.N) {
                         const int32_t zr = p.zp ? zp_s[tt] * p.rowsum[n + j] : 0;
                         y = finish_value(d[j], l4[j], __fmul_rn(p.alpha[n + j], scale_s[tt]),
                                          p.mu ? __fmul_rn(p.mu[n + j], scale_s[tt]) : 0.f, qsum_s[tt], zr, p.K * zp_s[tt]);
@@ -560,11 +603,11 @@ umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
 // -------------------------------------------------------------------------------------------------
 // host side
 // -------------------------------------------------------------------------------------------------
-template <int N_TOK, int WS, int BS, int TMEM_COLS, int NISS, int EW>
+template <int N_TOK, int WS, int BS, int TMEM_COLS, int NISS, int EW, int PL = 1>
 static int launch_umma_t(const CUtensorMap& wm, const CUtensorMap& bm, const CUtensorMap& tm, const UmmaParams& p,
                          dim3 grid, cudaStream_t s) {
     using L = UmmaCfg<N_TOK, WS, BS, TMEM_COLS, NISS, EW>;
-    auto kernel = umma_w1a_kernel<N_TOK, WS, BS, TMEM_COLS, NISS, EW>;
+    auto kernel = umma_w1a_kernel<N_TOK, WS, BS, TMEM_COLS, NISS, EW, PL>;
     static thread_local int configured = -1;
     int dev = 0;
     BWLA_CUDA_TRY(cudaGetDevice(&dev));
@@ -623,6 +666,41 @@ static int choose_wide_splits(int tiles, int units, int narrow_splits, int sms) 
     return wide < narrow ? s : 0;
 }
 
+// rows: of the codes, n_tok of them a tile; t_tok: tokens of T a tile
+static int make_umma_maps(const GemmArgs& a, const int8_t* codes_interleaved, int rows, int n_tok, int t_tok, CUtensorMap* wm, CUtensorMap* bm, CUtensorMap* tm) {
+    const uint64_t K = (uint64_t)a.K, N = (uint64_t)a.N, M = (uint64_t)a.M;
+    {
+        const uint64_t dims[2] = {K / 32, N};
+        const uint64_t strides[1] = {K / 8};
+        const uint32_t box[2] = {32, kRowsPerCta};
+        int st = make_map(wm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, a.packed, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+        if (st != BWLA_OK) return st;
+    }
+    {
+        const uint64_t dims[2] = {K, (uint64_t)rows};
+        const uint64_t strides[1] = {K};
+        const uint32_t box[2] = {kBlockK, (uint32_t)n_tok};
+        int st = make_map(bm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, codes_interleaved, dims, strides, box,
+                          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+        if (st != BWLA_OK) return st;
+    }
+    if (a.r > 0) {
+        const uint64_t dims[3] = {(uint64_t)kLowrankPad, M, 3};
+        const uint64_t strides[2] = {(uint64_t)kLowrankPad * 2, M * kLowrankPad * 2};
+        const uint32_t box[3] = {(uint32_t)kLowrankPad, (uint32_t)t_tok, 1};
+        return make_map(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, a.Thl, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+    }
+    *tm = *bm;   // never dereferenced
+    return BWLA_OK;
+}
+static void set_umma_params(UmmaParams* p, const GemmArgs& a, int rows, int units, int splits) {
+    p->M = (int)a.M; p->N = (int)a.N; p->K = (int)a.K; p->rows = rows; p->total_units = units; p->splits = splits; p->r = a.r;
+    p->scales = a.scales; p->qsum = a.qsum; p->alpha = a.alpha; p->mu = a.mu; p->zp = a.zp; p->rowsum = a.rowsum; p->U = (const __nv_bfloat16*)a.U;
+    p->out = (__nv_bfloat16*)a.out; p->ldo = a.ldo; p->acc_debug = a.acc_debug; p->status = a.status; p->dep_mode = a.dep_mode;
+}
+
 // codes_interleaved: int8 [M][K] in the interleaved order.  a.Thl: bf16 [3][M][64], T = hi + mid + lo.
 int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream) {
     const int M = (int)a.M, N = (int)a.N, K = (int)a.K;
@@ -645,37 +723,11 @@ int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStr
     if (wide_split) split = wide_split;
 
     CUtensorMap wm, bm, tm;
-    {
-        const uint64_t dims[2] = {(uint64_t)K / 32, (uint64_t)N};
-        const uint64_t strides[1] = {(uint64_t)K / 8};
-        const uint32_t box[2] = {32, kRowsPerCta};
-        int st = make_map(&wm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, a.packed, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-        if (st != BWLA_OK) return st;
-    }
-    {
-        const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
-        const uint64_t strides[1] = {(uint64_t)K};
-        const uint32_t box[2] = {kBlockK, (uint32_t)n_tok};
-        int st = make_map(&bm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, codes_interleaved, dims, strides, box,
-                          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-        if (st != BWLA_OK) return st;
-    }
-    if (a.r > 0) {
-        const uint64_t dims[3] = {(uint64_t)kLowrankPad, (uint64_t)M, 3};
-        const uint64_t strides[2] = {(uint64_t)kLowrankPad * 2, (uint64_t)M * kLowrankPad * 2};
-        const uint32_t box[3] = {(uint32_t)kLowrankPad, (uint32_t)n_tok, 1};
-        int st = make_map(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, a.Thl, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-        if (st != BWLA_OK) return st;
-    } else {
-        tm = bm;   // never dereferenced
-    }
+    const int st = make_umma_maps(a, codes_interleaved, M, n_tok, n_tok, &wm, &bm, &tm);
+    if (st != BWLA_OK) return st;
 
     UmmaParams p{};
-    p.M = M; p.N = N; p.K = K; p.total_units = units; p.splits = split; p.r = a.r;
-    p.scales = a.scales; p.qsum = a.qsum; p.alpha = a.alpha; p.mu = a.mu; p.zp = a.zp; p.rowsum = a.rowsum; p.U = (const __nv_bfloat16*)a.U;
-    p.out = (__nv_bfloat16*)a.out; p.ldo = a.ldo; p.acc_debug = a.acc_debug; p.status = a.status; p.dep_mode = a.dep_mode;
+    set_umma_params(&p, a, M, units, split);
 
     dim3 grid((unsigned)row_tiles, (unsigned)tok_tiles, (unsigned)split);
     switch (n_tok) {
@@ -689,6 +741,27 @@ int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStr
                                                        : launch_umma_t<64, 4, 3, 512, 2, 4>(wm, bm, tm, p, grid, stream);
     }
     return BWLA_ERR_UNSUPPORTED;
+}
+
+// The weight-only operating point, few tokens: three digit planes a value, codes int8 [3][M][K] in the interleaved order.
+bool umma_digits_supports(int64_t M, int64_t K, int64_t N, int r) {
+    return M >= 1 && 3 * M <= 96 && N > 0 && K % 128 == 0 && K <= 25600 && r <= kLowrankPad && M * N < (int64_t)1 << 31 && encode_tiled_fn() != nullptr;
+}
+int launch_gemm_umma_digits(const GemmArgs& a, cudaStream_t stream) {
+    const int rows = 3 * (int)a.M, n_tok = rows <= 48 ? 48 : 96;
+    const int row_tiles = (int)((a.N + kRowsPerCta - 1) / kRowsPerCta), units = (int)((a.K + kUnitK - 1) / kUnitK);
+    const int sms = sm_count();
+    if (sms <= 0) return BWLA_ERR_CUDA;
+    const int split = row_tiles > sms ? 1 : std::max(1, std::min(std::min(8, units), sms / row_tiles));
+    CUtensorMap wm, bm, tm;
+    const int st = make_umma_maps(a, a.codes, rows, n_tok, n_tok, &wm, &bm, &tm);
+    if (st != BWLA_OK) return st;
+    UmmaParams p{};
+    set_umma_params(&p, a, rows, units, split);
+    const dim3 grid((unsigned)row_tiles, 1, (unsigned)split);
+    if (n_tok == 48) return row_tiles > sms ? launch_umma_t<48, 2, 2, 256, 1, 2, 3>(wm, bm, tm, p, grid, stream)
+                                            : launch_umma_t<48, 4, 3, 512, 2, 4, 3>(wm, bm, tm, p, grid, stream);
+    return launch_umma_t<96, 4, 4, 512, 1, 4, 3>(wm, bm, tm, p, grid, stream);
 }
 
 }  // namespace bwla

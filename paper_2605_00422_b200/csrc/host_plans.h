@@ -233,8 +233,15 @@ inline bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) 
 constexpr int kSmallTokens = 16;
 
 // ---- the weight-only operating point ----
-// Up to how many tokens it runs on three int8 digits per value (gemm_small.cu)
-constexpr int kDigitTokens = 32;
+// Up to how many tokens it runs on three int8 digits per value: gemm_umma.cu, whose MMAs of 128 rows take 51 cycles whatever the 3 M columns
+// are up to 64 (mma.sync: 12 a column tile of 8, and 3.4 times as long for two of them), or gemm_small.cu for very few tokens where the codes
+// fit one CTA and the rows fill the device.  A call, us, gemm_small.cu | gemm_umma.cu, rank 32:
+//                       1 token      4            8            16           32
+//    4096 -> 4096      13.8 14.2   13.8 14.2    14.7 14.6    23.0 15.4    23.3 17.1
+//    5120 -> 25600     25.8 29.9   27.9 28.3    28.5 23.9    43.2 23.8   143.7 36.7
+//    5120 -> 1024      16.5 14.2   16.8 14.4    17.4 14.8    20.3 15.6    24.2 17.1     (split over clusters on gemm_small.cu)
+//   25600 -> 5120      45.2 29.5   45.7 32.3    46.0 32.3    69.1 33.5   115.7 46.4     (the same)
+constexpr int kDigitTokens = 32, kSmallDigitTokens = 4;
 constexpr int kQsumParts = 8;            // partial sums a token's code sum is kept as (one per CTA of its cluster)
 // bf16 values, or three digits of few tokens, and the sums of either: never less than fewer tokens need
 inline size_t a16_value_bytes(int64_t M, int64_t K) { return std::max((size_t)(M * K * 2), (size_t)(std::min<int64_t>(M, kDigitTokens) * K * 3)); }
