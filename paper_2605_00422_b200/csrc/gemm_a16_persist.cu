@@ -261,8 +261,8 @@ a16_persistent_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                         for (int h = 0; h < 3; ++h) {
                             const uint32_t t_addr = smem_u32(tbuf + h * b_bytes);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                mma_f16_ss(tmem_base + LR_COL, smem_desc_sw128(u_addr, 32 * j), smem_desc_sw128(t_addr, 32 * j),
+                            for (int j = 0; j < 4; ++j)      // (zeros beyond r)
+                                if (16 * j < p.r) mma_f16_ss(tmem_base + LR_COL, smem_desc_sw128(u_addr, 32 * j), smem_desc_sw128(t_addr, 32 * j),
                                            idesc, (h | j) ? 1u : 0u);
                         }
                         tc_commit(u_empty);

@@ -288,8 +288,8 @@ umma_w1a_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
                     for (int h = 0; h < 3; ++h) {
                         const uint32_t t_addr = smem_u32(tbuf + h * L::sub_bytes);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            mma_f16_ss(tmem_base + L::D2_COL, smem_desc_sw128(u_addr, 32 * i), smem_desc_sw128(t_addr, 32 * i),
+                        for (int i = 0; i < 4; ++i)      // (zeros beyond r)
+                            if (16 * i < p.r) mma_f16_ss(tmem_base + L::D2_COL, smem_desc_sw128(u_addr, 32 * i), smem_desc_sw128(t_addr, 32 * i),
                                        idesc_lr, (h | i) ? 1u : 0u);
                     }
                 }

@@ -5,8 +5,7 @@
 // A pair (cta_group::2, clusters of two) is one tensor core to the MMAs: each CTA holds 128 of the rows, in its own tensor memory, and
 // half of the tokens' codes, in its own shared memory.  One CTA alone needs 16 KB of codes for the 256 cycles of a k-block's MMAs, 64
 // bytes a cycle and SM, which is what the L2 delivers; a CTA of a pair needs half of that.  4096 tokens of 25600 -> 5120: 469 us before,
-// 394 now (2730 TOP/s, about what the power limit leaves: twice the sustained bf16 rate of cuBLAS); 5120 -> 25600, where the epilogue of
-// a tile takes longer than its K loop: 462 and 455.
+// 394 now (2730 TOP/s, about what the power limit leaves: twice the sustained bf16 rate of cuBLAS).
 //
 // One CTA per tile pays its set-up (barriers, tensor memory, the first loads from HBM) and its epilogue (read-back,
 // scaling, 32 KB of output) with the tensor core idle: at 128 tokens that was more than the tile's K loop.  Here the
@@ -27,6 +26,7 @@
 #include "bwla_common.cuh"
 #include "umma_ptx.cuh"
 #include "umma_wait.cuh"
+#include "rot_mma.cuh"
 #include "tensor_map.cuh"
 
 namespace bwla {
@@ -311,12 +311,13 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                     if (ok) {
                         tc_fence_after();
                         const uint32_t u_addr = smem_u32(ubuf);
+                        const int r = p.prob[tile_at(i).pi].r;      // (zeros beyond)
 #pragma unroll
                         for (int h = 0; h < 3; ++h) {
                             const uint32_t t_addr = smem_u32(tbuf + h * b_bytes);
 #pragma unroll
                             for (int j = 0; j < 4; ++j)
-                                mma_f16_ss_pair(tmem_base + LR_COL, smem_desc_sw128(u_addr, 32 * j), smem_desc_sw128(t_addr, 32 * j),
+                                if (16 * j < r) mma_f16_ss_pair(tmem_base + LR_COL, smem_desc_sw128(u_addr, 32 * j), smem_desc_sw128(t_addr, 32 * j),
                                            idesc_lr, (h | j) ? 1u : 0u);
                         }
                         tc_commit_pair(u_empty);
@@ -390,6 +391,7 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                 const uint32_t sel = odd ? 0x3276u : 0x5410u;
                 const int n_pair = n & ~1;
                 const bool pair_ok = ((reinterpret_cast<uintptr_t>(pr.out) & 3) == 0) && (pr.ldo & 1) == 0 && n_pair + 1 < pr.N;
+                const bool pairs_ok = __all_sync(0xFFFFFFFFu, pair_ok);
                 const uint32_t acc_addr = tmem_base + lane_addr + D_COL + (uint32_t)(i & 1) * kTok;
                 auto put = [&](uint32_t word, int tok) {          // word: tokens tok (low half) and tok + 1 of this lane's row
                     const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 1);
@@ -415,7 +417,35 @@ umma_w1a_persistent_kernel(const __grid_constant__ PersistMaps<NP> maps, const _
                         if (lane == 0) mbar_arrive_pair(issuer(acc_free));
                     }
                     if (t0 + 16 * c >= p.M) continue;            // warp-uniform; nothing of this chunk is stored
-                    if (pr.fast) {
+                    if (pr.fast && pairs_ok && t0 + 16 * c + 16 <= p.M) {
+                        // The usual case, a whole chunk: no conditions on single stores, a pointer that steps, packed additions.  A short K loop waits for
+                        // its epilogue, 2400 cycles a chunk without this (270 instructions beside the expanders): 4096 tokens of 2048 -> 25600 279 us,
+                        // 207 with it; of 5120 -> 25600, where most of it is hidden, 449 and 422.
+                        __nv_bfloat16* at = pr.out + (int64_t)(t0 + 16 * c + odd) * pr.ldo + n_pair;
+                        const int64_t step = 2 * pr.ldo;
+#pragma unroll
+                        for (int j = 0; j < 16; j += 4) {
+                            const float4 sc = sc_s[4 * c + (j >> 2)], co = co_s[4 * c + (j >> 2)];
+                            const float scs[4] = {sc.x, sc.y, sc.z, sc.w}, cos[4] = {co.x, co.y, co.z, co.w};
+                            float y[4];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) y[h] = __int_as_float(__float_as_int(cos[h]) - ((int32_t)v[j + h] >> 6));
+                            add2(y[0], y[1], -12582912.f, -12582912.f);
+                            add2(y[2], y[3], -12582912.f, -12582912.f);
+                            // (the product is rounded before the addition: the scalar multiplication is not contracted)
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) y[h] = __fmul_rn(__fmul_rn(alpha_n, scs[h]), y[h]);
+                            add2(y[0], y[1], lowrank ? __uint_as_float(l[j]) : 0.f, lowrank ? __uint_as_float(l[j + 1]) : 0.f);
+                            add2(y[2], y[3], lowrank ? __uint_as_float(l[j + 2]) : 0.f, lowrank ? __uint_as_float(l[j + 3]) : 0.f);
+#pragma unroll
+                            for (int h = 0; h < 4; h += 2) {
+                                const uint32_t word = pack_bf16x2(y[h], y[h + 1]);
+                                const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 1);
+                                *reinterpret_cast<uint32_t*>(at) = __byte_perm(word, other, sel);
+                                at += step;
+                            }
+                        }
+                    } else if (pr.fast) {
                         // the raw sum is -2^7 times the sum over the set bits; 1.5 * 2^23 + integer (below 2^22) is a float by its
                         // bits, and taking 1.5 * 2^23 off again is exact
 #pragma unroll
