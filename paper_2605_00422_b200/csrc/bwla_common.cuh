@@ -136,6 +136,7 @@ constexpr int kRotMaxProblems = 4;          // linears that share one x and are 
 struct RotProblem {
     const uint8_t* prepared;    // terms of P2^T and P1^T (launch_prepare_rot), or NULL: P1 and P2 are split by every CTA
     const float *P1, *P2;       // read only when `prepared` is NULL
+    const uint8_t* rows;        // beside `prepared`: the terms in the layout of rot_rows.cu, or NULL where that kernel is not chosen
     const uint8_t* okt;         // beside `prepared`: the terms in the layout of okt_umma.cu, or NULL where that kernel is not chosen
     // quantiser (yhat == NULL)
     int8_t* codes;              // [M][K]
@@ -169,6 +170,14 @@ int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits
 bool rot_umma_supports(const RotGeom& g, int n_problems, const RotProblem* problems);
 int launch_rot_umma(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                     const RotProblem* problems, uint32_t* status, cudaStream_t stream);
+// Many tokens of factors up to 128 x 128 (rot_rows.cu; launch_rot goes there by itself); x in 16-byte pieces
+bool rot_rows_supports(const RotGeom& g, int n_problems, const RotProblem* problems);
+int launch_prepare_rows(const RotRowsGeom& g, const float* P1, const float* P2, void* prepared, cudaStream_t stream);
+// (beside: the T = V x that its launch evaluates too, rows of V on 16 bytes)
+int launch_rot_rows(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
+                    const RotProblem* problems, const OktLowrank* beside, uint32_t* status, cudaStream_t stream);
+int launch_rows_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status, bool* taken,
+                         cudaStream_t stream);
 // how many clusters of a kernel the device holds at once
 int resident_clusters(const void* kernel, int dc, int threads, size_t smem);
 // ---- many tokens of factors up to 128 (okt_umma.cu; launch_rot goes there by itself) ----

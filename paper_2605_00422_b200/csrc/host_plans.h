@@ -163,18 +163,20 @@ inline size_t rot_prepared_bytes(const RotGeom& g) {
 }
 
 // ---- which kernel rotates many tokens (more than the device holds clusters for) ----
-// A call of one prepared linear of 32 outputs, us at 150, 1024 and 4096 (x 128: 2048) tokens, and the error of the rotation against 64
-// bits in 1e-7 of a row's 2-norm, on rot_mma.cu | okt_umma.cu | rot_umma.cu:
-//    64 x  64    21    31    64   1.4  |  26    43   103   1.7  |  22    38    88   1.4
-//    64 x  80    23    41    92   1.4  |  28    46   110   1.8  |  24    41    91   1.5
-//    64 x  88    27    50   121   1.5  |  29    47   111   2.0  |      -
-//    64 x 128    32    60   153   1.5  |  33    51   126   2.3  |  30    47   106   1.7
-//    86 x 128    46    94   288   1.5  |  39    61   152   2.5  |  45    80   230   1.9
-//   108 x 128    55   114   197   1.5  |  46    74   118   2.6  |  50    87   139   2.0
-//   128 x 128    66   155   273   1.5  |  50    78   125   2.7  |  50    79   126   2.0
-//   160 x 160   100   296     -   1.5  | 101   316     -   3.2  |  81   156     -   2.3
-// mma.sync wherever one warp holds all columns of a token and a CTA several tokens; rot_umma.cu (and for the bf16 values of the
-// weight-only operating point everywhere else); okt_umma.cu where a step of rot_umma.cu holds one token in half of its columns.
+// The kernel alone, us at 150, 1024 and 4096 tokens of one linear, and the error of 300 tokens against 64 bits in 1e-7 of a row's 2-norm:
+//                before                             rot_rows.cu
+//    48 x  64    13    21    46   1.35   rot_mma    13    19    41   1.34
+//    64 x  64    15    25    58   1.40   rot_mma    13    19    42   1.38
+//    64 x  80    17    33    86   1.43   rot_mma    13    21    50   1.40
+//    64 x 128    19    36    93   1.59   rot_umma   15    25    68   1.55
+//    86 x 128    21    44   137   2.45   okt_umma   17    36   113   1.83
+//   108 x 128    23    52   166   2.48   okt_umma   17    38   117   1.89
+//   128 x 128    23    50   162   2.64   okt_umma   19    39   124   1.9
+// rot_rows.cu wherever it can (n1 in (32, 128], n2 a multiple of 16 up to 128).  For the rest: mma.sync where one warp holds all columns of
+// a token and a CTA several tokens; okt_umma.cu for 81 to 128 columns, where a step of rot_umma.cu would hold one token in half of its
+// columns, and for n2 that is no multiple of 16; rot_umma.cu (160 x 160: 100 | 296 us at 150 and 1024 tokens on mma.sync, 81 | 156 here).
+// (As many tokens as the device holds at once stay on mma.sync, 1.45e-7 for every size: rot_rows.cu has 86 x 128 in 14.6 us of a call for
+// one token's 17.6, but 1.8e-7.)
 inline bool rot_mma_always(const RotGeom& g) { return g.cw == 1 && g.n2p <= 80; }
 inline bool rot_okt_factors(const RotGeom& g) {
     return !rot_mma_always(g) && g.na <= 16 && g.n2 <= 128 && (g.na > 10 || g.n2 % 16 != 0);
@@ -228,6 +230,53 @@ inline bool rot_umma_geometry(const RotGeom& g, int out_size, RotUmmaGeom* out) 
     }
     return false;
 }
+
+// ---- rotation of many tokens on tcgen05, output rows on the lanes (rot_rows.cu) ----
+constexpr int kRotRowsSharedBytes = 2048;      // its barriers and small per-CTA state
+struct RotRowsGeom {
+    int n1, n2, K;
+    int lanes, tps;         // tensor-memory lanes of a token (n1 rounded up to 64 or 128), tokens of a step
+    int groups, chunks;     // warps the columns are dealt to in every lane quarter, 16-column chunks of a warp
+    int nv;                 // accumulators for the first contraction
+    int y_chains;           // chains of sums of the second
+    int ks1, ks2;           // steps of 16 over a and over b
+    int atoms1, atoms2;     // K atoms of 32 elements
+    int xb;                 // buffers of x
+    int staged, out_bytes;  // outputs of a step go through shared memory (two buffers of out_bytes)
+    int p1_off, x_off, st_off, sh_off, total;   // the terms of P2^T at 0
+};
+// What follows the factors, with xb buffers of x.
+inline bool rot_rows_places(RotRowsGeom& g, int xb, int x_terms) {
+    g.xb = xb;
+    g.st_off = g.x_off + xb * x_terms * g.atoms2 * 128 * 64;
+    g.sh_off = (g.st_off + (g.staged ? 2 * g.out_bytes : 0) + 127) / 128 * 128;
+    g.total = g.sh_off + kRotRowsSharedBytes;
+    return g.total <= kRotMaxSmem;
+}
+// n1 in (32, 128] on the lanes; n2 a multiple of 16 up to 128: two accumulators for either contraction fill four (or six, up to 80
+// columns: two steps' V) times n2 columns of tensor memory.  A third chain of Y lies where V was, so that with one V the next step's V waits for it:
+// only for two tokens a step (108 x 128, 4096 tokens: 121 us with three chains, 117 with two, 1.73e-7 and 1.89e-7).  x_terms: 3 where rows are fp32.
+inline bool rot_rows_geometry(int n1, int n2, int out_size, RotRowsGeom* out, int x_terms = 1) {
+    if (n2 % 16 != 0 || n2 < 32 || n2 > 128 || n1 <= 32 || n1 > 128) return false;
+    RotRowsGeom g{};
+    g.n1 = n1; g.n2 = n2; g.K = n1 * n2;
+    g.lanes = n1 <= 64 ? 64 : 128; g.tps = 128 / g.lanes;
+    g.chunks = n2 <= 80 ? 1 : 2; g.groups = (n2 + 16 * g.chunks - 1) / (16 * g.chunks); g.nv = n2 <= 80 ? 2 : 1;
+    g.ks1 = (n1 + 15) / 16; g.ks2 = n2 / 16;
+    g.y_chains = g.ks2 == 2 || (g.nv == 1 && g.lanes == 128) ? 2 : 3;
+    g.atoms1 = (n1 + 31) / 32; g.atoms2 = (n2 + 31) / 32;
+    // Rows of a whole number of 32 outputs leave in 16-byte pieces from registers; others (half of a group of the codes' order would be
+    // two bytes of every four) through shared memory.
+    g.staged = n2 % 32 != 0;
+    g.out_bytes = g.tps * g.K * out_size;
+    g.p1_off = 2 * g.atoms2 * n2 * 64;         // (an MMA of the step's second token reads from 64 rows before P1's terms)
+    g.x_off = g.p1_off + 3 * g.atoms1 * g.lanes * 64;
+    for (int xb = x_terms == 1 ? 2 : 1; xb >= 1; --xb)
+        if (rot_rows_places(g, xb, x_terms)) { *out = g; return true; }
+    return false;
+}
+// once per layer: a header with the exponent of P2's scale, then both factors' terms as they lie in shared memory
+inline size_t rot_rows_prepared_bytes(const RotRowsGeom& g) { return kRotHeader + (size_t)g.x_off; }
 
 // Up to how many tokens the warp-level MMA kernel (gemm_small.cu) runs the int8 contraction.
 constexpr int kSmallTokens = 16;

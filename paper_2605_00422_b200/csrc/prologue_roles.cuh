@@ -213,9 +213,9 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uin
 // Up to 64 tokens: T for a tile of 16 tokens x 8 NTC columns and a part of K per block.  What such a block costs is latency:
 // V comes from HBM and is requested before the preceding kernel has finished (two or four chunks per warp), x follows
 // in one round trip, and K is cut into as many parts as give every warp about that many.
-template <int NTC>
+template <int NTC, int U = 8 / NTC>                          // U: chunks of a warp in registers at once
 static __device__ void lowrank_mma_role(const PrologueParams& p, int b, float* smem) {
-    constexpr int COLS = 8 * NTC, U = 8 / NTC;            // U: chunks of a warp in registers at once
+    constexpr int COLS = 8 * NTC;
     const int jtiles = (p.lr_cols + COLS - 1) / COLS;
     const int KS = p.lr_ks;
     const int jt = b % jtiles, j0 = jt * COLS;
@@ -314,10 +314,10 @@ static __device__ void lowrank_mma_role(const PrologueParams& p, int b, float* s
     if (KS > 1) {
         __threadfence();
         __syncthreads();
-        __shared__ uint32_t arrived;
-        if (threadIdx.x == 0) arrived = atomicAdd(p.lr_count + tile, 1u);
+        // (in place of the sums, which have been read)
+        if (threadIdx.x == 0) *reinterpret_cast<uint32_t*>(red) = atomicAdd(p.lr_count + tile, 1u);
         __syncthreads();
-        if (arrived != (uint32_t)(KS - 1)) return;
+        if (*reinterpret_cast<volatile uint32_t*>(red) != (uint32_t)(KS - 1)) return;
         __threadfence();
         for (int o = threadIdx.x; o < 16 * COLS; o += blockDim.x) {
             float s = 0.f;
@@ -438,7 +438,7 @@ inline int plan_lowrank(PrologueParams& p, float* lr_part, uint32_t* lr_count, i
         blocks *= p.lr_ks;
     }
     // shared memory of a low-rank block: per-warp partial sums, and its rows of V when those are staged (few tokens)
-    const size_t red_bytes = (size_t)kLrMaxWarps * 4 * (p.lr_wide == 3 ? 1024 : p.lr_wide == 2 || p.lr_wide == 4 ? 16 * cols : 64);
+    const size_t red_bytes = (size_t)std::max(kLrMaxWarps, warps) * 4 * (p.lr_wide == 3 ? 1024 : p.lr_wide == 2 || p.lr_wide == 4 ? 16 * cols : 64);
     const size_t stage_bytes = (size_t)2 * (size_t)K * 2;
     p.lr_stage = (p.lr_wide == 0 && red_bytes + stage_bytes <= smem_limit) ? 1 : 0;
     *smem = red_bytes + (p.lr_stage ? stage_bytes : 0);

@@ -918,6 +918,26 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
         // left: 32 tokens of 108 x 128 in clusters of four 36 us a call, in CTAs 28)
         return t.dc == 1 || ((base.dc > 1 || 2 * M * n_problems * t.dc <= sm_count()) && M * n_problems <= resident_clusters((const void*)rot_kernel_of(t, problems[0]), t.dc, 32 * t.warps, (size_t)(t.group_off + t.group_bytes)));
     });
+    // More tokens: rot_rows.cu wherever it can (T beside it by the warp-level MMA blocks only).  It also takes a few tokens of raw factors, whose
+    // split by every CTA is shorter there (64 x 80, us a call: 1 token 12.7 | 13.9, 4: 16.8 | 16.4, 32: 21.6 | 17.4, 129: 32.2 | 28.4), up to 80
+    // columns, where its error is no larger (host_plans.h; prepared, three linears with rank 64: 1 token 12.8 | 14.3, 24: 23.4 | 23.4, 50:
+    // 26.1 | 24.4).
+    const bool raw_few = !problems[0].prepared && M * n_problems > 3 && base.n1 <= 64 && base.n2 <= 80;
+    if (vec && (!few || raw_few) && rot_rows_supports(base, n_problems, problems)) {
+        if (any && M > 64) {
+            st = own_launch(true);
+            if (st != BWLA_OK) return st;
+        }
+        bool fits = true;
+        for (int i = 0; i < n_problems; ++i) {
+            if (!beside[i].V) continue;
+            PrologueParams probe{};
+            size_t bytes = 0;
+            plan_lowrank(probe, x, M, base.K, ldx, beside[i], kRotMaxWarps, kRotMaxSmem, &bytes);
+            fits = fits && (probe.lr_wide == 2 || probe.lr_wide == 4);
+        }
+        if (fits) return launch_rot_rows(base, x, M, ldx, bits, asym, n_problems, problems, beside, status, stream);
+    }
     if (!few && vec) {
         bool okt = rot_okt_factors(base) && !problems[0].yhat && !problems[0].digits;
         for (int i = 0; i < n_problems; ++i) okt = okt && (problems[i].okt || !problems[i].prepared);

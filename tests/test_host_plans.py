@@ -116,3 +116,28 @@ def test_operands_of_the_rotations_lie_inside_the_block(tmp_path):
             }
         }
     if (seen < 2000) std::printf("only %ld pairs\\n", seen);""") == ""
+
+
+def test_operands_of_the_rotation_with_rows_on_the_lanes_lie_inside_the_block(tmp_path):
+    """What its MMAs read of P1's terms (128 rows from any atom, and from 64 rows before them for a step's second token), its tensor memory and
+    shared memory, every column with a warp, no empty chain of sums; one x, and fp32 rows."""
+    assert violations(tmp_path, """
+    long seen = 0;
+    for (int n1 = 1; n1 <= 192; ++n1)
+        for (int n2 = 8; n2 <= 256; n2 += 8)
+            for (int size = 0; size <= 2; ++size)
+                for (int terms = 1; terms <= 3; terms += 2) {
+                    RotRowsGeom g{};
+                    if (!rot_rows_geometry(n1, n2, size, &g, terms)) continue;
+                    ++seen;
+                    for (int xb = g.xb; xb >= 1; --xb) {
+                        RotRowsGeom one = g;
+                        const bool ok = rot_rows_places(one, xb, terms) && one.total <= kRotMaxSmem && one.x_off - one.lanes * 64 + 128 * 64 <= one.total &&
+                                        one.p1_off >= (one.tps - 1) * 64 * 64 && (one.p1_off | one.x_off) % 1024 == 0 && (2 * one.nv + 2) * n2 <= 512 &&
+                                        one.groups * one.chunks * 16 >= n2 && (one.groups - 1) * one.chunks * 16 < n2 && one.groups <= 5 && one.tps * one.lanes == 128 &&
+                                        one.lanes >= n1 && one.ks1 >= 3 && one.ks1 <= 8 && one.ks2 >= 2 && one.ks2 <= 8 && one.ks2 * 16 == n2 &&
+                                        one.st_off + (one.staged ? 2 * one.out_bytes : 0) <= one.sh_off && (n1 * n2 % 32 != 0 || one.out_bytes % 16 == 0);
+                        if (!ok) { std::printf("%d x %d, %d bytes, %d terms\\n", n1, n2, size, terms); return 0; }
+                    }
+                }
+    if (seen < 1000) std::printf("only %ld\\n", seen);""") == ""

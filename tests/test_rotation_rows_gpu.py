@@ -1,0 +1,85 @@
+"""The tcgen05 rotation with output rows on the lanes at the edges of its work split: one and two tokens a step with a ragged last step,
+rows that do not fill the lanes, 2 to 5 warps a lane quarter, one and two chunks a warp, rows of outputs that are whole groups of 32 (written
+from registers) and that are not (through shared memory).
+
+Bounds as in tests/test_rotation_many_gpu.py: Y within 9e-7 of the token's full scale, codes, zero points and scales exactly those that follow
+from it, outputs those of the contraction on the codes in natural order."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2605_00422_b200 import inputs as gen
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(33, 32, 301), (40, 48, 297), (64, 64, 149), (62, 80, 298), (66, 112, 150), (128, 32, 151), (97, 64, 149), (90, 80, 150), (88, 96, 149), (128, 128, 297)]
+
+
+def _case(n1, n2, M, asym):
+    from paper_2605_00422_b200 import bwla
+    K, N = n1 * n2, 72
+    rng = np.random.default_rng([n1, n2, M])
+    P1, P2 = gen.orthogonal_f32(n1, rng), gen.orthogonal_f32(n2, rng)
+    x = rng.standard_t(3, size=(M, K)).astype(np.float32)
+    x[0, 0], x[M - 1], x[1] = 300.0, 0.0, np.abs(x[1])
+    packed = torch.from_numpy(rng.integers(-2 ** 31, 2 ** 31, size=(N, K // 32), dtype=np.int64).astype(np.int32)).cuda()
+    alpha, mu = torch.rand(N, device="cuda") + 0.5, 0.01 * torch.randn(N, device="cuda")
+    L = bwla.Layer(H.f32_to_dev(P1), H.f32_to_dev(P2), 8, packed, alpha, None, None, mu, asymmetric=asym)
+    return bwla, L, P1, P2, gen.bf16_bits_from_f32(x)
+
+
+@pytest.mark.parametrize("asym", [False, True])
+@pytest.mark.parametrize("n1,n2,M", SIZES)
+def test_codes(n1, n2, M, asym):
+    bwla, L, P1, P2, xb = _case(n1, n2, M, asym)
+    dx = H.bf16_to_dev(xb)
+    Y = oracle.rotate(xb, P1, P2)
+    full = np.maximum(np.abs(Y).max(axis=1, keepdims=True), 1e-30)
+    if asym:
+        u, s, z, y = (t.cpu().numpy() for t in bwla.bwla_layer_rotate_quant_asym(L, dx, want_y=True))
+        q = oracle.quantize_asym(y.astype(np.float64), 8, "f32")
+        assert np.array_equal(q["zeros"], z)
+    else:
+        u, s, y = (t.cpu().numpy() for t in bwla.bwla_layer_rotate_quant(L, dx, want_y=True))
+        q = oracle.quantize(y.astype(np.float64), 8, "f32")
+    assert float((np.abs(y.astype(np.float64) - Y) / full).max()) <= 9e-7
+    assert np.array_equal(q["codes"], u) and np.array_equal(q["scales"], s)
+    # the contraction's order, code sums and zero points: the accumulators that the codes in natural order have
+    out = bwla.bwla_w1ax_linear_group([L], dx)[0].float().cpu().numpy().astype(np.float64)
+    sign = oracle.unpack_signs(L.tensors[2].cpu().numpy().view(np.uint32), n1 * n2).astype(np.float64)
+    val = u.astype(np.float64) - (z[:, None] if asym else 0)
+    want = s[:, None].astype(np.float64) * (val @ sign.T * L.tensors[3].cpu().numpy().astype(np.float64) + val.sum(axis=1, keepdims=True) * L.tensors[6].cpu().numpy().astype(np.float64))
+    # bf16 rounding, and fp32 arithmetic on the terms before it
+    bound = 2.0 ** -8 * np.abs(want) + 2.0 ** -20 * s[:, None] * np.abs(val).sum(axis=1, keepdims=True) * float(L.tensors[3].max()) + 1e-30
+    assert np.all(np.abs(out - want) <= bound)
+
+
+@pytest.mark.parametrize("n1,n2,M", [(40, 48, 297), (36, 48, 150), (64, 64, 301), (96, 80, 150), (88, 96, 149)])
+def test_weight_only_values(n1, n2, M):
+    """bf16 values in either order and their sums, through the linear, against the bf16 rounding of the exact rotation."""
+    bwla, L, P1, P2, xb = _case(n1, n2, M, False)
+    Y = oracle.rotate(xb, P1, P2)
+    out = bwla.bwla_layer_w1a16_linear(L, H.bf16_to_dev(xb)).float().cpu().numpy().astype(np.float64)
+    yhat = torch.from_numpy(Y).float().bfloat16().double().numpy()
+    sign = oracle.unpack_signs(L.tensors[2].cpu().numpy().view(np.uint32), n1 * n2).astype(np.float64)
+    want = yhat @ sign.T * L.tensors[3].cpu().numpy().astype(np.float64) + yhat.sum(axis=1, keepdims=True) * L.tensors[6].cpu().numpy().astype(np.float64)
+    # bf16 output; a value within the rotation's error (9e-7 of full scale) of a rounding boundary moves by a bf16 step of its own: in 2-norm over
+    # K values far below the output's rounding, bounded here by one part in 2^8 of the values' 2-norm
+    bound = 2.0 ** -8 * np.abs(want) + 2.0 ** -8 * np.linalg.norm(yhat, axis=1, keepdims=True) * 2.0
+    assert np.all(np.abs(out - want) <= bound)
+    assert np.linalg.norm(out - want) <= 3e-3 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("n1,n2", [(64, 64), (40, 80), (64, 128)])
+def test_an_infinity_stays_in_its_token(n1, n2):
+    """Two tokens share a step's MMAs: the other one's codes and scale do not change."""
+    bwla, L, P1, P2, xb = _case(n1, n2, 300, False)
+    dx = H.bf16_to_dev(xb)
+    codes, scales = bwla.bwla_layer_rotate_quant(L, dx)[:2]
+    bad = dx.clone()
+    bad[4, 7] = float("inf"); bad[9, 100] = float("nan"); bad[131, :] = float("-inf")
+    c2, s2 = bwla.bwla_layer_rotate_quant(L, bad)[:2]
+    keep = torch.ones(300, dtype=torch.bool); keep[[4, 9, 131]] = False
+    assert torch.equal(codes.cpu()[keep], c2.cpu()[keep]) and torch.equal(scales.cpu()[keep], s2.cpu()[keep])
