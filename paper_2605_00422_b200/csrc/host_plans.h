@@ -52,12 +52,15 @@ inline size_t lowrank_split_bytes(int64_t M, int lr_cols) {
 // ---- T = V x for many tokens on tcgen05 (lowrank_umma.cu) ----
 constexpr int kLruTok = 128, kLruCols = 64, kLruBlockK = 64;        // tokens and columns of a tile, values of k per stage
 constexpr int kLruMaxParts = 16;         // parts of K per token tile
+constexpr int kLruClusterParts = 8;      // ... that a cluster adds up in shared memory; more (a second kernel adds them) only for a K above
+constexpr int kLruClusterK = 12288;
 constexpr int kLruTargetCtas = 160;      // parts are chosen so that tiles x parts comes near this, every part at least eight stages long
 inline int64_t lowrank_umma_tiles(int64_t M) { return (M + kLruTok - 1) / kLruTok; }
 inline int lowrank_umma_parts(int64_t M, int64_t K) {
     const int64_t tiles = lowrank_umma_tiles(M);
     int64_t ks = std::min<int64_t>(std::max<int64_t>(1, kLruTargetCtas / tiles), kLruMaxParts);
     ks = std::min<int64_t>(ks, std::max<int64_t>(1, K / (8 * kLruBlockK)));
+    if (ks > kLruClusterParts && K <= kLruClusterK) ks = kLruClusterParts;
     return (int)std::min<int64_t>(ks, std::max<int64_t>(1, M * K / (tiles * kLruCols * kLruTok * 4)));      // (their room: below)
 }
 // Which problems it takes; which of them go to it, launch_rot decides.

@@ -10,10 +10,10 @@
 // in registers, while the next 128 go into the second accumulator.
 //
 // Work of one CTA: a tile of 128 tokens (the accumulator's lanes) x all 64 columns x one part of K.  With fewer token
-// tiles than SMs, K is split into parts; the parts leave their sums in the workspace and a second small kernel adds
-// them in the order of the parts and splits the result into the three terms (so the result does not depend on which
-// CTA finished last).  Warp 0 copies (TMA: 64 values of k of the x tile and of V per stage), warp 1 issues the MMAs,
-// warps 2..5 are the epilogue, one per quarter of the accumulator's lanes.  Every wait is bounded.
+// tiles than SMs, K is split into parts.  Up to eight parts are a cluster: they leave their sums in their own shared memory, and each
+// adds its share of the columns over all of them, in the order of the parts, and splits it into the three terms.  (Through the workspace and
+// a second kernel, which more parts of a large K still take, four more microseconds stood before the rotation: a block of 333 tokens 205 us,
+// 199 now.)  Warp 0 copies (TMA: 64 values of k of the x tile and of V per stage), warp 1 issues the MMAs (all lanes in step), warps 2..5 are the epilogue, one per quarter of the accumulator's lanes.  Every wait is bounded.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -40,7 +40,7 @@ constexpr int kTmemCols = 2 * kCols;
 struct LrUmmaParams {
     int64_t M;
     int K, ks, tiles, n_problems;
-    float* part[kRotMaxProblems];                 // [tile][part][column][lane] fp32 (ks > 1)
+    float* part[kRotMaxProblems];                 // [tile][part][column][lane] fp32 (ks > kLruClusterParts)
     __nv_bfloat16* Thl[kRotMaxProblems];          // [3][M][64]
     uint32_t* status;
 };
@@ -79,11 +79,11 @@ lowrank_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_cons
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // blocks that share a token tile and a part of K (one per problem) are neighbours: the x tile is in the L2 for all but one
-    const int pi = (int)blockIdx.x % p.n_problems;
-    const int rest = (int)blockIdx.x / p.n_problems;
-    const int kp = rest % p.ks, tile = rest / p.ks;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
+    // the parts of a tile, then the problems that share its x, are neighbours
+    const int kp = (int)blockIdx.x % p.ks, rest = (int)blockIdx.x / p.ks;
+    const int pi = rest % p.n_problems, tile = rest / p.n_problems;
+    const bool cluster = p.ks > 1 && p.ks <= kLruClusterParts;
     const int nblocks = p.K / kBlockK;
     const int b_lo = (int)((int64_t)nblocks * kp / p.ks), b_hi = (int)((int64_t)nblocks * (kp + 1) / p.ks);
     const int nb = b_hi - b_lo;
@@ -124,29 +124,29 @@ lowrank_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_cons
             if (*abort_flag) for (int i = 0; i < 500; ++i) __nanosleep(100);   // let copies in flight land
         }
     } else if (warp == 1) {
-        if (elect_one()) {
-            // D = f32, A = B = bf16, both K-major, M = 128, N = 64
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kCols >> 3) << 17) | ((128u >> 4) << 24);
-            int s = 0; uint32_t ph = 0;
-            bool ok = true;
-            int b = b_lo;
-            for (int u = 0; u < units && ok; ++u) {
-                const int buf = u & 1;
-                if (u >= 2 && !wait_or_abort(&acc_free[buf], (uint32_t)(((u >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x220); break; }
+        // D = f32, A = B = bf16, both K-major, M = 128, N = 64
+        const bool one = elect_one();
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kCols >> 3) << 17) | ((128u >> 4) << 24);
+        const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0u, 0u) >> 32), x_lo0 = (uint32_t)smem_desc_sw128(smem_u32(smem), 0u);
+        int s = 0; uint32_t ph = 0;
+        bool ok = true;
+        int b = b_lo;
+        for (int u = 0; u < units && ok; ++u) {
+            const int buf = u & 1;
+            if (u >= 2 && !warp_wait(&acc_free[buf], (uint32_t)(((u >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x220); break; }
+            tc_fence_after();
+            const uint32_t d_addr = tmem_base + (uint32_t)(buf * kCols);
+            for (int i = 0; i < kFlushBlocks && b < b_hi; ++i, ++b) {
+                if (!warp_wait(&full[s], ph, abort_flag)) { give_up(p.status, abort_flag, 0x221); ok = false; break; }
                 tc_fence_after();
-                const uint32_t d_addr = tmem_base + (uint32_t)(buf * kCols);
-                for (int i = 0; i < kFlushBlocks && b < b_hi; ++i, ++b) {
-                    if (!wait_or_abort(&full[s], ph, abort_flag)) { give_up(p.status, abort_flag, 0x221); ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t xa = smem_u32(smem + s * stage_bytes), va = xa + x_bytes;
+                const uint32_t xa = x_lo0 + (uint32_t)s * (stage_bytes >> 4), va = xa + (x_bytes >> 4);
+                warp_mma_f16_ss(one, d_addr, xa, desc_hi, va, desc_hi, idesc, i > 0);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        mma_f16_ss(d_addr, smem_desc_sw128(xa, 32 * j), smem_desc_sw128(va, 32 * j), idesc, (i | j) ? 1u : 0u);
-                    tc_commit(&empty[s]);
-                    if (++s == kStages) { s = 0; ph ^= 1u; }
-                }
-                if (ok) tc_commit(&acc_full[buf]);
+                for (uint32_t j = 1; j < 4; ++j) warp_mma_f16_ss(one, d_addr, xa + 2u * j, desc_hi, va + 2u * j, desc_hi, idesc, 1u);
+                warp_commit(one, &empty[s]);
+                if (++s == kStages) { s = 0; ph ^= 1u; }
             }
+            if (ok) warp_commit(one, &acc_full[buf]);
         }
     } else {
         const int q = warp & 3;
@@ -184,7 +184,8 @@ lowrank_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_cons
                     }
                 }
             } else {
-                float* mine = p.part[pi] + ((size_t)tile * p.ks + kp) * (kCols * kTok) + lane_d;
+                // (all MMAs are complete, and with them every copy into the stages)
+                float* mine = (cluster ? reinterpret_cast<float*>(smem) : p.part[pi] + ((size_t)tile * p.ks + kp) * (kCols * kTok)) + lane_d;
 #pragma unroll
                 for (int c = 0; c < kCols; ++c) mine[c * kTok] = run[c];
             }
@@ -192,6 +193,35 @@ lowrank_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_cons
     }
     tc_fence_before();
     __syncthreads();
+    if (cluster) {
+        // every thread of every CTA takes part, whether or not its CTA gave up
+        cluster_arrive_release();
+        cluster_wait_acquire();
+        if (warp >= 2 && !*abort_flag) {
+            const int lane_d = (warp & 3) * 32 + lane;
+            const int64_t t = t0 + lane_d;
+            for (int cg = kp; cg < kCols / 8; cg += p.ks) {
+                const uint32_t at = smem_u32(smem) + (uint32_t)((8 * cg * kTok + lane_d) * 4);
+                float v[kLruClusterParts][8], s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int k = 0; k < kLruClusterParts; ++k)
+                    if (k < p.ks) {
+                        const uint32_t peer = map_shared_rank(at, (uint32_t)k);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) v[k][c] = ld_shared_cluster_f32(peer + (uint32_t)(c * kTok * 4));
+                    }
+#pragma unroll
+                for (int k = 0; k < kLruClusterParts; ++k)
+                    if (k < p.ks)
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) s[c] += v[k][c];
+                if (t < p.M) store_terms(p.Thl[pi], p.M, t, 8 * cg, s);
+            }
+        }
+        // nobody leaves while a neighbour may still read its shared memory
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    }
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
@@ -272,9 +302,12 @@ int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_
         BWLA_CUDA_TRY(cudaFuncSetAttribute(lowrank_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
         configured_device = dev;
     }
-    cudaLaunchAttribute attrs[1];
+    const bool cluster = p.ks > 1 && p.ks <= kLruClusterParts;
+    cudaLaunchAttribute attrs[2];
     attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attrs[0].val.programmaticStreamSerializationAllowed = launch_overlap_allowed();
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = (unsigned)p.ks; attrs[1].val.clusterDim.y = 1; attrs[1].val.clusterDim.z = 1;
     {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)(p.tiles * p.ks * n_problems), 1, 1);
@@ -282,14 +315,14 @@ int launch_lowrank_umma(const void* x, int64_t M, int64_t K, int64_t ldx, int n_
         cfg.dynamicSmemBytes = smem_bytes;
         cfg.stream = stream;
         cfg.attrs = attrs;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = cluster ? 2 : 1;
         ProfScope prof(kProfRotateQuant, stream);
         cudaError_t e = cudaLaunchKernelEx(&cfg, lowrank_umma_kernel, xm, maps, p);
         if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e); }
         int st = after_launch();
         if (st != BWLA_OK) return st;
     }
-    if (p.ks > 1) {
+    if (p.ks > 1 && !cluster) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)(p.tiles * (kCols / 8) * n_problems), 1, 1);
         cfg.blockDim = dim3(kTok, 1, 1);
