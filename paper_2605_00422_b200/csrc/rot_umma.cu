@@ -129,7 +129,7 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     const RotUmmaGeom& g = p.g;
     ru::Shared& sh = *reinterpret_cast<ru::Shared*>(smem + g.sh_off);
     volatile int* abort_flag = &sh.abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int rank = g.dc > 1 ? (int)cluster_ctarank() : 0;
     const int cl = (int)blockIdx.x / g.dc;
     const int prob_i = cl / p.clusters_per_problem;
@@ -216,52 +216,51 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             if (*abort_flag) for (int i = 0; i < 500; ++i) __nanosleep(100);
         }
     } else if (warp == 1) {
-        // ---------------- MMAs ----------------
-        if (elect_one()) {
-            const uint32_t idesc_a = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.ntot >> 3) << 17) | ((128u >> 4) << 24);
-            const uint32_t idesc_c = (1u << 4) | ((uint32_t)(g.nc >> 3) << 17) | ((128u >> 4) << 24);
-            const uint64_t d_p2 = smem_desc_kmajor(smem_u32(smem), 64), d_p1 = smem_desc_kmajor(smem_u32(smem + g.p1_off), 64);
-            const uint64_t d_x = smem_desc_kmajor(smem_u32(smem + g.x_off), 64);
-            const uint32_t blk2 = (uint32_t)(g.dt * 64) >> 4, blkx = (uint32_t)(g.ntot * 64) >> 4, blk1 = (uint32_t)(g.nc * 64) >> 4;
-            const int ks2 = g.n2 >> 4, ks1 = g.nc >> 4, half2 = (ks2 + 1) >> 1, half1 = (ks1 + 1) >> 1;
-            auto put_z = [&](int i) -> bool {
-                const int b = g.xb == 2 ? i & 1 : 0;
-                const uint32_t use = (uint32_t)(g.xb == 2 ? i >> 1 : i);
-                if (!wait_or_abort(&sh.x_full[b], use & 1u, abort_flag)) { give_up(p.status, abort_flag, 0x220); return false; }
-                if (i >= 1 && !wait_or_abort(&sh.d_free, phase_of(i) ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x221); return false; }
-                tc_fence_after();
-                const uint64_t xd = d_x + (uint64_t)((uint32_t)(b * g.atoms2) * blkx);
-                for (int term = 2; term >= 0; --term)
-                    for (int k = 0; k < ks2; ++k) {
-                        const int h = k >= half2;
-                        const uint32_t d = tmem + (uint32_t)(h * g.ntot);
-                        const uint32_t acc = (term == 2 && (k == 0 || k == half2)) ? 0u : 1u;
-                        mma_f16_ss(d, d_p2 + (uint64_t)((uint32_t)(term * g.atoms2 + (k >> 1)) * blk2 + 2u * (k & 1)),
-                                   xd + (uint64_t)((uint32_t)(k >> 1) * blkx + 2u * (k & 1)), idesc_a, acc);
-                    }
-                tc_commit(&sh.x_empty[b]);
-                tc_commit(&sh.z_full);
-                return true;
-            };
-            for (int i = 0; i < n; ++i) {
-                if (!put_z(i)) break;
-                if (!wait_or_abort(&sh.a_ready, (uint32_t)(i & 1), abort_flag)) { give_up(p.status, abort_flag, 0x222); break; }
-                tc_fence_after();
-                for (int tk = 0; tk < g.tps; ++tk) {
-                    const uint32_t a = tmem + (uint32_t)(2 * g.ntot + tk * (g.np >> 1));
-                    // lo hi, hi lo, hi hi
+        // ---------------- MMAs (all lanes in step: see umma_ptx.cuh) ----------------
+        const bool one = elect_one();
+        const uint32_t idesc_a = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.ntot >> 3) << 17) | ((128u >> 4) << 24);
+        const uint32_t idesc_c = (1u << 4) | ((uint32_t)(g.nc >> 3) << 17) | ((128u >> 4) << 24);
+        const uint64_t d_p2 = smem_desc_kmajor(smem_u32(smem), 64), d_p1 = smem_desc_kmajor(smem_u32(smem + g.p1_off), 64);
+        const uint64_t d_x = smem_desc_kmajor(smem_u32(smem + g.x_off), 64);
+        const uint32_t desc_hi = (uint32_t)(d_p2 >> 32);                      // (the same for all three)
+        const uint32_t blk2 = (uint32_t)(g.dt * 64) >> 4, blkx = (uint32_t)(g.ntot * 64) >> 4, blk1 = (uint32_t)(g.nc * 64) >> 4;
+        const int ks2 = g.n2 >> 4, ks1 = g.nc >> 4, half2 = (ks2 + 1) >> 1, half1 = (ks1 + 1) >> 1;
+        for (int i = 0; i < n; ++i) {
+            const int b = g.xb == 2 ? i & 1 : 0;
+            const uint32_t use = (uint32_t)(g.xb == 2 ? i >> 1 : i);
+            if (!warp_wait(&sh.x_full[b], use & 1u, abort_flag)) { give_up(p.status, abort_flag, 0x220); break; }
+            if (i >= 1 && !warp_wait(&sh.d_free, phase_of(i) ^ 1u, abort_flag)) { give_up(p.status, abort_flag, 0x221); break; }
+            tc_fence_after();
+            const uint32_t x0 = (uint32_t)d_x + (uint32_t)(b * g.atoms2) * blkx;
 #pragma unroll 1
-                    for (int q = 0; q < 3; ++q)
-                        for (int k = 0; k < ks1; ++k) {
-                            const int h = k >= half1;
-                            const uint32_t d = tmem + (uint32_t)(h * g.ntot + tk * g.np);
-                            mma_f16_ts(d, a + (q == 0 ? (uint32_t)(g.ntot >> 1) : 0u) + 8u * k,
-                                       d_p1 + (uint64_t)((uint32_t)((q == 1 ? g.atoms1 : 0) + (k >> 1)) * blk1 + 2u * (k & 1)), idesc_c,
-                                       (q == 0 && (k == 0 || k == half1)) ? 0u : 1u);
-                        }
+            for (int term = 2; term >= 0; --term) {
+                uint32_t at = (uint32_t)d_p2 + (uint32_t)(term * g.atoms2) * blk2, bt = x0;
+#pragma unroll 2
+                for (int k = 0; k < ks2; ++k) {
+                    warp_mma_f16_ss(one, k >= half2 ? tmem + (uint32_t)g.ntot : tmem, at, desc_hi, bt, desc_hi, idesc_a, (term == 2 && (k == 0 || k == half2)) ? 0u : 1u);
+                    at += k & 1 ? blk2 - 2u : 2u;
+                    bt += k & 1 ? blkx - 2u : 2u;
                 }
-                tc_commit(&sh.y_full);
             }
+            warp_commit(one, &sh.x_empty[b]);
+            warp_commit(one, &sh.z_full);
+            if (!warp_wait(&sh.a_ready, (uint32_t)(i & 1), abort_flag)) { give_up(p.status, abort_flag, 0x222); break; }
+            tc_fence_after();
+            for (int tk = 0; tk < g.tps; ++tk) {
+                const uint32_t a = tmem + (uint32_t)(2 * g.ntot + tk * (g.np >> 1)), y = tmem + (uint32_t)(tk * g.np);
+                // lo hi, hi lo, hi hi
+#pragma unroll 1
+                for (int q = 0; q < 3; ++q) {
+                    uint32_t at = a + (q == 0 ? (uint32_t)(g.ntot >> 1) : 0u), bt = (uint32_t)d_p1 + (q == 1 ? (uint32_t)g.atoms1 * blk1 : 0u);
+#pragma unroll 2
+                    for (int k = 0; k < ks1; ++k) {
+                        warp_mma_f16_ts(one, k >= half1 ? y + (uint32_t)g.ntot : y, at, bt, desc_hi, idesc_c, (q == 0 && (k == 0 || k == half1)) ? 0u : 1u);
+                        at += 8u;
+                        bt += k & 1 ? blk1 - 2u : 2u;
+                    }
+                }
+            }
+            warp_commit(one, &sh.y_full);
         }
     } else if (warp == 3) {
         // ---------------- code sums and staged outputs of a step ----------------
