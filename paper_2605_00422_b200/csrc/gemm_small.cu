@@ -82,9 +82,6 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
-__device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
 
 // NTP: token tiles of 8; PL: digit planes per token; SPLIT: clusters split K
 template <int NTP, int PL, bool SPLIT>
@@ -440,7 +437,9 @@ static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int 
         const int group_bytes = 2 * NT * 512;
         const int fit = (kSmemMax - off) / group_bytes;
         if (fit < 1) continue;
-        const int total = std::min((sms - spare) / S, S == 1 ? sms : resident_small_clusters(S));      // clusters the device holds
+        // Clusters the device holds.  Those that a rotation's cluster leaves no room would start, and fetch their constants, when it has ended: two
+        // are left out (a decode block of one token, 160 x 160 before the down projection: 83.1 us with all, 81.0 less one, 80.8 less two).
+        const int total = std::min((sms - spare) / S, S == 1 ? sms : resident_small_clusters(S) - (spare > 0 && PL == 1 ? 2 : 0));
         if (total < n) break;
         int groups[kRotMaxProblems], used = 0, longest = 1;
         int64_t all = 0;

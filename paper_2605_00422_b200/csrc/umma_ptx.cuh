@@ -346,6 +346,10 @@ __device__ __forceinline__ void warp_commit(bool one, uint64_t* bar) {
 // (the warp's index as a value that the compiler knows to be the same in all lanes)
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }
 
+__device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // ---- registers of a warpgroup, bulk copies out of shared memory ----
 template <int N>
 __device__ __forceinline__ void set_regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
