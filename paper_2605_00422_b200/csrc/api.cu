@@ -98,8 +98,7 @@ struct bwla_layer {
     uint8_t* prepared;
     bool rot;                 // the tensor-core rotation takes these factor sizes
     RotGeom geom;
-    uint8_t* rows;            // the factors once more in rot_rows.cu's form, inside `prepared`, or NULL where that kernel is not chosen
-    uint8_t* okt;             // the factors once more in okt_umma.cu's form, inside `prepared`, or NULL where that kernel is not chosen
+    uint8_t* many;            // the factors once more in the form of the kernel that many tokens of theirs go to (RotProblem), inside `prepared`, or NULL
     int asym;                 // activation quantiser: 0 symmetric, 1 asymmetric (per-token zero point)
     int32_t* rowsum;          // [N] sign sums of the rows, inside `prepared`
 };
@@ -293,15 +292,14 @@ int bwla_workspace_section(int64_t M, int64_t K, int64_t N, int r, int bits, int
 
 // ---- prepared layers -------------------------------------------------------------------------------------------
 
-struct PreparedLayout { bool rot; RotGeom geom; bool has_rows; RotRowsGeom rows_geom; bool has_okt; OktGeom okt_geom; size_t rows, okt, rowsum; };
+struct PreparedLayout { bool rot; RotGeom geom; bool has_rows; RotRowsGeom rows_geom; bool has_okt; OktGeom okt_geom; size_t many, rowsum; };
 static PreparedLayout prepared_layout(int n1, int n2) {
     PreparedLayout p{};
     p.rot = rot_geometry(n1, n2, &p.geom);
-    p.rows = p.rot ? align_up(rot_prepared_bytes(p.geom), 256) : 256;
-    p.has_rows = p.rot && rot_rows_geometry(n1, n2, 2, &p.rows_geom);      // (the factors' place does not depend on the outputs' size)
-    p.okt = p.rows + (p.has_rows ? align_up(rot_rows_prepared_bytes(p.rows_geom), 256) : 0);
-    p.has_okt = p.rot && rot_okt_factors(p.geom) && okt_geometry(n1, n2, &p.okt_geom);
-    p.rowsum = p.okt + (p.has_okt ? align_up(okt_prepared_bytes(p.okt_geom), 256) : 0);
+    p.many = p.rot ? align_up(rot_prepared_bytes(p.geom), 256) : 256;
+    p.has_rows = p.rot && rot_rows_geometry(n1, n2, 1, &p.rows_geom);      // (codes; where the factors lie does not depend on the outputs' size)
+    p.has_okt = p.rot && !p.has_rows && rot_okt_factors(p.geom) && okt_geometry(n1, n2, &p.okt_geom);
+    p.rowsum = p.many + (p.has_rows ? align_up(rot_rows_prepared_bytes(p.rows_geom), 256) : p.has_okt ? align_up(okt_prepared_bytes(p.okt_geom), 256) : 0);
     return p;
 }
 
@@ -331,14 +329,13 @@ int bwla_layer_create(bwla_layer** layer, int64_t K, int64_t N, const float* P1,
     L->prepared = (uint8_t*)prepared;
     const PreparedLayout lay = prepared_layout(n1, n2);
     L->rot = lay.rot; L->geom = lay.geom;
-    L->rows = lay.has_rows ? L->prepared + lay.rows : nullptr;
-    L->okt = lay.has_okt ? L->prepared + lay.okt : nullptr;
+    L->many = lay.has_rows || lay.has_okt ? L->prepared + lay.many : nullptr;
     L->asym = 0;
     L->rowsum = (int32_t*)(L->prepared + lay.rowsum);
     if (L->rot) {
         st = launch_prepare_rot(L->geom, P1, P2, prepared, (cudaStream_t)stream);
-        if (st == BWLA_OK && L->rows) st = launch_prepare_rows(lay.rows_geom, P1, P2, L->rows, (cudaStream_t)stream);
-        if (st == BWLA_OK && L->okt) st = launch_prepare_okt(lay.okt_geom, P1, P2, L->okt, (cudaStream_t)stream);
+        if (st == BWLA_OK && lay.has_rows) st = launch_prepare_rows(lay.rows_geom, P1, P2, L->many, (cudaStream_t)stream);
+        if (st == BWLA_OK && lay.has_okt) st = launch_prepare_okt(lay.okt_geom, P1, P2, L->many, (cudaStream_t)stream);
         if (st != BWLA_OK) { free(L); return st; }
     }
     st = launch_row_sums(packed, N, K, L->rowsum, (cudaStream_t)stream);
@@ -367,7 +364,7 @@ int bwla_layer_rotate_quant_asym(const bwla_layer* L, const void* x_bf16, int64_
     if (!L->rot || !rot_accepts_x(x_bf16, ldx)) return BWLA_ERR_UNSUPPORTED;
     // the kernel keeps u - 2^(b-1) so that codes fit int8; the bias puts u and the zero point back in [0, 2^b - 1]
     RotProblem pr{};
-    pr.prepared = L->prepared; pr.rows = L->rows; pr.okt = L->okt; pr.codes = (int8_t*)codes; pr.zp = zeros; pr.code_bias = 1 << (L->bits - 1); pr.scales = scales; pr.y = y_f32;
+    pr.prepared = L->prepared; pr.many = L->many; pr.codes = (int8_t*)codes; pr.zp = zeros; pr.code_bias = 1 << (L->bits - 1); pr.scales = scales; pr.y = y_f32;
     return launch_rot(L->geom, x_bf16, M, ldx, L->bits, 1, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
@@ -381,7 +378,7 @@ int bwla_layer_rotate_quant(const bwla_layer* L, const void* x_bf16, int64_t M, 
     if (st != BWLA_OK) return st;
     if (L->rot && g_forced_rotation != BWLA_ROT_SIMT) {
         RotProblem pr{};
-        pr.prepared = L->prepared; pr.rows = L->rows; pr.okt = L->okt; pr.codes = codes; pr.scales = scales; pr.y = y_f32;
+        pr.prepared = L->prepared; pr.many = L->many; pr.codes = codes; pr.scales = scales; pr.y = y_f32;
         return launch_rot(L->geom, x_bf16, M, ldx, L->bits, 0, 1, &pr, nullptr, nullptr, (cudaStream_t)stream);
     }
     if (y_f32) return BWLA_ERR_UNSUPPORTED;      // only the tensor-core kernel can hand out Y
@@ -441,7 +438,7 @@ int bwla_layer_w1a16_linear(const bwla_layer* L, const void* x_bf16, int64_t M, 
         }
     }
     RotProblem pr{};
-    pr.prepared = L->prepared; pr.rows = L->rows; pr.yhat = (__nv_bfloat16*)(base + w.yhat); pr.ysum = L->mu ? (float*)(base + w.ysum) : nullptr;
+    pr.prepared = L->prepared; pr.many = L->many; pr.yhat = (__nv_bfloat16*)(base + w.yhat); pr.ysum = L->mu ? (float*)(base + w.ysum) : nullptr;
     const bool persistent = a16_persistent_supports(L->K);
     pr.codes_layout = persistent ? 1 : 0;
     st = launch_rot(L->geom, x_bf16, M, ldx, 8, 0, 1, &pr, &lr, status, s);
@@ -509,7 +506,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         for (int i = 0; i < count; ++i) {
             const bwla_layer* L = layers[i];
             pr[i] = RotProblem{};
-            pr[i].prepared = L->prepared; pr[i].rows = L->rows; pr[i].okt = L->okt; pr[i].codes = (int8_t*)(wbase[i] + ws[i].codes); pr[i].codes_layout = path[i] == BWLA_PATH_I8 ? 1 : 0;
+            pr[i].prepared = L->prepared; pr[i].many = L->many; pr[i].codes = (int8_t*)(wbase[i] + ws[i].codes); pr[i].codes_layout = path[i] == BWLA_PATH_I8 ? 1 : 0;
             pr[i].zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr;
             pr[i].scales = (float*)(wbase[i] + ws[i].scales); pr[i].qsum = (int32_t*)(wbase[i] + ws[i].qsum);
             lr[i] = OktLowrank{L->V, L->r, wbase[i] + ws[i].T, L->r > 0 ? (float*)(wbase[i] + ws[i].lr_part) : nullptr,

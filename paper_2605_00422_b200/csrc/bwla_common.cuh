@@ -136,8 +136,7 @@ constexpr int kRotMaxProblems = 4;          // linears that share one x and are 
 struct RotProblem {
     const uint8_t* prepared;    // terms of P2^T and P1^T (launch_prepare_rot), or NULL: P1 and P2 are split by every CTA
     const float *P1, *P2;       // read only when `prepared` is NULL
-    const uint8_t* rows;        // beside `prepared`: the terms in the layout of rot_rows.cu, or NULL where that kernel is not chosen
-    const uint8_t* okt;         // beside `prepared`: the terms in the layout of okt_umma.cu, or NULL where that kernel is not chosen
+    const uint8_t* many;        // beside `prepared`: the terms in the layout of rot_rows.cu, or for factors that it does not take of okt_umma.cu, or NULL
     // quantiser (yhat == NULL)
     int8_t* codes;              // [M][K]
     int codes_layout;           // 0: natural k order; 1: the interleaved order of the tensor-core contraction

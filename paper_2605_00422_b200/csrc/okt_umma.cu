@@ -290,10 +290,10 @@ okt_umma_kernel(const __grid_constant__ CUtensorMap x_map, const OktKernelParams
         mbar_init(const_full, 1);
         fence_barrier_init();
         fence_proxy_async();
-        if (pr.okt) {
+        if (pr.many) {
             const int p2_region = (g.p2t_bytes + 1023) / 1024 * 1024, p1_region = (g.p1t_bytes + 1023) / 1024 * 1024;
-            const uint8_t* src2 = pr.okt + (size_t)dt * p2_region;
-            const uint8_t* src1 = pr.okt + (size_t)g.dt_count * p2_region + (size_t)cs * p1_region;
+            const uint8_t* src2 = pr.many + (size_t)dt * p2_region;
+            const uint8_t* src1 = pr.many + (size_t)g.dt_count * p2_region + (size_t)cs * p1_region;
             mbar_expect_tx(const_full, (uint32_t)(g.p2t_bytes + g.p1t_bytes));
             for (int off = 0; off < g.p2t_bytes; off += 16384)
                 tma_bulk_g2s(p2t + off, src2 + off, (uint32_t)min(16384, g.p2t_bytes - off), const_full);
@@ -317,7 +317,7 @@ okt_umma_kernel(const __grid_constant__ CUtensorMap x_map, const OktKernelParams
         tmem_alloc(tmem_slot, (uint32_t)g.tmem_cols);
         tmem_relinquish();
     }
-    if (!pr.okt) {
+    if (!pr.many) {
         // raw factors: every CTA splits what it needs of them, into the places where prepare_okt_kernel's terms would be copied
         auto place = [](uint8_t* at, int rows, int atom) {
             const int sh = 31 - __clz(atom);
@@ -381,7 +381,7 @@ okt_umma_kernel(const __grid_constant__ CUtensorMap x_map, const OktKernelParams
             const int steps2 = g.atom2 / 32, steps1 = g.atom1 / 32;           // MMAs (K = 16) per K-atom: 1, 2 or 4
             const uint32_t lo_p2 = (uint32_t)dP2, hi_p2 = (uint32_t)(dP2 >> 32), lo_x = (uint32_t)dX, hi_x = (uint32_t)(dX >> 32),
                            lo_p1 = (uint32_t)dP1, hi_p1 = (uint32_t)(dP1 >> 32);
-            bool ok = !pr.okt || wait_or_abort(const_full, 0, abort_flag);
+            bool ok = !pr.many || wait_or_abort(const_full, 0, abort_flag);
             if (!ok) give_up(p.status, abort_flag, 0x61);
             for (int it = 0; it < ntok && ok; ++it) {
                 const uint32_t ph = (uint32_t)(it & 1);

@@ -213,7 +213,8 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uin
 // Up to 64 tokens: T for a tile of 16 tokens x 8 NTC columns and a part of K per block.  What such a block costs is latency:
 // V comes from HBM and is requested before the preceding kernel has finished (two or four chunks per warp), x follows
 // in one round trip, and K is cut into as many parts as give every warp about that many.
-template <int NTC, int U = 8 / NTC>                          // U: chunks of a warp in registers at once
+// U: chunks of a warp in registers at once.  STATIC: a word of static shared memory (rot_rows.cu has no room for one before its dynamic memory)
+template <int NTC, int U = 8 / NTC, bool STATIC = true>
 static __device__ void lowrank_mma_role(const PrologueParams& p, int b, float* smem) {
     constexpr int COLS = 8 * NTC;
     const int jtiles = (p.lr_cols + COLS - 1) / COLS;
@@ -314,10 +315,14 @@ static __device__ void lowrank_mma_role(const PrologueParams& p, int b, float* s
     if (KS > 1) {
         __threadfence();
         __syncthreads();
-        // (in place of the sums, which have been read)
-        if (threadIdx.x == 0) *reinterpret_cast<uint32_t*>(red) = atomicAdd(p.lr_count + tile, 1u);
+        volatile uint32_t* arrived = reinterpret_cast<volatile uint32_t*>(red);          // (in place of the sums, which have been read)
+        if constexpr (STATIC) {
+            __shared__ uint32_t word;
+            arrived = &word;
+        }
+        if (threadIdx.x == 0) *arrived = atomicAdd(p.lr_count + tile, 1u);
         __syncthreads();
-        if (*reinterpret_cast<volatile uint32_t*>(red) != (uint32_t)(KS - 1)) return;
+        if (*arrived != (uint32_t)(KS - 1)) return;
         __threadfence();
         for (int o = threadIdx.x; o < 16 * COLS; o += blockDim.x) {
             float s = 0.f;

@@ -939,8 +939,9 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
         if (fits) return launch_rot_rows(base, x, M, ldx, bits, asym, n_problems, problems, beside, status, stream);
     }
     if (!few && vec) {
-        bool okt = rot_okt_factors(base) && !problems[0].yhat && !problems[0].digits;
-        for (int i = 0; i < n_problems; ++i) okt = okt && (problems[i].okt || !problems[i].prepared);
+        RotRowsGeom rows;
+        bool okt = rot_okt_factors(base) && !problems[0].yhat && !problems[0].digits && !rot_rows_geometry(base.n1, base.n2, 1, &rows);
+        for (int i = 0; i < n_problems; ++i) okt = okt && (problems[i].many || !problems[i].prepared);
         OktGeom og;
         if (okt && okt_geometry(base.n1, base.n2, &og)) {
             st = own_launch(false);

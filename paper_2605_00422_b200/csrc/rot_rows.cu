@@ -186,8 +186,8 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         const int lb = (int)blockIdx.x - p.rot_ctas;
         int j = 0;
         while (j + 1 < p.n_problems && lb >= p.lr_begin[j + 1]) ++j;
-        if (p.lr[j].lr_wide == 4) lowrank_mma_role<4, 1>(p.lr[j], lb - p.lr_begin[j], reinterpret_cast<float*>(smem));
-        else lowrank_mma_role<2, 2>(p.lr[j], lb - p.lr_begin[j], reinterpret_cast<float*>(smem));
+        if (p.lr[j].lr_wide == 4) lowrank_mma_role<4, 1, false>(p.lr[j], lb - p.lr_begin[j], reinterpret_cast<float*>(smem));
+        else lowrank_mma_role<2, 2, false>(p.lr[j], lb - p.lr_begin[j], reinterpret_cast<float*>(smem));
         return;
     }
     const int prob_i = (int)blockIdx.x / p.ctas_per_problem;
@@ -214,12 +214,12 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     // ---- the layer's factors (they do not depend on the preceding kernel; those of a binarisation may be what it has made) ----
     if (MODE == kRowsBinarize) griddep_wait();
     int e2;
-    if (pr.rows) {
-        e2 = __ldg(reinterpret_cast<const int*>(pr.rows));
+    if (pr.many) {
+        e2 = __ldg(reinterpret_cast<const int*>(pr.many));
         if (threadIdx.x == 0) {
             fence_proxy_async();
             mbar_expect_tx(&sh.fac_full, (uint32_t)g.x_off);
-            tma_bulk_g2s(smem, pr.rows + kRotHeader, (uint32_t)g.x_off, &sh.fac_full);
+            tma_bulk_g2s(smem, pr.many + kRotHeader, (uint32_t)g.x_off, &sh.fac_full);
         }
     } else {
         e2 = rot_rows_split(g, pr.P1, pr.P2, smem, sh.vmax[0][0], threadIdx.x, blockDim.x);
@@ -266,7 +266,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         const uint32_t p1_hi = (uint32_t)(d_p1 >> 32), x_hi = (uint32_t)(d_x >> 32);
         const uint32_t blk1 = (uint32_t)(g.lanes * 64) >> 4, n2 = (uint32_t)g.n2;
         bool ok = true;
-        if (pr.rows && !warp_wait(&sh.fac_full, 0u, abort_flag)) { give_up(p.status, abort_flag, 0x521); ok = false; }
+        if (pr.many && !warp_wait(&sh.fac_full, 0u, abort_flag)) { give_up(p.status, abort_flag, 0x521); ok = false; }
         for (int i = 0; i < n && ok; ++i) {
             const int b = g.xb == 2 ? i & 1 : 0;
             const uint32_t use = (uint32_t)(g.xb == 2 ? i >> 1 : i);
@@ -775,7 +775,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
 // ---------------------------------------------------------------------------------------------
 bool rot_rows_supports(const RotGeom& base, int n_problems, const RotProblem* problems) {
     for (int i = 0; i < n_problems; ++i)
-        if (problems[i].digits || problems[i].packed || (problems[i].prepared && !problems[i].rows)) return false;
+        if (problems[i].digits || problems[i].packed || (problems[i].prepared && !problems[i].many)) return false;
     RotRowsGeom g;
     return rot_rows_geometry(base.n1, base.n2, problems[0].yhat ? 2 : 1, &g);
 }
