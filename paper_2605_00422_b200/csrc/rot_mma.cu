@@ -516,7 +516,8 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             barrier();                                // Z^T is no longer needed: its place is x's again
             if (!F32 && more) { zero_padding(); fetch_x(t + stride); }
         }
-        // ---- back to true scale (exact: powers of two), then what the caller wants of Y
+        // ---- back to true scale (exact: powers of two; a binarisation scales its sums), then what the caller wants of Y
+        if (MODE != kRotBinarize) {
         const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
         const float f1 = pow2f(ey1);
 #pragma unroll
@@ -525,6 +526,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             const float f2 = pow2f(ey2);
 #pragma unroll
             for (int j = 0; j < NTW; ++j) { mul2(acc[j][0], acc[j][1], f2); mul2(acc[j][2], acc[j][3], f2); }
+        }
         }
         }
         float amax = 0.f, vmin = 0.f;                 // asymmetric: amax holds the largest value, zero included
@@ -712,7 +714,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             // the weight-only operating point: bf16 values (layout 1: inside each group of 32, position 2 (k % 16) +
             // (k % 32) / 16), and where asked for their sum
             __nv_bfloat16* yt = pr.yhat + t * (int64_t)g.K;
-            double s = 0.0;
+            float hi = 0.f, lo = 0.f;
 #pragma unroll
             for (int j = 0; j < NTW; ++j) {
 #pragma unroll
@@ -724,38 +726,43 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
                                 const int k = off_lo[e] + 8 * h + j * 8 * g.n2;
                                 const __nv_bfloat16 v = __float2bfloat16_rn(acc[j][2 * h + e]);
                                 yt[pr.codes_layout ? (k & ~31) + 2 * (k & 15) + ((k >> 4) & 1) : k] = v;
-                                if (pr.ysum) s += (double)__bfloat162float(v);
+                                if (pr.ysum) sum2(hi, lo, __bfloat162float(v));
                             }
                         }
                     }
                 }
             }
             if (pr.ysum) {
-                s = total_sum(s, par);
+                // (no error of an addition that left fp32's range)
+                const double s = total_sum((double)hi + (isfinite(hi) ? (double)lo : 0.0), par);
                 if (tid == 0 && rank == 0) pr.ysum[t] = (float)s;
             }
         } else {
             // Alg. 2, last step: the row's mean, its mean absolute deviation, and the signs about the mean
-            double s = 0.0;
+            float hi = 0.f, lo = 0.f;
 #pragma unroll
             for (int j = 0; j < NTW; ++j)             // (padding rows and columns are zeros)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) s += (double)acc[j][i];
-            const double mean = total_sum(s, 0) / (double)g.K;
-            double dev = 0.0;
+                for (int i = 0; i < 4; ++i) sum2(hi, lo, acc[j][i]);
+            const double mean = total_sum((double)hi + (double)lo, 0) / (double)g.K;
+            const float mean_hi = (float)mean, mean_lo = (float)(mean - (double)mean_hi);
+            float dev = 0.f, dev_lo = 0.f;
             uint32_t mine = 0u;                       // ballot number `lane` of the warp: column tile, row half, column parity
 #pragma unroll
             for (int j = 0; j < NTW; ++j) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const double x = (double)acc[j][i] - mean;
-                    if (8 * j < lim[i & 1] && (i < 2 || row_hi_ok)) dev += fabs(x);
-                    const uint32_t word = __ballot_sync(0xFFFFFFFFu, x > 0.0);
+                    const float x = less2(acc[j][i], mean_hi, mean_lo, 8 * j < lim[i & 1] && (i < 2 || row_hi_ok), dev, dev_lo);
+                    const uint32_t word = __ballot_sync(0xFFFFFFFFu, x > 0.f);
                     if (lane == 4 * j + i) mine = word;
                 }
             }
-            dev = total_sum(dev, 1) / (double)g.K;
-            if (tid == 0 && rank == 0) { pr.mu[t] = (float)mean; pr.alpha[t] = (float)dev; }
+            const double all = total_sum((double)dev + (double)dev_lo, 1) / (double)g.K;
+            if (tid == 0 && rank == 0) {
+                const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
+                const double scale = (double)pow2f(ey1) * (double)pow2f(ey2);
+                pr.mu[t] = (float)(mean * scale); pr.alpha[t] = (float)(all * scale);
+            }
             // bit 4 r + q of a ballot is row r (of the half), column pair q: the eight rows of a column are one byte of the row
             uint8_t* bytes = reinterpret_cast<uint8_t*>(pr.packed) + t * (int64_t)(g.K >> 3);
             const int j = lane >> 2, e = lane & 1, h = (lane >> 1) & 1;
@@ -979,6 +986,9 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
 int launch_rot_binarize(const RotGeom& g, const void* w, int dtype, int64_t N, int64_t ldw, const RotProblem& problem, uint32_t* status,
                         cudaStream_t stream) {
     if (N >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
+    bool taken = false;
+    const int st = launch_rows_binarize(g, w, dtype, N, ldw, problem, status, &taken, stream);
+    if (taken) return st;
     RotKernelParams p{};
     p.g = g; p.x = w; p.ldx = ldw; p.M = N; p.bits = 8; p.n_problems = 1; p.prob[0] = problem;
     p.status = status; p.groups = choose_groups(g, N, 1);

@@ -27,7 +27,7 @@
 // times as long), 50 now; of 86 x 128 137 and 113.  An MMA of 51 cycles took 110 to issue from run-time loops of one elected thread.
 //
 // Up to 64 x 80, fp32 rows of weights are split into three bf16 terms by the ALU warps, the next step's behind this step's V, and make six products with
-// P1's; mean and mean absolute deviation are summed in fp64, and a lane's signs are neighbouring bits.
+// P1's; mean and mean absolute deviation are summed in two floats, and a lane's signs are neighbouring bits.
 //
 // Launched with programmatic stream serialisation: the factors are fetched before the preceding kernel of the stream has finished; x is
 // read, and everything is stored, after it.  Every wait on an mbarrier is bounded (umma_wait.cuh); a warp whose wait ran out goes on
@@ -60,7 +60,7 @@ struct Shared {
     uint64_t a_ready[2];                  // the terms of V are in tensor memory (by step parity: the ALU warps may be a step ahead)
     uint64_t out_full[2], out_free[2];    // the step's outputs and code sums are staged; have left
     uint32_t vmax[2][2][kSlots], ymax[2][2][kSlots], ymin[2][2][kSlots];       // [step parity][token][warp of the token]
-    uint32_t dev[2][2][kSlots][2];        // ... fp64 sums of a binarisation
+    uint32_t dev[2][2][kSlots][2];        // ... two-float sums of a binarisation
     int qsum[2][2];                       // code sums of the step's tokens
     uint32_t tmem_slot;
     int abort_flag, skip;
@@ -370,11 +370,20 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         const bool gather = MODE != kRowsBinarize && CH == 1 && (g.n2 & 31) == 0;
         const int y0 = gather ? 32 * (wc >> 1) + RUN * (wc & 1) : c0;
         auto column = [&](int e) { return y0 + (gather ? e % RUN + (32 / (16 / RUN)) * (e / RUN) : e); };
+        const double inv = MODE == kRowsBinarize ? 1.0 / (double)g.K : 0.0;
+        const float inv_hi = (float)inv, inv_lo = (float)(inv - (double)inv_hi);
         bool ok = true;
         int z_exp = 0;
         auto token_barrier = [&]() { named_barrier(1 + tk, g.groups * g.lanes); };
         // ---- fp32 rows: eight values of step `i` to the three terms in x's place (rows beyond n1 and M are zeros)
         const int cpr = g.n2 >> 3, alu_threads = 32 * alu_warps;
+        // (the L2 is asked for a step's rows three steps before it: 5120 x 5120 143 us without, 129 with; the first pass over new pages 255 and 194)
+        auto ask_x = [&](int i) {
+            if (!F32 || !p.x_vec || threadIdx.x != rr::kControl || i >= n) return;
+            const int64_t t = (first + (int64_t)i * p.ctas_per_problem) * g.tps;
+            for (int j = 0; j < g.tps && t + j < p.M; ++j)
+                prefetch_l2_bulk(reinterpret_cast<const float*>(p.x) + (t + j) * p.ldx, (uint32_t)(g.K * 4));
+        };
         auto load_x = [&](int i, int j, float (&f)[8]) {
             const int r = j / cpr, a = r & (g.lanes - 1);
             const int64_t t = (first + (int64_t)i * p.ctas_per_problem) * g.tps + r / g.lanes;
@@ -409,6 +418,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         };
         // (128 n2 / 8 pieces a step for 8 n2 threads: two a thread)
         if (F32 && n > 0) {
+            ask_x(1); ask_x(2);
             float f[2][8];
             const int j = threadIdx.x - rr::kControl;
             const bool two = j + alu_threads < 128 * cpr;
@@ -521,14 +531,12 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 }
                 if (MODE == kRowsBf16 || MODE == kRowsBinarize) {
                     if (MODE == kRowsBinarize || pr.ysum) {
-                        // the sum of the (rounded) values goes where the quantiser's two extremes go
-                        double s = 0.0;
+                        // the sum of the values (scaled; or rounded) goes where the quantiser's two extremes go
+                        float hi = 0.f, lo = 0.f;
 #pragma unroll
-                        for (int e = 0; e < NC; ++e)
-                            if (valid) s += (double)(MODE == kRowsBinarize ? y[e] * f1 : __bfloat162float(__float2bfloat16_rn(y[e] * f1)));
-                        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                        const unsigned long long bits = (unsigned long long)__double_as_longlong(s);
-                        top = (uint32_t)bits; bottom = (uint32_t)(bits >> 32);
+                        for (int e = 0; e < NC; ++e) sum2(hi, lo, !valid ? 0.f : MODE == kRowsBinarize ? y[e] : __bfloat162float(__float2bfloat16_rn(y[e] * f1)));
+                        warp_sum2(hi, lo);
+                        top = __float_as_uint(hi); bottom = __float_as_uint(lo);
                     }
                 } else {
 #pragma unroll
@@ -554,7 +562,8 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     const int k0 = c * g.n2 + y0;
                     if (MODE == kRowsBf16) {
                         if (writer && pr.ysum) {
-                            double s = lane < slots ? __hiloint2double((int)s1, (int)s0) : 0.0;
+                            // (no error of an addition that left fp32's range)
+                            double s = lane < slots ? (double)__uint_as_float(s0) + (isfinite(__uint_as_float(s0)) ? (double)__uint_as_float(s1) : 0.0) : 0.0;
                             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
                             if (lane == 0) pr.ysum[t] = (float)s;
                         }
@@ -698,33 +707,34 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             };
             // ---- the step before, a binarisation (Alg. 2, last step): the row's mean, its mean absolute deviation, and the signs about the mean
             auto binarize = [&]() {
-                double s = lane < slots ? __hiloint2double((int)*reinterpret_cast<volatile uint32_t*>(&sh.ymin[par][tk][lane]),
-                                                           (int)*reinterpret_cast<volatile uint32_t*>(&sh.ymax[par][tk][lane])) : 0.0;
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                const double mean = s / (double)g.K;
-                double dev = 0.0;
+                float hi = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.ymax[par][tk][lane])) : 0.f;
+                float lo = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.ymin[par][tk][lane])) : 0.f;
+                warp_sum2(hi, lo);
+                hi = __shfl_sync(0xFFFFFFFFu, hi, 0); lo = __shfl_sync(0xFFFFFFFFu, lo, 0);
+                // the mean (of the scaled values) in two floats
+                const float prod = __fmul_rn(hi, inv_hi), rest = fmaf(hi, inv_hi, -prod) + fmaf(hi, inv_lo, __fmul_rn(lo, inv_hi));
+                const float mean = __fadd_rn(prod, rest), mean_lo = __fadd_rn(__fsub_rn(prod, mean), rest);
+                float dev = 0.f, dev_lo = 0.f;
                 uint32_t bits = 0u;
 #pragma unroll
                 for (int e = 0; e < NC; ++e) {
-                    const double d = (double)(y[e] * f1) - mean;
-                    if (e < have) {
-                        dev += fabs(d);
-                        bits |= d > 0.0 ? 1u << (e & 31) : 0u;
-                    }
+                    bits |= less2(y[e], mean, mean_lo, true, dev, dev_lo) > 0.f ? 1u << (e & 31) : 0u;
                 }
                 if (ok && valid && t < p.M) {
                     reinterpret_cast<uint16_t*>(pr.packed)[(t * (int64_t)g.K + c * g.n2 + y0) >> 4] = (uint16_t)bits;
                 }
-                if (!valid) dev = 0.0;
-                for (int o = 16; o > 0; o >>= 1) dev += __shfl_xor_sync(0xFFFFFFFFu, dev, o);
-                const unsigned long long word = (unsigned long long)__double_as_longlong(dev);
-                if (lane == 0) { sh.dev[par][tk][slot][0] = (uint32_t)word; sh.dev[par][tk][slot][1] = (uint32_t)(word >> 32); }
+                if (!valid) dev = dev_lo = 0.f;
+                warp_sum2(dev, dev_lo);
+                if (lane == 0) { sh.dev[par][tk][slot][0] = __float_as_uint(dev); sh.dev[par][tk][slot][1] = __float_as_uint(dev_lo); }
                 token_barrier();
                 if (slot == 0) {
-                    double all = lane < slots ? __hiloint2double((int)*reinterpret_cast<volatile uint32_t*>(&sh.dev[par][tk][lane][1]),
-                                                                 (int)*reinterpret_cast<volatile uint32_t*>(&sh.dev[par][tk][lane][0])) : 0.0;
-                    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xFFFFFFFFu, all, o);
-                    if (lane == 0 && ok && t < p.M) { pr.mu[t] = (float)mean; pr.alpha[t] = (float)(all / (double)g.K); }
+                    float all = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.dev[par][tk][lane][0])) : 0.f;
+                    float all_lo = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.dev[par][tk][lane][1])) : 0.f;
+                    warp_sum2(all, all_lo);
+                    if (lane == 0 && ok && t < p.M) {
+                        pr.mu[t] = mean * f1;
+                        pr.alpha[t] = (float)(((double)all + (double)all_lo) / (double)g.K * (double)f1);
+                    }
                 }
             };
             const int ze = z_exp;
@@ -734,6 +744,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     float f[2][8];
                     const int j = threadIdx.x - rr::kControl;
                     const bool more = F32 && i + 1 < n, two = j + alu_threads < 128 * cpr;
+                    ask_x(i + 3);
                     if (more) { load_x(i + 1, j, f[0]); if (two) load_x(i + 1, j + alu_threads, f[1]); }
                     load_v();
                     if (more) { put_x(j, f[0]); if (two) put_x(j + alu_threads, f[1]); x_done(); }

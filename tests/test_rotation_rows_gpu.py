@@ -83,3 +83,32 @@ def test_an_infinity_stays_in_its_token(n1, n2):
     c2, s2 = bwla.bwla_layer_rotate_quant(L, bad)[:2]
     keep = torch.ones(300, dtype=torch.bool); keep[[4, 9, 131]] = False
     assert torch.equal(codes.cpu()[keep], c2.cpu()[keep]) and torch.equal(scales.cpu()[keep], s2.cpu()[keep])
+
+
+@pytest.mark.parametrize("n1,n2,N,pad", [(33, 32, 149, 0), (40, 48, 301, 1), (64, 80, 75, 4)])
+def test_binarised_rows(n1, n2, N, pad):
+    """fp32 rows as three terms, in 16-byte pieces and in single loads, ragged last steps; the bounds of tests/test_binarize_gpu.py."""
+    from paper_2605_00422_b200 import bwla
+    from tests.test_binarize_gpu import _check
+    rng = np.random.default_rng([n1, n2, N])
+    P1, P2 = gen.orthogonal_f32(n1, rng), gen.orthogonal_f32(n2, rng)
+    W = (rng.standard_normal((N, n1 * n2)) * 0.02 + rng.uniform(-0.01, 0.01, (N, 1))).astype(np.float32)
+    big = torch.zeros(N, n1 * n2 + pad, device="cuda")
+    big[:, :n1 * n2] = torch.from_numpy(W).cuda()
+    _check(bwla, W, big[:, :n1 * n2], P1, P2)
+
+
+def test_a_linear_behind_binarised_rows():
+    """The linear's sign words, scales and shifts are fetched before it waits for its predecessor: it must see what that has written."""
+    from paper_2605_00422_b200 import bwla
+    n1, n2, N, K = 64, 64, 3000, 4096
+    rng = np.random.default_rng(6)
+    P1, P2 = H.f32_to_dev(gen.orthogonal_f32(n1, rng)), H.f32_to_dev(gen.orthogonal_f32(n2, rng))
+    x = H.bf16_to_dev(gen.bf16_bits_from_f32(rng.standard_normal((1, K)).astype(np.float32)))
+    for _ in range(4):
+        W = torch.from_numpy((rng.standard_normal((N, K)) * 0.02).astype(np.float32)).cuda()
+        torch.cuda.synchronize()
+        packed, alpha, mu = bwla.bwla_binarize_rows(W, P1, P2)
+        out = bwla.bwla_w1ax_linear(x, P1, P2, 6, packed, alpha, mu=mu)
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), bwla.bwla_w1ax_linear(x, P1, P2, 6, packed, alpha, mu=mu).view(torch.int16))
