@@ -713,8 +713,9 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
         } else if (MODE == kRotBf16) {
             // the weight-only operating point: bf16 values (layout 1: inside each group of 32, position 2 (k % 16) +
             // (k % 32) / 16), and where asked for their sum
+            // (in fp64: sums in two floats cost the call without a shift, which has no sum, registers, 8.4 -> 9.0 us at 73 tokens of 64 x 64)
             __nv_bfloat16* yt = pr.yhat + t * (int64_t)g.K;
-            float hi = 0.f, lo = 0.f;
+            double s = 0.0;
 #pragma unroll
             for (int j = 0; j < NTW; ++j) {
 #pragma unroll
@@ -726,15 +727,14 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
                                 const int k = off_lo[e] + 8 * h + j * 8 * g.n2;
                                 const __nv_bfloat16 v = __float2bfloat16_rn(acc[j][2 * h + e]);
                                 yt[pr.codes_layout ? (k & ~31) + 2 * (k & 15) + ((k >> 4) & 1) : k] = v;
-                                if (pr.ysum) sum2(hi, lo, __bfloat162float(v));
+                                if (pr.ysum) s += (double)__bfloat162float(v);
                             }
                         }
                     }
                 }
             }
             if (pr.ysum) {
-                // (no error of an addition that left fp32's range)
-                const double s = total_sum((double)hi + (isfinite(hi) ? (double)lo : 0.0), par);
+                s = total_sum(s, par);
                 if (tid == 0 && rank == 0) pr.ysum[t] = (float)s;
             }
         } else {
