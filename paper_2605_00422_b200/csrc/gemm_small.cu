@@ -23,7 +23,8 @@
 // memory (rows of 128 bytes, permuted so that every read is free of bank conflicts).  K is split over a cluster of S CTAs
 // where the codes would not fit or rows are few.  The epilogue, once per run, also evaluates U T (bf16 MMAs, three terms of T).
 //
-// PL = 3 is the weight-only operating point for up to 4 tokens whose codes fit one CTA (more: gemm_umma.cu): an activation is a 23-bit fixed-point number of a power-of-two scale, kept as
+// PL = 3 is the weight-only operating point for up to 4 tokens whose codes fit one CTA (more: gemm_umma.cu): an activation is a
+// 23-bit fixed-point number of a power-of-two scale, kept as
 // three signed base-256 digits (rot_mma.cu); the digits are contracted like three tokens' codes, exactly, and put together in
 // the epilogue.
 #include <cuda_bf16.h>

@@ -200,7 +200,9 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         sh.abort_flag = 0;
         mbar_init(&sh.fac_full, 1);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&sh.x_full[i], F32 ? alu_warps : 1); mbar_init(&sh.x_empty[i], 1); mbar_init(&sh.v_full[i], 1); mbar_init(&sh.v_empty[i], 1); mbar_init(&sh.a_ready[i], alu_warps); mbar_init(&sh.y_read[i], alu_warps);
+            mbar_init(&sh.x_full[i], F32 ? alu_warps : 1); mbar_init(&sh.x_empty[i], 1);
+            mbar_init(&sh.v_full[i], 1); mbar_init(&sh.v_empty[i], 1);
+            mbar_init(&sh.a_ready[i], alu_warps); mbar_init(&sh.y_read[i], alu_warps);
             mbar_init(&sh.out_full[i], alu_warps); mbar_init(&sh.out_free[i], 1);
             for (int j = 0; j < 2; ++j) sh.qsum[i][j] = 0;
         }
