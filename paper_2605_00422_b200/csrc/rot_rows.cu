@@ -230,18 +230,20 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
     if (MODE == kRowsBinarize) {
         // (no dependent starts before this kernel has ended: its outputs are constants of the calls behind it, which they read before they
         // wait; this call clears its status words itself)
-        if (threadIdx.x == 0) sh.skip = 0;
         if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) p.status[threadIdx.x] = 0u;
-    } else {
-        griddep_launch_dependents();
-        griddep_wait();                               // x may be the output of the preceding kernel
-        if (threadIdx.x == 0) sh.skip = p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0;  // the call already failed
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&sh.tmem_slot);
-    const int n = !sh.skip && first < steps_all ? (int)((steps_all - first + p.ctas_per_problem - 1) / p.ctas_per_problem) : 0;
+    if (MODE != kRowsBinarize) {
+        // (dependents start when every CTA has its tensor memory: one that got a CTA's columns first would wait for this grid with them)
+        griddep_launch_dependents();
+        griddep_wait();                               // x may be the output of the preceding kernel
+        if (threadIdx.x == 0) sh.skip = p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0;  // the call already failed
+        __syncthreads();                              // (one answer for all warps)
+    }
+    const int n = (MODE == kRowsBinarize || !sh.skip) && first < steps_all ? (int)((steps_all - first + p.ctas_per_problem - 1) / p.ctas_per_problem) : 0;
 
     if (warp < 4) {
     if (CH == 2) set_regs_dec<rr::kRegsControl>();
