@@ -278,6 +278,11 @@ inline bool rot_rows_geometry(int n1, int n2, int out_size, RotRowsGeom* out, in
         if (rot_rows_places(g, xb, x_terms)) { *out = g; return true; }
     return false;
 }
+// CTAs a problem gets, of as many as registers, threads and shared memory would let stay (`resident`): one an SM, because each takes all of
+// its tensor memory (384 threads, of factors with 32 columns, would fit twice).
+inline int rot_rows_ctas(int resident, int sms, int n_problems, int64_t steps) {
+    return (int)std::min<int64_t>(steps, std::min(resident, sms) / n_problems);
+}
 // once per layer: a header with the exponent of P2's scale, then both factors' terms as they lie in shared memory
 inline size_t rot_rows_prepared_bytes(const RotRowsGeom& g) { return kRotHeader + (size_t)g.x_off; }
 

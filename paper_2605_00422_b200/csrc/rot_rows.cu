@@ -810,9 +810,8 @@ static int launch_rows_kernel(RotRowsKernel k, const CUtensorMap& xm, RotRowsPar
     const int threads = rr::kControl + 128 * g.groups;
     // (a step a CTA: one x, so that blocks of the kernels before and behind find room beside these)
     if (g.xb == 2 && (p.M + g.tps - 1) / g.tps * p.n_problems + lr_blocks <= sm_count()) rot_rows_places(g, 1, 1);
-    const int room = resident_clusters((const void*)k, 1, threads, (size_t)g.total) / p.n_problems;
-    if (room < 1) return cuda_fail(cudaErrorInvalidConfiguration);
-    p.ctas_per_problem = (int)std::min<int64_t>((p.M + g.tps - 1) / g.tps, room);
+    p.ctas_per_problem = rot_rows_ctas(resident_clusters((const void*)k, 1, threads, (size_t)g.total), sm_count(), p.n_problems, (p.M + g.tps - 1) / g.tps);
+    if (p.ctas_per_problem < 1) return cuda_fail(cudaErrorInvalidConfiguration);
     cudaLaunchConfig_t cfg{};
     p.rot_ctas = p.n_problems * p.ctas_per_problem;
     cfg.gridDim = dim3((unsigned)(p.rot_ctas + lr_blocks), 1, 1);

@@ -141,3 +141,22 @@ def test_operands_of_the_rotation_with_rows_on_the_lanes_lie_inside_the_block(tm
                     }
                 }
     if (seen < 1000) std::printf("only %ld\\n", seen);""") == ""
+
+
+def test_a_rotation_that_takes_all_tensor_memory_has_one_block_an_sm(tmp_path):
+    """Whatever registers and shared memory would let stay: the problems' blocks together are no more than the SMs, every problem has one
+    and none more than it has steps."""
+    assert violations(tmp_path, """
+    for (int sms : {1, 4, 132, 148})
+        for (int per_sm = 1; per_sm <= 4; ++per_sm)
+            for (int n = 1; n <= 4; ++n)
+                for (long steps : {1L, 2L, 36L, 37L, 49L, 74L, 148L, 149L, 1000L}) {
+                    const int ctas = rot_rows_ctas(per_sm * sms, sms, n, steps);
+                    if (ctas * n > sms || ctas > steps || (n <= sms && ctas < 1)) { std::printf("%d SMs, %d an SM, %d problems, %ld steps: %d\\n", sms, per_sm, n, steps, ctas); return 0; }
+                }""") == ""
+
+
+def test_the_launch_asks_that_plan():
+    """The rows kernel's grid comes from rot_rows_ctas and from nowhere else."""
+    text = open(os.path.join(ROOT, "paper_2605_00422_b200", "csrc", "rot_rows.cu")).read()
+    assert text.count("p.ctas_per_problem = ") == 1 and "p.ctas_per_problem = rot_rows_ctas(" in text

@@ -56,6 +56,27 @@ def test_codes(n1, n2, M, asym):
     assert np.all(np.abs(out - want) <= bound)
 
 
+@pytest.mark.parametrize("n1,n2", [(40, 32), (128, 32)])
+def test_several_steps_an_sm_of_the_smallest_factors(n1, n2):
+    """Two of these blocks would fit an SM but for its tensor memory; calls behind one another, the contraction's blocks beside the rotation's."""
+    M = 2000
+    bwla, L, P1, P2, xb = _case(n1, n2, M, False)
+    dx = H.bf16_to_dev(xb)
+    codes, scales, y = bwla.bwla_layer_rotate_quant(L, dx, want_y=True)
+    Y = oracle.rotate(xb, P1, P2)
+    full = np.maximum(np.abs(Y).max(axis=1, keepdims=True), 1e-30)
+    assert float((np.abs(y.cpu().numpy().astype(np.float64) - Y) / full).max()) <= 9e-7
+    q = oracle.quantize(y.cpu().numpy().astype(np.float64), 8, "f32")
+    assert np.array_equal(q["codes"], codes.cpu().numpy()) and np.array_equal(q["scales"], scales.cpu().numpy())
+    want = bwla.bwla_w1a_gemm_codes(codes, scales, 8, L.tensors[2], L.tensors[3], mu=L.tensors[6])
+    want = want[0] if isinstance(want, tuple) else want
+    ws = torch.zeros(bwla.bwla_group_workspace_bytes([L], M), dtype=torch.uint8, device="cuda")
+    for _ in range(20):
+        out = bwla.bwla_w1ax_linear_group([L], dx, workspace=ws)[0]
+    assert bwla.bwla_check_status(ws) == 0
+    assert torch.equal(out.view(torch.int16), want.view(torch.int16))
+
+
 @pytest.mark.parametrize("n1,n2,M", [(40, 48, 297), (36, 48, 150), (64, 64, 301), (96, 80, 150), (88, 96, 149), (128, 112, 150)])
 def test_weight_only_values(n1, n2, M):
     """bf16 values in either order and their sums, through the linear, against the bf16 rounding of the exact rotation."""
