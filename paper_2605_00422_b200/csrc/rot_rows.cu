@@ -51,6 +51,7 @@ constexpr int kControl = 128;             // threads of the four control warps
 // registers with two chunks a warp: 96 a thread at launch (640 x 96 = 61440); 128 x 32 + 512 x 112 = 61440 after the split
 constexpr int kRegsControl = 32, kRegsAlu = 112;
 constexpr int kSlots = 20;                // warps of a token, at most
+constexpr int kNotFinite = 14 + 127 - 255;       // the exponent of V's scale where its largest magnitude is no number
 struct Shared {
     uint64_t fac_full;                    // the prepared factors have landed
     uint64_t x_full[2], x_empty[2];       // a step's x has landed; the MMAs that read it have completed
@@ -81,6 +82,11 @@ struct RotRowsParams {
     uint32_t* status;
 };
 
+__device__ __forceinline__ float max_nan(float a, float b) {       // (a NaN if one of them is)
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 // Where columns 2 k2, 2 k2 + 1 of row r lie in an operand of `rows` rows, 32 columns (64 bytes, swizzled) an atom.
 __host__ __device__ __forceinline__ int rot_rows_place(int rows, int r, int k2) {
     return ((k2 >> 4) * rows + r) * 64 + ((((k2 >> 2) ^ (r >> 1)) & 3) << 4) + 4 * (k2 & 3);
@@ -454,7 +460,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
 #pragma unroll
                             for (int e = 0; e < 16; e += 2) {
                                 add2(v[16 * ch + e], v[16 * ch + e + 1], __uint_as_float(u[e]), __uint_as_float(u[e + 1]));
-                                m = fmaxf(m, fmaxf(fabsf(v[16 * ch + e]), fabsf(v[16 * ch + e + 1])));
+                                m = max_nan(m, max_nan(fabsf(v[16 * ch + e]), fabsf(v[16 * ch + e + 1])));
                             }
                         }
                 }
@@ -463,7 +469,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             };
             auto convert = [&]() {
                 const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, lane < slots ? *reinterpret_cast<volatile uint32_t*>(&sh.vmax[par][tk][lane]) : 0u);
-                z_exp = max(-126, min(126, 14 + 127 - (int)(top >> 23)));
+                z_exp = max(-126, min(126, 14 + 127 - (int)(top >> 23)));      // (kNotFinite where V holds an infinity or a NaN)
                 const float scale = pow2f(z_exp);
                 if (ok) {
                     const uint32_t dst = tmem + lane_addr + (uint32_t)((i % NV) * 2 * g.n2 + c0);
@@ -556,7 +562,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (lane == 0) { sh.ymax[par][tk][slot] = top; if (MODE != kRowsSym) sh.ymin[par][tk][slot] = bottom; }
             };
             // ---- the step before: codes, scale and code sum, or bf16 values
-            auto emit = [&]() {
+            auto emit = [&](int ze) {
                 const uint32_t s0 = lane < slots ? *reinterpret_cast<volatile uint32_t*>(&sh.ymax[par][tk][lane]) : 0u;
                 const uint32_t s1 = MODE != kRowsSym && lane < slots ? *reinterpret_cast<volatile uint32_t*>(&sh.ymin[par][tk][lane]) : 0u;
                 if (ok && i >= 3 && !warp_wait(&sh.out_free[pi], (uint32_t)((((i - 1) >> 1) - 1) & 1), abort_flag)) { give_up(p.status, abort_flag, 0x534); ok = false; }
@@ -630,8 +636,18 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                         // fl(y inv) = fl(y_scaled (f inv)): f is a power of two, and where f inv leaves fp32's normal range the values are too
                         // small against the token's largest for any code but zero
                         const float f_inv = inv * f1;
+                        if (MODE == kRowsSym && (ze == rr::kNotFinite || inv > 3.402823466e38f)) {
+                            // as the other kernels have it: the code of a NaN is -1, and where the token is so small that inv overflows codes are 0
+                            // (the words below are put together by additions, which neither pattern may carry into)
 #pragma unroll
-                        for (int e = 0; e < NC; ++e) y[e] = __fmul_rn(y[e], f_inv);
+                            for (int e = 0; e < NC; ++e) {
+                                const float c0 = __fmul_rn(y[e], f_inv);
+                                y[e] = y[e] != y[e] ? -1.f : fabsf(c0) <= 128.f ? c0 : 0.f;
+                            }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < NC; ++e) y[e] = __fmul_rn(y[e], f_inv);
+                        }
 #pragma unroll
                         for (int e = 0; e < NC; e += 2) add2(y[e], y[e + 1], bias, bias);
                         if (MODE == kRowsAsym)
@@ -764,13 +780,13 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (i > 0) load_y(ze);
                 token_barrier();
                 if (i < n) convert();
-                if (i > 0) emit();
+                if (i > 0) emit(ze);
             } else {
                 if (i > 0) load_y(ze);
                 if (i < n) load_v();
                 token_barrier();
                 if (i < n) convert();
-                if (i > 0) emit();
+                if (i > 0) emit(ze);
             }
         }
         if (!ok) *abort_flag = 1;

@@ -68,8 +68,7 @@ def test_several_steps_an_sm_of_the_smallest_factors(n1, n2):
     assert float((np.abs(y.cpu().numpy().astype(np.float64) - Y) / full).max()) <= 9e-7
     q = oracle.quantize(y.cpu().numpy().astype(np.float64), 8, "f32")
     assert np.array_equal(q["codes"], codes.cpu().numpy()) and np.array_equal(q["scales"], scales.cpu().numpy())
-    want = bwla.bwla_w1a_gemm_codes(codes, scales, 8, L.tensors[2], L.tensors[3], mu=L.tensors[6])
-    want = want[0] if isinstance(want, tuple) else want
+    want = bwla.bwla_w1a_gemm_codes(codes, scales, 8, L.tensors[2], L.tensors[3], mu=L.tensors[6])[0]
     ws = torch.zeros(bwla.bwla_group_workspace_bytes([L], M), dtype=torch.uint8, device="cuda")
     for _ in range(20):
         out = bwla.bwla_w1ax_linear_group([L], dx, workspace=ws)[0]
@@ -104,6 +103,25 @@ def test_an_infinity_stays_in_its_token(n1, n2):
     c2, s2 = bwla.bwla_layer_rotate_quant(L, bad)[:2]
     keep = torch.ones(300, dtype=torch.bool); keep[[4, 9, 131]] = False
     assert torch.equal(codes.cpu()[keep], c2.cpu()[keep]) and torch.equal(scales.cpu()[keep], s2.cpu()[keep])
+
+
+@pytest.mark.parametrize("n1,n2", [(64, 64), (40, 80), (64, 128), (86, 128)])
+def test_tokens_without_numbers_have_the_codes_they_have_among_few(n1, n2):
+    """Infinities, NaNs, and a token so small that qmax / amax leaves fp32's range: the codes of the kernel for few tokens (-1 and 0), and the
+    code sums that belong to them.  qmax = 127 / amax overflows below 3.8e-37."""
+    bwla, L, P1, P2, xb = _case(n1, n2, 300, False)
+    odd = [3, 8, 131, 200, 299]
+    x = H.bf16_to_dev(xb)
+    x[3, 5], x[8, n1 * n2 - 1], x[131] = float("inf"), float("nan"), float("-inf")
+    x[200], x[299] = x[200] * 1e-39, x[299] * 0.0
+    codes, scales = bwla.bwla_layer_rotate_quant(L, x)[:2]
+    few, few_scales = bwla.bwla_layer_rotate_quant(L, x[odd].contiguous())[:2]
+    assert torch.equal(codes[odd], few)
+    assert torch.equal(scales[odd][[0, 1, 2, 4]], few_scales[[0, 1, 2, 4]])
+    assert abs(float(scales[200]) - float(few_scales[3])) <= 2e-6 * float(few_scales[3]) + 2.0 ** -148
+    out = bwla.bwla_w1ax_linear_group([L], x)[0]
+    again = bwla.bwla_w1a_gemm_codes(codes, scales, 8, L.tensors[2], L.tensors[3], mu=L.tensors[6])[0]
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
 
 
 @pytest.mark.parametrize("n1,n2,N,pad", [(33, 32, 149, 0), (40, 48, 301, 1), (64, 80, 75, 4)])
