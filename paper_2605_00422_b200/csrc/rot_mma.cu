@@ -516,8 +516,7 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             barrier();                                // Z^T is no longer needed: its place is x's again
             if (!F32 && more) { zero_padding(); fetch_x(t + stride); }
         }
-        // ---- back to true scale (exact: powers of two; a binarisation scales its sums), then what the caller wants of Y
-        if (MODE != kRotBinarize) {
+        // ---- back to true scale (exact: powers of two), then what the caller wants of Y
         const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
         const float f1 = pow2f(ey1);
 #pragma unroll
@@ -526,7 +525,6 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             const float f2 = pow2f(ey2);
 #pragma unroll
             for (int j = 0; j < NTW; ++j) { mul2(acc[j][0], acc[j][1], f2); mul2(acc[j][2], acc[j][3], f2); }
-        }
         }
         }
         float amax = 0.f, vmin = 0.f;                 // asymmetric: amax holds the largest value, zero included
@@ -739,30 +737,28 @@ __global__ void __launch_bounds__(32 * kRotMaxWarps, 1) rot_mma_kernel(const __g
             }
         } else {
             // Alg. 2, last step: the row's mean, its mean absolute deviation, and the signs about the mean
-            float hi = 0.f, lo = 0.f;
+            // (in fp64: sums in two floats, one chain of dependent additions a thread, took longer, us: 15505 rows of 32 x 32 98 for 90, 1998 of
+            // 32 x 64 27.6 for 25.3, 2348 of 86 x 128 187 for 172)
+            double s = 0.0;
 #pragma unroll
             for (int j = 0; j < NTW; ++j)             // (padding rows and columns are zeros)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) sum2(hi, lo, acc[j][i]);
-            const double mean = total_sum((double)hi + (double)lo, 0) / (double)g.K;
-            const float mean_hi = (float)mean, mean_lo = (float)(mean - (double)mean_hi);
-            float dev = 0.f, dev_lo = 0.f;
+                for (int i = 0; i < 4; ++i) s += (double)acc[j][i];
+            const double mean = total_sum(s, 0) / (double)g.K;
+            double dev = 0.0;
             uint32_t mine = 0u;                       // ballot number `lane` of the warp: column tile, row half, column parity
 #pragma unroll
             for (int j = 0; j < NTW; ++j) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float x = less2(acc[j][i], mean_hi, mean_lo, 8 * j < lim[i & 1] && (i < 2 || row_hi_ok), dev, dev_lo);
-                    const uint32_t word = __ballot_sync(0xFFFFFFFFu, x > 0.f);
+                    const double x = (double)acc[j][i] - mean;
+                    if (8 * j < lim[i & 1] && (i < 2 || row_hi_ok)) dev += fabs(x);
+                    const uint32_t word = __ballot_sync(0xFFFFFFFFu, x > 0.0);
                     if (lane == 4 * j + i) mine = word;
                 }
             }
-            const double all = total_sum((double)dev + (double)dev_lo, 1) / (double)g.K;
-            if (tid == 0 && rank == 0) {
-                const int ey = -(z_exp + e1), ey1 = max(-126, min(127, ey)), ey2 = max(-126, min(127, ey - ey1));
-                const double scale = (double)pow2f(ey1) * (double)pow2f(ey2);
-                pr.mu[t] = (float)(mean * scale); pr.alpha[t] = (float)(all * scale);
-            }
+            dev = total_sum(dev, 1) / (double)g.K;
+            if (tid == 0 && rank == 0) { pr.mu[t] = (float)mean; pr.alpha[t] = (float)dev; }
             // bit 4 r + q of a ballot is row r (of the half), column pair q: the eight rows of a column are one byte of the row
             uint8_t* bytes = reinterpret_cast<uint8_t*>(pr.packed) + t * (int64_t)(g.K >> 3);
             const int j = lane >> 2, e = lane & 1, h = (lane >> 1) & 1;
