@@ -26,6 +26,11 @@ __device__ __forceinline__ float less2(float v, float mean, float mean_lo, bool 
     }
     return d;
 }
+// (the same sum in every lane)
+__device__ __forceinline__ double warp_sum(double s) {
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    return s;
+}
 // (the whole sum in lane 0)
 __device__ __forceinline__ void warp_sum2(float& hi, float& lo) {
     for (int o = 16; o > 0; o >>= 1) {

@@ -540,13 +540,19 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     f1 = 1.f;
                 }
                 if (MODE == kRowsBf16 || MODE == kRowsBinarize) {
-                    if (MODE == kRowsBinarize || pr.ysum) {
-                        // the sum of the values (scaled; or rounded) goes where the quantiser's two extremes go
+                    // the sum of the values goes where the quantiser's two extremes go
+                    if (MODE == kRowsBinarize) {
                         float hi = 0.f, lo = 0.f;
 #pragma unroll
-                        for (int e = 0; e < NC; ++e) sum2(hi, lo, !valid ? 0.f : MODE == kRowsBinarize ? y[e] : __bfloat162float(__float2bfloat16_rn(y[e] * f1)));
+                        for (int e = 0; e < NC; ++e) sum2(hi, lo, !valid ? 0.f : y[e]);
                         warp_sum2(hi, lo);
                         top = __float_as_uint(hi); bottom = __float_as_uint(lo);
+                    } else if (pr.ysum) {
+                        double s = 0.0;
+#pragma unroll
+                        for (int e = 0; e < NC; ++e) s += (double)__bfloat162float(__float2bfloat16_rn(y[e] * f1));
+                        s = warp_sum(valid ? s : 0.0);
+                        top = (uint32_t)__double2loint(s); bottom = (uint32_t)__double2hiint(s);
                     }
                 } else {
 #pragma unroll
@@ -572,9 +578,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                     const int k0 = c * g.n2 + y0;
                     if (MODE == kRowsBf16) {
                         if (writer && pr.ysum) {
-                            // (no error of an addition that left fp32's range)
-                            double s = lane < slots ? (double)__uint_as_float(s0) + (isfinite(__uint_as_float(s0)) ? (double)__uint_as_float(s1) : 0.0) : 0.0;
-                            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                            const double s = warp_sum(__hiloint2double((int)s1, (int)s0));
                             if (lane == 0) pr.ysum[t] = (float)s;
                         }
                         // layout 1: inside each group of 32, position 2 (k % 16) + (k % 32) / 16

@@ -351,14 +351,14 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (MODE == kBf16) {
                     if (pr.ysum) {
                         // the sum of the rounded values goes where the quantiser's two extremes go
-                        float hi = 0.f, lo = 0.f;
+                        double s = 0.0;
 #pragma unroll
                         for (int j = 0; j < NC; ++j)
                             if (valid && 8 * j < have)
 #pragma unroll
-                                for (int e = 0; e < 8; ++e) sum2(hi, lo, __bfloat162float(__float2bfloat16_rn(y[8 * j + e] * f1)));
-                        warp_sum2(hi, lo);
-                        publish(__float_as_uint(__shfl_sync(0xFFFFFFFFu, hi, 0)), __float_as_uint(__shfl_sync(0xFFFFFFFFu, lo, 0)));
+                                for (int e = 0; e < 8; ++e) s += (double)__bfloat162float(__float2bfloat16_rn(y[8 * j + e] * f1));
+                        s = warp_sum(s);
+                        publish((uint32_t)__double2loint(s), (uint32_t)__double2hiint(s));
                     }
                 } else {
 #pragma unroll
@@ -474,9 +474,7 @@ rot_umma_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 if (t >= p.M) return true;
                 if (MODE == kBf16) {
                     if (writer) {
-                        // (no error of an addition that left fp32's range)
-                        double s = (double)__uint_as_float(s0) + (isfinite(__uint_as_float(s0)) ? (double)__uint_as_float(s1) : 0.0);
-                        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                        const double s = warp_sum(__hiloint2double((int)s1, (int)s0));
                         if (lane == 0) pr.ysum[t] = (float)s;
                     }
                     return true;
