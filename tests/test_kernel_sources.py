@@ -31,3 +31,12 @@ def test_dependents_start_behind_the_allocation_of_tensor_memory():
         line = body[body.rfind("\n", 0, sync) + 1:sync]
         assert line.strip() == "" and len(line) == 4, f"{path}: {name}: a barrier under a condition"
     assert seen >= 7, seen
+
+
+def test_an_edit_of_any_included_file_recompiles():
+    """Objects of two states of a header in one library would disagree on sizes and layouts."""
+    from paper_2605_00422_b200 import build
+    known = {os.path.basename(h) for h in build._headers()}
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")) + glob.glob(os.path.join(CSRC, "*.h")):
+        included = set(re.findall(r'#include "([^"]+)"', open(path).read()))
+        assert included <= known, f"{os.path.basename(path)}: {included - known}"
