@@ -180,10 +180,16 @@ inline size_t rot_prepared_bytes(const RotGeom& g) {
 // columns, and for n2 that is no multiple of 16; rot_umma.cu (160 x 160: 100 | 296 us at 150 and 1024 tokens on mma.sync, 81 | 156 here).
 // (As many tokens as the device holds at once stay on mma.sync, 1.45e-7 for every size: rot_rows.cu has 86 x 128 in 14.6 us of a call for
 // one token's 17.6, but 1.8e-7.)
+// With T = V x as blocks of the same launch (up to 64 tokens of several linears, or ranks that lowrank_umma.cu does not take) the kernel before was
+// rot_mma.cu unless okt_umma.cu took the factors, and its error is smaller beyond 80 columns or 64 rows (64 x 128: 1.44, 72 x 96: 1.49): they stay
+// there (rot_rows_exact).
 inline bool rot_mma_always(const RotGeom& g) { return g.cw == 1 && g.n2p <= 80; }
 inline bool rot_okt_factors(const RotGeom& g) {
     return !rot_mma_always(g) && g.na <= 16 && g.n2 <= 128 && (g.na > 10 || g.n2 % 16 != 0);
 }
+
+// Whether rot_rows.cu's error is no larger than that of the kernel these factors would go to otherwise.  beside: T in the same launch.
+inline bool rot_rows_exact(const RotGeom& g, bool beside) { return !beside || rot_mma_always(g) || rot_okt_factors(g); }
 
 // ---- rotation of many tokens on tcgen05 (rot_umma.cu) ----
 constexpr int kRotUmmaSharedBytes = 1792;      // its barriers and small per-CTA state
@@ -258,7 +264,8 @@ inline bool rot_rows_places(RotRowsGeom& g, int xb, int x_terms) {
 }
 // n1 in (32, 128] on the lanes; n2 a multiple of 16 up to 128: two accumulators for either contraction fill four (or six, up to 80
 // columns: two steps' V) times n2 columns of tensor memory.  A third chain of Y lies where V was, so that with one V the next step's V waits for it:
-// only for two tokens a step (108 x 128, 4096 tokens: 121 us with three chains, 117 with two, 1.73e-7 and 1.89e-7).  x_terms: 3 where rows are fp32.
+// two chains from 81 rows on, where okt_umma.cu was before (108 x 128, 4096 tokens: 121 us with three chains, 117 with two, 1.73e-7 and 1.89e-7, 2.48e-7
+// there), three below (80 x 128: 1.84e-7 with two, rot_umma.cu has 1.78e-7).  x_terms: 3 where rows are fp32.
 inline bool rot_rows_geometry(int n1, int n2, int out_size, RotRowsGeom* out, int x_terms = 1) {
     if (n2 % 16 != 0 || n2 < 32 || n2 > 128 || n1 <= 32 || n1 > 128) return false;
     RotRowsGeom g{};
@@ -266,7 +273,7 @@ inline bool rot_rows_geometry(int n1, int n2, int out_size, RotRowsGeom* out, in
     g.lanes = n1 <= 64 ? 64 : 128; g.tps = 128 / g.lanes;
     g.chunks = n2 <= 80 ? 1 : 2; g.groups = (n2 + 16 * g.chunks - 1) / (16 * g.chunks); g.nv = n2 <= 80 ? 2 : 1;
     g.ks1 = (n1 + 15) / 16; g.ks2 = n2 / 16;
-    g.y_chains = g.ks2 == 2 || (g.nv == 1 && g.lanes == 128) ? 2 : 3;
+    g.y_chains = g.ks2 == 2 || (g.nv == 1 && n1 > 80) ? 2 : 3;
     g.atoms1 = (n1 + 31) / 32; g.atoms2 = (n2 + 31) / 32;
     // Rows of a whole number of 32 outputs leave in 16-byte pieces from registers; others (half of a group of the codes' order would be
     // two bytes of every four) through shared memory.

@@ -926,7 +926,7 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
     // columns, where its error is no larger (host_plans.h; prepared, three linears with rank 64: 1 token 12.8 | 14.3, 24: 23.4 | 23.4, 50:
     // 26.1 | 24.4).
     const bool raw_few = !problems[0].prepared && M * n_problems > 3 && base.n1 <= 64 && base.n2 <= 80;
-    if (vec && (!few || raw_few) && rot_rows_supports(base, n_problems, problems)) {
+    if (vec && (!few || raw_few) && rot_rows_exact(base, any) && rot_rows_supports(base, n_problems, problems)) {
         if (any && M > 64) {
             st = own_launch(true);
             if (st != BWLA_OK) return st;

@@ -160,3 +160,20 @@ def test_the_launch_asks_that_plan():
     """The rows kernel's grid comes from rot_rows_ctas and from nowhere else."""
     text = open(os.path.join(ROOT, "paper_2605_00422_b200", "csrc", "rot_rows.cu")).read()
     assert text.count("p.ctas_per_problem = ") == 1 and "p.ctas_per_problem = rot_rows_ctas(" in text
+
+
+def test_the_rotation_with_rows_on_the_lanes_takes_no_factors_that_are_more_exact_elsewhere(tmp_path):
+    """T = V x in the same launch kept factors of up to 80 rows on the warp-level kernel unless it had more exact ones to offer: 64 x 128 1.44e-7 of a
+    row's 2-norm against 1.55e-7.  Up to 80 rows (whose other kernel is rot_umma.cu) the second contraction has three chains of sums."""
+    assert violations(tmp_path, """
+    long window = 0;
+    for (int n1 = 33; n1 <= 128; ++n1)
+        for (int n2 = 32; n2 <= 128; n2 += 16) {
+            RotGeom g{};
+            RotRowsGeom rows{};
+            if (n1 * n2 % 32 || !rot_geometry(n1, n2, &g) || !rot_rows_geometry(n1, n2, 1, &rows)) continue;
+            const bool larger = n1 <= 80 && (n1 > 64 || n2 > 80);
+            window += larger;
+            if (rot_rows_exact(g, true) == larger || !rot_rows_exact(g, false) || (n1 <= 80 && n2 > 32 && rows.y_chains != 3)) { std::printf("%d x %d\\n", n1, n2); return 0; }
+        }
+    if (window < 100) std::printf("only %ld\\n", window);""") == ""

@@ -151,3 +151,25 @@ def test_a_linear_behind_binarised_rows():
         out = bwla.bwla_w1ax_linear(x, P1, P2, 6, packed, alpha, mu=mu)
         torch.cuda.synchronize()
         assert torch.equal(out.view(torch.int16), bwla.bwla_w1ax_linear(x, P1, P2, 6, packed, alpha, mu=mu).view(torch.int16))
+
+
+@pytest.mark.parametrize("n1,n2,M,measured", [(64, 64, 800, 1.42), (64, 80, 800, 1.44), (64, 128, 800, 1.56), (72, 96, 800, 1.54), (80, 128, 800, 1.64), (86, 128, 800, 1.88),
+                                              (108, 128, 800, 1.95), (128, 128, 800, 1.95), (64, 80, 60, 1.45), (64, 128, 60, 1.45), (86, 128, 60, 1.50)])
+def test_error_of_the_present_kernels(n1, n2, M, measured):
+    """As test_error_against_64_bits of tests/test_rotation_many_gpu.py, at what the kernel for these factors and tokens has (1e-7 of a row's 2-norm;
+    seeds differ by less than 5 %)."""
+    from paper_2605_00422_b200 import bwla
+    K, errs = n1 * n2, []
+    for seed in range(6):
+        rng = np.random.default_rng([n1, n2, seed])
+        P1, P2 = H.f32_to_dev(gen.orthogonal_f32(n1, rng)), H.f32_to_dev(gen.orthogonal_f32(n2, rng))
+        x = torch.from_numpy(rng.standard_t(3, size=(M, K)).astype(np.float32)).cuda()
+        x[:, torch.from_numpy(rng.permutation(K)[:8]).cuda()] *= 50.0
+        x = x.bfloat16()
+        L = bwla.Layer(P1, P2, 6, torch.zeros((8, K // 32), dtype=torch.int32, device="cuda"), torch.ones(8, device="cuda"))
+        y = bwla.bwla_layer_rotate_quant(L, x, want_y=True)[2].double()
+        Y = (P1.double().t() @ x.double().view(M, n1, n2) @ P2.double()).reshape(M, K)
+        errs.append(float((((y - Y).norm(dim=1) / Y.norm(dim=1)) ** 2).mean()))
+    got = 1e7 * np.sqrt(np.mean(errs))
+    print(f"[{n1} x {n2}, {M} tokens] {got:.3f}")
+    assert got <= 1.05 * measured
