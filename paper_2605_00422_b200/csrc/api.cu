@@ -221,7 +221,13 @@ int bwla_w1ax_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, cons
         RotProblem pr{};
         pr.P1 = P1; pr.P2 = P2; pr.codes = codes; pr.codes_layout = path == BWLA_PATH_I8 ? 1 : 0; pr.scales = scales; pr.qsum = qsum;
         OktLowrank lr{V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status) + kLrCounterWord, (float*)codes};
-        st = launch_rot(geom, x_bf16, M, ldx, bits, 0, 1, &pr, &lr, (uint32_t*)(base + ws.status), s);
+        int behind = 0;
+        if (path == BWLA_PATH_I8 && M >= 3 && M <= sm_count()) {
+            GemmArgs g{};
+            g.M = M; g.K = K; g.N = N; g.r = r; g.bits = bits;
+            behind = M <= kSmallTokens ? gemm_small_blocks(g) : gemm_umma_sms(g);
+        }
+        st = launch_rot(geom, x_bf16, M, ldx, bits, 0, 1, &pr, &lr, (uint32_t*)(base + ws.status), s, behind);
     } else {
         st = launch_prologue(x_bf16, M, K, ldx, P1, n1, P2, n2, bits, codes, path == BWLA_PATH_I8 ? 1 : 0, scales, qsum,
                              V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status), s);

@@ -163,8 +163,9 @@ int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void*
 // asym == 0: symmetric codes in [-qmax, qmax], qmax = 2^(b-1) - 1.  asym == 1 (Sec. 4.1, per-token asymmetric): with
 // u in [0, 2^b - 1] and the integer zero point z of the token, the stored code is u - 2^(b-1) + code_bias and the
 // stored zero point z - 2^(b-1) + code_bias; a code minus the zero point times the scale is the value it stands for.
+// behind: SMs that the kernel behind it takes at once (0: not known; only asked for with raw factors and few tokens).
 int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
-               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream);
+               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream, int behind = 0);
 // The same for many tokens, on the tcgen05 tensor cores (rot_umma.cu); x in 16-byte pieces.  launch_rot goes there by itself.
 bool rot_umma_supports(const RotGeom& g, int n_problems, const RotProblem* problems);
 int launch_rot_umma(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
@@ -254,11 +255,13 @@ int launch_gemm_bitplane(const GemmArgs& a, cudaStream_t stream);
 // launch.  planes == 3: three digit planes per token (the weight-only operating point, up to kSmallDigitTokens).  *taken is false, and
 // nothing has been launched, for shapes whose codes do not fit shared memory: those go to the tcgen05 kernels.
 bool gemm_small_fits(const GemmArgs* a, int n, int planes);
+int gemm_small_blocks(const GemmArgs& a);      // of one linear's launch, one an SM; 0 where it does not fit
 int launch_gemm_small(const GemmArgs* a, int n, int planes, bool* taken, cudaStream_t stream);
 
 // tcgen05 path with the fused epilogue.  codes_interleaved: int8 [M][K] in the interleaved order.
 bool umma_supports(int64_t M, int64_t K, int64_t N, int r, int bits);
 int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream);
+int gemm_umma_sms(const GemmArgs& a);          // that its launch takes at once, or 0
 // The weight-only operating point for few tokens as three digit planes a value, a.codes int8 [3][M][K]: planes are tokens to the MMAs
 bool umma_digits_supports(int64_t M, int64_t K, int64_t N, int r);
 int launch_gemm_umma_digits(const GemmArgs& a, cudaStream_t stream);

@@ -515,6 +515,11 @@ bool gemm_small_fits(const GemmArgs* a, int n, int planes) {
     return small_plan(a, n, planes, &pl) && (planes == 1 || pl.S == 1);
 }
 
+int gemm_small_blocks(const GemmArgs& a) {
+    SmallPlan pl;
+    return small_plan(&a, 1, 1, &pl) ? pl.clusters[0] * pl.S : 0;
+}
+
 template <int NTP, int PL, bool SPLIT>
 static int launch_small_t(const SmallParams& p, int grid, int smem, cudaStream_t stream) {
     auto kernel = gemm_small_kernel<NTP, PL, SPLIT>;

@@ -701,44 +701,59 @@ static void set_umma_params(UmmaParams* p, const GemmArgs& a, int rows, int unit
     p->out = (__nv_bfloat16*)a.out; p->ldo = a.ldo; p->acc_debug = a.acc_debug; p->status = a.status; p->dep_mode = a.dep_mode;
 }
 
+struct UmmaPlan { int n_tok, row_tiles, tok_tiles, units, split; bool wide; };
+static UmmaPlan umma_plan(const GemmArgs& a, int sms) {
+    UmmaPlan u;
+    u.n_tok = a.M <= 16 ? 16 : a.M <= 32 ? 32 : 64;
+    u.row_tiles = (int)((a.N + kRowsPerCta - 1) / kRowsPerCta);
+    u.tok_tiles = (int)((a.M + u.n_tok - 1) / u.n_tok);
+    u.units = (int)((a.K + kUnitK - 1) / kUnitK);
+    // siblings that run beside one another plan for their share of the SMs
+    const int tiles = u.row_tiles * u.tok_tiles, plan_sms = a.sm_budget > 0 ? std::max(std::min(sms, a.sm_budget), tiles) : sms;
+    u.split = choose_splits(tiles, u.units, u.n_tok <= 64, plan_sms);
+    const int wide_split = u.n_tok <= 32 ? choose_wide_splits(tiles, u.units, u.split, plan_sms) : 0;
+    if (wide_split) u.split = wide_split;
+    // (64 tokens: a grid larger than the SM count would run in two waves with one CTA per SM, two smaller CTAs per SM instead)
+    u.wide = u.n_tok <= 32 ? wide_split != 0 : tiles * u.split <= sms;
+    return u;
+}
+int gemm_umma_sms(const GemmArgs& a) {
+    const int sms = sm_count();
+    if (umma_persistent_supports(a.M, a.K, a.N, a.r)) return (int)std::min<int64_t>(sms, 2 * ((a.N + 255) / 256) * ((a.M + 127) / 128));
+    if (a.M > 64 || sms <= 0) return 0;
+    const UmmaPlan u = umma_plan(a, sms);
+    const int blocks = u.row_tiles * u.tok_tiles * u.split;
+    return std::min(sms, u.wide ? blocks : (blocks + 1) / 2);
+}
+
 // codes_interleaved: int8 [M][K] in the interleaved order.  a.Thl: bf16 [3][M][64], T = hi + mid + lo.
 int launch_gemm_umma(const GemmArgs& a, const int8_t* codes_interleaved, cudaStream_t stream) {
-    const int M = (int)a.M, N = (int)a.N, K = (int)a.K;
     if (umma_persistent_supports(a.M, a.K, a.N, a.r)) {
         GemmArgs one = a;
         one.codes = codes_interleaved;
         return launch_gemm_umma_persistent(&one, 1, stream);
     }
-    if (M > 64) return BWLA_ERR_UNSUPPORTED;                  // (every such problem this path takes went to the persistent kernel)
-    const int n_tok = M <= 16 ? 16 : M <= 32 ? 32 : 64;
-    const int row_tiles = (N + kRowsPerCta - 1) / kRowsPerCta;
-    const int tok_tiles = (M + n_tok - 1) / n_tok;
-    const int units = (K + kUnitK - 1) / kUnitK;
+    if (a.M > 64) return BWLA_ERR_UNSUPPORTED;                // (every such problem this path takes went to the persistent kernel)
     const int sms = sm_count();
     if (sms <= 0) return BWLA_ERR_CUDA;
-    // siblings that run beside one another plan for their share of the SMs
-    const int plan_sms = a.sm_budget > 0 ? std::max(std::min(sms, a.sm_budget), row_tiles * tok_tiles) : sms;
-    int split = choose_splits(row_tiles * tok_tiles, units, n_tok <= 64, plan_sms);
-    const int wide_split = n_tok <= 32 ? choose_wide_splits(row_tiles * tok_tiles, units, split, plan_sms) : 0;
-    if (wide_split) split = wide_split;
+    const UmmaPlan u = umma_plan(a, sms);
 
     CUtensorMap wm, bm, tm;
-    const int st = make_umma_maps(a, codes_interleaved, M, n_tok, n_tok, &wm, &bm, &tm);
+    const int st = make_umma_maps(a, codes_interleaved, (int)a.M, u.n_tok, u.n_tok, &wm, &bm, &tm);
     if (st != BWLA_OK) return st;
 
     UmmaParams p{};
-    set_umma_params(&p, a, M, units, split);
+    set_umma_params(&p, a, (int)a.M, u.units, u.split);
 
-    dim3 grid((unsigned)row_tiles, (unsigned)tok_tiles, (unsigned)split);
-    switch (n_tok) {
+    dim3 grid((unsigned)u.row_tiles, (unsigned)u.tok_tiles, (unsigned)u.split);
+    switch (u.n_tok) {
         // (up to 16 tokens only where the codes of a K above 100 thousand do not fit gemm_small.cu's shared memory)
-        case 16: return wide_split ? launch_umma_t<16, 3, 2, 512, 2, 4>(wm, bm, tm, p, grid, stream)
-                                   : launch_umma_t<16, 3, 2, 256, 2, 2>(wm, bm, tm, p, grid, stream);
-        case 32: return wide_split ? launch_umma_t<32, 3, 2, 512, 2, 4>(wm, bm, tm, p, grid, stream)
-                                   : launch_umma_t<32, 3, 2, 256, 2, 2>(wm, bm, tm, p, grid, stream);
-        // a grid larger than the SM count would run in two waves with one CTA per SM: two smaller CTAs per SM instead
-        case 64: return grid.x * grid.y * grid.z > (unsigned)sms ? launch_umma_t<64, 2, 2, 256, 1, 2>(wm, bm, tm, p, grid, stream)
-                                                       : launch_umma_t<64, 4, 3, 512, 2, 4>(wm, bm, tm, p, grid, stream);
+        case 16: return u.wide ? launch_umma_t<16, 3, 2, 512, 2, 4>(wm, bm, tm, p, grid, stream)
+                               : launch_umma_t<16, 3, 2, 256, 2, 2>(wm, bm, tm, p, grid, stream);
+        case 32: return u.wide ? launch_umma_t<32, 3, 2, 512, 2, 4>(wm, bm, tm, p, grid, stream)
+                               : launch_umma_t<32, 3, 2, 256, 2, 2>(wm, bm, tm, p, grid, stream);
+        case 64: return u.wide ? launch_umma_t<64, 4, 3, 512, 2, 4>(wm, bm, tm, p, grid, stream)
+                               : launch_umma_t<64, 2, 2, 256, 1, 2>(wm, bm, tm, p, grid, stream);
     }
     return BWLA_ERR_UNSUPPORTED;
 }

@@ -190,6 +190,40 @@ inline bool rot_okt_factors(const RotGeom& g) {
 
 // Whether rot_rows.cu's error is no larger than that of the kernel these factors would go to otherwise.  beside: T in the same launch.
 inline bool rot_rows_exact(const RotGeom& g, bool beside) { return !beside || rot_mma_always(g) || rot_okt_factors(g); }
+// Whether it is the faster one for more tokens than rot_mma.cu has places for at once; t: tokens x linears.  A step of rot_rows.cu takes its time
+// whatever n1 and n2 are, and all SMs take a multiple of two tokens (n1 <= 64), so that it pays where the lanes are full and either the first
+// step or many steps count.  A call with it in percent of a call with the other kernel (1536 outputs, one linear, r = 0; calls repeat to 1 %):
+//     tokens          149 185 200 260 296 333 400 450 512 600 1024 2048
+//    64 x 64           91  90 100  96 100 104 100 100  96  87   89   85        rank 32      96  96  99  99  99 100  98  98  96  88   91   87
+//    64 x 64, raw      93  91  97 101 106 108  93  95  92  93   88   86        bf16 values  90  93  97  93  94  97  98  95  96  86   90   86
+//    64 x 80           96  95  97  99  99 101  97  83  84  85   81   79        rank 32      98  97  98  99 100  98  96  86  86  84   83   81
+//    64 x 80, raw      98  97  98  96  95 110  93  92  92  96   87   81        bf16 values 102 101 101 101 102 108 107  93  93 101   99   95
+//    48 x 64           99  97 108 106 108 115 107 108 104  97  100   98        48 x 80     102 102 104 105 105 112 104  95  95  96   95   93
+//    72 x 96          104 104 103  99 103  97  99 104 102  99  100  103        80 x 64     101 101 101  98 101  90  90  95  94  89   91   92
+//    64 x 96           98  98  99  96  99  91  93  93  92  90   85   83        48 x 48, 64 x 48, 64 x 32: 100 to 145 up to 600 tokens
+// (64 x 128 and more than 80 rows: 67 to 100.  With T beside, three linears of 64 x 64 and 64 tokens take 108 % of the time; without 95.)
+// t_first: T = V x in a launch of its own before.
+inline bool rot_rows_faster(const RotGeom& g, bool values, bool raw, bool beside, bool t_first, int64_t t, int sms) {
+    if (rot_mma_always(g)) {
+        if (g.n2 < 64 || g.K < 3072) return false;
+        if (values) return g.n2 % 32 == 0 ? g.K >= 4096 || t > 4 * sms : g.K >= 5120 && t > 3 * sms;
+        if (g.K < 4096) return t > (g.n2 >= 80 ? 3 : 4) * sms;
+        if (beside && g.K < 5120) return 4 * t <= 5 * sms;
+        return t_first || 2 * t > 5 * sms || 4 * t <= (raw ? 7 : 8) * sms;
+    }
+    if (g.n1 > 64 && !rot_okt_factors(g)) return (values || g.n2 <= 80) && 2 * t > 3 * (int64_t)sms;
+    return true;
+}
+// The same for t tokens that rot_mma.cu has places for (on `few_sms` SMs), raw factors.  It is the faster one by 5 to 10 % unless its blocks do not
+// find SMs beside those of the contraction behind it (`behind`), as which the call after it takes 4 to 6 us more; rot_rows.cu has half
+// as many.  us, rot_mma.cu | rot_rows.cu, 64 x 80 to 4096 outputs (128 blocks): 20 tokens 14.6 | 16.9, 25 20.2 | 16.5, 40 20.9 | 17.2, 64 22.2 | 21.3; to
+// 4700 (148 blocks): 25 tokens 21.8 | 22.4; to 8192 (64 blocks): 80 tokens 25.2 | 27.9, 100 31.4 | 27.9, 128 31.3 | 27.9.  64 x 64 to 5120, 4 tokens
+// (148 blocks): 15.5 | 13.7.  With t_first most of it is hidden up to one tile of 128 tokens (64 x 80 to 5120, 128 tokens 101 %, 140 92 %).
+inline bool rot_rows_crowded(const RotGeom& g, bool t_first, int64_t t, int few_sms, int behind, int sms) {
+    if (!rot_mma_always(g) || g.n2 < 64 || g.K < 3072 || t < 3 || behind == 0) return false;
+    if (behind + few_sms <= sms || (t_first && (g.K < 5120 || t <= 128))) return false;
+    return t <= 16 || t > 64 || (behind < sms - 2 && behind + (t + 1) / 2 <= sms + 24);
+}
 
 // ---- rotation of many tokens on tcgen05 (rot_umma.cu) ----
 constexpr int kRotUmmaSharedBytes = 1792;      // its barriers and small per-CTA state

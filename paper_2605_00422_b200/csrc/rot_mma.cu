@@ -875,7 +875,7 @@ static RotKernel rot_kernel_of(const RotGeom& g, const RotProblem& pr) {
 }
 
 int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
-               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream) {
+               const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream, int behind) {
     if (M == 0 || n_problems == 0) return BWLA_OK;
     if (n_problems > kRotMaxProblems || M >= ((int64_t)1 << 31)) return BWLA_ERR_INVALID_ARG;
     const bool vec = rot_accepts_x(x, ldx);
@@ -921,12 +921,17 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
         // left: 32 tokens of 108 x 128 in clusters of four 36 us a call, in CTAs 28)
         return t.dc == 1 || ((base.dc > 1 || 2 * M * n_problems * t.dc <= sm_count()) && M * n_problems <= resident_clusters((const void*)rot_kernel_of(t, problems[0]), t.dc, 32 * t.warps, (size_t)(t.group_off + t.group_bytes)));
     });
-    // More tokens: rot_rows.cu wherever it can (T beside it by the warp-level MMA blocks only).  It also takes a few tokens of raw factors, whose
-    // split by every CTA is shorter there (64 x 80, us a call: 1 token 12.7 | 13.9, 4: 16.8 | 16.4, 32: 21.6 | 17.4, 129: 32.2 | 28.4), up to 80
-    // columns, where its error is no larger (host_plans.h; prepared, three linears with rank 64: 1 token 12.8 | 14.3, 24: 23.4 | 23.4, 50:
-    // 26.1 | 24.4).
-    const bool raw_few = !problems[0].prepared && M * n_problems > 3 && base.n1 <= 64 && base.n2 <= 80;
-    if (vec && (!few || raw_few) && rot_rows_exact(base, any) && rot_rows_supports(base, n_problems, problems)) {
+    // rot_rows.cu where it can and is no less exact and faster (T beside it by the warp-level MMA blocks only)
+    auto rows_faster = [&]() {
+        const int sms = sm_count();
+        const bool t_first = M > 64 && lowrank && lowrank[0].r > 0;
+        if (!few) return rot_rows_faster(base, problems[0].yhat != nullptr, !problems[0].prepared, any && M <= 64, t_first, M * n_problems, sms);
+        if (problems[0].prepared || behind == 0 || M < 3 || sms < 1) return false;
+        const int at_once = resident_clusters((const void*)rot_kernel_of(g, problems[0]), g.dc, 32 * g.warps, (size_t)(g.group_off + g.group_bytes)) * g.dc;
+        const int per_sm = std::max(1, at_once / sms);
+        return rot_rows_crowded(base, t_first, M * n_problems, (int)((M * n_problems * g.dc + per_sm - 1) / per_sm), behind, sms);
+    };
+    if (vec && rot_rows_exact(base, any) && rows_faster() && rot_rows_supports(base, n_problems, problems)) {
         if (any && M > 64) {
             st = own_launch(true);
             if (st != BWLA_OK) return st;

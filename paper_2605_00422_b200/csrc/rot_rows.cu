@@ -237,6 +237,10 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         // (no dependent starts before this kernel has ended: its outputs are constants of the calls behind it, which they read before they
         // wait; this call clears its status words itself)
         if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) p.status[threadIdx.x] = 0u;
+    } else if (threadIdx.x == 0) {
+        // the call (or one before it) already failed: one answer for all warps, looked up while the factors and the tensor memory are on their way (a
+        // failure of the kernel before that comes later is not seen, and this one's work is then done for nothing)
+        sh.skip = p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0;
     }
     tc_fence_before();
     __syncthreads();
@@ -246,8 +250,6 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         // (dependents start when every CTA has its tensor memory: one that got a CTA's columns first would wait for this grid with them)
         griddep_launch_dependents();
         griddep_wait();                               // x may be the output of the preceding kernel
-        if (threadIdx.x == 0) sh.skip = p.status && *reinterpret_cast<volatile uint32_t*>(p.status) != 0;  // the call already failed
-        __syncthreads();                              // (one answer for all warps)
     }
     const int n = (MODE == kRowsBinarize || !sh.skip) && first < steps_all ? (int)((steps_all - first + p.ctas_per_problem - 1) / p.ctas_per_problem) : 0;
 

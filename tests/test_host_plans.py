@@ -177,3 +177,29 @@ def test_the_rotation_with_rows_on_the_lanes_takes_no_factors_that_are_more_exac
             if (rot_rows_exact(g, true) == larger || !rot_rows_exact(g, false) || (n1 <= 80 && n2 > 32 && rows.y_chains != 3)) { std::printf("%d x %d\\n", n1, n2); return 0; }
         }
     if (window < 100) std::printf("only %ld\\n", window);""") == ""
+
+
+def test_which_kernel_rotates(tmp_path):
+    """The rule's two sides at its lines, on 148 SMs: r(factors, values, raw, T beside, T first, tokens x linears) and c(factors, T first, tokens,
+    SMs of either kernel)."""
+    got = violations(tmp_path, """
+    auto geom = [](int n1, int n2) { RotGeom g{}; if (!rot_geometry(n1, n2, &g)) std::printf("no geometry "); return g; };
+    auto r = [&](int n1, int n2, bool values, bool raw, bool beside, bool first, long t) {
+        std::printf("%d", (int)rot_rows_faster(geom(n1, n2), values, raw, beside, first, t, 148));
+    };
+    auto c = [&](int n1, int n2, bool first, long t, int few, int behind) { std::printf("%d", (int)rot_rows_crowded(geom(n1, n2), first, t, few, behind, 148)); };
+    for (long t : {149, 259, 260, 296, 297, 370, 371}) { r(64, 64, 0, 0, 0, 0, t); r(64, 64, 0, 1, 0, 0, t); r(64, 80, 0, 0, 0, 1, t); }
+    std::printf(" ");
+    for (long t : {150, 185, 186, 256}) { r(64, 64, 0, 0, 1, 0, t); r(64, 80, 0, 0, 1, 0, t); }
+    std::printf(" ");
+    for (long t : {444, 445, 592, 593}) { r(48, 64, 0, 0, 0, 0, t); r(48, 64, 1, 0, 0, 0, t); r(48, 80, 0, 0, 0, 0, t); r(64, 80, 1, 0, 0, 0, t); }
+    std::printf(" ");
+    for (long t : {149, 4096}) { r(36, 64, 0, 0, 0, 0, t); r(64, 48, 0, 0, 0, 0, t); r(48, 80, 1, 0, 0, 0, t); r(64, 64, 1, 0, 0, 0, t); r(64, 128, 0, 1, 0, 0, t); r(128, 64, 0, 0, 0, 0, t); }
+    std::printf(" ");
+    for (long t : {149, 222, 223}) { r(80, 64, 0, 0, 0, 0, t); r(72, 96, 0, 0, 0, 0, t); r(72, 96, 1, 0, 0, 0, t); }
+    std::printf(" ");
+    c(64, 80, 0, 20, 20, 128); c(64, 80, 0, 25, 25, 128); c(64, 80, 0, 64, 64, 140); c(64, 80, 0, 64, 64, 141); c(64, 80, 0, 17, 17, 146); c(64, 80, 0, 4, 4, 144); c(64, 80, 0, 5, 5, 144);
+    std::printf(" ");
+    c(64, 64, 0, 2, 2, 148); c(64, 64, 0, 3, 3, 148); c(64, 64, 0, 50, 25, 0); c(64, 80, 1, 128, 128, 40); c(64, 80, 1, 129, 129, 40); c(64, 64, 1, 140, 70, 148);
+    c(64, 128, 0, 50, 50, 128); c(64, 48, 0, 50, 50, 128);""")
+    assert got.split() == ["111111101101001001111", "11110101", "0000001100111111", "000111000111", "000000101", "0110001", "01001000"], got
