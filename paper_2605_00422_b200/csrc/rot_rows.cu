@@ -61,7 +61,7 @@ struct Shared {
     uint64_t a_ready[2];                  // the terms of V are in tensor memory (by step parity: the ALU warps may be a step ahead)
     uint64_t out_full[2], out_free[2];    // the step's outputs and code sums are staged; have left
     uint32_t vmax[2][2][kSlots], ymax[2][2][kSlots], ymin[2][2][kSlots];       // [step parity][token][warp of the token]
-    uint32_t dev[2][2][kSlots][2];        // ... two-float sums of a binarisation
+    double dev[2][2][kSlots];             // ... sums of a binarisation's deviations
     int qsum[2][2];                       // code sums of the step's tokens
     uint32_t tmem_slot;
     int abort_flag, skip;
@@ -382,8 +382,6 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         const bool gather = MODE != kRowsBinarize && CH == 1 && (g.n2 & 31) == 0;
         const int y0 = gather ? 32 * (wc >> 1) + RUN * (wc & 1) : c0;
         auto column = [&](int e) { return y0 + (gather ? e % RUN + (32 / (16 / RUN)) * (e / RUN) : e); };
-        const double inv = MODE == kRowsBinarize ? 1.0 / (double)g.K : 0.0;
-        const float inv_hi = (float)inv, inv_lo = (float)(inv - (double)inv_hi);
         bool ok = true;
         int z_exp = 0;
         auto token_barrier = [&]() { named_barrier(1 + tk, g.groups * g.lanes); };
@@ -543,17 +541,14 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
                 }
                 if (MODE == kRowsBf16 || MODE == kRowsBinarize) {
                     // the sum of the values goes where the quantiser's two extremes go
-                    if (MODE == kRowsBinarize) {
-                        float hi = 0.f, lo = 0.f;
+                    if (MODE == kRowsBinarize || pr.ysum) {
+                        double s = 0.0, s1 = 0.0;             // (of the scaled, or the rounded values; two chains)
 #pragma unroll
-                        for (int e = 0; e < NC; ++e) sum2(hi, lo, !valid ? 0.f : y[e]);
-                        warp_sum2(hi, lo);
-                        top = __float_as_uint(hi); bottom = __float_as_uint(lo);
-                    } else if (pr.ysum) {
-                        double s = 0.0;
-#pragma unroll
-                        for (int e = 0; e < NC; ++e) s += (double)__bfloat162float(__float2bfloat16_rn(y[e] * f1));
-                        s = warp_sum(valid ? s : 0.0);
+                        for (int e = 0; e < NC; e += 2) {
+                            s += (double)(MODE == kRowsBinarize ? y[e] : __bfloat162float(__float2bfloat16_rn(y[e] * f1)));
+                            s1 += (double)(MODE == kRowsBinarize ? y[e + 1] : __bfloat162float(__float2bfloat16_rn(y[e + 1] * f1)));
+                        }
+                        s = warp_sum(valid ? s + s1 : 0.0);
                         top = (uint32_t)__double2loint(s); bottom = (uint32_t)__double2hiint(s);
                     }
                 } else {
@@ -733,33 +728,29 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
             };
             // ---- the step before, a binarisation (Alg. 2, last step): the row's mean, its mean absolute deviation, and the signs about the mean
             auto binarize = [&]() {
-                float hi = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.ymax[par][tk][lane])) : 0.f;
-                float lo = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.ymin[par][tk][lane])) : 0.f;
-                warp_sum2(hi, lo);
-                hi = __shfl_sync(0xFFFFFFFFu, hi, 0); lo = __shfl_sync(0xFFFFFFFFu, lo, 0);
-                // the mean (of the scaled values) in two floats
-                const float prod = __fmul_rn(hi, inv_hi), rest = fmaf(hi, inv_hi, -prod) + fmaf(hi, inv_lo, __fmul_rn(lo, inv_hi));
-                const float mean = __fadd_rn(prod, rest), mean_lo = __fadd_rn(__fsub_rn(prod, mean), rest);
-                float dev = 0.f, dev_lo = 0.f;
+                const uint32_t s0 = lane < slots ? *reinterpret_cast<volatile uint32_t*>(&sh.ymax[par][tk][lane]) : 0u;
+                const uint32_t s1 = lane < slots ? *reinterpret_cast<volatile uint32_t*>(&sh.ymin[par][tk][lane]) : 0u;
+                const double mean = warp_sum(__hiloint2double((int)s1, (int)s0)) / (double)g.K;          // (of the scaled values)
+                const float below = __double2float_rd(mean);                                             // (a float is above the mean where it is above this)
+                double dev = 0.0, dev1 = 0.0;
                 uint32_t bits = 0u;
 #pragma unroll
-                for (int e = 0; e < NC; ++e) {
-                    bits |= less2(y[e], mean, mean_lo, true, dev, dev_lo) > 0.f ? 1u << (e & 31) : 0u;
+                for (int e = 0; e < NC; e += 2) {
+                    bits |= (y[e] > below ? 1u << (e & 31) : 0u) | (y[e + 1] > below ? 2u << (e & 31) : 0u);
+                    dev += fabs((double)y[e] - mean);
+                    dev1 += fabs((double)y[e + 1] - mean);
                 }
                 if (ok && valid && t < p.M) {
                     reinterpret_cast<uint16_t*>(pr.packed)[(t * (int64_t)g.K + c * g.n2 + y0) >> 4] = (uint16_t)bits;
                 }
-                if (!valid) dev = dev_lo = 0.f;
-                warp_sum2(dev, dev_lo);
-                if (lane == 0) { sh.dev[par][tk][slot][0] = __float_as_uint(dev); sh.dev[par][tk][slot][1] = __float_as_uint(dev_lo); }
+                dev = warp_sum(valid ? dev + dev1 : 0.0);
+                if (lane == 0) sh.dev[par][tk][slot] = dev;
                 token_barrier();
                 if (slot == 0) {
-                    float all = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.dev[par][tk][lane][0])) : 0.f;
-                    float all_lo = lane < slots ? __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&sh.dev[par][tk][lane][1])) : 0.f;
-                    warp_sum2(all, all_lo);
+                    const double all = warp_sum(lane < slots ? *reinterpret_cast<volatile double*>(&sh.dev[par][tk][lane]) : 0.0);
                     if (lane == 0 && ok && t < p.M) {
-                        pr.mu[t] = mean * f1;
-                        pr.alpha[t] = (float)(((double)all + (double)all_lo) / (double)g.K * (double)f1);
+                        pr.mu[t] = (float)(mean * (double)f1);
+                        pr.alpha[t] = (float)(all / (double)g.K * (double)f1);
                     }
                 }
             };

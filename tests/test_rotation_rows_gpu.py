@@ -187,6 +187,53 @@ def test_binarised_rows(n1, n2, N, pad):
     _check(bwla, W, big[:, :n1 * n2], P1, P2)
 
 
+@pytest.mark.parametrize("n1,n2,N,dtype", [(64, 64, 160, torch.float32), (56, 80, 160, torch.float32), (64, 80, 160, torch.float32), (64, 64, 160, torch.bfloat16)])
+def test_sums_of_a_binarisation_hold_what_cancels(n1, n2, N, dtype):
+    """Identity factors, so that the rotated row is the row: values of 22 bits (8 as bf16) near 2^14, their negatives in the other half, and eight small
+    ones down to 2^-25 whose sum is all that is left: 50 bits (38) of one sum."""
+    from paper_2605_00422_b200 import bwla
+    K = n1 * n2
+    rng = np.random.default_rng([n1, n2])
+    unit = 2.0 ** -8 if dtype == torch.float32 else 2.0 ** 6
+    W = np.zeros((N, n1, n2))
+    W[:, : n1 // 2] = rng.integers(int(2 ** 13 / unit), int(2 ** 14 / unit), size=(N, n1 // 2, n2)) * unit
+    W[:, :8, 3] = 0.0
+    W[:, n1 // 2: 2 * (n1 // 2)] = -W[:, : n1 // 2]
+    W[:, :8, 3] = (2 * rng.integers(0, 4, size=(N, 8)) + 1) * 2.0 ** -25
+    w = torch.from_numpy(W.reshape(N, K)).to(dtype).cuda()
+    assert np.array_equal(w.cpu().double().numpy().reshape(W.shape), W)
+    packed, alpha, mu = bwla.bwla_binarize_rows(w, torch.eye(n1, device="cuda"), torch.eye(n2, device="cuda"))
+    flat = W.reshape(N, K)
+    mean = flat.sum(axis=1) / K                       # (exact: numpy's partial sums of these fit 53 bits)
+    assert np.all(np.abs(mu.cpu().numpy().astype(np.float64) - mean) <= 1e-7 * mean)
+    np.testing.assert_allclose(alpha.cpu().numpy(), np.abs(flat - mean[:, None]).mean(axis=1), rtol=1e-7)
+    assert np.array_equal(oracle.unpack_signs(packed.cpu().numpy().view(np.uint32), K) > 0, flat > mean[:, None])
+
+
+@pytest.mark.parametrize("n1,n2,dtype", [(64, 64, torch.float32), (56, 80, torch.float32), (64, 80, torch.bfloat16), (32, 64, torch.float32), (64, 128, torch.float32)])
+def test_binarised_rows_without_numbers_and_at_the_ends_of_the_range(n1, n2, dtype):
+    """Infinities and NaNs: no set bits, scale and shift NaN, and neighbours that keep theirs; a row of zeros: zeros; rows of 2^-100 and 2^100."""
+    from paper_2605_00422_b200 import bwla
+    N, K = 160, n1 * n2
+    rng = np.random.default_rng([n1, n2, 7])
+    P1, P2 = H.f32_to_dev(gen.orthogonal_f32(n1, rng)), H.f32_to_dev(gen.orthogonal_f32(n2, rng))
+    w = torch.from_numpy((rng.standard_normal((N, K)) + 0.1).astype(np.float32)).cuda()
+    w[4] *= 2.0 ** -100
+    w[5] *= 2.0 ** 100
+    w = w.to(dtype)
+    want = [t.cpu() for t in bwla.bwla_binarize_rows(w, P1, P2)[:3]]
+    w[1, 5], w[2, K - 1], w[9], w[12] = float("inf"), float("nan"), float("-inf"), 0.0
+    packed, alpha, mu = (t.cpu() for t in bwla.bwla_binarize_rows(w, P1, P2)[:3])
+    bad, keep = [1, 2, 9], [i for i in range(N) if i not in (1, 2, 9, 12)]
+    assert bool((packed[bad] == 0).all()) and bool(alpha[bad].isnan().all()) and bool(mu[bad].isnan().all())
+    assert bool((packed[12] == 0).all()) and float(alpha[12]) == 0.0 and float(mu[12]) == 0.0
+    assert all(torch.equal(a[keep], b[keep]) for a, b in zip((packed, alpha, mu), want))
+    Y = (P1.double().t() @ w[4:6].double().view(2, n1, n2) @ P2.double()).reshape(2, K).cpu()
+    mean = Y.mean(dim=1)
+    dev = (Y - mean[:, None]).abs().mean(dim=1)
+    assert bool(((alpha[4:6] - dev).abs() <= 1e-6 * dev).all()) and bool(((mu[4:6] - mean).abs() <= 1e-6 * dev).all())
+
+
 def test_a_linear_behind_binarised_rows():
     """The linear's sign words, scales and shifts are fetched before it waits for its predecessor: it must see what that has written."""
     from paper_2605_00422_b200 import bwla
