@@ -319,6 +319,14 @@ inline bool rot_rows_geometry(int n1, int n2, int out_size, RotRowsGeom* out, in
         if (rot_rows_places(g, xb, x_terms)) { *out = g; return true; }
     return false;
 }
+// Whether rows of weights are binarised there and not by rot_mma.cu: up to 80 columns (its error is smaller then), more rows than half of the SMs, and
+// factors for which a step, whose time does not depend on n1, is the shorter one.  us of 4000 to 5120 rows, rot_mma.cu | rot_rows.cu, fp32 and bf16:
+//    64 x 64  94 |  85   64 | 51      64 x 48  76 | 75   55 | 45      48 x 48  58 | 70   42 | 43      64 x 32  49 | 66   36 | 39
+//    64 x 80 187 | 128  117 | 73      56 x 64  93 | 84   64 | 51      48 x 64  91 | 99   62 | 61      36 x 64  71 | 78   50 | 49
+//    48 x 80 110 |  89   74 | 57
+inline bool rot_rows_binarizes(const RotGeom& g, bool f32, int64_t rows, int sms) {
+    return 2 * rows > sms && g.n1 <= 64 && g.n2 >= 48 && g.n2 <= 80 && (g.n1 > 48 || g.n2 >= (f32 ? 80 : 64));
+}
 // CTAs a problem gets, of as many as registers, threads and shared memory would let stay (`resident`): one an SM, because each takes all of
 // its tensor memory (384 threads, of factors with 32 columns, would fit twice).
 inline int rot_rows_ctas(int resident, int sms, int n_problems, int64_t steps) {

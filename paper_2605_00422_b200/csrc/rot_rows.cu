@@ -874,7 +874,7 @@ int launch_rows_binarize(const RotGeom& base, const void* w, int dtype, int64_t 
                          cudaStream_t stream) {
     RotRowsParams p{};
     const bool f32 = dtype == BWLA_DTYPE_F32;
-    *taken = (f32 || rot_accepts_x(w, ldw)) && (int64_t)N * 2 > sm_count() && base.n1 <= 64 && base.n2 <= 80 && rot_rows_geometry(base.n1, base.n2, 0, &p.g, f32 ? 3 : 1);
+    *taken = (f32 || rot_accepts_x(w, ldw)) && rot_rows_binarizes(base, f32, N, sm_count()) && rot_rows_geometry(base.n1, base.n2, 0, &p.g, f32 ? 3 : 1);
     if (!*taken) return BWLA_OK;
     p.M = N; p.bits = 8; p.n_problems = 1; p.prob[0] = problem; p.status = status; p.x = w; p.ldx = ldw;
     p.x_vec = (reinterpret_cast<uintptr_t>(w) & 15) == 0 && ldw % 4 == 0;

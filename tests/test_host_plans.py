@@ -203,3 +203,10 @@ def test_which_kernel_rotates(tmp_path):
     c(64, 64, 0, 2, 2, 148); c(64, 64, 0, 3, 3, 148); c(64, 64, 0, 50, 25, 0); c(64, 80, 1, 128, 128, 40); c(64, 80, 1, 129, 129, 40); c(64, 64, 1, 140, 70, 148);
     c(64, 128, 0, 50, 50, 128); c(64, 48, 0, 50, 50, 128);""")
     assert got.split() == ["111111101101001001111", "11110101", "0000001100111111", "000111000111", "000000101", "0110001", "01001000"], got
+
+
+def test_which_kernel_binarises(tmp_path):
+    got = violations(tmp_path, """
+    auto b = [](int n1, int n2, bool f32, long rows) { RotGeom g{}; rot_geometry(n1, n2, &g); std::printf("%d", (int)rot_rows_binarizes(g, f32, rows, 148)); };
+    for (int f32 = 0; f32 < 2; ++f32) { b(64, 64, f32, 74); b(64, 64, f32, 75); b(48, 64, f32, 4000); b(48, 80, f32, 4000); b(56, 48, f32, 4000); b(48, 48, f32, 4000); b(64, 32, f32, 4000); b(64, 128, f32, 4000); std::printf(" "); }""")
+    assert got.split() == ["01111000", "01011000"], got
