@@ -215,12 +215,14 @@ int bwla_w1ax_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, cons
     const int path = resolve_path(M, K, N, r, bits);
 
     RotGeom geom;
+    int rot_cluster = 0;
     if (g_forced_rotation != BWLA_ROT_SIMT && rot_geometry(n1, n2, &geom)) {
         // the Kronecker factors are handed over raw: every CTA of the rotation splits what it needs of them (a prepared
         // layer has that done once)
         RotProblem pr{};
         pr.P1 = P1; pr.P2 = P2; pr.codes = codes; pr.codes_layout = path == BWLA_PATH_I8 ? 1 : 0; pr.scales = scales; pr.qsum = qsum;
         OktLowrank lr{V_bf16, r, Thl, r > 0 ? (float*)(base + ws.lr_part) : nullptr, (uint32_t*)(base + ws.status) + kLrCounterWord, (float*)codes};
+        if (path == BWLA_PATH_I8 && M <= 2) rot_cluster = rot_few_cluster(geom, M, 1, &pr);
         int behind = 0;
         if (path == BWLA_PATH_I8 && M >= 3 && M <= sm_count()) {
             GemmArgs g{};
@@ -236,7 +238,7 @@ int bwla_w1ax_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, cons
     GemmArgs g{};
     g.scales = scales; g.qsum = qsum; g.M = M; g.K = K; g.N = N; g.bits = bits; g.packed = packed; g.alpha = alpha;
     g.mu = mu; g.Thl = r > 0 ? Thl : nullptr; g.U = U_bf16; g.r = r; g.out = out_bf16; g.ldo = ldo; g.acc_debug = nullptr;
-    g.status = (uint32_t*)(base + ws.status);
+    g.status = (uint32_t*)(base + ws.status); g.rot_cluster = rot_cluster;
     return run_contraction(path, g, codes, s);
 }
 
@@ -506,6 +508,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
     const bool rot = L0->rot && g_forced_rotation != BWLA_ROT_SIMT;      // (the layers share n1 and n2)
     // the asymmetric quantiser lives in the tensor-core rotation
     if (L0->asym && (!rot || !rot_accepts_x(x_bf16, ldx))) return BWLA_ERR_UNSUPPORTED;
+    int rot_cluster = 0;
     if (rot) {
         RotProblem pr[kRotMaxProblems];
         OktLowrank lr[kRotMaxProblems];
@@ -520,6 +523,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         }
         st = launch_rot(L0->geom, x_bf16, M, ldx, L0->bits, L0->asym, count, pr, lr, status, s);
         if (st != BWLA_OK) return st;
+        if (M <= 2) rot_cluster = rot_few_cluster(L0->geom, M, count, pr);
     } else {
         for (int i = 0; i < count; ++i) {
             const bwla_layer* L = layers[i];
@@ -539,7 +543,7 @@ int bwla_w1ax_linear_group(const bwla_layer* const* layers, int count, const voi
         g.codes = (int8_t*)(wbase[i] + ws[i].codes);
         g.scales = (float*)(wbase[i] + ws[i].scales); g.qsum = (int32_t*)(wbase[i] + ws[i].qsum);
         g.M = M; g.K = L->K; g.N = L->N; g.bits = L->bits; g.packed = L->packed; g.alpha = L->alpha; g.mu = L->mu;
-        g.zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr; g.rowsum = L->rowsum;
+        g.zp = L->asym ? (int32_t*)(wbase[i] + ws[i].zp) : nullptr; g.rowsum = L->rowsum; g.rot_cluster = rot_cluster;
         g.Thl = L->r > 0 ? wbase[i] + ws[i].T : nullptr; g.U = L->U; g.r = L->r; g.out = outs[i]; g.ldo = ldos[i];
         g.status = status;
         all_i8 = all_i8 && path[i] == BWLA_PATH_I8;

@@ -167,6 +167,7 @@ int launch_prepare_rot(const RotGeom& g, const float* P1, const float* P2, void*
 int launch_rot(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream, int behind = 0);
 // The same for many tokens, on the tcgen05 tensor cores (rot_umma.cu); x in 16-byte pieces.  launch_rot goes there by itself.
+int rot_few_cluster(const RotGeom& g, int64_t M, int n_problems, const RotProblem* problems);      // CTAs of a cluster where it takes few tokens in clusters, or 1
 bool rot_umma_supports(const RotGeom& g, int n_problems, const RotProblem* problems);
 int launch_rot_umma(const RotGeom& g, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                     const RotProblem* problems, uint32_t* status, cudaStream_t stream);
@@ -229,6 +230,7 @@ struct GemmArgs {
     // kDepChain: the ordinary chain (wait for the predecessor before reading its results).
     int dep_mode;
     int sm_budget;            // SMs this launch should plan for (0: all): siblings share the device
+    int rot_cluster;          // CTAs of a cluster of the rotation before (few tokens; 0: not known, or no clusters)
 };
 enum { kDepChain = 0, kDepHead = 1, kDepSibling = 2 };
 

@@ -422,7 +422,7 @@ static int resident_small_clusters(int S) {
 // Picks S by an estimate of cycles: the items of the longest run chain at the measured rate of the loop (32 and 52 cycles per
 // 128 k, row group and scheduler-quarter at 8 and 16 tokens), a round of barriers and epilogue per run, filling the CTA's codes from
 // the L2, and the cluster's barriers.
-static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int n, bool lowrank, int sms, int spare, SmallPlan* best) {
+static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int n, bool lowrank, int sms, int spare, int room, SmallPlan* best) {
     using namespace small_;
     const int NT = NTP * PL, tok = 8 * NT;
     double best_cost = 0.0;
@@ -438,9 +438,7 @@ static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int 
         const int group_bytes = 2 * NT * 512;
         const int fit = (kSmemMax - off) / group_bytes;
         if (fit < 1) continue;
-        // Clusters the device holds.  Those that a rotation's cluster leaves no room would start, and fetch their constants, when it has ended: two
-        // are left out (a decode block of one token, 160 x 160 before the down projection: 83.1 us with all, 81.0 less one, 80.8 less two).
-        const int total = std::min((sms - spare) / S, S == 1 ? sms : resident_small_clusters(S) - (spare > 0 && PL == 1 ? 2 : 0));
+        const int total = std::min((sms - spare) / S, S == 1 ? sms : resident_small_clusters(S) - room);      // clusters the device holds
         if (total < n) break;
         int groups[kRotMaxProblems], used = 0, longest = 1;
         int64_t all = 0;
@@ -478,7 +476,7 @@ static bool small_plan_search(int NTP, int PL, int units, const int64_t* N, int 
 // The plans of the shapes a thread has called lately: a decode loop asks for the same few on every step.
 static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     using namespace small_;
-    struct Key { int dev, NTP, PL, units, n, lowrank, spare; int64_t N[kRotMaxProblems]; };
+    struct Key { int dev, NTP, PL, units, n, lowrank, spare, room; int64_t N[kRotMaxProblems]; };
     struct Known { Key k; bool ok; SmallPlan plan; };
     static thread_local Known known[16];
     static thread_local int used = 0;
@@ -495,8 +493,12 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     // With very few tokens the rotation kernels before and after have a handful of CTAs: a few SMs are left to them, so that this
     // kernel starts whole while the one before still runs, and the next one's constants arrive under this one.
     k.spare = M <= 2 ? 8 : 0;
+    // Clusters of this kernel that a rotation in clusters leaves no room would start, and fetch their constants, when it has ended: two are left out
+    // (one token, 160 x 160 to 1024 and 12288 outputs, raw: 26.5 -> 19.0 us, 42.1 -> 32.2; 108 x 128 to 5120: 23.5 -> 21.5; a rotation in single CTAs needs
+    // none, 86 x 128 to 5120: 20.3 us, 21.3 with two left out).
+    k.room = k.spare > 0 && planes == 1 && a[0].rot_cluster > 1 ? 2 : 0;
     auto same = [&](const Key& o) {
-        return o.dev == k.dev && o.NTP == k.NTP && o.PL == k.PL && o.units == k.units && o.n == k.n && o.lowrank == k.lowrank && o.spare == k.spare &&
+        return o.dev == k.dev && o.NTP == k.NTP && o.PL == k.PL && o.units == k.units && o.n == k.n && o.lowrank == k.lowrank && o.spare == k.spare && o.room == k.room &&
                std::equal(k.N, k.N + kRotMaxProblems, o.N);
     };
     for (int i = 0; i < 16 && i < used; ++i)
@@ -504,7 +506,7 @@ static bool small_plan(const GemmArgs* a, int n, int planes, SmallPlan* out) {
     const int sms = sm_count();
     Known& slot = known[used % 16];
     slot.k = k;
-    slot.ok = sms > 0 && small_plan_search(k.NTP, k.PL, k.units, k.N, n, k.lowrank != 0, sms, k.spare, &slot.plan);
+    slot.ok = sms > 0 && small_plan_search(k.NTP, k.PL, k.units, k.N, n, k.lowrank != 0, sms, k.spare, k.room, &slot.plan);
     ++used;
     *out = slot.plan;
     return slot.ok;

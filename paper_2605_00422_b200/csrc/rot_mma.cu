@@ -874,6 +874,19 @@ static RotKernel rot_kernel_of(const RotGeom& g, const RotProblem& pr) {
     return pr.yhat ? pick_kernel<kRotBf16, false>(g) : pr.digits ? pick_kernel<kRotDigits, false>(g) : pick_kernel<kRotQuant, false>(g);
 }
 
+// Whether the device holds a cluster for every token at once, and the geometry that is spread for the time of one token.
+static bool few_geometry(const RotGeom& base, int64_t M, int n_problems, const RotProblem* problems, RotGeom* g) {
+    return M * n_problems <= sm_count() && few_tokens_geometry(base, !problems[0].prepared, g, [&](const RotGeom& t) {
+        // (behind another kernel a cluster finds its place later than single CTAs do, where these are possible half of the SMs must be
+        // left: 32 tokens of 108 x 128 in clusters of four 36 us a call, in CTAs 28)
+        return t.dc == 1 || ((base.dc > 1 || 2 * M * n_problems * t.dc <= sm_count()) && M * n_problems <= resident_clusters((const void*)rot_kernel_of(t, problems[0]), t.dc, 32 * t.warps, (size_t)(t.group_off + t.group_bytes)));
+    });
+}
+int rot_few_cluster(const RotGeom& base, int64_t M, int n_problems, const RotProblem* problems) {
+    RotGeom g = base;
+    return few_geometry(base, M, n_problems, problems, &g) ? g.dc : 1;
+}
+
 int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int bits, int asym, int n_problems,
                const RotProblem* problems, const OktLowrank* lowrank, uint32_t* status, cudaStream_t stream, int behind) {
     if (M == 0 || n_problems == 0) return BWLA_OK;
@@ -916,11 +929,7 @@ int launch_rot(const RotGeom& base, const void* x, int64_t M, int64_t ldx, int b
     if (st != BWLA_OK) return st;
     // ---- the kernel: while the device holds a cluster for every token, mma.sync, spread for the time of one token ----
     RotGeom g = base;
-    const bool few = M * n_problems <= sm_count() && few_tokens_geometry(base, !problems[0].prepared, &g, [&](const RotGeom& t) {
-        // (behind another kernel a cluster finds its place later than single CTAs do, where these are possible half of the SMs must be
-        // left: 32 tokens of 108 x 128 in clusters of four 36 us a call, in CTAs 28)
-        return t.dc == 1 || ((base.dc > 1 || 2 * M * n_problems * t.dc <= sm_count()) && M * n_problems <= resident_clusters((const void*)rot_kernel_of(t, problems[0]), t.dc, 32 * t.warps, (size_t)(t.group_off + t.group_bytes)));
-    });
+    const bool few = few_geometry(base, M, n_problems, problems, &g);
     // rot_rows.cu where it can and is no less exact and faster (T beside it by the warp-level MMA blocks only)
     auto rows_faster = [&]() {
         const int sms = sm_count();
