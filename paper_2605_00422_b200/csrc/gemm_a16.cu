@@ -6,7 +6,7 @@
 //   out[t][n] = bf16( alpha[n] * sum_k s[n][k] * yhat[t][k] + U[n,:] . T[t,:] + mu[n] * sum_k yhat[t][k] )
 //
 // This kernel serves K that is not a multiple of 128 (and more than 32 tokens); gemm_a16_persist.cu and the digits of gemm_small.cu
-// serve the rest.
+// (up to 4 tokens) and gemm_umma.cu (up to 32) serve the rest.
 //
 // Tile of one CTA: 128 tokens (the accumulator's lanes) x 128 weight rows (its columns) x all of K.
 //   A operand: yhat, K-major, by TMA (64 values of k = one 128-byte swizzle atom per stage);

@@ -4,8 +4,8 @@
 //
 // A pair (cta_group::2, clusters of two) is one tensor core to the MMAs: each CTA holds 128 of the rows, in its own tensor memory, and
 // half of the tokens' codes, in its own shared memory.  One CTA alone needs 16 KB of codes for the 256 cycles of a k-block's MMAs, 64
-// bytes a cycle and SM, which is what the L2 delivers; a CTA of a pair needs half of that.  4096 tokens of 25600 -> 5120: 469 us before,
-// 394 now (2730 TOP/s, about what the power limit leaves: twice the sustained bf16 rate of cuBLAS).
+// bytes a cycle and SM, which is what the L2 delivers; a CTA of a pair needs half of that.  4096 tokens of 25600 -> 5120: 469 us in single
+// CTAs, 394 in pairs (2730 TOP/s, about what the power limit leaves: twice the sustained bf16 rate of cuBLAS).
 //
 // One CTA per tile pays its set-up (barriers, tensor memory, the first loads from HBM) and its epilogue (read-back,
 // scaling, 32 KB of output) with the tensor core idle: at 128 tokens that was more than the tile's K loop.  Here the

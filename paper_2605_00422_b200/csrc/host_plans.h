@@ -52,7 +52,10 @@ inline size_t lowrank_split_bytes(int64_t M, int lr_cols) {
 // ---- T = V x for many tokens on tcgen05 (lowrank_umma.cu) ----
 constexpr int kLruTok = 128, kLruCols = 64, kLruBlockK = 64;        // tokens and columns of a tile, values of k per stage
 constexpr int kLruMaxParts = 16;         // parts of K per token tile
-constexpr int kLruClusterParts = 8;      // ... that a cluster adds up in shared memory; more (a second kernel adds them) only for a K above
+// Up to eight are added up in a cluster's shared memory; more, which a second kernel adds, only for a K above kLruClusterK: a call of 129 | 333
+// tokens, rank 64, 5120 outputs, us, eight in a cluster and up to sixteen apart: K = 8192 40.2, 40.8 | 44.6, 45.4; 11008 49.5, 49.9 | 54.4, 53.7; 12288 50.6, 50.7 |
+// 57.7, 56.3; 13824 58.2, 57.3 | 61.9, 59.7; 25600 94.3, 90.0 | 118.3, 113.4 (1024 tokens: 108.8, 110.6 at 11008, 126.2, 127.0 at 13824, 262, 259 at 25600).
+constexpr int kLruClusterParts = 8;
 constexpr int kLruClusterK = 12288;
 constexpr int kLruTargetCtas = 160;      // parts are chosen so that tiles x parts comes near this, every part at least eight stages long
 inline int64_t lowrank_umma_tiles(int64_t M) { return (M + kLruTok - 1) / kLruTok; }

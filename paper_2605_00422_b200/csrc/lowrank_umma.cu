@@ -13,7 +13,7 @@
 // tiles than SMs, K is split into parts.  Up to eight parts are a cluster: they leave their sums in their own shared memory, and each
 // adds its share of the columns over all of them, in the order of the parts, and splits it into the three terms.  (Through the workspace and
 // a second kernel, which more parts of a large K still take, four more microseconds stood before the rotation: a block of 333 tokens 205 us,
-// 199 now.)  Warp 0 copies (TMA: 64 values of k of the x tile and of V per stage), warp 1 issues the MMAs (all lanes in step), warps
+// 199 with clusters.)  Warp 0 copies (TMA: 64 values of k of the x tile and of V per stage), warp 1 issues the MMAs (all lanes in step), warps
 // 2..5 are the epilogue, one per quarter of the accumulator's lanes.  Every wait is bounded.
 #include <cuda_bf16.h>
 

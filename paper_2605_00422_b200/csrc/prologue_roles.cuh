@@ -14,7 +14,7 @@ namespace bwla {
 
 using namespace ptx;
 
-constexpr int kLrMaxWarps = 16;   // blocks have at most 512 threads
+constexpr int kLrMaxWarps = 16;   // of the blocks that plan with it (512 threads); rot_rows.cu runs lowrank_mma_role with up to 24
 
 struct PrologueParams {
     const __nv_bfloat16* x; int64_t M; int K; int64_t ldx;

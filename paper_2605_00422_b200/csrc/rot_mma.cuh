@@ -8,38 +8,11 @@
 
 namespace bwla {
 
-// Sums in two floats, hi + lo, each addition's rounding error (Knuth's TwoSum) kept in lo: 2^-47 of the sum.  (fp64 additions and conversions run at
-// a few a cycle and SM: with them the binarisation of a step took 12600 of 17000 cycles.)
-__device__ __forceinline__ void sum2(float& hi, float& lo, float v) {
-    const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
-    hi = s;
-}
-// v less a mean of two floats, with the errors of both subtractions; its magnitude is added to hi + lo where `counts`.
-__device__ __forceinline__ float less2(float v, float mean, float mean_lo, bool counts, float& hi, float& lo) {
-    const float s = __fsub_rn(v, mean), b = __fsub_rn(s, v);
-    const float err = __fsub_rn(__fsub_rn(__fsub_rn(v, __fsub_rn(s, b)), __fadd_rn(mean, b)), mean_lo);
-    const float d = __fadd_rn(s, err), left = __fadd_rn(__fsub_rn(s, d), err);
-    if (counts) {
-        sum2(hi, lo, fabsf(d));
-        lo = __fadd_rn(lo, d < 0.f ? -left : left);
-    }
-    return d;
-}
 // (the same sum in every lane)
 __device__ __forceinline__ double warp_sum(double s) {
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     return s;
 }
-// (the whole sum in lane 0)
-__device__ __forceinline__ void warp_sum2(float& hi, float& lo) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h = __shfl_xor_sync(0xFFFFFFFFu, hi, o), l = __shfl_xor_sync(0xFFFFFFFFu, lo, o);
-        sum2(hi, lo, h);
-        lo = __fadd_rn(lo, l);
-    }
-}
-
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));

@@ -12,8 +12,8 @@
 //   second: A = two fp16 terms of V in tensor memory, B = two fp16 terms of P2^T; three products
 // Small products first.  V is scaled by a power of two of the token (its largest magnitude goes to [2^14, 2^15)), which leaves exactly
 // with the scale of P2.  The tensor core truncates when it adds to its accumulator, so the first contraction is summed in two chains and the
-// second in three (two beyond 64 x 80 of one token: host_plans.h), in accumulators of their own, and added with rounded additions.  (With two for
-// the second 64 x 80 had 1.56e-7 of a row's 2-norm and 64 x 128 1.74e-7; 1.47e-7 and 1.64e-7 on the kernels that this one replaced.)
+// second in three (two for more than 80 rows and columns: host_plans.h), in accumulators of their own, and added with rounded additions.  (With two
+// for the second 64 x 80 has 1.56e-7 of a row's 2-norm and 64 x 128 1.74e-7; with three 1.44e-7 and 1.55e-7.)
 //
 // The terms of V take the place of the first of its accumulators (a warp writes the lanes and columns that it has read), the third chain of
 // Y that of the second.  Up to 80 columns there is a second pair for the next step's V; the MMAs then run a step ahead and are never waited for:
@@ -23,11 +23,11 @@
 // With more columns Y(i-1) is read first and quantised under the MMAs of Y(i) and V(i+1).
 //
 // Bounds: up to 80 columns the ALU warps' instructions (a step of two tokens of 64 x 64 4000 cycles, 1000 of them MMAs); beyond, the chain V, exchange
-// and terms, Y of a token (86 x 128: 6200 cycles, 3100 of them MMAs).  4096 tokens of 64 x 80 86 us before (mma.sync, whose MMAs take eight
-// times as long), 50 now; of 86 x 128 137 and 113.  An MMA of 51 cycles took 110 to issue from run-time loops of one elected thread.
+// and terms, Y of a token (86 x 128: 6200 cycles, 3100 of them MMAs).  4096 tokens of 64 x 80 50 us (rot_mma.cu, whose MMAs take eight
+// times as long, 86); of 86 x 128 113 (okt_umma.cu 137).  An MMA of 51 cycles took 110 to issue from run-time loops of one elected thread.
 //
 // Up to 64 x 80, fp32 rows of weights are split into three bf16 terms by the ALU warps, the next step's behind this step's V, and make six products with
-// P1's; mean and mean absolute deviation are summed in two floats, and a lane's signs are neighbouring bits.
+// P1's; mean and mean absolute deviation are summed in fp64, and a lane's signs are neighbouring bits.
 //
 // Launched with programmatic stream serialisation: the factors are fetched before the preceding kernel of the stream has finished; x is
 // read, and everything is stored, after it.  Every wait on an mbarrier is bounded (umma_wait.cuh); a warp whose wait ran out goes on
@@ -111,7 +111,7 @@ int launch_prepare_rows(const RotRowsGeom& g, const float* P1, const float* P2, 
     return after_launch();
 }
 
-// Steps of 16 values of the contractions: the first has two chains of sums, the second three (two where it has two steps).
+// Steps of 16 values of the contractions: the first has two chains of sums, the second two or three (RotRowsGeom::y_chains).
 __host__ __device__ constexpr int chain_end(int ks, int chains, int h) { return (ks * (h + 1) + chains - 1) / chains; }
 
 // The MMAs of one product of the first contraction (one term of P1^T, one of x) into chain H, KS steps of 16 in all.  Unrolled: the issuing
@@ -387,7 +387,7 @@ rot_rows_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant
         auto token_barrier = [&]() { named_barrier(1 + tk, g.groups * g.lanes); };
         // ---- fp32 rows: eight values of step `i` to the three terms in x's place (rows beyond n1 and M are zeros)
         const int cpr = g.n2 >> 3, alu_threads = 32 * alu_warps;
-        // (the L2 is asked for a step's rows three steps before it: 5120 x 5120 143 us without, 129 with; the first pass over new pages 255 and 194)
+        // (the L2 is asked for a step's rows three steps before it: 5120 x 5120 143 us without, 129 with (sums in two floats); the first pass over new pages 255 and 194)
         auto ask_x = [&](int i) {
             if (!F32 || !p.x_vec || threadIdx.x != rr::kControl || i >= n) return;
             const int64_t t = (first + (int64_t)i * p.ctas_per_problem) * g.tps;
