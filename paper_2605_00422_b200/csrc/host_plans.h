@@ -208,7 +208,7 @@ inline bool rot_rows_exact(const RotGeom& g, bool beside) { return !beside || ro
 // t_first: T = V x in a launch of its own before.
 inline bool rot_rows_faster(const RotGeom& g, bool values, bool raw, bool beside, bool t_first, int64_t t, int sms) {
     if (rot_mma_always(g)) {
-        if (g.n2 < 64 || g.K < 3072) return false;
+        if (g.n1 < 48 || g.n2 < 64) return false;          // (36 x 80 has 1.45e-7 here and 1.44e-7 on rot_mma.cu)
         if (values) return g.n2 % 32 == 0 ? g.K >= 4096 || t > 4 * sms : g.K >= 5120 && t > 3 * sms;
         if (g.K < 4096) return t > (g.n2 >= 80 ? 3 : 4) * sms;
         if (beside && g.K < 5120) return 4 * t <= 5 * sms;
@@ -223,7 +223,7 @@ inline bool rot_rows_faster(const RotGeom& g, bool values, bool raw, bool beside
 // 4700 (148 blocks): 25 tokens 21.8 | 22.4; to 8192 (64 blocks): 80 tokens 25.2 | 27.9, 100 31.4 | 27.9, 128 31.3 | 27.9.  64 x 64 to 5120, 4 tokens
 // (148 blocks): 15.5 | 13.7.  With t_first most of it is hidden up to one tile of 128 tokens (64 x 80 to 5120, 128 tokens 101 %, 140 92 %).
 inline bool rot_rows_crowded(const RotGeom& g, bool t_first, int64_t t, int few_sms, int behind, int sms) {
-    if (!rot_mma_always(g) || g.n2 < 64 || g.K < 3072 || t < 3 || behind == 0) return false;
+    if (!rot_mma_always(g) || g.n1 < 48 || g.n2 < 64 || t < 3 || behind == 0) return false;
     if (behind + few_sms <= sms || (t_first && (g.K < 5120 || t <= 128))) return false;
     return t <= 16 || t > 64 || (behind < sms - 2 && behind + (t + 1) / 2 <= sms + 24);
 }
@@ -301,8 +301,8 @@ inline bool rot_rows_places(RotRowsGeom& g, int xb, int x_terms) {
 }
 // n1 in (32, 128] on the lanes; n2 a multiple of 16 up to 128: two accumulators for either contraction fill four (or six, up to 80
 // columns: two steps' V) times n2 columns of tensor memory.  A third chain of Y lies where V was, so that with one V the next step's V waits for it:
-// two chains from 81 rows on, where okt_umma.cu was before (108 x 128, 4096 tokens: 121 us with three chains, 117 with two, 1.73e-7 and 1.89e-7, 2.48e-7
-// there), three below (80 x 128: 1.84e-7 with two, rot_umma.cu has 1.78e-7).  x_terms: 3 where rows are fp32.
+// two chains for codes from 81 rows on, where okt_umma.cu was before (108 x 128, 4096 tokens: 121 us with three chains, 117 with two, 1.73e-7 and
+// 1.89e-7, 2.48e-7 there), three where rot_umma.cu was: bf16 values, whose error was 1.87e-7 there, and fewer rows (80 x 128: 1.84e-7 with two, 1.78e-7).  x_terms: 3 where rows are fp32.
 inline bool rot_rows_geometry(int n1, int n2, int out_size, RotRowsGeom* out, int x_terms = 1) {
     if (n2 % 16 != 0 || n2 < 32 || n2 > 128 || n1 <= 32 || n1 > 128) return false;
     RotRowsGeom g{};
@@ -310,7 +310,7 @@ inline bool rot_rows_geometry(int n1, int n2, int out_size, RotRowsGeom* out, in
     g.lanes = n1 <= 64 ? 64 : 128; g.tps = 128 / g.lanes;
     g.chunks = n2 <= 80 ? 1 : 2; g.groups = (n2 + 16 * g.chunks - 1) / (16 * g.chunks); g.nv = n2 <= 80 ? 2 : 1;
     g.ks1 = (n1 + 15) / 16; g.ks2 = n2 / 16;
-    g.y_chains = g.ks2 == 2 || (g.nv == 1 && n1 > 80) ? 2 : 3;
+    g.y_chains = g.ks2 == 2 || (g.nv == 1 && n1 > 80 && out_size == 1) ? 2 : 3;
     g.atoms1 = (n1 + 31) / 32; g.atoms2 = (n2 + 31) / 32;
     // Rows of a whole number of 32 outputs leave in 16-byte pieces from registers; others (half of a group of the codes' order would be
     // two bytes of every four) through shared memory.
