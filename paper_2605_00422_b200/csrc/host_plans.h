@@ -170,7 +170,7 @@ inline size_t rot_prepared_bytes(const RotGeom& g) {
 
 // ---- which kernel rotates many tokens (more than the device holds clusters for) ----
 // The kernel alone, us at 150, 1024 and 4096 tokens of one linear, and the error of 300 tokens against 64 bits in 1e-7 of a row's 2-norm:
-//                before                             rot_rows.cu
+//                the other kernel                   rot_rows.cu
 //    48 x  64    13    21    46   1.35   rot_mma    13    19    41   1.34
 //    64 x  64    15    25    58   1.40   rot_mma    13    19    42   1.38
 //    64 x  80    17    33    86   1.43   rot_mma    13    21    50   1.40
@@ -178,7 +178,7 @@ inline size_t rot_prepared_bytes(const RotGeom& g) {
 //    86 x 128    21    44   137   2.45   okt_umma   17    36   113   1.83
 //   108 x 128    23    52   166   2.48   okt_umma   17    38   117   1.89
 //   128 x 128    23    50   162   2.64   okt_umma   19    39   124   1.9
-// rot_rows.cu wherever it can (n1 in (32, 128], n2 a multiple of 16 up to 128).  For the rest: mma.sync where one warp holds all columns of
+// rot_rows.cu where it can (n1 in (32, 128], n2 a multiple of 16 up to 128) and is the faster one (rot_rows_faster).  For the rest: mma.sync where one warp holds all columns of
 // a token and a CTA several tokens; okt_umma.cu for 81 to 128 columns, where a step of rot_umma.cu would hold one token in half of its
 // columns, and for n2 that is no multiple of 16; rot_umma.cu (160 x 160: 100 | 296 us at 150 and 1024 tokens on mma.sync, 81 | 156 here).
 // (As many tokens as the device holds at once stay on mma.sync, 1.45e-7 for every size: rot_rows.cu has 86 x 128 in 14.6 us of a call for
